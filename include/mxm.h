@@ -136,14 +136,18 @@ mxm_status mxm_gemm(int mode, const double* A, const double* B, double* C, int64
  *   raster    C tiles are walked by the persistent grid in groups of
  *             `raster` tile-rows (tile-row pairs on CTA pairs), column by
  *             column inside a group, so that the CTAs working at the same
- *             time share operand tiles in L2; 0: 8 (4 tile-row pairs).
+ *             time share operand tiles in L2; 0: 8 (4 tile-row pairs, 8 for
+ *             256 x 256 C tiles).
  *   kb_order  the k-block order of the slice GEMM: 0 the default (2), 1
  *             every diagonal (pair) walks k forwards, 2 every other one
  *             walks k backwards (it starts on the tiles the previous one
  *             read last, still in L2).
- *   cta       the slice GEMM on bf16 digits: 0 the rule (CTA pairs,
- *             cta_group::2 with 256 x 128 C tiles, for two or more tile-rows
- *             of A without split-k), 1 single CTAs (128 x 128 C tiles).
+ *   cta       the slice GEMM on bf16 digits: 0 the rule (difference
+ *             products on CTA pairs, cta_group::2 with 256 x 256 C tiles, where
+ *             they apply and their workspace can be had; else CTA pairs with
+ *             256 x 128 C tiles for two or more tile-rows of A without
+ *             split-k), 1 single CTAs (128 x 128 C tiles), the digit products
+ *             one by one.
  *   splitk    k ranges per C tile: 0 the rule (products with fewer C tiles
  *             than 152 split k towards 304 work units), 1 never, s > 1 that
  *             many (at most the number of k-blocks: 16-wide for the native
@@ -188,7 +192,10 @@ mxm_status mxm_gemm_host(int mode, const double* hA, const double* hB, double* h
  * `mode` on an m x k by k x n product (Sec. 3.1 shapes) with `slices` slices
  * needs (the FP64 path: zero-padded tile copies of A and B, plus split-k
  * partials; the emulated modes: row and column scales, the digit planes of
- * the Ozaki split, the running sums or split-k partials).  Host arithmetic
+ * the Ozaki split and of the difference products, the segment sums, running
+ * sums or split-k partials).  An emulated call on a smaller caller workspace
+ * runs without the difference products (same bits) as long as it holds
+ * mxm_workspace_size_plan of a plan with cta = 1.  Host arithmetic
  * only, no device call.  Returns 0 for an empty product (m, n or k <= 0),
  * an unknown mode or a slice count the mode does not take.  The paper has no
  * counterpart; size a buffer for mxm_set_workspace with it.

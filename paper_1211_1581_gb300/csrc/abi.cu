@@ -167,7 +167,9 @@ F64Dims native_dims(int64_t m, int64_t k, int64_t n, const mxm_plan& p) {
 }
 
 // Dims of an emulated product (bf16 digits) under a plan.
-OzakiDims emul_dims(int mode, int64_t m, int64_t k, int64_t n, int slices, const mxm_plan& p) {
+// kara: difference products allowed (their planes need more workspace).
+OzakiDims emul_dims(int mode, int64_t m, int64_t k, int64_t n, int slices, const mxm_plan& p,
+                    bool kara = true) {
   OzakiDims d = ozaki_dims_splitk(m, k, n, slices, mode_beta(mode), mode_rn(mode));
   if (p.splitk == 1) {
     d.splits = 1;
@@ -182,6 +184,16 @@ OzakiDims emul_dims(int mode, int64_t m, int64_t k, int64_t n, int slices, const
   // against 73.4 GB for groups of 8 going forwards (same time within 0.5 %)
   d.raster = p.raster > 0 ? p.raster : (d.pair ? kPairRaster : kDefaultRaster);
   d.kb_alt = p.kb_order == 1 ? 0 : 1;
+  if (kara && p.cta == 0 && p.splitk <= 1) {
+    OzakiDims w = d;
+    w.splits = 1;
+    if (kara_chosen(w)) {
+      w.kara = 1;
+      w.pair = 1;
+      w.raster = p.raster > 0 ? p.raster : kDefaultRaster;
+      return w;
+    }
+  }
   return d;
 }
 
@@ -193,10 +205,10 @@ OzakiDims fp8_dims(int64_t m, int64_t k, int64_t n, int slices, const mxm_plan& 
 }
 
 size_t workspace_bytes(int mode, int64_t m, int64_t k, int64_t n, int slices,
-                       const mxm_plan& p = kNoPlan) {
+                       const mxm_plan& p = kNoPlan, bool kara = true) {
   if (m <= 0 || n <= 0 || k <= 0) return 0;
   if (mode == MXM_MODE_F64) return f64_workspace(native_dims(m, k, n, p));
-  if (emul_mode(mode)) return ozaki_layout(emul_dims(mode, m, k, n, slices, p)).total;
+  if (emul_mode(mode)) return ozaki_layout(emul_dims(mode, m, k, n, slices, p, kara)).total;
   if (mode == MXM_MODE_EMUL_FP8) return ozaki_layout(fp8_dims(m, k, n, slices, p)).total;
   if (mode == MXM_MODE_BF16_F32ACC) return ozaki_layout(ozaki_dims(m, k, n, 1, 8)).total;
   return 0;
@@ -205,7 +217,7 @@ size_t workspace_bytes(int mode, int64_t m, int64_t k, int64_t n, int slices,
 // Launch sequence of one product whose workspace is already in place.
 mxm_status run_gemm(int mode, const double* A, const double* B, double* C, int64_t m, int64_t k,
                     int64_t n, int slices, uint8_t* ws, int* status, cudaStream_t s,
-                    const mxm_plan& plan = kNoPlan) {
+                    const mxm_plan& plan = kNoPlan, bool kara = true) {
   if (m == 0 || n == 0) return MXM_OK;
   if (k == 0) return launch_zero_fill(C, m * n, s) == cudaSuccess ? MXM_OK : cuda_fail();
   cudaError_t e = cudaSuccess;
@@ -218,7 +230,7 @@ mxm_status run_gemm(int mode, const double* A, const double* B, double* C, int64
     if (e == cudaSuccess) e = launch_f64_gemm(ws, C, d, status, s);
     profile_mark(ce, 3, s);
   } else if (emul_mode(mode)) {
-    const OzakiDims d = emul_dims(mode, m, k, n, slices, plan);
+    const OzakiDims d = emul_dims(mode, m, k, n, slices, plan, kara);
     const OzakiLayout L = ozaki_layout(d);
     uint64_t* rowbits = reinterpret_cast<uint64_t*>(ws + L.rowbits);
     uint64_t* colbits = reinterpret_cast<uint64_t*>(ws + L.colbits);
@@ -332,10 +344,17 @@ mxm_status mxm_gemm_plan(int mode, const double* A, const double* B, double* C, 
   std::lock_guard<std::mutex> lock(g_mutex);
   DeviceState* ds = nullptr;
   if ((st = current_state(&ds)) != MXM_OK) return st;
-  const size_t need = workspace_bytes(mode, m, k, n, slices, p);
-  if ((st = ensure_workspace(ds, need, s)) != MXM_OK) return st;
-  return run_gemm(mode, A, B, C, m, k, n, slices, static_cast<uint8_t*>(ds->ws), ds->status, s,
-                  p);
+  // the difference products where their workspace can be had, else (a caller
+  // workspace sized for less, a capture, no memory) the products one by one:
+  // the same bits either way
+  bool kara = true;
+  if (ensure_workspace(ds, workspace_bytes(mode, m, k, n, slices, p), s) != MXM_OK) {
+    kara = false;
+    st = ensure_workspace(ds, workspace_bytes(mode, m, k, n, slices, p, false), s);
+    if (st != MXM_OK) return st;
+  }
+  return run_gemm(mode, A, B, C, m, k, n, slices, static_cast<uint8_t*>(ds->ws), ds->status, s, p,
+                  kara);
 }
 
 mxm_status mxm_gemm(int mode, const double* A, const double* B, double* C, int64_t m, int64_t k,
@@ -395,12 +414,13 @@ static int64_t host_panel_cols(int64_t h, int64_t n, int sms) {
 
 static mxm_status gemm_host_panels(DeviceState* ds, int mode, const double* hA, const double* hB,
                                    double* hC, int64_t m, int64_t k, int64_t n, int slices,
-                                   int64_t h, cudaStream_t s) {
+                                   int64_t h, cudaStream_t s, bool kara) {
   const int beta = mode_beta(mode);
   const bool rn = mode_rn(mode);
   const int64_t w = host_panel_cols(h, n, ds->sm_count);
   const int64_t P = (m + h - 1) / h, Q = (n + w - 1) / w;
-  const OzakiDims dp = ozaki_dims(h, k, w, slices, beta, rn);  // the largest block, no split-k
+  OzakiDims dp = ozaki_dims(h, k, w, slices, beta, rn);  // the largest block, no split-k
+  dp.kara = kara && kara_chosen(dp) ? 1 : 0;
   const OzakiLayout L = ozaki_layout(dp);
   // per compute stream: row scales, A planes, running sums of one block
   const size_t rb_bytes = align_up(sizeof(uint64_t) * size_t(h), 1024);
@@ -480,6 +500,7 @@ static mxm_status gemm_host_panels(DeviceState* ds, int mode, const double* hA, 
     uint8_t* bplanes = cw + (L.aslices - L.colbits);
     OzakiDims db = ozaki_dims(0, k, colw(j), slices, beta, rn);
     db.pair = dp.pair;  // every block's product reads these B planes
+    db.kara = dp.kara;
     if (cudaStreamWaitEvent(ds->c2, eBc[j], 0) != cudaSuccess ||
         launch_ozaki_scale(nullptr, dB + j * w * k, db, nullptr, colbits, ds->status, ds->c2) !=
             cudaSuccess ||
@@ -497,6 +518,7 @@ static mxm_status gemm_host_panels(DeviceState* ds, int mode, const double* hA, 
     uint64_t* sums = reinterpret_cast<uint64_t*>(buf + rb_bytes + ap_bytes);
     OzakiDims da = ozaki_dims(hp, k, 0, slices, beta, rn);
     da.pair = dp.pair;
+    da.kara = dp.kara;
     if (cudaStreamWaitEvent(c, eA[i], 0) != cudaSuccess ||
         launch_ozaki_scale(dA + r0 * k, nullptr, da, rowbits, nullptr, ds->status, c) !=
             cudaSuccess ||
@@ -512,7 +534,8 @@ static mxm_status gemm_host_panels(DeviceState* ds, int mode, const double* hA, 
       double* blk = dC + r0 * n + j * w * hp;  // h x wj, row-major, contiguous
       OzakiDims dg = ozaki_dims(hp, k, wj, slices, beta, rn);
       dg.pair = dp.pair;
-      dg.raster = dg.pair ? kPairRaster : kDefaultRaster;
+      dg.kara = dp.kara;
+      dg.raster = dg.pair && !dg.kara ? kPairRaster : kDefaultRaster;
       dg.kb_alt = 1;
       cudaEvent_t done = eC[i * Q + j];
       if (cudaStreamWaitEvent(c, eBs[j], 0) != cudaSuccess ||
@@ -555,13 +578,25 @@ mxm_status mxm_gemm_host(int mode, const double* hA, const double* hB, double* h
   if ((st = current_state(&ds)) != MXM_OK) return st;
   if (emul_mode(mode) && k > 0) {
     const int64_t h = host_panel_rows(m, n, ds->sm_count);
-    if (h > 0) return gemm_host_panels(ds, mode, hA, hB, hC, m, k, n, slices, h, s);
+    if (h > 0) {
+      // as mxm_gemm: without the difference products where their workspace
+      // cannot be had
+      st = gemm_host_panels(ds, mode, hA, hB, hC, m, k, n, slices, h, s, true);
+      if (st == MXM_ERR_WORKSPACE_TOO_SMALL || (st == MXM_ERR_CUDA && ds->ws == nullptr))
+        st = gemm_host_panels(ds, mode, hA, hB, hC, m, k, n, slices, h, s, false);
+      return st;
+    }
   }
   const size_t ab = align_up(sizeof(double) * size_t(m) * size_t(k), 1024);
   const size_t bb = align_up(sizeof(double) * size_t(k) * size_t(n), 1024);
   const size_t cb = align_up(sizeof(double) * size_t(m) * size_t(n), 1024);
-  const size_t need = ab + bb + cb + workspace_bytes(mode, m, k, n, slices);
-  if ((st = ensure_workspace(ds, need, s)) != MXM_OK) return st;
+  bool kara = true;
+  if (ensure_workspace(ds, ab + bb + cb + workspace_bytes(mode, m, k, n, slices), s) != MXM_OK) {
+    kara = false;
+    st = ensure_workspace(ds, ab + bb + cb + workspace_bytes(mode, m, k, n, slices, kNoPlan, false),
+                          s);
+    if (st != MXM_OK) return st;
+  }
   uint8_t* base = static_cast<uint8_t*>(ds->ws);
   double* dA = reinterpret_cast<double*>(base);
   double* dB = reinterpret_cast<double*>(base + ab);
@@ -573,7 +608,8 @@ mxm_status mxm_gemm_host(int mode, const double* hA, const double* hB, double* h
             cudaSuccess)
       return cuda_fail();
   }
-  st = run_gemm(mode, dA, dB, dC, m, k, n, slices, base + ab + bb + cb, ds->status, s);
+  st = run_gemm(mode, dA, dB, dC, m, k, n, slices, base + ab + bb + cb, ds->status, s,
+                kNoPlan, kara);
   if (st != MXM_OK) return st;
   if (cudaMemcpyAsync(hC, dC, sizeof(double) * size_t(m) * size_t(n), cudaMemcpyDeviceToHost, s) !=
       cudaSuccess)

@@ -1,6 +1,7 @@
 // mxm_internal.h -- declarations shared by the translation units of
 // libmxm.so (not part of the public C ABI in include/mxm.h).
 #pragma once
+#include <cmath>
 #include <cstddef>
 #include <cstdint>
 
@@ -101,6 +102,8 @@ struct OzakiDims {
                        //    persistent walk over C tiles
   int kb_alt;          // 1: alternate the k-block direction from one diagonal
                        //    (pair) to the next
+  int kara;            // 1: difference products on 256 x 256 C tiles (ozaki_kara.cu);
+                       //    the operands have kara_planes(S) digit planes
 };
 
 // Default walk: groups of 8 tile-rows (4 pair-rows on CTA pairs); the
@@ -121,6 +124,7 @@ inline OzakiDims ozaki_dims(int64_t m, int64_t k, int64_t n, int S, int beta, bo
   d.pair = d.Mt >= 2 ? 1 : 0;
   d.raster = kDefaultRaster;
   d.kb_alt = 0;
+  d.kara = 0;
   return d;
 }
 
@@ -156,7 +160,7 @@ inline OzakiDims ozaki_dims_splitk(int64_t m, int64_t k, int64_t n, int S, int b
 // tiles): bf16 digits without split-k, chosen where the dims are made (two
 // or more tile-rows of A; products that share B planes share the choice,
 // a single tile-row then leaving the second CTA of its pairs idle).
-inline bool ozaki_b_halves(const OzakiDims& d) { return d.pair != 0 && !d.fp8; }
+inline bool ozaki_b_halves(const OzakiDims& d) { return d.pair != 0 && !d.fp8 && !d.kara; }
 inline bool ozaki_cta2(const OzakiDims& d) {
   return ozaki_b_halves(d) && d.splits <= 1 && d.Mt >= 1;
 }
@@ -206,37 +210,6 @@ inline size_t ozaki_spill_bytes(const OzakiDims& d) {
   return (size_t)ctas * 2 * kOzTileRows * kOzTileRows * 8;
 }
 
-inline OzakiLayout ozaki_layout(const OzakiDims& d) {
-  OzakiLayout L;
-  size_t off = 0;
-  L.rowbits = off; off = align_up(off + sizeof(uint64_t) * (size_t)(d.m > 0 ? d.m : 1), 1024);
-  L.colbits = off; off = align_up(off + sizeof(uint64_t) * (size_t)(d.n > 0 ? d.n : 1), 1024);
-  L.aslices = off; off = align_up(off + (size_t)d.S * d.Mt * d.Kt * ozaki_tile_bytes(d), 1024);
-  L.bslices = off; off = align_up(off + (size_t)d.S * d.Nt * d.Kt * ozaki_tile_bytes(d), 1024);
-  // running sums of the recombination between diagonal pairs: per C tile
-  // 128 x 128 x 8 bytes, column-major inside the tile (so that a warp, which
-  // owns 32 consecutive rows, touches 256 contiguous bytes per column).
-  // Under split-k the region holds instead the int64 partial sums D_g of
-  // every k range: [splits][Mt x Nt tiles][S diagonals] x 128 x 128,
-  // column-major inside the tile.  The spill area (if any) follows the sums.
-  L.sums = off; off = align_up(off + ozaki_sums_bytes(d), 1024);
-  off = align_up(off + ozaki_spill_bytes(d), 1024);
-  L.total = off;
-  return L;
-}
-
-
-// The plan of ozaki_dims_splitk when its workspace fits `cap` bytes, else
-// the same product without split-k (the split-k partials are exact integers
-// added exactly, so both plans give the same bits).  The caller checks
-// whether the returned plan fits.
-inline OzakiDims ozaki_dims_capped(int64_t m, int64_t k, int64_t n, int S, int beta,
-                                   size_t cap) {
-  OzakiDims d = ozaki_dims_splitk(m, k, n, S, beta);
-  if (d.splits > 1 && ozaki_layout(d).total > cap) d = ozaki_dims(m, k, n, S, beta);
-  return d;
-}
-
 // Largest number of K=16 MMAs whose integer products can be summed in an
 // FP32 accumulator without rounding: every product is at most (2^beta-1)^2
 // in magnitude and 16 of them enter per MMA, so the running sum stays within
@@ -253,6 +226,123 @@ inline int ozaki_window_stages(int beta, bool rn = false) {
   return ozaki_window_mmas(beta, rn) / (kOzTileK / 16);
 }
 
+// ---------------------------------------------------------------- difference products
+// (ozaki_kara.cu; the identity is stated there.)  Digit planes of an operand:
+// the S digits, then one difference plane for every pair s < t with
+// s + t <= S + 1 except (1, S), ordered by s + t, then s.
+constexpr int kKaraMaxSlices = 9;
+__host__ __device__ inline int kara_pairs(int S) {
+  int n = -1;
+  for (int g = 3; g <= S + 1; ++g) n += (g - 1) / 2;
+  return n > 0 ? n : 0;
+}
+__host__ __device__ inline int kara_planes(int S) { return S + kara_pairs(S); }
+inline int kara_pair_plane(int S, int s, int t) {
+  int idx = S;
+  for (int g = 3; g < s + t; ++g) idx += (g - 1) / 2;
+  idx += s - 1;
+  if (s + t == S + 1) --idx;  // (1, S) has no plane
+  return idx;
+}
+
+// Exact FP32 windows (k-blocks) of the difference products: truncated digits
+// of one value have one sign, so their differences keep the digit bound;
+// balanced digits differ by at most 256.
+inline int kara_window_stages(const OzakiDims& d) {
+  return d.rn ? static_cast<int>((1ll << 24) / (256ll * 256 * 16)) / (kOzTileK / 16)
+              : ozaki_window_stages(d.beta, false);
+}
+
+// Most products in one segment: N_{S+1} (the pair (1, S) counts twice).
+inline int kara_max_segment(int S) { return S / 2 + 1; }
+
+// 256 x 256 C tiles of the CTA pairs; the pairs of a 152-SM GPU (a constant,
+// so that the workspace is host arithmetic); the scratch: S slots per tile
+// and CTA of the pair, and those of the tiles cut into units (fewer than the
+// pairs, 2 S - 2 slots each and k range; the cut stays within them).
+constexpr int64_t kKaraPairs = 76;
+constexpr size_t kKaraSlotBytes = (size_t)kOzTileRows * 256 * 4;
+inline int64_t kara_tiles(const OzakiDims& d) { return (d.Mt + 1) / 2 * ((d.Nt + 1) / 2); }
+inline size_t kara_cut_slots(const OzakiDims& d) {
+  const int64_t t = kara_tiles(d), cut = t < kKaraPairs ? t : kKaraPairs;
+  const size_t slots = (size_t)cut * (2 * d.S - 2);
+  return slots > 3 * (size_t)kKaraPairs ? slots : 3 * (size_t)kKaraPairs;
+}
+inline size_t kara_scratch_bytes(const OzakiDims& d) {
+  return 2 * kKaraSlotBytes * ((size_t)kara_tiles(d) * d.S + kara_cut_slots(d));
+}
+
+// Host form of the kernels' oz_exact_from: the first diagonal of the FP64
+// phase of the fold.
+inline int ozaki_exact_from(int S, int beta, int64_t Kt) {
+  const double dmax = static_cast<double>((1 << beta) - 1);
+  int gx = S + 1;
+  double yb = 0.0;
+  for (int g = S + 1; g >= 2; --g) {
+    yb += std::ldexp((g - 1) * dmax * dmax * kOzTileK * static_cast<double>(Kt),
+                     beta * (S + 1 - g));
+    if (yb >= 4503599627370496.0) break;  // 2^52
+    gx = g;
+  }
+  return gx;
+}
+
+// Which products can take the difference products.
+inline bool kara_fits(const OzakiDims& d) {
+  return !d.fp8 && d.S >= 3 && d.S <= kKaraMaxSlices && d.beta * d.S <= 64 && ozaki_narrow(d) &&
+         d.Kt > 0 && d.Mt >= 2 && d.Nt >= 2 && kara_tiles(d) < (1 << 24);
+}
+
+inline OzakiLayout ozaki_layout(const OzakiDims& d) {
+  OzakiLayout L;
+  size_t off = 0;
+  L.rowbits = off; off = align_up(off + sizeof(uint64_t) * (size_t)(d.m > 0 ? d.m : 1), 1024);
+  L.colbits = off; off = align_up(off + sizeof(uint64_t) * (size_t)(d.n > 0 ? d.n : 1), 1024);
+  const size_t planes = d.kara ? kara_planes(d.S) : d.S;
+  L.aslices = off; off = align_up(off + planes * d.Mt * d.Kt * ozaki_tile_bytes(d), 1024);
+  L.bslices = off; off = align_up(off + planes * d.Nt * d.Kt * ozaki_tile_bytes(d), 1024);
+  if (d.kara) {  // the segment sums of the difference-product kernel
+    L.sums = off;
+    L.total = align_up(off + kara_scratch_bytes(d), 1024);
+    return L;
+  }
+  // running sums of the recombination between diagonal pairs: per C tile
+  // 128 x 128 x 8 bytes, column-major inside the tile (so that a warp, which
+  // owns 32 consecutive rows, touches 256 contiguous bytes per column).
+  // Under split-k the region holds instead the int64 partial sums D_g of
+  // every k range: [splits][Mt x Nt tiles][S diagonals] x 128 x 128,
+  // column-major inside the tile.  The spill area (if any) follows the sums.
+  L.sums = off; off = align_up(off + ozaki_sums_bytes(d), 1024);
+  off = align_up(off + ozaki_spill_bytes(d), 1024);
+  L.total = off;
+  return L;
+}
+
+
+// The choice: the workspace (digit and difference planes, segment slots) up
+// to kKaraMaxBytes (6.8 GB at 8192^3, 27 GB at 16384^3), and not for a part of a
+// wave with little k, where the planes and slots cost more than the products
+// save (measured at 512 x 512 x 4096, S = 7: 154 us against 148).
+constexpr size_t kKaraMaxBytes = (size_t)32 << 30;
+inline bool kara_chosen(const OzakiDims& d) {
+  if (!kara_fits(d)) return false;
+  if (d.Kt <= 4 && kara_tiles(d) > 16 && kara_tiles(d) < 48) return false;
+  OzakiDims w = d;
+  w.kara = 1;
+  return ozaki_layout(w).total <= kKaraMaxBytes;
+}
+
+// The plan of ozaki_dims_splitk when its workspace fits `cap` bytes, else
+// the same product without split-k (the split-k partials are exact integers
+// added exactly, so both plans give the same bits).  The caller checks
+// whether the returned plan fits.
+inline OzakiDims ozaki_dims_capped(int64_t m, int64_t k, int64_t n, int S, int beta,
+                                   size_t cap) {
+  OzakiDims d = ozaki_dims_splitk(m, k, n, S, beta);
+  if (d.splits > 1 && ozaki_layout(d).total > cap) d = ozaki_dims(m, k, n, S, beta);
+  return d;
+}
+
 cudaError_t launch_ozaki_scale(const double* A, const double* B, const OzakiDims& d,
                                uint64_t* rowbits, uint64_t* colbits, int* status,
                                cudaStream_t s);
@@ -265,6 +355,10 @@ cudaError_t launch_ozaki_split(const double* A, const double* B, const OzakiDims
 cudaError_t launch_ozaki_gemm(const uint8_t* aslices, const uint8_t* bslices,
                               const uint64_t* rowbits, const uint64_t* colbits, double* C,
                               const OzakiDims& d, uint64_t* sums, int* status, cudaStream_t s);
+// The same by difference products (d.kara; scratch: kara_scratch_bytes(d)).
+cudaError_t launch_ozaki_kara(const uint8_t* aslices, const uint8_t* bslices,
+                              const uint64_t* rowbits, const uint64_t* colbits, double* C,
+                              const OzakiDims& d, uint8_t* scratch, int* status, cudaStream_t s);
 
 // ---------------------------------------------------------------- FP64
 constexpr int kF64BM = 128, kF64BN = 128, kF64BK = 16;

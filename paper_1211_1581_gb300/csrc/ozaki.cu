@@ -35,6 +35,7 @@
 #include <type_traits>
 
 #include "mxm_internal.h"
+#include "ozaki_fold.cuh"
 #include "ptx.cuh"
 
 namespace mxm {
@@ -209,10 +210,12 @@ __device__ __forceinline__ uint32_t bf16_pair(uint32_t q0, uint32_t q1, uint32_t
   return __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);  // the upper halves
 }
 
+// diff: +1 (A) or -1 (B): the planes of the difference products follow the
+// digits (kara_pair_plane order): d_s - d_t for A, d_t - d_s for B; 0: none.
 template <int V>
 __device__ __forceinline__ void split_chunk_store_w64(const double (&x)[V], int e, int S,
                                                       int beta, uint8_t* dst,
-                                                      size_t slice_stride) {
+                                                      size_t slice_stride, int diff = 0) {
   uint32_t Fh[V], Fl[V], mg[V];
 #pragma unroll
   for (int j = 0; j < V; ++j) {
@@ -260,6 +263,34 @@ __device__ __forceinline__ void split_chunk_store_w64(const double (&x)[V], int 
     *reinterpret_cast<uint4*>(dst + static_cast<size_t>(s - 1) * slice_stride) =
         make_uint4(packed[0], packed[1], packed[2], packed[3]);
   }
+  if constexpr (V == 8) {
+    if (diff == 0) return;
+    uint8_t* out = dst + static_cast<size_t>(S) * slice_stride;
+    for (int g = 3; g <= S + 1; ++g)
+      for (int s = g == S + 1 ? 2 : 1; s < g - s; ++s) {
+        // the larger-weight digit first for A, second for B
+        const int pa = beta * (S - (diff > 0 ? s : g - s)), pb = beta * (S - (diff > 0 ? g - s : s));
+        uint32_t packed[4];
+#pragma unroll
+        for (int j = 0; j < 8; j += 2) {
+          uint32_t f[2];
+#pragma unroll
+          for (int h = 0; h < 2; ++h) {
+            const uint32_t da = (pa >= 32 ? Fh[j + h] >> (pa - 32)
+                                          : __funnelshift_r(Fl[j + h], Fh[j + h], pa)) & mask;
+            const uint32_t db = (pb >= 32 ? Fh[j + h] >> (pb - 32)
+                                          : __funnelshift_r(Fl[j + h], Fh[j + h], pb)) & mask;
+            // 1.5 2^23 + (da - db) as a float pattern, minus 1.5 2^23, with
+            // the sign of x
+            f[h] = __float_as_uint(__uint_as_float(0x4B400000u + da - db) - 12582912.0f) ^
+                   (mg[j + h] & 0x80000000u);
+          }
+          packed[j >> 1] = __byte_perm(f[0], f[1], 0x7632);  // the upper halves
+        }
+        *reinterpret_cast<uint4*>(out) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
+        out += slice_stride;
+      }
+  }
 }
 
 // Balanced 8-bit digits (the round-to-nearest split): with e1 = e + 1,
@@ -270,7 +301,8 @@ __device__ __forceinline__ void split_chunk_store_w64(const double (&x)[V], int 
 // same digits as taking V mod 256 in [-128, 127] from the bottom up.  Each
 // digit is an integer of at most 8 bits, exact in bf16.
 __device__ __forceinline__ void split_chunk_store_rn8(const double (&x)[8], int e1, int S,
-                                                      uint8_t* dst, size_t slice_stride) {
+                                                      uint8_t* dst, size_t slice_stride,
+                                                      int diff = 0) {
   long long W[8];
   const long long Boff =
       S > 1 ? static_cast<long long>(0x8080808080808080ull >> (8 * (9 - S))) : 0ll;
@@ -316,19 +348,43 @@ __device__ __forceinline__ void split_chunk_store_rn8(const double (&x)[8], int 
     *reinterpret_cast<uint4*>(dst + static_cast<size_t>(s - 1) * slice_stride) =
         make_uint4(packed[0], packed[1], packed[2], packed[3]);
   }
+  if (diff == 0) return;
+  uint8_t* out = dst + static_cast<size_t>(S) * slice_stride;
+  for (int g = 3; g <= S + 1; ++g)
+    for (int s = g == S + 1 ? 2 : 1; s < g - s; ++s) {
+      // byte differences (the offsets of 128 cancel below the top digit)
+      const int ps = 8 * (S - s), pt = 8 * (S - (g - s));
+      uint32_t packed[4];
+#pragma unroll
+      for (int j = 0; j < 8; j += 2) {
+        uint32_t q[2];
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int ds = s == 1 ? static_cast<int>(W[j + h] >> ps)
+                                : static_cast<int>((W[j + h] >> ps) & 255) - 128;
+          const int dt = static_cast<int>((W[j + h] >> pt) & 255) - 128;
+          q[h] = kMagic + static_cast<uint32_t>(diff > 0 ? ds - dt : dt - ds);
+        }
+        packed[j >> 1] = bf16_pair(q[0], q[1], kNegMagic, kNegMagic);
+      }
+      *reinterpret_cast<uint4*>(out) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
+      out += slice_stride;
+    }
 }
 
 __device__ __forceinline__ void split_chunk(const double (&x)[8], int e, int S, int beta,
-                                            uint8_t* dst, size_t slice_stride, bool rn = false) {
+                                            uint8_t* dst, size_t slice_stride, bool rn = false,
+                                            int diff = 0) {
   if (rn)
-    split_chunk_store_rn8(x, e + 1, S, dst, slice_stride);
+    split_chunk_store_rn8(x, e + 1, S, dst, slice_stride, diff);
   else if (beta * S <= 64)
-    split_chunk_store_w64<8>(x, e, S, beta, dst, slice_stride);
+    split_chunk_store_w64<8>(x, e, S, beta, dst, slice_stride, diff);
   else
     split_chunk_store(x, e, S, beta, dst, slice_stride);
 }
 __device__ __forceinline__ void split_chunk(const double (&x)[16], int e, int S, int beta,
-                                            uint8_t* dst, size_t slice_stride, bool = false) {
+                                            uint8_t* dst, size_t slice_stride, bool = false,
+                                            int = 0) {
   split_chunk_store_w64<16>(x, e, S, beta, dst, slice_stride);  // beta = 4, S <= 16
 }
 
@@ -354,7 +410,8 @@ __device__ __forceinline__ void split_a_tile(const double* __restrict__ A, int64
                                              int beta, int64_t tm, int64_t tk, uint8_t* tile,
                                              size_t slice_stride, bool rn = false,
                                              int row_lim = kOzTileRows,
-                                             int chunk_lim = SplitGeo<V>::kChunksPerRow) {
+                                             int chunk_lim = SplitGeo<V>::kChunksPerRow,
+                                             int diff = 0) {
   using G = SplitGeo<V>;
   const bool pairs = ((k & 1) == 0) && ((reinterpret_cast<uintptr_t>(A) & 15) == 0);
   const int total = row_lim * chunk_lim;
@@ -389,7 +446,8 @@ __device__ __forceinline__ void split_a_tile(const double* __restrict__ A, int64
 #pragma unroll
     for (int h = 0; h < 2; ++h)
       if (p0 + h * static_cast<int>(blockDim.x) < total)
-        split_chunk(v[h], e[h], S, beta, tile + G::offset(rr[h], cc[h]), slice_stride, rn);
+        split_chunk(v[h], e[h], S, beta, tile + G::offset(rr[h], cc[h]), slice_stride, rn,
+                    diff);
   }
 }
 
@@ -406,11 +464,13 @@ __device__ __forceinline__ void split_b_tile(const double* __restrict__ B, int64
                                              size_t slice_stride,
                                              double (*sb)[kOzTileRows + 1], bool rn = false,
                                              bool halves = false, int row_lim = kOzTileRows,
-                                             int chunk_lim = SplitGeo<V>::kChunksPerRow) {
+                                             int chunk_lim = SplitGeo<V>::kChunksPerRow,
+                                             int diff = 0, int pass0 = 0,
+                                             int pass1 = kOzTileK / kSplitBRows) {
   using G = SplitGeo<V>;
   const int64_t col0 = tn * kOzTileRows;
   constexpr int kChunksPerPass = kSplitBRows / V;
-  for (int pass = 0; pass < kOzTileK / kSplitBRows; ++pass) {
+  for (int pass = pass0; pass < pass1; ++pass) {
     if (pass * kChunksPerPass >= chunk_lim) break;  // block-uniform
     const int64_t l0 = tk * kOzTileK + pass * kSplitBRows;
     if (blockDim.x == kSplitThreads) {  // every launch: all of a thread's loads in flight at once
@@ -449,7 +509,7 @@ __device__ __forceinline__ void split_b_tile(const double* __restrict__ B, int64
       for (int j = 0; j < V; ++j) v[j] = sb[cl * V + j][r];
       const int c = pass * kChunks + cl;
       const int off = (V == 8 && halves) ? oz_chunk_offset_halves(r, c) : G::offset(r, c);
-      split_chunk(v, f, S, beta, tile + off, slice_stride, rn);
+      split_chunk(v, f, S, beta, tile + off, slice_stride, rn, diff);
     }
     __syncthreads();
   }
@@ -459,12 +519,13 @@ __device__ __forceinline__ void split_b_tile(const double* __restrict__ B, int64
 template <int V>
 __global__ void __launch_bounds__(256) oz_split_a_kernel(
     const double* __restrict__ A, int64_t m, int64_t k, const uint64_t* __restrict__ rowbits,
-    int S, int beta, int64_t Mt, int64_t Kt, uint8_t* __restrict__ aslices, bool rn) {
+    int S, int beta, int64_t Mt, int64_t Kt, uint8_t* __restrict__ aslices, bool rn, int diff) {
   constexpr size_t kTile = SplitGeo<V>::kTileBytes;
   const int64_t tk = blockIdx.x, tm = blockIdx.y;
   split_a_tile<V>(A, m, k, rowbits, S, beta, tm, tk,
                   aslices + (static_cast<size_t>(tm) * Kt + tk) * kTile,
-                  static_cast<size_t>(Mt) * Kt * kTile, rn);
+                  static_cast<size_t>(Mt) * Kt * kTile, rn, kOzTileRows,
+                  SplitGeo<V>::kChunksPerRow, diff);
 }
 
 // Steps 1 and 2 for A in one pass: one block per row of A (and per padding
@@ -478,7 +539,7 @@ constexpr int64_t kFusedRowMaxK = 24576;  // k doubles held in shared memory (19
 
 __global__ void __launch_bounds__(256) oz_scale_split_a_kernel(
     const double* __restrict__ A, int64_t m, int64_t k, uint64_t* __restrict__ rowbits, int S,
-    int beta, int64_t Mt, int64_t Kt, uint8_t* __restrict__ aslices, bool rn,
+    int beta, int64_t Mt, int64_t Kt, uint8_t* __restrict__ aslices, bool rn, int diff,
     int* __restrict__ status) {
   extern __shared__ double row[];
   __shared__ uint32_t wmax[32];
@@ -539,7 +600,7 @@ __global__ void __launch_bounds__(256) oz_scale_split_a_kernel(
 #pragma unroll
     for (int j = 0; j < 8; ++j) v[j] = row[tk * kOzTileK + c * 8 + j];
     split_chunk(v, e, S, beta, base + tk * kOzTileBytes + oz_chunk_offset(r, c), slice_stride,
-                rn);
+                rn, diff);
   }
 }
 
@@ -549,18 +610,21 @@ __host__ __device__ inline bool oz_fused_a(const OzakiDims& d) {
   return !d.fp8 && d.Kt * kOzTileK <= kFusedRowMaxK;
 }
 
-// B -> B_t tiles [S][Nt][Kt]; halves: the CTA-pair layout of each tile.
+// B -> B_t tiles [S][Nt][Kt]; halves: the CTA-pair layout of each tile.  A block
+// takes one 32-row pass of a tile (blockIdx.z): with whole tiles a small
+// product filled a few SMs with four passes in a row (512 x 512: 34 us).
 template <int V>
 __global__ void __launch_bounds__(256) oz_split_b_kernel(
     const double* __restrict__ B, int64_t k, int64_t n, const uint64_t* __restrict__ colbits,
     int S, int beta, int64_t Nt, int64_t Kt, uint8_t* __restrict__ bslices, bool rn,
-    bool halves) {
+    bool halves, int diff) {
   constexpr size_t kTile = SplitGeo<V>::kTileBytes;
   __shared__ double sb[kSplitBRows][kOzTileRows + 1];
   const int64_t tk = blockIdx.x, tn = blockIdx.y;
   split_b_tile<V>(B, k, n, colbits, S, beta, tn, tk,
                   bslices + (static_cast<size_t>(tn) * Kt + tk) * kTile,
-                  static_cast<size_t>(Nt) * Kt * kTile, sb, rn, halves);
+                  static_cast<size_t>(Nt) * Kt * kTile, sb, rn, halves, kOzTileRows,
+                  SplitGeo<V>::kChunksPerRow, diff, blockIdx.z, blockIdx.z + 1);
 }
 
 // ---------------------------------------------------------------- grouped steps 1-2
@@ -829,19 +893,6 @@ constexpr int kAccSlotCols = 64;
 constexpr int kMmaK = 16;           // K per tcgen05.mma kind::f16
 constexpr int kMmaPerStage = kOzTileK / kMmaK;
 
-__device__ __forceinline__ void tile_coords(int64_t tile, int64_t Mt, int64_t Nt, int64_t G,
-                                            int64_t& tm, int64_t& tn) {
-  // groups of G tile-rows, column-major inside a group: CTAs working at the
-  // same time share A tiles and B tiles in L2
-  const int64_t per_group = G * Nt;
-  const int64_t grp = tile / per_group;
-  const int64_t first = grp * G;
-  const int64_t gsz = (Mt - first) < G ? (Mt - first) : G;
-  const int64_t in = tile - grp * per_group;
-  tm = first + in % gsz;
-  tn = in / gsz;
-}
-
 // One 128 x 128 tile of C and where its operand tiles live.
 struct OzTile {
   const uint8_t* a;          // slice 1 of A tile-row tm, k-block 0
@@ -1062,24 +1113,6 @@ struct OzGrouped {
     return j;
   }
 };
-
-// First diagonal of the FP64 phase of the fold: diagonals g >= the returned
-// value are combined exactly in int64 (the partial sum
-// Y = sum_g D_g 2^{beta (S+1-g)} stays below 2^52 by the bound
-// |D_g| <= (g-1)(2^beta-1)^2 128 Kt, so the FP64 fold of those steps is
-// exact and doing them in integers gives the same bits).
-__device__ __forceinline__ int oz_exact_from(int S, int beta, int64_t Kt) {
-  const double dmax = static_cast<double>((1 << beta) - 1);
-  int gx = S + 1;
-  double yb = 0.0;
-  for (int g = S + 1; g >= 2; --g) {
-    yb += (g - 1) * dmax * dmax * static_cast<double>(kOzTileK) * static_cast<double>(Kt) *
-          pow2_normal(beta * (S + 1 - g));
-    if (yb >= 4503599627370496.0) break;  // 2^52
-    gx = g;
-  }
-  return gx;
-}
 
 // The final scaling of one result.  Inline: the folds that call it are
 // rolled loops over a few columns at a time, so the code stays small (the
@@ -2286,24 +2319,25 @@ cudaError_t launch_ozaki_split(const double* A, const double* B, const OzakiDims
                                          static_cast<int>(smem));
     if (e != cudaSuccess) return e;
     oz_scale_split_a_kernel<<<static_cast<unsigned>(d.Mt * kOzTileRows), 256, smem, s>>>(
-        A, d.m, d.k, rowbits, d.S, d.beta, d.Mt, d.Kt, aslices, d.rn != 0, status);
+        A, d.m, d.k, rowbits, d.S, d.beta, d.Mt, d.Kt, aslices, d.rn != 0, d.kara, status);
   } else if (d.Mt > 0) {
     dim3 grid(static_cast<unsigned>(d.Kt), static_cast<unsigned>(d.Mt));
     if (d.fp8)
       oz_split_a_kernel<16><<<grid, 256, 0, s>>>(A, d.m, d.k, rowbits, d.S, d.beta, d.Mt, d.Kt,
-                                                 aslices, false);
+                                                 aslices, false, 0);
     else
       oz_split_a_kernel<8><<<grid, 256, 0, s>>>(A, d.m, d.k, rowbits, d.S, d.beta, d.Mt, d.Kt,
-                                                aslices, d.rn != 0);
+                                                aslices, d.rn != 0, d.kara);
   }
   if (d.Nt > 0) {
-    dim3 grid(static_cast<unsigned>(d.Kt), static_cast<unsigned>(d.Nt));
+    dim3 grid(static_cast<unsigned>(d.Kt), static_cast<unsigned>(d.Nt), kOzTileK / kSplitBRows);
     if (d.fp8)
       oz_split_b_kernel<16><<<grid, 256, 0, s>>>(B, d.k, d.n, colbits, d.S, d.beta, d.Nt, d.Kt,
-                                                 bslices, false, false);
+                                                 bslices, false, false, 0);
     else
       oz_split_b_kernel<8><<<grid, 256, 0, s>>>(B, d.k, d.n, colbits, d.S, d.beta, d.Nt, d.Kt,
-                                                bslices, d.rn != 0, ozaki_b_halves(d));
+                                                bslices, d.rn != 0, ozaki_b_halves(d),
+                                                d.kara ? -1 : 0);
   }
   return cudaGetLastError();
 }
@@ -2403,6 +2437,9 @@ cudaError_t launch_ozaki_gemm(const uint8_t* aslices, const uint8_t* bslices,
                               const uint64_t* rowbits, const uint64_t* colbits, double* C,
                               const OzakiDims& d, uint64_t* sums, int* status, cudaStream_t s) {
   if (d.Mt == 0 || d.Nt == 0) return cudaSuccess;
+  if (d.kara)
+    return launch_ozaki_kara(aslices, bslices, rowbits, colbits, C, d,
+                             reinterpret_cast<uint8_t*>(sums), status, s);
   const int window = ozaki_window_stages(d.beta, d.rn != 0);
   const int64_t splits = d.splits > 1 ? d.splits : 1;
   OzSingle tiles{aslices, bslices, rowbits, colbits, C,      d.m, d.n,

@@ -1,0 +1,100 @@
+"""The difference-product slice GEMM (256 x 256 C tiles on CTA pairs): results
+bit-identical to the oracle's emulation, which takes the digit products one
+by one.  Sizes at the edges of its rules: one row, column or k past a tile,
+odd tile-row and tile-column counts (a CTA of a pair without a tile), one
+k-block, several FP32 windows, tiles cut by segments and by ranges of k, whole
+waves with a cut rest; every slice count it takes."""
+import ctypes
+
+import numpy as np
+import pytest
+import torch
+
+import oracle
+from paper_1211_1581_gb300 import inputs, mxm
+from helpers import assert_bitwise
+
+pytestmark = pytest.mark.gpu
+
+
+def _emulated(A, B, mode, S):
+    if mode == mxm.MODE_EMUL_RN8:
+        return oracle.ozaki_gemm_rn8(A, B, S)
+    return oracle.ozaki_gemm(A, B, S=S, beta=7 if mode == mxm.MODE_EMUL_I8 else 8)
+
+
+@pytest.mark.parametrize("mode,S,m,k,n", [
+    (mxm.MODE_EMUL_I8, 7, 256, 128, 256),      # one tile, one k-block
+    (mxm.MODE_EMUL_I8, 7, 129, 129, 129),      # a second tile row, column, k-block of one
+    (mxm.MODE_EMUL_I8, 8, 385, 1040, 257),     # odd tile counts; 9 k-blocks: two windows
+    (mxm.MODE_EMUL_I8, 3, 300, 200, 257),
+    (mxm.MODE_EMUL_I8, 4, 260, 300, 513),
+    (mxm.MODE_EMUL_I8, 5, 513, 17, 300),
+    (mxm.MODE_EMUL_I8, 6, 257, 2100, 130),     # few tiles: cut along k too
+    (mxm.MODE_EMUL_I8, 9, 300, 260, 300),
+    (mxm.MODE_EMUL_BF16, 3, 200, 300, 200),
+    (mxm.MODE_EMUL_BF16, 6, 300, 1777, 257),   # windows of two k-blocks
+    (mxm.MODE_EMUL_BF16, 8, 257, 400, 513),
+    (mxm.MODE_EMUL_RN8, 3, 129, 100, 257),
+    (mxm.MODE_EMUL_RN8, 6, 385, 1300, 300),
+    (mxm.MODE_EMUL_RN8, 7, 300, 140, 300),
+])
+def test_bit_identical_to_oracle(mode, S, m, k, n):
+    A, B = inputs.gemm_operands("spread", m, k, n, seed=S, cfg=41)
+    C = torch.full((m, n), float("nan"), dtype=torch.float64, device="cuda")
+    mxm.mxm_gemm(mode, torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda(), C, slices=S)
+    assert mxm.mxm_get_device_status() == mxm.MXM_OK
+    assert_bitwise(C.cpu().numpy(), _emulated(A, B, mode, S), f"mode {mode} S={S} {m}x{k}x{n}")
+
+
+@pytest.mark.parametrize("m,k,n,raster", [(2300, 200, 2300, 0), (2300, 200, 2300, 3),
+                                          (5000, 130, 4870, 0)])
+def test_many_tiles_match_the_products_one_by_one(m, k, n, raster):
+    """More tiles than CTA pairs (81 and 380 on 76): whole waves and the cut
+    rest, against the single-CTA kernel, which takes no difference products,
+    and on sampled entries against the oracle."""
+    A, B = inputs.gemm_operands("spread", m, k, n, seed=2, cfg=42)
+    dA, dB = torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda()
+    C = torch.full((m, n), float("nan"), dtype=torch.float64, device="cuda")
+    D = torch.full((m, n), float("nan"), dtype=torch.float64, device="cuda")
+    mxm.mxm_gemm_plan(mxm.MODE_EMUL_I8, dA, dB, C, slices=7, plan=mxm.Plan(raster, 0, 0, 0))
+    mxm.mxm_gemm_plan(mxm.MODE_EMUL_I8, dA, dB, D, slices=7, plan=mxm.Plan(0, 0, 1, 1))
+    assert mxm.mxm_get_device_status() == mxm.MXM_OK
+    assert torch.equal(C, D)
+    rng = np.random.default_rng(m + raster)
+    ii, jj = rng.integers(0, m, 200), rng.integers(0, n, 200)
+    assert_bitwise(C.cpu().numpy()[ii, jj], oracle.ozaki_entries(A, B, ii, jj, S=7, beta=7),
+                   "sampled entries")
+
+
+def test_smaller_caller_workspace_takes_the_products_one_by_one():
+    """A caller workspace of the size the products one by one need (what
+    mxm_workspace_size gives under a single-CTA plan) still runs, with the same
+    bits; one byte less is refused."""
+    m, k, n = 600, 300, 600
+    A, B = inputs.gemm_operands("spread", m, k, n, seed=3, cfg=43)
+    dA, dB = torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda()
+    less = mxm.mxm_workspace_size_plan(mxm.MODE_EMUL_I8, m, k, n, 7, mxm.Plan(0, 0, 1, 0))
+    full = mxm.mxm_workspace_size(mxm.MODE_EMUL_I8, m, k, n, 7)
+    assert 0 < less < full
+    want = oracle.ozaki_gemm(A, B, S=7, beta=7)
+    ws = torch.empty(full, dtype=torch.uint8, device="cuda")
+    lib = mxm.load()
+    try:
+        for size, status in ((full, mxm.MXM_OK), (full - 1, mxm.MXM_OK), (less, mxm.MXM_OK),
+                             (less - 1, mxm.MXM_ERR_WORKSPACE_TOO_SMALL)):
+            assert lib.mxm_set_workspace(ws.data_ptr(), size, None) == mxm.MXM_OK
+            C = torch.full((m, n), 7.0, dtype=torch.float64, device="cuda")
+            torch.cuda.synchronize()
+            st = lib.mxm_gemm(mxm.MODE_EMUL_I8, ctypes.c_void_p(dA.data_ptr()),
+                              ctypes.c_void_p(dB.data_ptr()), ctypes.c_void_p(C.data_ptr()),
+                              m, k, n, 7, None)
+            assert st == status
+            torch.cuda.synchronize()
+            if st == mxm.MXM_OK:
+                assert_bitwise(C.cpu().numpy(), want, f"workspace {size}")
+            else:
+                assert torch.all(C == 7.0)
+    finally:
+        torch.cuda.synchronize()
+        mxm.mxm_set_workspace(None)
