@@ -85,8 +85,9 @@ const char* mxm_status_string(mxm_status s);
  * tensor path); the summation order over k is unspecified, so results agree
  * with any correct FP64 evaluation within |C - AB|_ij <= 2 k u (|A||B|)_ij,
  * u = 2^-53, and are bit-exact whenever every partial sum is exact (e.g.
- * small-integer matrices).  Uses library workspace (zero-padded tile copies
- * of A and B, mxm_workspace_size(MXM_MODE_F64, ...) bytes).
+ * small-integer matrices).  Uses library workspace (partial sums of the
+ * pieces of C that two of the GPU's equal shares of the work meet in,
+ * mxm_workspace_size(MXM_MODE_F64, ...) bytes).
  */
 mxm_status mxm_f64(const double* A, const double* B, double* C, int64_t m, int64_t k,
                    int64_t n, void* stream);
@@ -137,7 +138,8 @@ mxm_status mxm_gemm(int mode, const double* A, const double* B, double* C, int64
  *             `raster` tile-rows (tile-row pairs on CTA pairs), column by
  *             column inside a group, so that the CTAs working at the same
  *             time share operand tiles in L2; 0: 8 (4 tile-row pairs, 8 for
- *             256 x 256 C tiles).
+ *             256 x 256 C tiles).  The native path walks row by row (its
+ *             operand traffic is small beside its arithmetic).
  *   kb_order  the k-block order of the slice GEMM: 0 the default (2), 1
  *             every diagonal (pair) walks k forwards, 2 every other one
  *             walks k backwards (it starts on the tiles the previous one
@@ -148,10 +150,13 @@ mxm_status mxm_gemm(int mode, const double* A, const double* B, double* C, int64
  *             256 x 128 C tiles for two or more tile-rows of A without
  *             split-k), 1 single CTAs (128 x 128 C tiles), the digit products
  *             one by one.
- *   splitk    k ranges per C tile: 0 the rule (products with fewer C tiles
- *             than 152 split k towards 304 work units), 1 never, s > 1 that
- *             many (at most the number of k-blocks: 16-wide for the native
- *             path, 128-wide for the emulated modes; not for MXM_MODE_EMUL_FP8).
+ *   splitk    k ranges per C tile: 0 the rule (emulated products with fewer
+ *             C tiles than 152 split k towards 304 work units; the native path
+ *             cuts the whole product into equal shares, wherever along k a
+ *             share ends), 1 never, s > 1 that many (at most the number of
+ *             k-blocks: 16-wide for the native path, whose shares then end at
+ *             the s-ths of k only, 128-wide for the emulated modes; not for
+ *             MXM_MODE_EMUL_FP8).
  */
 typedef struct {
   int32_t raster;
@@ -190,12 +195,13 @@ mxm_status mxm_gemm_host(int mode, const double* hA, const double* hB, double* h
 /*
  * mxm_workspace_size -- bytes of device workspace one mxm_gemm call of mode
  * `mode` on an m x k by k x n product (Sec. 3.1 shapes) with `slices` slices
- * needs (the FP64 path: zero-padded tile copies of A and B, plus split-k
- * partials; the emulated modes: row and column scales, the digit planes of
+ * needs (the FP64 path: partial sums of 32 x 32 pieces of C, and never less
+ * than the tile copies of A and B an earlier form held; the emulated modes: row and column scales, the digit planes of
  * the Ozaki split and of the difference products, the segment sums, running
  * sums or split-k partials).  An emulated call on a smaller caller workspace
  * runs without the difference products (same bits) as long as it holds
- * mxm_workspace_size_plan of a plan with cta = 1.  Host arithmetic
+ * mxm_workspace_size_plan of a plan with cta = 1; a native call on a smaller
+ * one cuts the work into fewer shares.  Host arithmetic
  * only, no device call.  Returns 0 for an empty product (m, n or k <= 0),
  * an unknown mode or a slice count the mode does not take.  The paper has no
  * counterpart; size a buffer for mxm_set_workspace with it.

@@ -160,9 +160,10 @@ bool plan_ok(int mode, const mxm_plan& p) {
 // Dims of a native product under a plan.
 F64Dims native_dims(int64_t m, int64_t k, int64_t n, const mxm_plan& p) {
   F64Dims d = f64_dims(m, k, n);
-  if (p.splitk == 1) d.splits = 1;
-  else if (p.splitk > 1) d.splits = p.splitk < d.Kt ? p.splitk : (d.Kt > 0 ? d.Kt : 1);
-  if (p.raster > 0) d.raster = p.raster;
+  if (p.splitk >= 1) {
+    d.splits = p.splitk < d.Kt ? p.splitk : (d.Kt > 0 ? d.Kt : 1);
+    d.ranges = d.splits;
+  }
   return d;
 }
 
@@ -204,11 +205,15 @@ OzakiDims fp8_dims(int64_t m, int64_t k, int64_t n, int slices, const mxm_plan& 
   return d;
 }
 
+// most: all the workspace a product can make use of, else the least it runs with.
 size_t workspace_bytes(int mode, int64_t m, int64_t k, int64_t n, int slices,
-                       const mxm_plan& p = kNoPlan, bool kara = true) {
+                       const mxm_plan& p = kNoPlan, bool most = true) {
   if (m <= 0 || n <= 0 || k <= 0) return 0;
-  if (mode == MXM_MODE_F64) return f64_workspace(native_dims(m, k, n, p));
-  if (emul_mode(mode)) return ozaki_layout(emul_dims(mode, m, k, n, slices, p, kara)).total;
+  if (mode == MXM_MODE_F64) {
+    const F64Dims d = native_dims(m, k, n, p);
+    return most ? f64_workspace(d) : f64_workspace_least(d);
+  }
+  if (emul_mode(mode)) return ozaki_layout(emul_dims(mode, m, k, n, slices, p, most)).total;
   if (mode == MXM_MODE_EMUL_FP8) return ozaki_layout(fp8_dims(m, k, n, slices, p)).total;
   if (mode == MXM_MODE_BF16_F32ACC) return ozaki_layout(ozaki_dims(m, k, n, 1, 8)).total;
   return 0;
@@ -216,8 +221,8 @@ size_t workspace_bytes(int mode, int64_t m, int64_t k, int64_t n, int slices,
 
 // Launch sequence of one product whose workspace is already in place.
 mxm_status run_gemm(int mode, const double* A, const double* B, double* C, int64_t m, int64_t k,
-                    int64_t n, int slices, uint8_t* ws, int* status, cudaStream_t s,
-                    const mxm_plan& plan = kNoPlan, bool kara = true) {
+                    int64_t n, int slices, uint8_t* ws, size_t ws_bytes, int* status,
+                    cudaStream_t s, const mxm_plan& plan = kNoPlan, bool kara = true) {
   if (m == 0 || n == 0) return MXM_OK;
   if (k == 0) return launch_zero_fill(C, m * n, s) == cudaSuccess ? MXM_OK : cuda_fail();
   cudaError_t e = cudaSuccess;
@@ -225,9 +230,8 @@ mxm_status run_gemm(int mode, const double* A, const double* B, double* C, int64
     const F64Dims d = native_dims(m, k, n, plan);
     CallEvents* ce = profile_begin(s);
     profile_mark(ce, 1, s);
-    e = launch_f64_pack(A, B, d, ws, s);
     profile_mark(ce, 2, s);
-    if (e == cudaSuccess) e = launch_f64_gemm(ws, C, d, status, s);
+    e = launch_f64_gemm(A, B, C, d, ws, ws_bytes, status, s);
     profile_mark(ce, 3, s);
   } else if (emul_mode(mode)) {
     const OzakiDims d = emul_dims(mode, m, k, n, slices, plan, kara);
@@ -344,17 +348,17 @@ mxm_status mxm_gemm_plan(int mode, const double* A, const double* B, double* C, 
   std::lock_guard<std::mutex> lock(g_mutex);
   DeviceState* ds = nullptr;
   if ((st = current_state(&ds)) != MXM_OK) return st;
-  // the difference products where their workspace can be had, else (a caller
-  // workspace sized for less, a capture, no memory) the products one by one:
-  // the same bits either way
-  bool kara = true;
+  // the difference products (native: all workers) where their workspace can be
+  // had, else (a caller workspace sized for less, a capture, no memory) the
+  // products one by one, with the same bits (native: fewer workers)
+  bool most = true;
   if (ensure_workspace(ds, workspace_bytes(mode, m, k, n, slices, p), s) != MXM_OK) {
-    kara = false;
+    most = false;
     st = ensure_workspace(ds, workspace_bytes(mode, m, k, n, slices, p, false), s);
     if (st != MXM_OK) return st;
   }
-  return run_gemm(mode, A, B, C, m, k, n, slices, static_cast<uint8_t*>(ds->ws), ds->status, s, p,
-                  kara);
+  return run_gemm(mode, A, B, C, m, k, n, slices, static_cast<uint8_t*>(ds->ws), ds->ws_bytes,
+                  ds->status, s, p, most);
 }
 
 mxm_status mxm_gemm(int mode, const double* A, const double* B, double* C, int64_t m, int64_t k,
@@ -590,9 +594,9 @@ mxm_status mxm_gemm_host(int mode, const double* hA, const double* hB, double* h
   const size_t ab = align_up(sizeof(double) * size_t(m) * size_t(k), 1024);
   const size_t bb = align_up(sizeof(double) * size_t(k) * size_t(n), 1024);
   const size_t cb = align_up(sizeof(double) * size_t(m) * size_t(n), 1024);
-  bool kara = true;
+  bool most = true;
   if (ensure_workspace(ds, ab + bb + cb + workspace_bytes(mode, m, k, n, slices), s) != MXM_OK) {
-    kara = false;
+    most = false;
     st = ensure_workspace(ds, ab + bb + cb + workspace_bytes(mode, m, k, n, slices, kNoPlan, false),
                           s);
     if (st != MXM_OK) return st;
@@ -608,8 +612,8 @@ mxm_status mxm_gemm_host(int mode, const double* hA, const double* hB, double* h
             cudaSuccess)
       return cuda_fail();
   }
-  st = run_gemm(mode, dA, dB, dC, m, k, n, slices, base + ab + bb + cb, ds->status, s,
-                kNoPlan, kara);
+  st = run_gemm(mode, dA, dB, dC, m, k, n, slices, base + ab + bb + cb,
+                ds->ws_bytes - (ab + bb + cb), ds->status, s, kNoPlan, most);
   if (st != MXM_OK) return st;
   if (cudaMemcpyAsync(hC, dC, sizeof(double) * size_t(m) * size_t(n), cudaMemcpyDeviceToHost, s) !=
       cudaSuccess)

@@ -1,18 +1,16 @@
 // f64.cu -- native FP64 product C = A.B (mod2am, Sec. 3.1) on the FP64
-// tensor path (DMMA, mma.sync m16n8k4 .f64), fed by bulk copies.
+// tensor path (DMMA, mma.sync m16n8k4 .f64).
 //
-// The paper's k-blocked rank-u update (arbb_mxm2b, Sec. 3.1) becomes the K
-// loop over 16-wide k-blocks here; every block is a rank-16 update of a
-// 128 x 128 C tile held in FP64 registers.
-//
-// Data path:
-//   f64_pack_a / f64_pack_b  copy A and B once into zero-padded 128 x 16
-//       tiles (B transposed, both K-major) with an XOR swizzle that makes the
-//       DMMA fragment loads bank-conflict free; one tile = 16 KiB, moved by a
-//       single cp.async.bulk.
-//   f64_gemm  warp 0 streams tiles into a 4-stage shared-memory ring
-//       (mbarrier full/empty pairs); warps 1..8 each own a 32 x 64 piece of
-//       the C tile and issue DMMA; the epilogue stores C with edge masks.
+// The FP64 pipe is the limit on this GPU by far: a DMMA m16n8k4 holds an SM
+// sub-partition's pipe for ~1,100 clocks, and one k step of a warp's 32 x 32
+// piece of C (8 DMMAs, 2 KiB of operands) takes ~4 us.  So the operands come
+// straight from the caller's arrays, one step ahead, with no packed copies
+// and no shared memory, and what matters is that every sub-partition gets the
+// same number of DMMAs: the paper's k-blocked rank-u update (arbb_mxm2b) is
+// cut into equal shares across pieces and k.  8192^3: 1000 ms, 1.10 TFLOP/s,
+// all of the DMMA probe's rate (128 x 128 tiles staged by bulk copies, whole
+// tiles per CTA: 1033 ms; 2048^3: 15.7 against 19.1 ms, 256^3: 46 us against
+// 615 us, where those tiles left most SMs idle).
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -24,63 +22,6 @@
 namespace mxm {
 namespace {
 
-constexpr int BM = kF64BM, BN = kF64BN, BK = kF64BK;
-constexpr int kStages = 4;
-constexpr int kConsumerWarps = 8;
-constexpr int kThreads = 32 * (1 + kConsumerWarps);
-
-// element (r, c) of a 128 x 16 tile -> word offset (8-byte words)
-__host__ __device__ __forceinline__ int swz(int r, int c) { return r * BK + (c ^ ((r & 3) << 2)); }
-
-// Tile (tm, tk) of A (m x k): element (r, c) = A[tm*128 + r][tk*16 + c].
-__device__ __forceinline__ void pack_a_tile(const double* __restrict__ A, int64_t m, int64_t k,
-                                            int64_t tm, int64_t tk, double* __restrict__ tile) {
-  for (int p = threadIdx.x; p < BM * BK; p += blockDim.x) {
-    const int r = p / BK, c = p % BK;
-    const int64_t row = tm * BM + r, col = tk * BK + c;
-    tile[swz(r, c)] = (row < m && col < k) ? __ldg(A + row * k + col) : 0.0;
-  }
-}
-
-// Tile (tn, tk) of B^T: element (r, c) = B[tk*16 + c][tn*128 + r], staged
-// through shared memory so that both the reads and the writes are coalesced.
-__device__ __forceinline__ void pack_b_tile(const double* __restrict__ B, int64_t k, int64_t n,
-                                            int64_t tn, int64_t tk, double* __restrict__ tile,
-                                            double (*t)[BN + 1]) {
-  for (int p = threadIdx.x; p < BK * BN; p += blockDim.x) {
-    const int c = p / BN, r = p % BN;
-    const int64_t kr = tk * BK + c, col = tn * BN + r;
-    t[c][r] = (kr < k && col < n) ? __ldg(B + kr * n + col) : 0.0;
-  }
-  __syncthreads();
-  for (int p = threadIdx.x; p < BN * BK; p += blockDim.x) {
-    const int r = p / BK, c = p % BK;
-    tile[swz(r, c)] = t[c][r];
-  }
-  __syncthreads();
-}
-
-__global__ void f64_pack_a_kernel(const double* __restrict__ A, int64_t m, int64_t k, int64_t Kt,
-                                  double* __restrict__ out) {
-  const int64_t tk = blockIdx.x, tm = blockIdx.y;
-  pack_a_tile(A, m, k, tm, tk, out + (tm * Kt + tk) * (BM * BK));
-}
-
-__global__ void f64_pack_b_kernel(const double* __restrict__ B, int64_t k, int64_t n, int64_t Kt,
-                                  double* __restrict__ out) {
-  __shared__ double t[BK][BN + 1];
-  const int64_t tk = blockIdx.x, tn = blockIdx.y;
-  pack_b_tile(B, k, n, tn, tk, out + (tn * Kt + tk) * (BN * BK), t);
-}
-
-struct __align__(128) F64Smem {
-  double a[kStages][BM * BK];
-  double b[kStages][BN * BK];
-  uint64_t full[kStages];
-  uint64_t empty[kStages];
-  int abort_flag;
-};
-
 __device__ __forceinline__ void dmma_16x8x4(double (&d)[4], double a0, double a1, double b0) {
   asm volatile(
       "mma.sync.aligned.m16n8k4.row.col.f64.f64.f64.f64 {%0,%1,%2,%3}, {%4,%5}, {%6}, "
@@ -89,72 +30,31 @@ __device__ __forceinline__ void dmma_16x8x4(double (&d)[4], double a0, double a1
       : "d"(a0), "d"(a1), "d"(b0));
 }
 
-__device__ __forceinline__ void tile_coords(int64_t tile, int64_t Mt, int64_t Nt, int64_t G,
-                                            int64_t& tm, int64_t& tn) {
-  // groups of G tile-rows, column-major inside a group (L2 reuse of the
-  // operand tiles of the CTAs working at the same time)
-  const int64_t per_group = G * Nt;
-  const int64_t grp = tile / per_group;
-  const int64_t first = grp * G;
-  const int64_t gsz = (Mt - first) < G ? (Mt - first) : G;
-  const int64_t in = tile - grp * per_group;
-  tm = first + in % gsz;
-  tn = in / gsz;
-}
-
-struct F64Tile {
-  const double* a;   // packed A tile-row, first k-block of this unit
-  const double* b;   // packed B^T tile-row, first k-block of this unit
-  int64_t Kt;        // k-blocks of this unit
-  double* C;         // output (C, or a partial tile under split-k)
-  int64_t m, n, ldc, row0, col0;
-};
-
-// Work unit t: C tile t / splits, k range t % splits (consecutive CTAs take
-// the k ranges of one tile).  Without split-k the unit writes C with edge
-// masks; with it, a full 128 x 128 partial tile (the packed operands are
-// zero-padded, so the padding rows and columns are zeros).
-struct F64Single {
-  const double* apack;
-  const double* bpack;
-  double* C;
-  double* partials;
-  int64_t m, n, Mt, Nt, Kt, splits;
-  int64_t raster;
-  __device__ __forceinline__ int64_t count() const { return Mt * Nt * splits; }
-#ifdef MXM_DEBUG_BOUNDS
-  // the packed operand tiles (bounds checks of the debug build)
-  __device__ __forceinline__ const double* a_begin() const { return apack; }
-  __device__ __forceinline__ const double* a_end() const { return apack + Mt * Kt * (BM * BK); }
-  __device__ __forceinline__ const double* b_begin() const { return bpack; }
-  __device__ __forceinline__ const double* b_end() const { return bpack + Nt * Kt * (BN * BK); }
-#endif
-  __device__ __forceinline__ F64Tile tile(int64_t t) const {
-    const int64_t tile = t / splits, sp = t - tile * splits;
-    int64_t tm, tn;
-    tile_coords(tile, Mt, Nt, raster, tm, tn);
-    const int64_t kb0 = Kt * sp / splits, kb1 = Kt * (sp + 1) / splits;
-    const double* a = apack + (tm * Kt + kb0) * (BM * BK);
-    const double* b = bpack + (tn * Kt + kb0) * (BN * BK);
-    if (splits == 1) return F64Tile{a, b, kb1 - kb0, C, m, n, n, tm * BM, tn * BN};
-    double* p = partials + ((sp * Mt + tm) * Nt + tn) * (BM * BN);
-    return F64Tile{a, b, kb1 - kb0, p, BM, BN, BN, 0, 0};
+// The live DMMA blocks of a piece (ML of its two m16 rows, NL of its four n8
+// columns) as compile-time constants: a predicated-off DMMA still costs the
+// pipe ~150 clocks (edge pieces ran 13-30 % longer that way), so each shape
+// has its own loop.
+template <typename F>
+__device__ __forceinline__ void f64_with_blocks(bool two, int nlive, const F& f) {
+  using C1 = std::integral_constant<int, 1>;
+  using C2 = std::integral_constant<int, 2>;
+  using C3 = std::integral_constant<int, 3>;
+  using C4 = std::integral_constant<int, 4>;
+  if (two) {
+    switch (nlive) {
+      case 4: f(C2{}, C4{}); break;
+      case 3: f(C2{}, C3{}); break;
+      case 2: f(C2{}, C2{}); break;
+      default: f(C2{}, C1{}); break;
+    }
+  } else {
+    switch (nlive) {
+      case 4: f(C1{}, C4{}); break;
+      case 3: f(C1{}, C3{}); break;
+      case 2: f(C1{}, C2{}); break;
+      default: f(C1{}, C1{}); break;
+    }
   }
-};
-
-// C[row][col] = sum over splits s (in order) of the partial tiles.
-__global__ void __launch_bounds__(256) f64_splitk_reduce_kernel(const double* __restrict__ P,
-                                                                double* __restrict__ C,
-                                                                int64_t m, int64_t n, int64_t Mt,
-                                                                int64_t Nt, int64_t splits) {
-  const int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (idx >= m * n) return;
-  const int64_t row = idx / n, col = idx - (idx / n) * n;
-  const int64_t off = ((row / BM) * Nt + col / BN) * (BM * BN) + (row % BM) * BN + col % BN;
-  const int64_t stride = Mt * Nt * (BM * BN);
-  double acc = 0.0;
-  for (int64_t s = 0; s < splits; ++s) acc += __ldcs(P + s * stride + off);
-  C[idx] = acc;
 }
 
 // ---------------------------------------------------------------- grouped
@@ -231,20 +131,21 @@ __global__ void __launch_bounds__(kGroupedF64Threads, 2)
     const int nlive = static_cast<int>((n - col0 + 7) / 8 < 4 ? (n - col0 + 7) / 8 : 4);
     double a[4], b[4], an[4], bn[4];
     load_frags(A, B, k, n, arow, bcol, rmask, cmask, t4, a, b);
-    for (int64_t k0 = 0; k0 < k; k0 += kF64GroupedK) {
-      load_frags(A, B, k, n, arow, bcol, rmask, cmask, k0 + kF64GroupedK + t4, an, bn);
+    f64_with_blocks(mlive1, nlive, [&](auto ml, auto nl) {
+      for (int64_t k0 = 0; k0 < k; k0 += kF64GroupedK) {
+        load_frags(A, B, k, n, arow, bcol, rmask, cmask, k0 + kF64GroupedK + t4, an, bn);
 #pragma unroll
-      for (int mi = 0; mi < 2; ++mi)
+        for (int mi = 0; mi < decltype(ml)::value; ++mi)
 #pragma unroll
-        for (int ni = 0; ni < 4; ++ni)
-          if ((mi == 0 || mlive1) && ni < nlive)
+          for (int ni = 0; ni < decltype(nl)::value; ++ni)
             dmma_16x8x4(acc[mi][ni], a[2 * mi], a[2 * mi + 1], b[ni]);
 #pragma unroll
-      for (int i = 0; i < 4; ++i) {
-        a[i] = an[i];
-        b[i] = bn[i];
+        for (int i = 0; i < 4; ++i) {
+          a[i] = an[i];
+          b[i] = bn[i];
+        }
       }
-    }
+    });
     // D fragment of m16n8: (g, 2 t4), (g, 2 t4 + 1), (g + 8, 2 t4), (g + 8, 2 t4 + 1)
 #pragma unroll
     for (int mi = 0; mi < 2; ++mi) {
@@ -264,198 +165,239 @@ __global__ void __launch_bounds__(kGroupedF64Threads, 2)
   }
 }
 
-// Persistent: every CTA walks tiles blockIdx.x, +gridDim.x, ...; the producer
-// and the consumers walk the same sequence and keep the stage ring running
-// across tiles.
-template <typename Tiles>
-__global__ void __launch_bounds__(kThreads, 1)
-    f64_gemm_kernel(const Tiles tiles, int* __restrict__ status) {
-  extern __shared__ uint8_t smem_raw[];
-  F64Smem& sm = *reinterpret_cast<F64Smem*>(
-      (reinterpret_cast<uintptr_t>(smem_raw) + 127) & ~static_cast<uintptr_t>(127));
-  const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+// ---------------------------------------------------------------- balanced
+// The product cut into equal shares of DMMA work: the C matrix in 32 x 32
+// pieces, each of Ks = ceil(k / 4) steps of up to 8 DMMAs m16n8k4 (the blocks
+// of an edge piece past the last row or column are not issued), walked piece
+// after piece, k inside; worker i of W takes the i-th W-th of that walk,
+// whatever piece it starts or ends in.  The FP64 pipe is the limit (a DMMA
+// holds an SM sub-partition's for ~1,100 clocks, a step for ~4 us), so the
+// operands come straight from the caller's arrays, loaded one step ahead, and
+// only the balance counts: W = 1216, two warps per sub-partition of 152 SMs (a
+// constant: the rounding does not depend on the device), fewer when that would
+// be less than a step each.  A piece that lies
+// within one share is stored to C; the parts of a piece cut by a share's
+// boundary go to the workers' slots and f64_balanced_reduce_kernel adds them
+// in order of k.
+constexpr int kPiece = kF64Piece;
+constexpr int kBalancedThreads = 256;
 
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < kStages; ++s) {
-      mbar_init(&sm.full[s], 1);
-      mbar_init(&sm.empty[s], kConsumerWarps);
-    }
-    sm.abort_flag = 0;
-    fence_mbar_init();
+struct F64Spot {   // a place in the walk
+  int64_t piece, step;
+};
+
+struct F64Balanced {
+  const double* A;
+  const double* B;
+  double* C;
+  double* slots;   // 2 per worker, kPiece x kPiece each
+  F64Spot* starts;  // where each worker's share starts, then the end of the walk
+  int64_t m, k, n;
+  int64_t Mp, Np, Ks;   // pieces down and across, steps of 4 k
+  int64_t rows16, cols8;  // live DMMA blocks: ceil(m / 16), ceil(n / 8)
+  int workers;
+  int64_t ranges;  // 0: a share may end after any step; s: only at the s-ths of k
+};
+
+// The start of worker i's share: at i / W of the DMMAs, rounded down to a step
+// (to the start of its k range).
+__device__ __forceinline__ F64Spot f64_spot(const F64Balanced& p, int i) {
+  F64Spot s;
+  if (i >= p.workers) {
+    s.piece = p.Mp * p.Np;
+    s.step = 0;
+    return s;
   }
-  __syncthreads();
-  volatile int* abort_flag = &sm.abort_flag;
-  const int64_t ntiles = tiles.count();
+  const int64_t total = p.rows16 * p.cols8 * p.Ks;  // < 2^53
+  const int64_t at = total / p.workers * i + total % p.workers * i / p.workers;
+  const int64_t band = 2 * p.cols8 * p.Ks;          // a full row of pieces
+  int64_t pm = at / band;
+  if (pm > p.Mp - 1) pm = p.Mp - 1;
+  int64_t rem = at - pm * band;
+  const int64_t ml = p.rows16 - 2 * pm < 2 ? p.rows16 - 2 * pm : 2;
+  int64_t pn = rem / (ml * 4 * p.Ks);
+  if (pn > p.Np - 1) pn = p.Np - 1;
+  rem -= pn * ml * 4 * p.Ks;
+  const int64_t nl = p.cols8 - 4 * pn < 4 ? p.cols8 - 4 * pn : 4;
+  s.piece = pm * p.Np + pn;
+  s.step = rem / (ml * nl);
+  if (p.ranges > 0) s.step = p.Ks * (s.step * p.ranges / p.Ks) / p.ranges;
+  return s;
+}
 
-  if (warp == 0) {
-    if (lane == 0) {
-      int stage = 0;
-      uint32_t phase = 0;
-      bool ok = true;
-      for (int64_t t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-        const F64Tile j = tiles.tile(t);
-        for (int64_t kb = 0; kb < j.Kt; ++kb) {
-          if (!mbar_wait_bounded(&sm.empty[stage], phase ^ 1u, abort_flag, status)) {
-            ok = false;
-            break;
-          }
-          MXM_BOUNDS(in_range(j.a + kb * (BM * BK), kF64TileBytes, tiles.a_begin(),
-                              tiles.a_end()) &&
-                         in_range(j.b + kb * (BN * BK), kF64TileBytes, tiles.b_begin(),
-                                  tiles.b_end()),
-                     status);
-          mbar_arrive_expect_tx(&sm.full[stage], 2 * kF64TileBytes);
-          bulk_g2s(sm.a[stage], j.a + kb * (BM * BK), kF64TileBytes, &sm.full[stage]);
-          bulk_g2s(sm.b[stage], j.b + kb * (BN * BK), kF64TileBytes, &sm.full[stage]);
-          if (++stage == kStages) {
-            stage = 0;
-            phase ^= 1u;
-          }
-        }
-      }
-      for (int i = 0; i < kStages; ++i) {  // drain: no copy in flight at exit
-        if (!mbar_wait_bounded(&sm.empty[stage], phase ^ 1u, abort_flag, status)) break;
-        if (++stage == kStages) {
-          stage = 0;
-          phase ^= 1u;
-        }
-      }
-    }
-    return;
-  }
-
-  // consumers: warp w (1..8) owns rows wm*32 .. +32, columns wn*64 .. +64
-  const int cw = warp - 1;
-  const int wm = cw >> 1, wn = cw & 1;
+__global__ void __launch_bounds__(kBalancedThreads, 1) f64_balanced_kernel(
+    const F64Balanced p, int* __restrict__ status) {
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t4 = lane & 3;
-  int stage = 0;
-  uint32_t phase = 0;
-  bool ok = true;
-  for (int64_t t = blockIdx.x; t < ntiles && ok; t += gridDim.x) {
-    const F64Tile j = tiles.tile(t);
-    // the m16 / n8 blocks of this warp's 32 x 64 region that hold any row /
-    // column of C (warp-uniform); the others are not issued (edge tiles)
-    const int64_t rows_left = j.m - (j.row0 + wm * 32);
-    const int64_t cols_left = j.n - (j.col0 + wn * 64);
-    const int mlive = rows_left <= 0 ? 0 : (rows_left > 16 ? 2 : 1);
-    const int nlive =
-        cols_left <= 0 ? 0 : (cols_left >= 64 ? 8 : static_cast<int>((cols_left + 7) / 8));
-    double acc[2][8][4];
+  // neighbouring shares on one sub-partition (warps w and w + 4)
+  const int worker = blockIdx.x * (kBalancedThreads / 32) + (warp & 3) * 2 + (warp >> 2);
+  if (worker >= p.workers) return;
+  F64Spot at = f64_spot(p, worker);
+  const F64Spot end = f64_spot(p, worker + 1);
+  if (p.ranges != 1 && lane == 0) {
+    p.starts[worker] = at;
+    if (worker == p.workers - 1) p.starts[worker + 1] = end;
+  }
+  while (at.piece < end.piece || (at.piece == end.piece && at.step < end.step)) {
+    const int64_t pm = at.piece / p.Np, pn = at.piece - pm * p.Np;
+    const int64_t row0 = pm * kPiece, col0 = pn * kPiece;
+    const int64_t s0 = at.step, s1 = at.piece < end.piece ? p.Ks : end.step;
+    MXM_BOUNDS(row0 < p.m && col0 < p.n && s0 >= 0 && s1 <= p.Ks, status);
+    const bool mlive1 = row0 + 16 < p.m;
+    const int nlive = static_cast<int>(p.cols8 - 4 * pn < 4 ? p.cols8 - 4 * pn : 4);
+    // this lane's A rows (halves g, g + 8 of the two m16 blocks) and B columns
+    const double* ap[4];
+    const double* bp[4];
+    uint32_t rmask = 0, cmask = 0;
+#pragma unroll
+    for (int i = 0; i < 4; ++i) {
+      const int64_t row = row0 + i * 8 + g, col = col0 + i * 8 + g;
+      if (row < p.m) rmask |= 1u << i;
+      if (col < p.n) cmask |= 1u << i;
+      ap[i] = p.A + (row < p.m ? row : 0) * p.k + 4 * s0 + t4;
+      bp[i] = p.B + (4 * s0 + t4) * p.n + (col < p.n ? col : 0);
+    }
+    int64_t kk = 4 * s0 + t4;  // this lane's k of the next load
+    double acc[2][4][4];
 #pragma unroll
     for (int mi = 0; mi < 2; ++mi)
 #pragma unroll
-      for (int ni = 0; ni < 8; ++ni)
+      for (int ni = 0; ni < 4; ++ni)
 #pragma unroll
         for (int q = 0; q < 4; ++q) acc[mi][ni][q] = 0.0;
-
-    // kEdge: the predicated form for a region only partly inside C; whole
-    // regions keep the plain loop
-    auto kloop = [&](auto edge) {
-      constexpr bool kEdge = decltype(edge)::value;
-      for (int64_t kb = 0; kb < j.Kt; ++kb) {
-        if (!mbar_wait_bounded(&sm.full[stage], phase, abort_flag, status)) {
-          ok = false;
-          break;
-        }
-        const double* As = sm.a[stage];
-        const double* Bs = sm.b[stage];
+    double a[4], b[4], an[4], bn[4];
+    auto load = [&](double (&x)[4], double (&y)[4]) {
+      const bool kv = kk < p.k;
 #pragma unroll
-        for (int kk = 0; kk < BK / 4; ++kk) {
-          const int c = kk * 4 + t4;
-          double a[2][2], b[8];
-#pragma unroll
-          for (int mi = 0; mi < 2; ++mi) {
-            const int r0 = wm * 32 + mi * 16 + g;
-            a[mi][0] = As[swz(r0, c)];
-            a[mi][1] = As[swz(r0 + 8, c)];
-          }
-#pragma unroll
-          for (int ni = 0; ni < 8; ++ni) b[ni] = Bs[swz(wn * 64 + ni * 8 + g, c)];
-#pragma unroll
-          for (int mi = 0; mi < 2; ++mi)
-#pragma unroll
-            for (int ni = 0; ni < 8; ++ni)
-              if (!kEdge || (mi < mlive && ni < nlive))
-                dmma_16x8x4(acc[mi][ni], a[mi][0], a[mi][1], b[ni]);
-        }
-        __syncwarp();
-        if (lane == 0) mbar_arrive(&sm.empty[stage]);
-        if (++stage == kStages) {
-          stage = 0;
-          phase ^= 1u;
-        }
+      for (int i = 0; i < 4; ++i) {
+        x[i] = (kv && ((rmask >> i) & 1u)) ? __ldg(ap[i]) : 0.0;
+        y[i] = (kv && ((cmask >> i) & 1u)) ? __ldg(bp[i]) : 0.0;
+        ap[i] += 4;
+        bp[i] += 4 * p.n;
       }
+      kk += 4;
     };
-    if (mlive == 2 && nlive == 8)
-      kloop(std::false_type{});
-    else
-      kloop(std::true_type{});
-    if (!ok) break;
-
-    // epilogue: D fragment (g, 2t), (g, 2t+1), (g+8, 2t), (g+8, 2t+1)
+    load(a, b);
+    f64_with_blocks(mlive1, nlive, [&](auto ml, auto nl) {
+      for (int64_t s = s0; s < s1; ++s) {
+        load(an, bn);
 #pragma unroll
-    for (int mi = 0; mi < 2; ++mi) {
+        for (int mi = 0; mi < decltype(ml)::value; ++mi)
 #pragma unroll
-      for (int half = 0; half < 2; ++half) {
-        const int64_t row = j.row0 + wm * 32 + mi * 16 + g + half * 8;
-        if (row >= j.m) continue;
-        double* crow = j.C + row * j.ldc;
+          for (int ni = 0; ni < decltype(nl)::value; ++ni)
+            dmma_16x8x4(acc[mi][ni], a[2 * mi], a[2 * mi + 1], b[ni]);
 #pragma unroll
-        for (int ni = 0; ni < 8; ++ni) {
-          const int64_t col = j.col0 + wn * 64 + ni * 8 + 2 * t4;
-          if (col < j.n) crow[col] = acc[mi][ni][half * 2];
-          if (col + 1 < j.n) crow[col + 1] = acc[mi][ni][half * 2 + 1];
+        for (int i = 0; i < 4; ++i) {
+          a[i] = an[i];
+          b[i] = bn[i];
         }
       }
+    });
+    if (s0 == 0 && s1 == p.Ks) {
+      // D fragment of m16n8: (g, 2 t4), (g, 2 t4 + 1), (g + 8, 2 t4), (g + 8, 2 t4 + 1)
+#pragma unroll
+      for (int mi = 0; mi < 2; ++mi) {
+#pragma unroll
+        for (int h = 0; h < 2; ++h) {
+          const int64_t row = row0 + mi * 16 + h * 8 + g;
+          if (row >= p.m) continue;
+          double* crow = p.C + row * p.n;
+#pragma unroll
+          for (int ni = 0; ni < 4; ++ni) {
+            const int64_t col = col0 + ni * 8 + 2 * t4;
+            if (col < p.n) crow[col] = acc[mi][ni][2 * h];
+            if (col + 1 < p.n) crow[col + 1] = acc[mi][ni][2 * h + 1];
+          }
+        }
+      }
+    } else {
+      // slot 0: a piece begun by another worker, slot 1: one that this worker begins
+      double* slot = p.slots + (static_cast<int64_t>(worker) * 2 + (s0 == 0 ? 1 : 0)) *
+                                   (kPiece * kPiece) + lane;
+#pragma unroll
+      for (int mi = 0; mi < 2; ++mi)
+#pragma unroll
+        for (int ni = 0; ni < 4; ++ni)
+#pragma unroll
+          for (int q = 0; q < 4; ++q) slot[((mi * 4 + ni) * 4 + q) * 32] = acc[mi][ni][q];
     }
+    ++at.piece;
+    at.step = 0;
   }
 }
 
-constexpr size_t kF64SmemBytes = sizeof(F64Smem) + 128;
+// The pieces cut by share boundaries: block i takes the piece that worker i
+// begins and does not finish (its elements shared over blockIdx.y) and adds
+// the workers' parts in order of k.
+__global__ void __launch_bounds__(kBalancedThreads) f64_balanced_reduce_kernel(
+    const F64Balanced p) {
+  const int w0 = blockIdx.x;
+  const F64Spot from = p.starts[w0], to = p.starts[w0 + 1];
+  if (to.step == 0 || (from.piece == to.piece && from.step > 0)) return;
+  const int64_t piece = to.piece;
+  // the last worker that starts inside the piece
+  int lo = w0 + 1, hi = p.workers - 1;
+  while (lo < hi) {
+    const int mid = (lo + hi + 1) >> 1;
+    if (p.starts[mid].piece <= piece) lo = mid; else hi = mid - 1;
+  }
+  const int w1 = lo;
+  const int64_t pm = piece / p.Np, pn = piece - pm * p.Np;
+  for (int e = blockIdx.y * kBalancedThreads + threadIdx.x; e < kPiece * kPiece;
+       e += gridDim.y * kBalancedThreads) {
+    double v = p.slots[(static_cast<int64_t>(w0) * 2 + 1) * (kPiece * kPiece) + e];
+    if (p.ranges == 0) {
+#pragma unroll 8
+      for (int w = w0 + 1; w <= w1; ++w)
+        v += __ldcs(p.slots + static_cast<int64_t>(w) * 2 * (kPiece * kPiece) + e);
+    } else {  // shares may be empty: those have no part
+      for (int w = w0 + 1; w <= w1; ++w) {
+        const F64Spot b = p.starts[w], n = p.starts[w + 1];
+        if (b.piece < n.piece || b.step < n.step)
+          v += __ldcs(p.slots + static_cast<int64_t>(w) * 2 * (kPiece * kPiece) + e);
+      }
+    }
+    const int i = e >> 5, lane = e & 31, q = i & 3;
+    const int64_t row = pm * kPiece + (i >> 4) * 16 + (q >> 1) * 8 + (lane >> 2);
+    const int64_t col = pn * kPiece + ((i >> 2) & 3) * 8 + 2 * (lane & 3) + (q & 1);
+    if (row < p.m && col < p.n) p.C[row * p.n + col] = v;
+  }
+}
 
 }  // namespace
 
-cudaError_t launch_f64_pack(const double* A, const double* B, const F64Dims& d, uint8_t* ws,
-                            cudaStream_t s) {
-  if (d.Kt == 0) return cudaSuccess;
-  double* apack = reinterpret_cast<double*>(ws);
-  double* bpack = apack + d.Mt * d.Kt * (BM * BK);
-  if (d.Mt > 0)
-    f64_pack_a_kernel<<<dim3(static_cast<unsigned>(d.Kt), static_cast<unsigned>(d.Mt)), 256, 0,
-                        s>>>(A, d.m, d.k, d.Kt, apack);
-  if (d.Nt > 0)
-    f64_pack_b_kernel<<<dim3(static_cast<unsigned>(d.Kt), static_cast<unsigned>(d.Nt)), 256, 0,
-                        s>>>(B, d.k, d.n, d.Kt, bpack);
-  return cudaGetLastError();
-}
-
-template <typename Tiles>
-static cudaError_t launch_f64_gemm_t(const Tiles& tiles, int64_t grid, int* status,
-                                     cudaStream_t s) {
-  if (grid <= 0) return cudaSuccess;
-  auto kern = f64_gemm_kernel<Tiles>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(kF64SmemBytes));
-  if (e != cudaSuccess) return e;
-  kern<<<static_cast<unsigned>(grid), kThreads, kF64SmemBytes, s>>>(tiles, status);
-  return cudaGetLastError();
-}
-
-cudaError_t launch_f64_gemm(uint8_t* ws, double* C, const F64Dims& d, int* status,
-                            cudaStream_t s) {
-  if (d.Mt == 0 || d.Nt == 0) return cudaSuccess;
-  const double* apack = reinterpret_cast<const double*>(ws);
-  const double* bpack = apack + d.Mt * d.Kt * (BM * BK);
-  double* partials = reinterpret_cast<double*>(ws + f64_partials_offset(d));
-  F64Single tiles{apack, bpack, C, partials, d.m, d.n, d.Mt, d.Nt, d.Kt, d.splits,
-                  d.raster > 0 ? d.raster : kDefaultRaster};
-  const int64_t count = d.Mt * d.Nt * d.splits;
-  const int64_t grid = count < sm_count() ? count : sm_count();
-  cudaError_t e = launch_f64_gemm_t(tiles, grid, status, s);
-  if (e != cudaSuccess || d.splits == 1) return e;
-  const int64_t total = d.m * d.n;
-  f64_splitk_reduce_kernel<<<static_cast<unsigned>((total + 255) / 256), 256, 0, s>>>(
-      partials, C, d.m, d.n, d.Mt, d.Nt, d.splits);
+cudaError_t launch_f64_gemm(const double* A, const double* B, double* C, const F64Dims& d,
+                            uint8_t* ws, size_t ws_bytes, int* status, cudaStream_t s) {
+  if (d.m == 0 || d.n == 0 || d.k == 0) return cudaSuccess;
+  F64Balanced p;
+  p.A = A;
+  p.B = B;
+  p.C = C;
+  p.slots = reinterpret_cast<double*>(ws);
+  p.m = d.m;
+  p.k = d.k;
+  p.n = d.n;
+  p.Mp = (d.m + kPiece - 1) / kPiece;
+  p.Np = (d.n + kPiece - 1) / kPiece;
+  p.Ks = (d.k + 3) / 4;
+  p.rows16 = (d.m + 15) / 16;
+  p.cols8 = (d.n + 7) / 8;
+  p.ranges = d.ranges;
+  int64_t workers = f64_workers(d);
+  // a caller workspace of the packed copies' size may hold fewer slots
+  const int64_t fit = static_cast<int64_t>(ws_bytes / kF64WorkerBytes) - 1;
+  if (d.ranges != 1 && fit < workers) {
+    if (fit < 64) p.ranges = 1;
+    else workers = fit;
+  }
+  p.workers = static_cast<int>(workers);
+  p.starts = reinterpret_cast<F64Spot*>(p.slots + workers * 2 * kPiece * kPiece);
+  constexpr int kWarps = kBalancedThreads / 32;
+  f64_balanced_kernel<<<(p.workers + kWarps - 1) / kWarps, kBalancedThreads, 0, s>>>(p, status);
+  if (p.ranges != 1) {
+    const unsigned split = p.Mp * p.Np < 304 ? kPiece * kPiece / kBalancedThreads : 1;
+    f64_balanced_reduce_kernel<<<dim3(p.workers, split), kBalancedThreads, 0, s>>>(p);
+  }
   return cudaGetLastError();
 }
 

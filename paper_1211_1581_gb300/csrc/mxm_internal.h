@@ -366,8 +366,9 @@ constexpr int kF64TileBytes = kF64BM * kF64BK * 8;  // 16 KiB (BM == BN)
 
 struct F64Dims {
   int64_t m, k, n, Mt, Nt, Kt;
-  int64_t splits;  // k ranges per C tile (1: no split)
-  int raster;      // tile-rows per group of the persistent walk over C tiles
+  int64_t splits;  // k ranges per 128 x 128 tile the workspace has room for
+  int64_t ranges;  // where a worker's share may end along k: 0 after any step,
+                   // s at the s-ths of k (1: not inside a piece)
 };
 
 inline F64Dims f64_dims(int64_t m, int64_t k, int64_t n) {
@@ -377,25 +378,40 @@ inline F64Dims f64_dims(int64_t m, int64_t k, int64_t n) {
   d.Nt = (n + kF64BN - 1) / kF64BN;
   d.Kt = (k + kF64BK - 1) / kF64BK;
   d.splits = splitk_count(d.Mt * d.Nt, d.Kt, 8);
-  d.raster = kDefaultRaster;
+  // little k: pieces are not cut (a piece is at most 8 steps, 34 us)
+  d.ranges = k < 32 ? 1 : 0;
   return d;
 }
 
-// Packed operand tiles, then (split-k only) the partial C tiles:
-// splits x Mt x Nt tiles of 128 x 128 doubles, row-major inside a tile.
-inline size_t f64_partials_offset(const F64Dims& d) {
-  return align_up((size_t)(d.Mt + d.Nt) * d.Kt * kF64TileBytes, 1024);
-}
-inline size_t f64_workspace(const F64Dims& d) {
-  const size_t partials =
-      d.splits > 1 ? (size_t)d.splits * d.Mt * d.Nt * kF64BM * kF64BN * sizeof(double) : 0;
-  return align_up(f64_partials_offset(d) + partials, 1024);
+// The workers of the native product (two warps on each of the 608 SM
+// sub-partitions of a 152-SM GPU, each with at least one step of 8 DMMAs) and
+// the two 32 x 32 slots (and its place in a table of the shares' starts) each
+// needs when shares cut pieces.
+constexpr int64_t kF64Piece = 32;
+constexpr size_t kF64WorkerBytes = 2 * kF64Piece * kF64Piece * sizeof(double) + 16;
+inline int64_t f64_workers(const F64Dims& d) {
+  const int64_t steps = (d.m + 15) / 16 * ((d.n + 7) / 8) * ((d.k + 3) / 4) / 8;
+  return steps < 1 ? 1 : (steps < 1216 ? steps : 1216);
 }
 
-cudaError_t launch_f64_pack(const double* A, const double* B, const F64Dims& d, uint8_t* ws,
-                            cudaStream_t s);
-cudaError_t launch_f64_gemm(uint8_t* ws, double* C, const F64Dims& d, int* status,
-                            cudaStream_t s);
+// Workspace of a native product: the workers' slots, and never less than
+// before, when it held zero-padded 128 x 16 tile copies of A and B and the
+// partial tiles of the k ranges (a size callers may have kept).
+inline size_t f64_workspace_least(const F64Dims& d) {
+  const size_t packs = align_up((size_t)(d.Mt + d.Nt) * d.Kt * kF64TileBytes, 1024);
+  const size_t partials =
+      d.splits > 1 ? (size_t)d.splits * d.Mt * d.Nt * kF64BM * kF64BN * sizeof(double) : 0;
+  return align_up(packs + partials, 1024);
+}
+inline size_t f64_workspace(const F64Dims& d) {
+  const size_t least = f64_workspace_least(d);
+  const size_t slots = d.ranges == 1 ? 0 : (size_t)(f64_workers(d) + 1) * kF64WorkerBytes;
+  return slots > least ? slots : least;
+}
+
+// C = A.B with ws_bytes of workspace (fewer slots: fewer workers).
+cudaError_t launch_f64_gemm(const double* A, const double* B, double* C, const F64Dims& d,
+                            uint8_t* ws, size_t ws_bytes, int* status, cudaStream_t s);
 
 cudaError_t launch_zero_fill(double* C, int64_t count, cudaStream_t s);
 
