@@ -259,17 +259,29 @@ inline int kara_max_segment(int S) { return S / 2 + 1; }
 // 256 x 256 C tiles of the CTA pairs; the pairs of a 152-SM GPU (a constant,
 // so that the workspace is host arithmetic); the scratch: S slots per tile
 // and CTA of the pair, and those of the tiles cut into units (fewer than the
-// pairs, 2 S - 2 slots each and k range; the cut stays within them).
+// pairs, or all where k is cut for the sums' sake; 2 S - 2 slots per tile and
+// k range; the cut stays within them).
 constexpr int64_t kKaraPairs = 76;
 constexpr size_t kKaraSlotBytes = (size_t)kOzTileRows * 256 * 4;
 inline int64_t kara_tiles(const OzakiDims& d) { return (d.Mt + 1) / 2 * ((d.Nt + 1) / 2); }
+// The k ranges that keep every sum of a range in int32 (1 unless k is long
+// for the digits: S = 6 of 8 bits beyond 4,718).
+inline int kara_min_ranges(const OzakiDims& d) {
+  if (ozaki_narrow(d)) return 1;
+  const double dmax = static_cast<double>(ozaki_dmax(d));
+  const int64_t most =
+      static_cast<int64_t>(2147483647.0 / ((d.S + 1) * dmax * dmax * kOzTileK));
+  return most < 1 ? 0 : static_cast<int>((d.Kt + most - 1) / most);
+}
 inline size_t kara_cut_slots(const OzakiDims& d) {
-  const int64_t t = kara_tiles(d), cut = t < kKaraPairs ? t : kKaraPairs;
-  const size_t slots = (size_t)cut * (2 * d.S - 2);
+  const int64_t t = kara_tiles(d), r = kara_min_ranges(d);
+  const int64_t cut = t < kKaraPairs || r > 1 ? t : kKaraPairs;
+  const size_t slots = (size_t)cut * r * (2 * d.S - 2);
   return slots > 3 * (size_t)kKaraPairs ? slots : 3 * (size_t)kKaraPairs;
 }
 inline size_t kara_scratch_bytes(const OzakiDims& d) {
-  return 2 * kKaraSlotBytes * ((size_t)kara_tiles(d) * d.S + kara_cut_slots(d));
+  const size_t whole = kara_min_ranges(d) > 1 ? 0 : (size_t)kara_tiles(d) * d.S;
+  return 2 * kKaraSlotBytes * (whole + kara_cut_slots(d));
 }
 
 // Host form of the kernels' oz_exact_from: the first diagonal of the FP64
@@ -289,8 +301,8 @@ inline int ozaki_exact_from(int S, int beta, int64_t Kt) {
 
 // Which products can take the difference products.
 inline bool kara_fits(const OzakiDims& d) {
-  return !d.fp8 && d.S >= 3 && d.S <= kKaraMaxSlices && d.beta * d.S <= 64 && ozaki_narrow(d) &&
-         d.Kt > 0 && d.Mt >= 2 && d.Nt >= 2 && kara_tiles(d) < (1 << 24);
+  return !d.fp8 && d.S >= 3 && d.S <= kKaraMaxSlices && d.beta * d.S <= 64 && d.Kt > 0 &&
+         kara_min_ranges(d) >= 1 && kara_min_ranges(d) <= 16 && d.Mt >= 2 && d.Nt >= 2 && kara_tiles(d) < (1 << 24);
 }
 
 inline OzakiLayout ozaki_layout(const OzakiDims& d) {

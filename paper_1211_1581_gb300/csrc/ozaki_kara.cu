@@ -204,13 +204,20 @@ __device__ __forceinline__ double i64_pow2(long long y, int p) {
 // g >= gx, FP64 additions after).  Straight-line over the longest list (D_2
 // apart: indexed by S it would put the list into local memory); the bounds
 // are uniform.
-__device__ __forceinline__ void fold_columns(const int (&d)[kMaxS - 1][4], const int (&d2)[4],
+// Sum: int, or long long where a D_g may pass 2^31.
+__device__ __forceinline__ double sum_pow2(int d, int p) { return i32_times_pow2(d, p); }
+__device__ __forceinline__ double sum_pow2(long long d, int p) { return i64_pow2(d, p); }
+template <typename Sum>
+__device__ __forceinline__ void fold_columns(const Sum (&d)[kMaxS - 1][4], const Sum (&d2)[4],
                                              int S, int beta, int gx, double (&out)[4]) {
   long long y[4];
 #pragma unroll
   for (int c = 0; c < 4; ++c) y[c] = d[0][c];  // diagonal S + 1 is always exact
-  auto exact = [&](const int (&v)[4], int sh) {
-    if (sh < 31) {
+  auto exact = [&](const Sum (&v)[4], int sh) {
+    if constexpr (sizeof(Sum) == 8) {
+#pragma unroll
+      for (int c = 0; c < 4; ++c) y[c] += static_cast<long long>(static_cast<uint64_t>(v[c]) << sh);
+    } else if (sh < 31) {
       const int w = 1 << sh;
 #pragma unroll
       for (int c = 0; c < 4; ++c) y[c] += static_cast<long long>(v[c]) * w;  // one IMAD.WIDE
@@ -232,12 +239,12 @@ __device__ __forceinline__ void fold_columns(const int (&d)[kMaxS - 1][4], const
     const int g = S + 1 - i;
     if (g >= 3 && g < gx) {  // uniform
 #pragma unroll
-      for (int c = 0; c < 4; ++c) out[c] = __dadd_rn(out[c], i32_times_pow2(d[i][c], -beta * g));
+      for (int c = 0; c < 4; ++c) out[c] = __dadd_rn(out[c], sum_pow2(d[i][c], -beta * g));
     }
   }
   if (gx > 2) {
 #pragma unroll
-    for (int c = 0; c < 4; ++c) out[c] = __dadd_rn(out[c], i32_times_pow2(d2[c], -beta * 2));
+    for (int c = 0; c < 4; ++c) out[c] = __dadd_rn(out[c], sum_pow2(d2[c], -beta * 2));
   }
 }
 
@@ -556,8 +563,9 @@ __device__ __forceinline__ void add4(int (&v)[4], const int4& x) {
 // with all its slot reads in flight at once.  Bound by HBM (4 S bytes read and
 // 8 written per element; S = 7 at 8192^2: 2.4 GB).  kCut: the tiles cut into
 // units (2 S - 2 slots per k range), else the whole tiles (S slots).
+// Sum: the type of D_g; every k range's part of it fits int32.
 constexpr int kFoldThreads = 128;
-template <bool kCut>
+template <bool kCut, typename Sum>
 __global__ void __launch_bounds__(kFoldThreads) oz_kara_fold_kernel(
     const __grid_constant__ KaraArgs a, int part0) {
   constexpr int kSlotVec = kSlotInts / 4;
@@ -570,20 +578,23 @@ __global__ void __launch_bounds__(kFoldThreads) oz_kara_fold_kernel(
   const int64_t row = (2 * static_cast<int64_t>(tm) + rank) * kOzTileRows + (v & 127);
   const int64_t col = static_cast<int64_t>(tn) * kN + 4 * (v >> 7);
   if (row >= a.m || col >= a.n) return;
-  int d[kMaxS - 1][4], d2[4];  // D_{S+1} .. D_3, and D_2
+  Sum d[kMaxS - 1][4], d2[4];  // D_{S+1} .. D_3, and D_2
   if constexpr (kCut) {
-    // N_g and P_s, added over the k ranges; T_g = P_1 + .. + P_{g-1},
-    // D_g = T_g + N_g (and T_S for D_{S+1}), D_2 = P_1
+    // N_g and P_s; T_g = P_1 + .. + P_{g-1}, D_g = T_g + N_g (and T_S for
+    // D_{S+1}), D_2 = P_1.  With int32 D_g the k ranges' N_g and P_s are
+    // added first, with 64-bit ones each range's D_g are.
+    constexpr bool kWide = sizeof(Sum) == 8;
     const size_t range = 2 * static_cast<size_t>(2 * S - 2) * kSlotVec;
     const int4* p = a.cut_scratch + static_cast<size_t>(part >> 1) * a.ranges * range +
                     static_cast<size_t>(rank) * (2 * S - 2) * kSlotVec + v;
-    int sq[kMaxS - 1][4];  // P_{S-1} .. P_1
+    int ng[kMaxS - 1][4], sq[kMaxS - 1][4];  // N_{S+1} .. N_3, P_{S-1} .. P_1
+    auto clear = [&]() {
 #pragma unroll
-    for (int i = 0; i < kMaxS - 1; ++i)
+      for (int i = 0; i < kMaxS - 1; ++i)
 #pragma unroll
-      for (int j = 0; j < 4; ++j) d[i][j] = sq[i][j] = 0;
-#pragma unroll 1
-    for (int r = 0; r < a.ranges; ++r) {
+        for (int j = 0; j < 4; ++j) ng[i][j] = sq[i][j] = 0;
+    };
+    auto read = [&]() {
       int4 x[kMaxS - 1], y[kMaxS - 1];
 #pragma unroll
       for (int i = 0; i < kMaxS - 1; ++i)
@@ -594,24 +605,44 @@ __global__ void __launch_bounds__(kFoldThreads) oz_kara_fold_kernel(
 #pragma unroll
       for (int i = 0; i < kMaxS - 1; ++i)
         if (i < S - 1) {
-          add4(d[i], x[i]);
+          add4(ng[i], x[i]);
           add4(sq[i], y[i]);
         }
       p += range;
-    }
-    int T[4] = {0, 0, 0, 0};
-#pragma unroll
-    for (int i = kMaxS - 1; i >= 1; --i) {  // up from P_1 (zeros before it): sq[i - 1] = P_{S-i}
+    };
+    auto combine = [&]() {
+      int T[4];
 #pragma unroll
       for (int j = 0; j < 4; ++j) {
-        T[j] += sq[i - 1][j];
-        if (i == kMaxS - 1) d2[j] = T[j];
-        else if (i < S - 1) d[i][j] += T[j];
-        if (i <= S - 1 && i + 1 > S - 1) d2[j] = T[j];  // P_1 alone
+        T[j] = sq[kMaxS - 2][j];  // up from P_1 (zeros before it): sq[i - 1] = P_{S-i}
+        if (S == kMaxS) d2[j] += T[j];
       }
-    }
 #pragma unroll
-    for (int j = 0; j < 4; ++j) d[0][j] += T[j];
+      for (int i = kMaxS - 2; i >= 1; --i) {
+#pragma unroll
+        for (int j = 0; j < 4; ++j) {
+          T[j] += sq[i - 1][j];
+          if (i == S - 1) d2[j] += T[j];  // P_1 alone
+          if (i < S - 1) d[i][j] += ng[i][j] + T[j];
+        }
+      }
+#pragma unroll
+      for (int j = 0; j < 4; ++j) d[0][j] += ng[0][j] + T[j];
+    };
+#pragma unroll
+    for (int j = 0; j < 4; ++j) {
+      d2[j] = 0;
+#pragma unroll
+      for (int i = 0; i < kMaxS - 1; ++i) d[i][j] = 0;
+    }
+    clear();
+#pragma unroll 1
+    for (int r = 0; r < a.ranges; ++r) {
+      if (kWide && r > 0) clear();
+      read();
+      if (kWide) combine();
+    }
+    if (!kWide) combine();
   } else {
     const int4* p = a.full_scratch + static_cast<size_t>(part) * S * kSlotVec + v;
 #pragma unroll
@@ -697,16 +728,19 @@ int cut_segments(const KaraProg& pr, int parts, uint8_t* part) {
 // segments times ranges of k), by an estimate in k-blocks of one product (0.53
 // us): the waves of units, each with its longest run of products, 2 per
 // segment for its slot, and the fold's reading of the slots.  false: whole.
+// Never fewer ranges than keep a range's sums in int32.
 bool choose_cut(const OzakiDims& d, int64_t rest, int64_t pairs, KaraArgs& a) {
+  const int least = kara_min_ranges(d);
   const int total = a.prog.end[a.prog.nseg - 1], nslots = 2 * d.S - 2;
   const double slot_read = 0.25;  // 2 x 128 KiB at about 2 TB/s
   double best = static_cast<double>(d.Kt) * total + 2.0 * a.prog.nseg + slot_read * rest * d.S;
+  if (least > 1) best = 1e30;
   int best_parts = 1, best_ranges = 1;
   uint8_t part[kMaxSegs + 1];
   for (int parts = 1; parts <= a.prog.nseg; ++parts) {
     const int worst = cut_segments(a.prog, parts, part);
     const int segs = (a.prog.nseg + parts - 1) / parts;
-    for (int ranges = 1; ranges <= 16 && ranges <= d.Kt; ++ranges) {
+    for (int ranges = least; ranges < least + 16 && ranges <= d.Kt; ++ranges) {
       if (static_cast<size_t>(rest * ranges * nslots) > kara_cut_slots(d)) break;
       const int64_t waves = (rest * parts * ranges + pairs - 1) / pairs;
       const double cost = waves * (static_cast<double>((d.Kt + ranges - 1) / ranges) * worst +
@@ -777,7 +811,8 @@ cudaError_t launch_ozaki_kara(const uint8_t* aslices, const uint8_t* bslices,
   // whole waves of tiles, then the rest, cut where that is shorter
   const int64_t tiles = kara_tiles(d);
   a.tiles = static_cast<int>(tiles);
-  const int64_t rest = tiles % pairs;
+  const bool wide = kara_min_ranges(d) > 1;  // every tile is cut along k
+  const int64_t rest = wide ? tiles : tiles % pairs;
   a.full_tiles = static_cast<int>(tiles - rest);
   a.parts = a.ranges = 1;
   if (rest > 0 && !choose_cut(d, rest, pairs, a)) a.full_tiles = a.tiles;
@@ -790,15 +825,17 @@ cudaError_t launch_ozaki_kara(const uint8_t* aslices, const uint8_t* bslices,
   if (e != cudaSuccess) return e;
   // (tile, rank) parts on the y axis of the grid, at most kFoldParts per launch
   constexpr int64_t kFoldParts = 32768;
-  const unsigned bx = kSlotInts / 4 / kFoldThreads;
-  for (int64_t p0 = 0, all = 2 * static_cast<int64_t>(a.full_tiles); p0 < all; p0 += kFoldParts) {
-    const int64_t now = all - p0 < kFoldParts ? all - p0 : kFoldParts;
-    oz_kara_fold_kernel<false><<<dim3(bx, static_cast<unsigned>(now)), kFoldThreads, 0, s>>>(
-        a, static_cast<int>(p0));
-  }
-  if (a.tiles > a.full_tiles)
-    oz_kara_fold_kernel<true><<<dim3(bx, 2u * static_cast<unsigned>(a.tiles - a.full_tiles)),
-                                kFoldThreads, 0, s>>>(a, 0);
+  auto fold = [&](auto kern, int64_t parts) {
+    for (int64_t p0 = 0; p0 < parts; p0 += kFoldParts) {
+      const int64_t now = parts - p0 < kFoldParts ? parts - p0 : kFoldParts;
+      kern<<<dim3(kSlotInts / 4 / kFoldThreads, static_cast<unsigned>(now)), kFoldThreads, 0, s>>>(
+          a, static_cast<int>(p0));
+    }
+  };
+  fold(oz_kara_fold_kernel<false, int>, 2 * static_cast<int64_t>(a.full_tiles));
+  const int64_t cut = 2 * (tiles - a.full_tiles);
+  if (wide) fold(oz_kara_fold_kernel<true, long long>, cut);
+  else fold(oz_kara_fold_kernel<true, int>, cut);
   return cudaGetLastError();
 }
 

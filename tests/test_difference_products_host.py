@@ -49,7 +49,10 @@ int main() {
   CHECK(!kara_chosen(ozaki_dims(1024, 1024, 1024, 2, 7)));
   CHECK(!kara_chosen(ozaki_dims(1024, 1024, 1024, 10, 7)));
   CHECK(kara_chosen(ozaki_dims(8192, 8192, 8192, 7, 7)));
-  CHECK(!kara_chosen(ozaki_dims(8192, 8192, 8192, 6, 8)));      // D_g beyond int32
+  d = ozaki_dims(8192, 8192, 8192, 6, 8);  // D_g beyond int32: k in ranges within it
+  CHECK(kara_chosen(d) && kara_min_ranges(d) == 2 && !ozaki_narrow(d));
+  CHECK(7.0 * 255 * 255 * 128 * ((d.Kt + 1) / 2) < 2147483648.0);
+  CHECK(kara_min_ranges(ozaki_dims(8192, 8192, 8192, 7, 7)) == 1);
   CHECK(kara_chosen(ozaki_dims(8192, 8192, 8192, 6, 8, true)));
   CHECK(!kara_chosen(ozaki_dims(65536, 16384, 65536, 7, 7)));   // memory
   std::printf("%s %d\n", fails ? "FAILED" : "ok", fails);

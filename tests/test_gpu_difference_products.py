@@ -35,6 +35,8 @@ def _emulated(A, B, mode, S):
     (mxm.MODE_EMUL_BF16, 3, 200, 300, 200),
     (mxm.MODE_EMUL_BF16, 6, 300, 1777, 257),   # windows of two k-blocks
     (mxm.MODE_EMUL_BF16, 8, 257, 400, 513),
+    (mxm.MODE_EMUL_BF16, 6, 257, 6000, 300),   # sums beyond int32: k in ranges
+    (mxm.MODE_EMUL_I8, 7, 130, 20000, 257),
     (mxm.MODE_EMUL_RN8, 3, 129, 100, 257),
     (mxm.MODE_EMUL_RN8, 6, 385, 1300, 300),
     (mxm.MODE_EMUL_RN8, 7, 300, 140, 300),
