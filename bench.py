@@ -758,7 +758,7 @@ def run_cg_suite(emit, stream, only=""):
     """Conjugate gradients (Sec. 3.4): the Table 2 orders and bandwidths,
     the largest order of the cluster engine and a 10^6 order, each solved
     to r2 <= 1e-24 (b, b) by each engine that takes it (the cluster engine:
-    one launch; the graph engine: one graph launch).  Rate in the paper's
+    one launch on a cluster; over all SMs: one cooperative launch).  Rate in the paper's
     terms: FP64 operations of the steps taken (2 nnz + 10 n per step) over
     the solve time (CUDA events).  The CPU line is the oracle's solve,
     timed on the host."""

@@ -336,11 +336,11 @@ mxm_status mxm_spmv(const double* matvals, const int32_t* indx, const int32_t* r
 
 /* Engines of mxm_cg. */
 enum {
-  MXM_CG_AUTO = 0,     /* the cluster engine for n <= mxm_cg_max_n() and small nnz
-                          (or when work is NULL), else the graph engine */
+  MXM_CG_AUTO = 0,     /* the cluster engine for n <= mxm_cg_max_n() and small n and nnz
+                          (or when work is NULL), else the engine over all SMs */
   MXM_CG_CLUSTER = 1,  /* one launch on a thread-block cluster of up to 16 CTAs */
-  MXM_CG_GRAPH = 2     /* a CUDA graph: the loop is a conditional WHILE node over three
-                          kernels on all SMs; needs `work`; not inside a stream capture */
+  MXM_CG_GRAPH = 2     /* one cooperative launch over all SMs; needs `work`; not inside a
+                          stream capture */
 };
 
 /*
@@ -359,7 +359,7 @@ enum {
  *   x                     the solution, n doubles (written);
  *   engine                MXM_CG_AUTO, MXM_CG_CLUSTER or MXM_CG_GRAPH;
  *   work                  mxm_cg_workspace_size(n) bytes of scratch for the
- *                         graph engine (may be NULL for the cluster engine);
+ *                         engine over all SMs (may be NULL for the cluster engine);
  *   iters                 one int32: the number of steps taken;
  *   r2                    one double: the last (r, r) (the recursive
  *                         residual, as the paper's loop test uses it);
@@ -371,9 +371,9 @@ enum {
  * row pointer or column outside the arrays) is skipped and recorded as
  * MXM_ERR_INVALID_ARG in the device status word; x is then unspecified.
  * Host-side errors: n <= 0, max_iters < 0, an unknown engine, NULL or
- * overlapping arrays, the graph engine without work: MXM_ERR_INVALID_ARG;
- * the cluster engine with n > mxm_cg_max_n(), n or nnz > INT32_MAX, the graph
- * engine inside a stream capture: MXM_ERR_UNSUPPORTED; misaligned
+ * overlapping arrays, the engine over all SMs without work: MXM_ERR_INVALID_ARG;
+ * the cluster engine with n > mxm_cg_max_n(), n or nnz > INT32_MAX, the engine
+ * over all SMs inside a stream capture: MXM_ERR_UNSUPPORTED; misaligned
  * pointers: MXM_ERR_ALIGNMENT; a failed launch: MXM_ERR_CUDA.
  */
 mxm_status mxm_cg(const double* matvals, const int32_t* indx, const int32_t* rowp,
@@ -381,7 +381,7 @@ mxm_status mxm_cg(const double* matvals, const int32_t* indx, const int32_t* row
                   int32_t max_iters, int32_t engine, double* work, int32_t* iters, double* r2,
                   double* r2_hist, void* stream);
 
-/* mxm_cg_workspace_size -- bytes of `work` the graph engine needs for order n
+/* mxm_cg_workspace_size -- bytes of `work` the engine over all SMs needs for order n
  * (r, p, q and the blocks' shares of the dot products). */
 size_t mxm_cg_workspace_size(int64_t n);
 

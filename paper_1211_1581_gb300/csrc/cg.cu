@@ -48,8 +48,8 @@
 namespace mxm {
 
 int* device_status_word();  // abi.cu
-size_t cg_graph_workspace_bytes(int64_t n);  // cg_graph.cu
-mxm_status cg_graph_solve(const double* vals, const int32_t* indx, const int32_t* rowp,
+size_t cg_grid_workspace_bytes(int64_t n);  // cg_grid.cu
+mxm_status cg_grid_solve(const double* vals, const int32_t* indx, const int32_t* rowp,
                           const double* b, double* x, double* work, int32_t* iters, double* r2,
                           double* r2_hist, int64_t n, int64_t nnz, double stop,
                           int32_t max_iters, int* status, cudaStream_t s);
@@ -440,13 +440,24 @@ using namespace mxm;
 extern "C" int64_t mxm_cg_max_n(void) { return kCgMaxN; }
 
 extern "C" size_t mxm_cg_workspace_size(int64_t n) {
-  return n > 0 ? cg_graph_workspace_bytes(n) : 0;
+  return n > 0 ? cg_grid_workspace_bytes(n) : 0;
 }
 
-// Matrices whose product has more values than this go to the graph engine
-// by default: one cluster's 16 SMs then spend longer on the FP64 work of a
-// step than the graph engine's three launches over all SMs cost.
-constexpr int64_t kCgClusterMaxNnz = 524288;
+// The automatic choice.  Measured per step: the cluster engine 4.7 us plus
+// 0.58 ns a row plus 0.020 ns a value (one cluster's 16 SMs: n = 1024 with 127
+// diagonals 8.0 us, 511 14.3 us; n = 12288 with 3 diagonals 11.6 us), the
+// engine over all SMs 11 us and little more (13.3, 11.3 us): the line is where
+// the two meet.  Inside a stream capture, which the engine over all SMs
+// refuses, the cluster engine keeps every matrix of up to kCgCaptureMaxNnz
+// values.
+constexpr int64_t kCgCaptureMaxNnz = 524288;
+static bool cg_auto_cluster(int64_t n, int64_t nnz, bool no_work, cudaStream_t s) {
+  if (n > kCgMaxN) return false;
+  if (no_work || 29 * n + nnz <= 375000) return true;
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  return nnz <= kCgCaptureMaxNnz && cudaStreamIsCapturing(s, &cap) == cudaSuccess &&
+         cap != cudaStreamCaptureStatusNone;
+}
 
 extern "C" mxm_status mxm_cg(const double* matvals, const int32_t* indx, const int32_t* rowp,
                              const double* b, double* x, int64_t n, int64_t nnz, double stop,
@@ -459,8 +470,9 @@ extern "C" mxm_status mxm_cg(const double* matvals, const int32_t* indx, const i
     return MXM_ERR_INVALID_ARG;
   if (nnz > INT32_MAX || n > INT32_MAX) return MXM_ERR_UNSUPPORTED;
   if (engine == MXM_CG_AUTO)
-    engine = (n <= kCgMaxN && (nnz <= kCgClusterMaxNnz || work == nullptr)) ? MXM_CG_CLUSTER
-                                                                           : MXM_CG_GRAPH;
+    engine = cg_auto_cluster(n, nnz, work == nullptr, static_cast<cudaStream_t>(stream))
+                 ? MXM_CG_CLUSTER
+                 : MXM_CG_GRAPH;
   if (engine == MXM_CG_CLUSTER && n > kCgMaxN) return MXM_ERR_UNSUPPORTED;
   if (rowp == nullptr || b == nullptr || x == nullptr || iters == nullptr ||
       r2 == nullptr || (nnz > 0 && (matvals == nullptr || indx == nullptr)) ||
@@ -478,7 +490,7 @@ extern "C" mxm_status mxm_cg(const double* matvals, const int32_t* indx, const i
     return a0 < b0 + qb && b0 < a0 + pb;
   };
   const size_t vb = static_cast<size_t>(n) * sizeof(double);
-  const size_t wb = engine == MXM_CG_GRAPH ? cg_graph_workspace_bytes(n) : 0;
+  const size_t wb = engine == MXM_CG_GRAPH ? cg_grid_workspace_bytes(n) : 0;
   const void* outs[2] = {x, work};
   const size_t outb[2] = {vb, wb};
   for (int o = 0; o < 2; ++o) {
@@ -493,7 +505,7 @@ extern "C" mxm_status mxm_cg(const double* matvals, const int32_t* indx, const i
   int* status = device_status_word();
   if (status == nullptr) return MXM_ERR_CUDA;
   if (engine == MXM_CG_GRAPH)
-    return cg_graph_solve(matvals, indx, rowp, b, x, work, iters, r2, r2_hist, n, nnz, stop,
+    return cg_grid_solve(matvals, indx, rowp, b, x, work, iters, r2, r2_hist, n, nnz, stop,
                           max_iters, status, static_cast<cudaStream_t>(stream));
   CgArgs a;
   a.vals = matvals;

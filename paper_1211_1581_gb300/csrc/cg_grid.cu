@@ -1,0 +1,421 @@
+// cg_grid.cu -- conjugate gradients (Sec. 3.4) for systems too large for one
+// thread-block cluster: the paper's `_while` loop runs inside one cooperative
+// launch over all SMs, a block per SM, with three grid barriers a step:
+//
+//   product    q = A p on the block's own rows and its share of (p, q);
+//   residual   (p, q) = the shares added in block order (the same sum in
+//              every block); alpha = r2 / (p, q); r -= alpha q and the
+//              block's share of (r, r);
+//   direction  r2_new = the shares in block order; beta = r2_new / r2;
+//              x += alpha p, p = r + beta p.
+//
+// Measured per step against three kernels in a conditional graph node (12 us
+// of launches a step, every vector through memory): n = 10^6 with 7 diagonals
+// 36.1 against 98.6 us (the FP64 pipe's share of it 19 us), 300,000 with 21
+// 30.9 against 57.6, 12,288 with 511 25.7 against 46, 13,000 with 3 11.5
+// against 16.2 (three barriers of 1.2 us, two dot products of 2 us each and
+// the latency of one gather).
+//
+// Rows are shared out by number: block b of kCgBlocks owns rows
+// [b n / kCgBlocks, (b + 1) n / kCgBlocks), its q, r and x live in shared
+// memory when they fit (n up to ~1.4 million), p, gathered by everybody, in
+// global memory.  The product is bound by the FP64 pipe on this GPU (a
+// warp-wide fused multiply-add holds an SM sub-partition 64 clocks, however
+// many lanes are live) and by latency, so a row is given as few lanes as keep
+// every thread on rows (one lane a row from 156,000 rows on: no shuffle tree,
+// all 32 lanes live; the lanes' strided loads of values and columns meet in
+// L1), and a lane has eight values, columns and gathers in flight.
+//
+// The number of blocks and the lanes per row depend on n and nnz only, and
+// every sum has a fixed order: the rounding of a solve does not depend on the
+// device (a device with room for fewer blocks gives each several).  Every
+// wait at a barrier is bounded: after kWaitLimitNs it raises the abort word,
+// records MXM_ERR_TIMEOUT and every block leaves.
+#include <cuda_runtime.h>
+
+#include <cstdint>
+
+#include "mxm.h"
+#include "mxm_internal.h"
+
+namespace mxm {
+
+namespace {
+
+constexpr int kCgGThreads = 1024;
+constexpr int kCgGWarps = kCgGThreads / 32;
+constexpr int kCgBlocks = 152;        // row shares (one per SM of a GB300), as a constant
+constexpr int64_t kCgGMaxShares = 1216;  // doubles per share table in the workspace
+constexpr int kBatch = 8;             // values, columns and gathers of a lane in flight
+
+struct CgState {
+  unsigned long long arrived;  // barrier arrivals since the start
+  int abort;
+};
+
+struct CgWork {  // layout of the caller's workspace
+  double* r;
+  double* p;
+  double* q;
+  double* part_pq;
+  double* part_rr;
+  CgState* st;
+};
+
+size_t cg_workspace(int64_t n) {
+  return static_cast<size_t>(3 * n + 2 * kCgGMaxShares + 4) * sizeof(double) + 256;
+}
+
+CgWork cg_work(double* w, int64_t n) {
+  CgWork c;
+  c.r = w;
+  c.p = w + n;
+  c.q = w + 2 * n;
+  c.part_pq = w + 3 * n;
+  c.part_rr = c.part_pq + kCgGMaxShares;
+  c.st = reinterpret_cast<CgState*>(c.part_rr + kCgGMaxShares);
+  return c;
+}
+
+struct CgGridArgs {
+  const double* vals;
+  const int32_t* indx;
+  const int32_t* rowp;
+  const double* b;
+  double* x;
+  CgWork w;
+  int64_t n, nnz;
+  int64_t rows_cap;   // most rows of a share
+  int in_smem;        // q, r and x of the shares in shared memory
+  double stop;
+  int32_t max_iters;
+  int32_t* iters;
+  double* r2;
+  double* r2_hist;
+  int* status;
+};
+
+// Sum of one double per thread in a fixed order; thread 0 gets it.  Four
+// warps (one per sub-partition) add eight values each before their shuffle
+// trees: every warp's own tree would hold the FP64 pipe four times as long.
+__device__ __forceinline__ double block_total(double v, double* red) {
+  const int tid = threadIdx.x;
+  red[tid] = v;
+  __syncthreads();
+  if (tid < 128) {
+    v = 0.0;
+#pragma unroll
+    for (int i = 0; i < kCgGThreads; i += 256) v += red[tid + i] + red[tid + i + 128];
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
+    if ((tid & 31) == 0) red[kCgGThreads + (tid >> 5)] = v;
+  }
+  __syncthreads();
+  if (tid == 0)
+    v = (red[kCgGThreads] + red[kCgGThreads + 1]) + (red[kCgGThreads + 2] + red[kCgGThreads + 3]);
+  return v;
+}
+
+// The shares added in a fixed order by the first warp, and the step's
+// quotient of the sum and r2 by one thread (an FP64 division by all of them
+// would take a microsecond of the pipe): every thread gets both, the same in
+// every block.
+__device__ __forceinline__ void shares_total(const double* part, double* red, double r2,
+                                             bool over, double& total, double& ratio) {
+  double* const out = red + kCgGThreads + 4;
+  if (threadIdx.x < 32) {
+    double t = 0.0;
+#pragma unroll
+    for (int i = 0; i < (kCgBlocks + 31) / 32; ++i) {
+      const int s = i * 32 + threadIdx.x;
+      const double v = s < kCgBlocks ? __ldcg(part + s) : 0.0;
+      t = i == 0 ? v : t + v;
+    }
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
+    if (threadIdx.x == 0) {
+      out[0] = t;
+      out[1] = over ? r2 / t : t / r2;
+    }
+  }
+  __syncthreads();
+  total = out[0];
+  ratio = out[1];
+}
+
+__device__ __forceinline__ uint64_t timer_ns() {
+  uint64_t t;
+  asm volatile("mov.u64 %0, %%globaltimer;" : "=l"(t));
+  return t;
+}
+
+// All blocks; what each wrote before is visible to all after.  false: a wait
+// gave up (here or in another block).
+__device__ bool grid_barrier(CgState* st, unsigned long long& target, int* flag, int* status) {
+  target += gridDim.x;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    unsigned long long seen;
+    asm volatile("atom.add.release.gpu.global.u64 %0, [%1], 1;"
+                 : "=l"(seen)
+                 : "l"(&st->arrived)
+                 : "memory");
+    int ok = 1;
+    const uint64_t t0 = timer_ns();
+    for (uint32_t it = 1;; ++it) {
+      asm volatile("ld.acquire.gpu.global.u64 %0, [%1];" : "=l"(seen) : "l"(&st->arrived) : "memory");
+      if (seen >= target) break;
+      if ((it & 63u) == 0) {
+        if (*reinterpret_cast<volatile int*>(&st->abort)) {
+          ok = 0;
+          break;
+        }
+        if (timer_ns() - t0 > kWaitLimitNs) {
+          atomicExch(&st->abort, 1);
+          atomicOr(status, kStatusTimeout);
+          ok = 0;
+          break;
+        }
+      }
+    }
+    *flag = ok;
+  }
+  __syncthreads();
+  return *flag != 0;
+}
+
+// q = A p on rows [lo, hi) (qs[row - lo]); returns this thread's part of
+// (p, q).  G lanes a row; a warp takes 32 / G rows at a time.
+template <int G>
+__device__ __forceinline__ double cg_product(const CgGridArgs& a, int64_t lo, int64_t hi,
+                                             double* qs, bool& bad) {
+  constexpr int R = 32 / G;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int sub = lane & (G - 1), grp = lane / G;
+  const double* const p = a.w.p;
+  const int n = static_cast<int>(a.n);
+  double pq = 0.0;
+  for (int64_t base = lo + static_cast<int64_t>(warp) * R; base < hi;
+       base += static_cast<int64_t>(kCgGWarps) * R) {
+    const int64_t row = base + grp;
+    int b = 0, e = 0;
+    double prow = 0.0;
+    if (row < hi) {
+      b = __ldg(a.rowp + row);
+      e = __ldg(a.rowp + row + 1);
+      if (b < 0 || e < b || e > a.nnz) {
+        bad = true;
+        b = e = 0;
+      }
+      if (sub == 0) prow = __ldcg(p + row);
+    }
+    int j = b + sub;
+    double t = 0.0;
+    // the most values any lane of the warp has left (the warp runs together)
+    int m = __reduce_max_sync(0xFFFFFFFFu, j < e ? (e - j + G - 1) / G : 0);
+    for (; m > 0; m -= kBatch) {
+      double v[kBatch], pv[kBatch];
+      int c[kBatch];
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        c[u] = -1;
+        v[u] = 0.0;
+        if (j + u * G < e) {
+          c[u] = __ldg(a.indx + j + u * G);
+          v[u] = __ldg(a.vals + j + u * G);
+          bad |= c[u] < 0 || c[u] >= n;
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u) {
+        pv[u] = 0.0;
+        if (c[u] >= 0 && c[u] < n) pv[u] = __ldcg(p + c[u]);
+        else v[u] = 0.0;
+      }
+#pragma unroll
+      for (int u = 0; u < kBatch; ++u)
+        if (u < m) t = fma(v[u], pv[u], t);  // uniform
+      j = j + kBatch * G;
+    }
+#pragma unroll
+    for (int o = G / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
+    if (row < hi && sub == 0) {
+      qs[row - lo] = t;
+      pq = fma(prow, t, pq);
+    }
+  }
+  return pq;
+}
+
+template <int G>
+__global__ void __launch_bounds__(kCgGThreads, 1) cg_grid_kernel(const CgGridArgs a) {
+  extern __shared__ double dsm[];
+  __shared__ double red[kCgGThreads + 6];
+  __shared__ int flag;
+  const int tid = threadIdx.x;
+  const bool many = gridDim.x < kCgBlocks;  // several shares a block: their vectors in memory
+  const bool smem = a.in_smem && !many;
+  CgState* const st = a.w.st;
+  unsigned long long target = 0;
+  bool bad = false;
+  auto lo_of = [&](int s) { return a.n * s / kCgBlocks; };
+  auto q_of = [&](int64_t lo) { return smem ? dsm : a.w.q + lo; };
+  auto r_of = [&](int64_t lo) { return smem ? dsm + a.rows_cap : a.w.r + lo; };
+  auto x_of = [&](int64_t lo) { return smem ? dsm + 2 * a.rows_cap : a.x + lo; };
+
+  // x0 = 0, r0 = p0 = b, shares of (b, b)
+  for (int s = blockIdx.x; s < kCgBlocks; s += gridDim.x) {
+    const int64_t lo = lo_of(s), hi = lo_of(s + 1);
+    double* const r = r_of(lo);
+    double* const x = x_of(lo);
+    double bb = 0.0;
+    for (int64_t i = lo + tid; i < hi; i += kCgGThreads) {
+      const double bi = __ldg(a.b + i);
+      x[i - lo] = 0.0;
+      r[i - lo] = bi;
+      a.w.p[i] = bi;
+      bb = fma(bi, bi, bb);
+    }
+    bb = block_total(bb, red);
+    if (tid == 0) a.w.part_rr[s] = bb;
+  }
+  bool ok = grid_barrier(st, target, &flag, a.status);
+  double r2 = 0.0, unused;
+  if (ok) shares_total(a.w.part_rr, red, 1.0, false, r2, unused);
+  int32_t k = 0;
+  bool brk = false;
+  while (ok && r2 > a.stop && k < a.max_iters) {
+    for (int s = blockIdx.x; s < kCgBlocks; s += gridDim.x) {
+      const int64_t lo = lo_of(s), hi = lo_of(s + 1);
+      const double pq = block_total(cg_product<G>(a, lo, hi, q_of(lo), bad), red);
+      if (tid == 0) a.w.part_pq[s] = pq;
+    }
+    if (!(ok = grid_barrier(st, target, &flag, a.status))) break;
+    double pAp, alpha, r2n, beta;
+    shares_total(a.w.part_pq, red, r2, true, pAp, alpha);
+    if (!(pAp > 0.0)) {  // the same in every block: the same shares, the same order
+      brk = true;
+      break;
+    }
+    for (int s = blockIdx.x; s < kCgBlocks; s += gridDim.x) {
+      const int64_t lo = lo_of(s), own = lo_of(s + 1) - lo;
+      const double* const q = q_of(lo);
+      double* const r = r_of(lo);
+      double rr = 0.0;
+      for (int64_t i = tid; i < own; i += kCgGThreads) {
+        const double ri = fma(-alpha, q[i], r[i]);
+        r[i] = ri;
+        rr = fma(ri, ri, rr);
+      }
+      rr = block_total(rr, red);
+      if (tid == 0) a.w.part_rr[s] = rr;
+    }
+    if (!(ok = grid_barrier(st, target, &flag, a.status))) break;
+    shares_total(a.w.part_rr, red, r2, false, r2n, beta);
+    r2 = r2n;
+    for (int s = blockIdx.x; s < kCgBlocks; s += gridDim.x) {
+      const int64_t lo = lo_of(s), own = lo_of(s + 1) - lo;
+      const double* const r = r_of(lo);
+      double* const x = x_of(lo);
+#pragma unroll 4
+      for (int64_t i = tid; i < own; i += kCgGThreads) {
+        const double pi = __ldcg(a.w.p + lo + i);
+        x[i] = fma(alpha, pi, x[i]);
+        __stcg(a.w.p + lo + i, fma(beta, pi, r[i]));
+      }
+    }
+    if (blockIdx.x == 0 && tid == 0 && a.r2_hist != nullptr) a.r2_hist[k] = r2;
+    ++k;
+    if (!(ok = grid_barrier(st, target, &flag, a.status))) break;
+  }
+  if (smem) {  // each thread's own elements
+    const int64_t lo = lo_of(blockIdx.x), own = lo_of(blockIdx.x + 1) - lo;
+    for (int64_t i = tid; i < own; i += kCgGThreads) a.x[lo + i] = x_of(lo)[i];
+  }
+  if (blockIdx.x == 0 && tid == 0) {
+    *a.iters = k;
+    *a.r2 = r2;
+    if (brk) atomicOr(a.status, kStatusBreakdown);
+  }
+  if (bad) atomicOr(a.status, kStatusBounds);
+}
+
+// Lanes per row: the fewest that give every thread of a share a row.
+int cg_grid_group(int64_t n, int64_t nnz) {
+  const int64_t rows = (n + kCgBlocks - 1) / kCgBlocks;
+  const int64_t avg = n > 0 ? (nnz + n - 1) / n : 0;
+  int g = 1;
+  while (g < 32 && rows * g < kCgGThreads && g < avg) g *= 2;
+  return g;
+}
+
+template <int G>
+mxm_status launch_grid(CgGridArgs a, cudaStream_t s) {
+  int dev = 0, optin = 0, sms = 0, per_sm = 0;
+  cudaFuncAttributes fa;
+  if (cudaGetDevice(&dev) != cudaSuccess ||
+      cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
+          cudaSuccess ||
+      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
+      cudaFuncGetAttributes(&fa, cg_grid_kernel<G>) != cudaSuccess)
+    return MXM_ERR_CUDA;
+  a.rows_cap = (a.n + kCgBlocks - 1) / kCgBlocks;
+  size_t smem = 3 * static_cast<size_t>(a.rows_cap) * sizeof(double);
+  a.in_smem = smem + fa.sharedSizeBytes <= static_cast<size_t>(optin) ? 1 : 0;
+  if (!a.in_smem) smem = 0;
+  if (cudaFuncSetAttribute(cg_grid_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                           static_cast<int>(smem)) != cudaSuccess ||
+      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cg_grid_kernel<G>, kCgGThreads,
+                                                    smem) != cudaSuccess)
+    return MXM_ERR_CUDA;
+  int blocks = sms * per_sm;
+  if (blocks > kCgBlocks) blocks = kCgBlocks;
+  if (blocks < 1) return MXM_ERR_CUDA;
+  if (cudaMemsetAsync(a.w.st, 0, sizeof(CgState), s) != cudaSuccess) return MXM_ERR_CUDA;
+  void* args[] = {&a};
+  return cudaLaunchCooperativeKernel(reinterpret_cast<void*>(cg_grid_kernel<G>), dim3(blocks),
+                                     dim3(kCgGThreads), args, smem, s) == cudaSuccess
+             ? MXM_OK
+             : MXM_ERR_CUDA;
+}
+
+}  // namespace
+
+size_t cg_grid_workspace_bytes(int64_t n) { return cg_workspace(n); }
+
+// One solve by the engine over all SMs (arguments checked by the caller).
+mxm_status cg_grid_solve(const double* vals, const int32_t* indx, const int32_t* rowp,
+                         const double* b, double* x, double* work, int32_t* iters, double* r2,
+                         double* r2_hist, int64_t n, int64_t nnz, double stop,
+                         int32_t max_iters, int* status, cudaStream_t s) {
+  cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing(s, &cap) != cudaSuccess) return MXM_ERR_CUDA;
+  if (cap != cudaStreamCaptureStatusNone) return MXM_ERR_UNSUPPORTED;
+  CgGridArgs a;
+  a.vals = vals;
+  a.indx = indx;
+  a.rowp = rowp;
+  a.b = b;
+  a.x = x;
+  a.w = cg_work(work, n);
+  a.n = n;
+  a.nnz = nnz;
+  a.rows_cap = 0;
+  a.in_smem = 0;
+  a.stop = stop;
+  a.max_iters = max_iters;
+  a.iters = iters;
+  a.r2 = r2;
+  a.r2_hist = r2_hist;
+  a.status = status;
+  switch (cg_grid_group(n, nnz)) {
+    case 1: return launch_grid<1>(a, s);
+    case 2: return launch_grid<2>(a, s);
+    case 4: return launch_grid<4>(a, s);
+    case 8: return launch_grid<8>(a, s);
+    case 16: return launch_grid<16>(a, s);
+    default: return launch_grid<32>(a, s);
+  }
+}
+
+}  // namespace mxm

@@ -329,7 +329,7 @@ def mxm_cg(matvals, indx, rowp, b, x, stop, max_iters, iters=None, r2=None, r2_h
     """Conjugate gradients for A x = b (Sec. 3.4), A SPD in CSR (CUDA
     tensors: matvals float64, indx and rowp int32, b and x float64), the
     loop on the device (``engine``: CG_AUTO, CG_CLUSTER or CG_GRAPH).
-    ``iters`` (int32[1]), ``r2`` (float64[1]) and, for the graph engine,
+    ``iters`` (int32[1]), ``r2`` (float64[1]) and, for the engine over all SMs,
     ``work`` (mxm_cg_workspace_size(n) bytes) are allocated when not given;
     ``r2_hist`` (float64[max_iters]) is optional.  Returns (iters, r2) as
     device tensors; read them after the stream (and check
