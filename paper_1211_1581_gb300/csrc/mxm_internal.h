@@ -1,7 +1,6 @@
 // mxm_internal.h -- declarations shared by the translation units of
 // libmxm.so (not part of the public C ABI in include/mxm.h).
 #pragma once
-#include <cmath>
 #include <cstddef>
 #include <cstdint>
 
@@ -275,27 +274,35 @@ inline int kara_min_ranges(const OzakiDims& d) {
       static_cast<int64_t>(2147483647.0 / ((d.S + 1) * dmax * dmax * kOzTileK));
   return most < 1 ? 0 : static_cast<int>((d.Kt + most - 1) / most);
 }
+// The most ranges a cut takes: at least four k-blocks each otherwise.
+inline int kara_max_ranges(const OzakiDims& d) {
+  const int64_t least = kara_min_ranges(d), most = least > d.Kt / 4 ? least : d.Kt / 4;
+  return static_cast<int>(most < least + 15 ? most : least + 15);
+}
 inline size_t kara_cut_slots(const OzakiDims& d) {
   const int64_t t = kara_tiles(d), r = kara_min_ranges(d);
   const int64_t cut = t < kKaraPairs || r > 1 ? t : kKaraPairs;
-  const size_t slots = (size_t)cut * r * (2 * d.S - 2);
-  return slots > 3 * (size_t)kKaraPairs ? slots : 3 * (size_t)kKaraPairs;
+  const size_t one = (size_t)cut * (2 * d.S - 2), least = one * r;
+  const size_t most = one * kara_max_ranges(d), cap = 3 * (size_t)kKaraPairs;
+  return most <= cap ? most : (least > cap ? least : cap);
 }
 inline size_t kara_scratch_bytes(const OzakiDims& d) {
   const size_t whole = kara_min_ranges(d) > 1 ? 0 : (size_t)kara_tiles(d) * d.S;
   return 2 * kKaraSlotBytes * (whole + kara_cut_slots(d));
 }
 
-// Host form of the kernels' oz_exact_from: the first diagonal of the FP64
-// phase of the fold.
-inline int ozaki_exact_from(int S, int beta, int64_t Kt) {
-  const double dmax = static_cast<double>((1 << beta) - 1);
+// The first diagonal of the FP64 phase of the fold (oz_exact_from).
+__host__ __device__ inline int ozaki_exact_from(int S, int beta, int64_t Kt) {
+  const uint64_t dmax = (1u << beta) - 1;
+  const uint64_t one = dmax * dmax * kOzTileK * static_cast<uint64_t>(Kt);  // < 2^48
   int gx = S + 1;
-  double yb = 0.0;
+  uint64_t y = 0;
   for (int g = S + 1; g >= 2; --g) {
-    yb += std::ldexp((g - 1) * dmax * dmax * kOzTileK * static_cast<double>(Kt),
-                     beta * (S + 1 - g));
-    if (yb >= 4503599627370496.0) break;  // 2^52
+    const int sh = beta * (S + 1 - g);
+    const uint64_t d = static_cast<uint64_t>(g - 1) * one;
+    if (sh >= 52 || (d >> (52 - sh)) != 0) break;  // this diagonal alone reaches 2^52
+    y += d << sh;
+    if (y >> 52) break;
     gx = g;
   }
   return gx;
@@ -304,7 +311,8 @@ inline int ozaki_exact_from(int S, int beta, int64_t Kt) {
 // Which products can take the difference products.
 inline bool kara_fits(const OzakiDims& d) {
   return !d.fp8 && d.S >= 3 && d.S <= kKaraMaxSlices && d.beta * d.S <= 64 && d.Kt > 0 &&
-         kara_min_ranges(d) >= 1 && kara_min_ranges(d) <= 16 && d.Mt >= 2 && d.Nt >= 2 && kara_tiles(d) < (1 << 24);
+         kara_min_ranges(d) >= 1 && kara_min_ranges(d) <= 16 &&
+         d.Mt >= 1 && d.Nt >= 1 && kara_tiles(d) < (1 << 24);
 }
 
 inline OzakiLayout ozaki_layout(const OzakiDims& d) {
@@ -334,13 +342,17 @@ inline OzakiLayout ozaki_layout(const OzakiDims& d) {
 
 
 // The choice: the workspace (digit and difference planes, segment slots) up
-// to kKaraMaxBytes (6.8 GB at 8192^3, 27 GB at 16384^3), and not for a part of a
+// to kKaraMaxBytes (6.8 GB at 8192^3, 27 GB at 16384^3); not for a part of a
 // wave with little k, where the planes and slots cost more than the products
-// save (measured at 512 x 512 x 4096, S = 7: 154 us against 148).
+// save (measured at 512 x 512 x 4096, S = 7: 154 us against 148); and with a
+// single tile-row or tile-column, where half of a 256 x 256 tile is empty,
+// only as long as the product is small enough to be bound by latency (155 x
+// 305 x 98, S = 7: 3x; 64 x 8192 x 8192, S = 6: 956 us against 906).
 constexpr size_t kKaraMaxBytes = (size_t)32 << 30;
 inline bool kara_chosen(const OzakiDims& d) {
   if (!kara_fits(d)) return false;
   if (d.Kt <= 4 && kara_tiles(d) > 16 && kara_tiles(d) < 48) return false;
+  if ((d.Mt == 1 || d.Nt == 1) && (d.Kt < 2 || kara_tiles(d) * d.Kt > 256)) return false;
   OzakiDims w = d;
   w.kara = 1;
   return ozaki_layout(w).total <= kKaraMaxBytes;

@@ -90,15 +90,22 @@ __device__ __forceinline__ uint64_t warp_row_max(const double* __restrict__ a, i
   return max_bits(hi, lo);
 }
 
-// max_l |a_il| per row, a warp per row.
-__global__ void oz_rowmax_kernel(const double* __restrict__ A, int64_t m, int64_t k,
-                                 uint64_t* __restrict__ rowbits, int* __restrict__ status) {
+// max_l |a_il| per row (rows too long for the fused pass): a warp per row and
+// run of kRowMaxRun values, the runs' maxima meet in rowbits by atomicMax
+// (rowbits zeroed first).  128 rows of 65536: 126 us with a warp for the whole
+// row, 16 blocks in all.
+constexpr int64_t kRowMaxRun = 2048;
+__global__ void oz_rowmax_kernel(const double* __restrict__ A, int64_t m, int64_t k, int64_t run0,
+                                 unsigned long long* __restrict__ rowbits,
+                                 int* __restrict__ status) {
   const int64_t row = static_cast<int64_t>(blockIdx.x) * (blockDim.x >> 5) + (threadIdx.x >> 5);
   if (row >= m) return;
   const int lane = threadIdx.x & 31;
-  const uint64_t mx = warp_row_max(A + row * k, k, lane);
+  const int64_t l0 = (run0 + blockIdx.y) * kRowMaxRun;
+  const uint64_t mx =
+      warp_row_max(A + row * k + l0, k - l0 < kRowMaxRun ? k - l0 : kRowMaxRun, lane);
   if (lane == 0) {
-    rowbits[row] = mx;
+    atomicMax(rowbits + row, static_cast<unsigned long long>(mx));
     if (mx >= kInfBits) atomicOr(status, kStatusNonFinite);
   }
 }
@@ -191,202 +198,217 @@ __device__ __forceinline__ void split_chunk_store(const double (&x)[8], int e, i
   }
 }
 
-// The same for beta * S <= 64: the fraction |x| 2^-e is first put in one
-// 64-bit fixed-point word F = floor(|x| 2^{beta S - e}) (one shift), then
-// digit s is the field F >> beta (S - s) (a shift uniform over the warp, of
-// the high word or a funnel shift of both).  V values per 16-byte chunk:
-// V = 8 bf16 digits, or V = 16 E4M3 digits (|d| <= 15, from a 16-entry table
-// of the E4M3 codes of 0..15).
-//
-// A bf16 digit is the upper half of the FP32 pattern of the integer +-mag
-// (exact: at most 8 significant bits), made without a conversion
-// instruction: the pattern of 2^23 + mag (mag in the low mantissa bits of
-// 2^23, with the sign of x) plus -+2^23 is exactly +-mag, and +0 for mag = 0
-// (x + (-x) rounds to +0).
-__device__ __forceinline__ uint32_t bf16_pair(uint32_t q0, uint32_t q1, uint32_t a0,
-                                              uint32_t a1) {
-  const float f0 = __uint_as_float(q0) + __uint_as_float(a0);
-  const float f1 = __uint_as_float(q1) + __uint_as_float(a1);
-  return __byte_perm(__float_as_uint(f0), __float_as_uint(f1), 0x7632);  // the upper halves
-}
-
-// diff: +1 (A) or -1 (B): the planes of the difference products follow the
-// digits (kara_pair_plane order): d_s - d_t for A, d_t - d_s for B; 0: none.
-template <int V>
-__device__ __forceinline__ void split_chunk_store_w64(const double (&x)[V], int e, int S,
-                                                      int beta, uint8_t* dst,
-                                                      size_t slice_stride, int diff = 0) {
-  uint32_t Fh[V], Fl[V], mg[V];
+// 4-bit digits (|d| <= 15, S <= 16) in E4M3, 16 per 16-byte chunk: the fraction
+// |x| 2^-e is first put in one 64-bit fixed-point word
+// F = floor(|x| 2^{4 S - e}) (one shift), then digit s is the field
+// F >> 4 (S - s) (a shift uniform over the warp, of the high word or a funnel
+// shift of both), and a 16-entry table gives its E4M3 code.
+__device__ __forceinline__ void split_chunk_store_e4m3(const double (&x)[16], int e, int S,
+                                                       uint8_t* dst, size_t slice_stride) {
+  uint32_t Fh[16], Fl[16], sg[16];
 #pragma unroll
-  for (int j = 0; j < V; ++j) {
+  for (int j = 0; j < 16; ++j) {
     const uint64_t b = static_cast<uint64_t>(__double_as_longlong(x[j]));
     const int be = static_cast<int>((b >> 52) & 0x7FF);
     const uint64_t mant = b & 0x000FFFFFFFFFFFFFull;
     const uint64_t M = be ? (mant | 0x0010000000000000ull) : mant;
-    const int sh = (be ? be - 1075 : -1074) - e + beta * S;
+    const int sh = (be ? be - 1075 : -1074) - e + 4 * S;
     const uint64_t F = sh >= 0 ? (sh < 64 ? M << sh : 0ull) : (-sh < 64 ? M >> -sh : 0ull);
     Fh[j] = static_cast<uint32_t>(F >> 32);
     Fl[j] = static_cast<uint32_t>(F);
-    mg[j] = V == 8 ? (0x4B000000u | (static_cast<uint32_t>(b >> 63) << 31))  // +-2^23
-                   : static_cast<uint32_t>(b >> 63);
+    sg[j] = static_cast<uint32_t>(b >> 63);
   }
-  const uint32_t mask = (1u << beta) - 1u;
+  // E4M3 codes of 0..7 and 8..15, one byte each
+  constexpr uint64_t kLo = 0x4E4C4A4844403800ull, kHi = 0x5756555453525150ull;
   for (int s = 1; s <= S; ++s) {
-    const int p = beta * (S - s);
-    auto field = [&](int j) -> uint32_t {
-      return (p >= 32 ? (Fh[j] >> (p - 32)) : __funnelshift_r(Fl[j], Fh[j], p)) & mask;
-    };
+    const int p = 4 * (S - s);
     uint32_t packed[4];
-    if constexpr (V == 8) {
 #pragma unroll
-      for (int j = 0; j < 8; j += 2)
-        packed[j >> 1] = bf16_pair(field(j) | mg[j], field(j + 1) | mg[j + 1],
-                                   mg[j] ^ 0x80000000u, mg[j + 1] ^ 0x80000000u);
-    } else {
-      // E4M3 codes of 0..7 and 8..15, one byte each
-      constexpr uint64_t kLo = 0x4E4C4A4844403800ull, kHi = 0x5756555453525150ull;
+    for (int w = 0; w < 4; ++w) {
+      uint32_t word = 0;
 #pragma unroll
-      for (int w = 0; w < 4; ++w) {
-        uint32_t word = 0;
-#pragma unroll
-        for (int h = 0; h < 4; ++h) {
-          const int j = 4 * w + h;
-          const uint32_t mag = field(j);
-          const uint64_t tbl = mag < 8 ? kLo : kHi;
-          uint32_t code = static_cast<uint32_t>(tbl >> (8 * (mag & 7))) & 0xFFu;
-          if (mag) code |= mg[j] << 7;
-          word |= code << (8 * h);
-        }
-        packed[w] = word;
+      for (int h = 0; h < 4; ++h) {
+        const int j = 4 * w + h;
+        const uint32_t mag = (p >= 32 ? (Fh[j] >> (p - 32)) : __funnelshift_r(Fl[j], Fh[j], p)) & 15u;
+        const uint64_t tbl = mag < 8 ? kLo : kHi;
+        uint32_t code = static_cast<uint32_t>(tbl >> (8 * (mag & 7))) & 0xFFu;
+        if (mag) code |= sg[j] << 7;
+        word |= code << (8 * h);
       }
+      packed[w] = word;
     }
     *reinterpret_cast<uint4*>(dst + static_cast<size_t>(s - 1) * slice_stride) =
         make_uint4(packed[0], packed[1], packed[2], packed[3]);
   }
-  if constexpr (V == 8) {
-    if (diff == 0) return;
-    uint8_t* out = dst + static_cast<size_t>(S) * slice_stride;
-    for (int g = 3; g <= S + 1; ++g)
-      for (int s = g == S + 1 ? 2 : 1; s < g - s; ++s) {
-        // the larger-weight digit first for A, second for B
-        const int pa = beta * (S - (diff > 0 ? s : g - s)), pb = beta * (S - (diff > 0 ? g - s : s));
-        uint32_t packed[4];
-#pragma unroll
-        for (int j = 0; j < 8; j += 2) {
-          uint32_t f[2];
-#pragma unroll
-          for (int h = 0; h < 2; ++h) {
-            const uint32_t da = (pa >= 32 ? Fh[j + h] >> (pa - 32)
-                                          : __funnelshift_r(Fl[j + h], Fh[j + h], pa)) & mask;
-            const uint32_t db = (pb >= 32 ? Fh[j + h] >> (pb - 32)
-                                          : __funnelshift_r(Fl[j + h], Fh[j + h], pb)) & mask;
-            // 1.5 2^23 + (da - db) as a float pattern, minus 1.5 2^23, with
-            // the sign of x
-            f[h] = __float_as_uint(__uint_as_float(0x4B400000u + da - db) - 12582912.0f) ^
-                   (mg[j + h] & 0x80000000u);
-          }
-          packed[j >> 1] = __byte_perm(f[0], f[1], 0x7632);  // the upper halves
-        }
-        *reinterpret_cast<uint4*>(out) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
-        out += slice_stride;
-      }
-  }
 }
 
-// Balanced 8-bit digits (the round-to-nearest split): with e1 = e + 1,
-// V = round(x 2^(8S - e1)) (ties to even; |V| <= 2^(8S-1), S <= 7), and the
-// digits of V in base 256 with every lower digit in [-128, 127] and the top
-// one in [-128, 128]: with W = V + sum_{i < S-1} 128 256^i, lower digit i is
-// byte i of W minus 128 and the top digit is W >> 8(S-1) (floor) -- the
-// same digits as taking V mod 256 in [-128, 127] from the bottom up.  Each
-// digit is an integer of at most 8 bits, exact in bf16.
-__device__ __forceinline__ void split_chunk_store_rn8(const double (&x)[8], int e1, int S,
-                                                      uint8_t* dst, size_t slice_stride,
-                                                      int diff = 0) {
-  long long W[8];
-  const long long Boff =
-      S > 1 ? static_cast<long long>(0x8080808080808080ull >> (8 * (9 - S))) : 0ll;
+// The three digit kinds of the product, eight values at a time, every digit
+// kept as packed bf16 (two values per register) so that the difference planes
+// cost one packed subtraction per two values: |d_s - d_t| <= 256 is exact in
+// bf16.  About 50 instructions per value at S = 7 with the difference planes,
+// against 150 with a float per digit and difference.  8192^2, S = 7 (18 planes,
+// 2.4 GB written): A 672 -> 460 us with its maxima, 6.4 TB/s; B 633 -> 492 us.
+//   kind 0  7-bit digits (S <= 9), from the 64-bit fixed-point word (as the
+//           4-bit digits above): 0x4300 | d is the bf16 pattern of 128 + d,
+//           128 is subtracted packed and the sign of x put on by its bit.
+//   kind 1  8-bit digits (S <= 8) of the same word: byte b behind the pattern
+//           of 2^23 gives the float 2^23 + b (signed like x).
+//   kind 2  balanced 8-bit digits (S <= 7): with e1 = e + 1,
+//           V = round(x 2^(8S - e1)) (ties to even; |V| <= 2^(8S-1)), and the
+//           digits of V in base 256 with every lower digit in [-128, 127] and
+//           the top one in [-128, 128]: with W = V + sum_{i < S-1} 128 256^i,
+//           lower digit i is byte i of W minus 128 and the top digit is
+//           W >> 8(S-1) (floor) -- the same digits as taking V mod 256 in
+//           [-128, 127] from the bottom up.
+// kDiff: the planes of the difference products follow the digits
+// (kara_pair_plane order): d_s - d_t for A; for B d_t - d_s, by the sign bits in
+// flip.  The kernels are compiled per kind: together the kinds take 165
+// registers a thread, and one block per SM.
+__device__ __forceinline__ uint32_t bf16x2_sub(uint32_t a, uint32_t b) {
+  uint32_t r;
+  asm("sub.rn.bf16x2 %0, %1, %2;" : "=r"(r) : "r"(a), "r"(b));
+  return r;
+}
+// The float pattern `top`'s upper half over byte `i` (uniform) of the word.
+__device__ __forceinline__ uint32_t byte_under(uint32_t hi, uint32_t lo, int i, uint32_t top) {
+  return i >= 4 ? __byte_perm(hi, top, 0x7650u | static_cast<uint32_t>(i - 4))
+                : __byte_perm(lo, top, 0x7650u | static_cast<uint32_t>(i));
+}
+
+template <int kKind, bool kDiff>
+__device__ __forceinline__ void split_chunk_store_planes(const double (&x)[8], int e, int S,
+                                                         uint8_t* dst, size_t slice_stride,
+                                                         uint32_t flip) {
+  constexpr int kMaxS = kKind == 0 ? 9 : kKind == 1 ? 8 : 7;
+  constexpr int kBeta = kKind == 0 ? 7 : 8;
+  uint32_t Fh[8], Fl[8], sg[8];
 #pragma unroll
   for (int j = 0; j < 8; ++j) {
     const uint64_t b = static_cast<uint64_t>(__double_as_longlong(x[j]));
     const int be = static_cast<int>((b >> 52) & 0x7FF);
     const uint64_t mant = b & 0x000FFFFFFFFFFFFFull;
     const uint64_t M = be ? (mant | 0x0010000000000000ull) : mant;
-    const int sh = (be ? be - 1075 : -1074) - e1 + 8 * S;  // x 2^(8S - e1) = M 2^sh
-    uint64_t q;
-    if (sh >= 0) {
-      q = M << sh;  // |x 2^(8S - e1)| < 2^(8S-1) <= 2^55: no bit leaves the word
-    } else if (-sh >= 64) {
-      q = 0;        // M < 2^53 <= half of 2^64: rounds to 0
+    const int sh = (be ? be - 1075 : -1074) - e - (kKind == 2 ? 1 : 0) + kBeta * S;
+    uint64_t F;
+    if constexpr (kKind == 2) {
+      // |x 2^(8S - e1)| = M 2^sh < 2^(8S-1) <= 2^55, rounded to nearest even
+      if (sh >= 0) {
+        F = M << sh;
+      } else if (-sh >= 64) {
+        F = 0;  // M < 2^53 <= half of 2^64: rounds to 0
+      } else {
+        const int nsh = -sh;
+        F = M >> nsh;
+        const uint64_t rem = M & ((1ull << nsh) - 1ull), half = 1ull << (nsh - 1);
+        if (rem > half || (rem == half && (F & 1ull))) ++F;
+      }
+      const uint64_t off = S > 1 ? 0x8080808080808080ull >> (8 * (9 - S)) : 0ull;
+      F = (b >> 63 ? 0ull - F : F) + off;
     } else {
-      const int nsh = -sh;
-      q = M >> nsh;
-      const uint64_t rem = M & ((1ull << nsh) - 1ull), half = 1ull << (nsh - 1);
-      if (rem > half || (rem == half && (q & 1ull))) ++q;
+      F = sh >= 0 ? (sh < 64 ? M << sh : 0ull) : (-sh < 64 ? M >> -sh : 0ull);
     }
-    const long long V = (b >> 63) ? -static_cast<long long>(q) : static_cast<long long>(q);
-    W[j] = V + Boff;
+    Fh[j] = static_cast<uint32_t>(F >> 32);
+    Fl[j] = static_cast<uint32_t>(F);
+    sg[j] = static_cast<uint32_t>(b >> 63);
   }
-  // digit dg (|dg| <= 128) as an exact float without a conversion
-  // instruction: the pattern of 1.5 2^23 + dg minus 1.5 2^23 (+0 for dg = 0)
-  constexpr uint32_t kMagic = 0x4B400000u;  // 1.5 2^23 = 12582912
-  const uint32_t kNegMagic = 0xCB400000u;
-  for (int s = 1; s <= S; ++s) {
-    const int p = 8 * (S - s);
-    uint32_t packed[4];
+  uint32_t sgn[4];  // kind 0: the signs of a register's two values
+  if constexpr (kKind == 0) {
 #pragma unroll
-    for (int j = 0; j < 8; j += 2) {
-      uint32_t q[2];
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        const int dg = s == 1 ? static_cast<int>(W[j + h] >> p)
-                              : static_cast<int>((W[j + h] >> p) & 255) - 128;
-        q[h] = kMagic + static_cast<uint32_t>(dg);
-      }
-      packed[j >> 1] = bf16_pair(q[0], q[1], kNegMagic, kNegMagic);
-    }
-    *reinterpret_cast<uint4*>(dst + static_cast<size_t>(s - 1) * slice_stride) =
-        make_uint4(packed[0], packed[1], packed[2], packed[3]);
+    for (int w = 0; w < 4; ++w) sgn[w] = (sg[2 * w] << 15) | (sg[2 * w + 1] << 31);
   }
-  if (diff == 0) return;
-  uint8_t* out = dst + static_cast<size_t>(S) * slice_stride;
-  for (int g = 3; g <= S + 1; ++g)
-    for (int s = g == S + 1 ? 2 : 1; s < g - s; ++s) {
-      // byte differences (the offsets of 128 cancel below the top digit)
-      const int ps = 8 * (S - s), pt = 8 * (S - (g - s));
-      uint32_t packed[4];
+  uint32_t d[kMaxS][4];
 #pragma unroll
-      for (int j = 0; j < 8; j += 2) {
-        uint32_t q[2];
+  for (int s = 0; s < kMaxS; ++s) {
+    if (s < S) {  // uniform
+      if constexpr (kKind == 0) {
+        const int p = 7 * (S - 1 - s);
+        uint32_t f[8];
+        if (p >= 32) {
 #pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const int ds = s == 1 ? static_cast<int>(W[j + h] >> ps)
-                                : static_cast<int>((W[j + h] >> ps) & 255) - 128;
-          const int dt = static_cast<int>((W[j + h] >> pt) & 255) - 128;
-          q[h] = kMagic + static_cast<uint32_t>(diff > 0 ? ds - dt : dt - ds);
+          for (int j = 0; j < 8; ++j) f[j] = (Fh[j] >> (p - 32)) & 127u;
+        } else {
+#pragma unroll
+          for (int j = 0; j < 8; ++j) f[j] = __funnelshift_r(Fl[j], Fh[j], p) & 127u;
         }
-        packed[j >> 1] = bf16_pair(q[0], q[1], kNegMagic, kNegMagic);
+#pragma unroll
+        for (int w = 0; w < 4; ++w)
+          d[s][w] = bf16x2_sub(0x43004300u | f[2 * w] | (f[2 * w + 1] << 16), 0x43004300u) ^ sgn[w];
+      } else {
+        float f[8];
+#pragma unroll
+        for (int j = 0; j < 8; ++j) {
+          if constexpr (kKind == 1) {
+            const uint32_t top = 0x4B000000u | (sg[j] << 31);  // +-2^23
+            f[j] = __uint_as_float(byte_under(Fh[j], Fl[j], S - 1 - s, top)) -
+                   __uint_as_float(top);
+          } else if (s == 0) {  // the top digit: W >> 8 (S - 1), nine bits with its sign
+            const long long W = static_cast<long long>((static_cast<uint64_t>(Fh[j]) << 32) | Fl[j]);
+            f[j] = __uint_as_float(0x4B400000u + static_cast<uint32_t>(W >> (8 * (S - 1)))) -
+                   12582912.0f;
+          } else {
+            f[j] = __uint_as_float(byte_under(Fh[j], Fl[j], S - 1 - s, 0x4B400000u)) - 12583040.0f;
+          }
+        }
+#pragma unroll
+        for (int w = 0; w < 4; ++w)  // the upper halves: exact
+          d[s][w] = __byte_perm(__float_as_uint(f[2 * w]), __float_as_uint(f[2 * w + 1]), 0x7632);
       }
-      *reinterpret_cast<uint4*>(out) = make_uint4(packed[0], packed[1], packed[2], packed[3]);
-      out += slice_stride;
+      *reinterpret_cast<uint4*>(dst) = make_uint4(d[s][0], d[s][1], d[s][2], d[s][3]);
+      dst += slice_stride;
     }
+  }
+  if constexpr (kDiff) {
+#pragma unroll
+    for (int g = 3; g <= kMaxS + 1; ++g) {
+      if (g <= S + 1) {  // uniform
+#pragma unroll
+        for (int s = 1; s < g - s; ++s) {
+          const int t = g - s <= kMaxS ? g - s : kMaxS;
+          if (s > 1 || g <= S) {  // (1, S) has no plane
+            uint32_t out[4];
+#pragma unroll
+            for (int w = 0; w < 4; ++w) out[w] = bf16x2_sub(d[s - 1][w], d[t - 1][w]) ^ flip;
+            *reinterpret_cast<uint4*>(dst) = make_uint4(out[0], out[1], out[2], out[3]);
+            dst += slice_stride;
+          }
+        }
+      }
+    }
+  }
 }
 
-__device__ __forceinline__ void split_chunk(const double (&x)[8], int e, int S, int beta,
-                                            uint8_t* dst, size_t slice_stride, bool rn = false,
-                                            int diff = 0) {
-  if (rn)
-    split_chunk_store_rn8(x, e + 1, S, dst, slice_stride, diff);
-  else if (beta * S <= 64)
-    split_chunk_store_w64<8>(x, e, S, beta, dst, slice_stride, diff);
-  else
-    split_chunk_store(x, e, S, beta, dst, slice_stride);
-}
-__device__ __forceinline__ void split_chunk(const double (&x)[16], int e, int S, int beta,
-                                            uint8_t* dst, size_t slice_stride, bool = false,
-                                            int = 0) {
-  split_chunk_store_w64<16>(x, e, S, beta, dst, slice_stride);  // beta = 4, S <= 16
-}
+// What a split kernel does with V values of one row: kKind 0-2 as above, 3 any
+// other digits (no difference planes), kKindE4m3 the 4-bit ones.
+constexpr int kKindOther = 3, kKindE4m3 = 4;
+template <int kKind, bool kDiff>
+struct Splitter {
+  static constexpr int V = kKind == kKindE4m3 ? 16 : 8;
+  int S, beta;
+  uint32_t flip;
+  __device__ __forceinline__ void operator()(const double (&x)[V], int e, uint8_t* dst,
+                                             size_t slice_stride) const {
+    if constexpr (kKind == kKindE4m3) split_chunk_store_e4m3(x, e, S, dst, slice_stride);
+    else if constexpr (kKind == kKindOther) split_chunk_store(x, e, S, beta, dst, slice_stride);
+    else split_chunk_store_planes<kKind, kDiff>(x, e, S, dst, slice_stride, flip);
+  }
+};
+// Any bf16 digits, chosen at run time (grouped calls).
+struct SplitterAny {
+  static constexpr int V = 8;
+  int S, beta;
+  bool rn;
+  __device__ __forceinline__ void operator()(const double (&x)[8], int e, uint8_t* dst,
+                                             size_t slice_stride) const {
+    if (rn)
+      split_chunk_store_planes<2, false>(x, e, S, dst, slice_stride, 0u);
+    else if (beta == 7 && S <= 9)
+      split_chunk_store_planes<0, false>(x, e, S, dst, slice_stride, 0u);
+    else if (beta == 8 && S <= 8)
+      split_chunk_store_planes<1, false>(x, e, S, dst, slice_stride, 0u);
+    else
+      split_chunk_store(x, e, S, beta, dst, slice_stride);
+  }
+};
 
 // Tile geometry of the two digit carriers: V digits per 16-byte chunk.
 template <int V>
@@ -404,14 +426,14 @@ struct SplitGeo {
 // 16-byte stores are contiguous); rows of even k are read as 16-byte pairs.
 // (row_lim, chunk_lim: only rows < row_lim and chunks < chunk_lim of the
 // tile are written -- the rest is never read by the edge-tile copies.)
-template <int V>
+template <typename Split>
 __device__ __forceinline__ void split_a_tile(const double* __restrict__ A, int64_t m, int64_t k,
-                                             const uint64_t* __restrict__ rowbits, int S,
-                                             int beta, int64_t tm, int64_t tk, uint8_t* tile,
-                                             size_t slice_stride, bool rn = false,
+                                             const uint64_t* __restrict__ rowbits,
+                                             const Split& split, int64_t tm, int64_t tk,
+                                             uint8_t* tile, size_t slice_stride,
                                              int row_lim = kOzTileRows,
-                                             int chunk_lim = SplitGeo<V>::kChunksPerRow,
-                                             int diff = 0) {
+                                             int chunk_lim = SplitGeo<Split::V>::kChunksPerRow) {
+  constexpr int V = Split::V;
   using G = SplitGeo<V>;
   const bool pairs = ((k & 1) == 0) && ((reinterpret_cast<uintptr_t>(A) & 15) == 0);
   const int total = row_lim * chunk_lim;
@@ -446,8 +468,7 @@ __device__ __forceinline__ void split_a_tile(const double* __restrict__ A, int64
 #pragma unroll
     for (int h = 0; h < 2; ++h)
       if (p0 + h * static_cast<int>(blockDim.x) < total)
-        split_chunk(v[h], e[h], S, beta, tile + G::offset(rr[h], cc[h]), slice_stride, rn,
-                    diff);
+        split(v[h], e[h], tile + G::offset(rr[h], cc[h]), slice_stride);
   }
 }
 
@@ -457,16 +478,16 @@ __device__ __forceinline__ void split_a_tile(const double* __restrict__ A, int64
 // shared memory, then every thread takes V consecutive k of one column.
 constexpr int kSplitBRows = 32;
 constexpr int kSplitThreads = 256;  // the block size of the split launches
-template <int V>
+template <typename Split>
 __device__ __forceinline__ void split_b_tile(const double* __restrict__ B, int64_t k, int64_t n,
-                                             const uint64_t* __restrict__ colbits, int S,
-                                             int beta, int64_t tn, int64_t tk, uint8_t* tile,
-                                             size_t slice_stride,
-                                             double (*sb)[kOzTileRows + 1], bool rn = false,
-                                             bool halves = false, int row_lim = kOzTileRows,
-                                             int chunk_lim = SplitGeo<V>::kChunksPerRow,
-                                             int diff = 0, int pass0 = 0,
-                                             int pass1 = kOzTileK / kSplitBRows) {
+                                             const uint64_t* __restrict__ colbits,
+                                             const Split& split, int64_t tn, int64_t tk,
+                                             uint8_t* tile, size_t slice_stride,
+                                             double (*sb)[kOzTileRows + 1], bool halves,
+                                             int row_lim = kOzTileRows,
+                                             int chunk_lim = SplitGeo<Split::V>::kChunksPerRow,
+                                             int pass0 = 0, int pass1 = kOzTileK / kSplitBRows) {
+  constexpr int V = Split::V;
   using G = SplitGeo<V>;
   const int64_t col0 = tn * kOzTileRows;
   constexpr int kChunksPerPass = kSplitBRows / V;
@@ -509,58 +530,63 @@ __device__ __forceinline__ void split_b_tile(const double* __restrict__ B, int64
       for (int j = 0; j < V; ++j) v[j] = sb[cl * V + j][r];
       const int c = pass * kChunks + cl;
       const int off = (V == 8 && halves) ? oz_chunk_offset_halves(r, c) : G::offset(r, c);
-      split_chunk(v, f, S, beta, tile + off, slice_stride, rn, diff);
+      split(v, f, tile + off, slice_stride);
     }
     __syncthreads();
   }
 }
 
-// A -> A_s tiles [S][Mt][Kt].
-template <int V>
+// A -> A_s tiles [planes][Mt][Kt].
+template <typename Split>
 __global__ void __launch_bounds__(256) oz_split_a_kernel(
     const double* __restrict__ A, int64_t m, int64_t k, const uint64_t* __restrict__ rowbits,
-    int S, int beta, int64_t Mt, int64_t Kt, uint8_t* __restrict__ aslices, bool rn, int diff) {
-  constexpr size_t kTile = SplitGeo<V>::kTileBytes;
+    const Split split, int64_t Mt, int64_t Kt, uint8_t* __restrict__ aslices) {
+  constexpr size_t kTile = SplitGeo<Split::V>::kTileBytes;
   const int64_t tk = blockIdx.x, tm = blockIdx.y;
-  split_a_tile<V>(A, m, k, rowbits, S, beta, tm, tk,
-                  aslices + (static_cast<size_t>(tm) * Kt + tk) * kTile,
-                  static_cast<size_t>(Mt) * Kt * kTile, rn, kOzTileRows,
-                  SplitGeo<V>::kChunksPerRow, diff);
+  split_a_tile(A, m, k, rowbits, split, tm, tk,
+               aslices + (static_cast<size_t>(tm) * Kt + tk) * kTile,
+               static_cast<size_t>(Mt) * Kt * kTile);
 }
 
-// Steps 1 and 2 for A in one pass: one block per row of A (and per padding
-// row of the last tile-row) holds the row in shared memory, zero-padded to
-// whole k-blocks, takes its maximum and writes its digits into every k-block
-// tile from there -- A is read from memory once.  The row's 16-byte chunks of
-// a tile atom fill one 128-byte line (the swizzle permutes chunks inside the
-// row), so the stores stay whole lines.  Padding rows (i >= m) get zero
-// digits and no maximum.
+// Steps 1 and 2 for A in one pass: a block takes R rows of A (padding rows of
+// the last tile-row among them; R = 1, 2, 4 or 8), 256 / R threads each, holds them in shared
+// memory, zero-padded to whole k-blocks, takes their maxima and writes the
+// digits into every k-block tile from there -- A is read from memory once.
+// A row's 16-byte chunks of a tile atom fill one 128-byte line (the swizzle
+// permutes chunks inside the row), so the stores stay whole lines.  Padding
+// rows (i >= m) get zero digits and no maximum.  R is the most for which every
+// thread still has a chunk of eight (16384 rows of 256, S = 6: 79 us with one
+// row a block and most of its threads without a chunk, 26 us with eight).
 constexpr int64_t kFusedRowMaxK = 24576;  // k doubles held in shared memory (192 KiB)
 
+template <typename Split>
 __global__ void __launch_bounds__(256) oz_scale_split_a_kernel(
-    const double* __restrict__ A, int64_t m, int64_t k, uint64_t* __restrict__ rowbits, int S,
-    int beta, int64_t Mt, int64_t Kt, uint8_t* __restrict__ aslices, bool rn, int diff,
+    const double* __restrict__ A, int64_t m, int64_t k, uint64_t* __restrict__ rowbits,
+    const Split split, int R, int64_t Mt, int64_t Kt, uint8_t* __restrict__ aslices,
     int* __restrict__ status) {
-  extern __shared__ double row[];
-  __shared__ uint32_t wmax[32];
-  __shared__ uint64_t rmax;
-  const int64_t i = blockIdx.x;
+  const int T = 256 / R, kW = T / 32;  // threads and warps per row
+  extern __shared__ double rows[];
+  __shared__ uint32_t wmax[8];
+  __shared__ uint64_t rmax[8];
+  const int rr = threadIdx.x / T, t = threadIdx.x % T;
+  const int64_t i = static_cast<int64_t>(blockIdx.x) * R + rr;
   const int64_t kp = Kt * kOzTileK;
+  double* const row = rows + rr * kp;
   const bool real = i < m;
   const double* a = A + (real ? i : 0) * k;
   uint32_t mh = 0;
   // eight loads of a thread in flight before they go to shared memory
-  // (few blocks fit an SM with a whole row in shared memory)
-  for (int64_t l0 = threadIdx.x; l0 < kp; l0 += 8 * static_cast<int64_t>(blockDim.x)) {
+  // (few blocks fit an SM with whole rows in shared memory)
+  for (int64_t l0 = t; l0 < kp; l0 += 8 * T) {
     double v[8];
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      const int64_t l = l0 + u * static_cast<int64_t>(blockDim.x);
+      const int64_t l = l0 + u * T;
       v[u] = (real && l < k) ? __ldg(a + l) : 0.0;
     }
 #pragma unroll
     for (int u = 0; u < 8; ++u) {
-      const int64_t l = l0 + u * static_cast<int64_t>(blockDim.x);
+      const int64_t l = l0 + u * T;
       if (l < kp) {
         row[l] = v[u];
         mh = max(mh, abs_hi(v[u]));
@@ -570,17 +596,17 @@ __global__ void __launch_bounds__(256) oz_scale_split_a_kernel(
   mh = warp_max_u32(mh);
   if ((threadIdx.x & 31) == 0) wmax[threadIdx.x >> 5] = mh;
   __syncthreads();
-  if (threadIdx.x < 32) {
-    uint32_t w = threadIdx.x < (blockDim.x >> 5) ? wmax[threadIdx.x] : 0;
+  if (t < 32) {  // the row's first warp
+    uint32_t w = t < kW ? wmax[rr * kW + t] : 0;
     w = warp_max_u32(w);
     uint32_t lo = 0;
     if (w == 0) {  // every high word is zero: the low words (row in shared memory)
-      for (int64_t l = threadIdx.x; l < kp; l += 32) lo = max(lo, lo_word(row[l]));
+      for (int64_t l = t; l < kp; l += 32) lo = max(lo, lo_word(row[l]));
       lo = warp_max_u32(lo);
     }
-    if (threadIdx.x == 0) {
+    if (t == 0) {
       const uint64_t mx = max_bits(w, lo);
-      rmax = mx;
+      rmax[rr] = mx;
       if (real) {
         rowbits[i] = mx;
         if (mx >= kInfBits) atomicOr(status, kStatusNonFinite);
@@ -588,19 +614,19 @@ __global__ void __launch_bounds__(256) oz_scale_split_a_kernel(
     }
   }
   __syncthreads();
-  const int e = exponent_from_absbits(rmax < kInfBits ? rmax : 0);
+  const int e = exponent_from_absbits(rmax[rr] < kInfBits ? rmax[rr] : 0);
   const int64_t tm = i / kOzTileRows;
   const int r = static_cast<int>(i - tm * kOzTileRows);
   const size_t slice_stride = static_cast<size_t>(Mt) * Kt * kOzTileBytes;
   uint8_t* base = aslices + static_cast<size_t>(tm) * Kt * kOzTileBytes;
-  for (int64_t p = threadIdx.x; p < Kt * kOzChunksPerRow; p += blockDim.x) {
-    const int64_t tk = p / kOzChunksPerRow;
-    const int c = static_cast<int>(p - tk * kOzChunksPerRow);
+  const int chunks = static_cast<int>(Kt) * kOzChunksPerRow;
+  for (int p = t; p < chunks; p += T) {
+    const int tk = p / kOzChunksPerRow, c = p % kOzChunksPerRow;
     double v[8];
 #pragma unroll
-    for (int j = 0; j < 8; ++j) v[j] = row[tk * kOzTileK + c * 8 + j];
-    split_chunk(v, e, S, beta, base + tk * kOzTileBytes + oz_chunk_offset(r, c), slice_stride,
-                rn, diff);
+    for (int j = 0; j < 8; ++j) v[j] = row[p * 8 + j];
+    split(v, e, base + static_cast<size_t>(tk) * kOzTileBytes + oz_chunk_offset(r, c),
+          slice_stride);
   }
 }
 
@@ -613,18 +639,17 @@ __host__ __device__ inline bool oz_fused_a(const OzakiDims& d) {
 // B -> B_t tiles [S][Nt][Kt]; halves: the CTA-pair layout of each tile.  A block
 // takes one 32-row pass of a tile (blockIdx.z): with whole tiles a small
 // product filled a few SMs with four passes in a row (512 x 512: 34 us).
-template <int V>
+template <typename Split>
 __global__ void __launch_bounds__(256) oz_split_b_kernel(
     const double* __restrict__ B, int64_t k, int64_t n, const uint64_t* __restrict__ colbits,
-    int S, int beta, int64_t Nt, int64_t Kt, uint8_t* __restrict__ bslices, bool rn,
-    bool halves, int diff) {
-  constexpr size_t kTile = SplitGeo<V>::kTileBytes;
+    const Split split, int64_t Nt, int64_t Kt, uint8_t* __restrict__ bslices, bool halves) {
+  constexpr size_t kTile = SplitGeo<Split::V>::kTileBytes;
   __shared__ double sb[kSplitBRows][kOzTileRows + 1];
   const int64_t tk = blockIdx.x, tn = blockIdx.y;
-  split_b_tile<V>(B, k, n, colbits, S, beta, tn, tk,
-                  bslices + (static_cast<size_t>(tn) * Kt + tk) * kTile,
-                  static_cast<size_t>(Nt) * Kt * kTile, sb, rn, halves, kOzTileRows,
-                  SplitGeo<V>::kChunksPerRow, diff, blockIdx.z, blockIdx.z + 1);
+  split_b_tile(B, k, n, colbits, split, tn, tk,
+               bslices + (static_cast<size_t>(tn) * Kt + tk) * kTile,
+               static_cast<size_t>(Nt) * Kt * kTile, sb, halves, kOzTileRows,
+               SplitGeo<Split::V>::kChunksPerRow, blockIdx.z, blockIdx.z + 1);
 }
 
 // ---------------------------------------------------------------- grouped steps 1-2
@@ -795,6 +820,7 @@ __global__ void __launch_bounds__(256, 3) oz_grouped_split_kernel(uint8_t* __res
   const uint64_t* colbits = reinterpret_cast<const uint64_t*>(ws + hdr->off_colbits);
   const int32_t* owner = reinterpret_cast<const int32_t*>(ws + hdr->off_owner);
   __shared__ double sb[kSplitBRows][kOzTileRows + 1];
+  const SplitterAny split{S, beta, rn};
   const int64_t atiles = hdr->atiles, total = atiles + hdr->btiles;
   for (int64_t u = blockIdx.x; u < total; u += gridDim.x) {  // block-uniform
     const bool in_b = u >= atiles;
@@ -806,17 +832,16 @@ __global__ void __launch_bounds__(256, 3) oz_grouped_split_kernel(uint8_t* __res
     if (!in_b) {
       const int64_t rows = r.m - tr * kOzTileRows;
       const int row_lim = rows >= kOzTileRows ? kOzTileRows : static_cast<int>((rows + 7) / 8 * 8);
-      split_a_tile<8>(r.A, r.m, r.k, rowbits + r.row_begin, S, beta, tr, tk,
-                      ws + hdr->off_a + static_cast<size_t>(t) * kOzTileBytes,
-                      static_cast<size_t>(atiles) * kOzTileBytes, rn, row_lim, lim);
+      split_a_tile(r.A, r.m, r.k, rowbits + r.row_begin, split, tr, tk,
+                   ws + hdr->off_a + static_cast<size_t>(t) * kOzTileBytes,
+                   static_cast<size_t>(atiles) * kOzTileBytes, row_lim, lim);
     } else {
       const int64_t cols = r.n - tr * kOzTileRows;
       const int row_lim =
           cols >= kOzTileRows ? kOzTileRows : static_cast<int>((cols + 15) / 16 * 16);
-      split_b_tile<8>(r.B, r.k, r.n, colbits + r.col_begin, S, beta, tr, tk,
-                      ws + hdr->off_b + static_cast<size_t>(t) * kOzTileBytes,
-                      static_cast<size_t>(hdr->btiles) * kOzTileBytes, sb, rn, false, row_lim,
-                      lim);
+      split_b_tile(r.B, r.k, r.n, colbits + r.col_begin, split, tr, tk,
+                   ws + hdr->off_b + static_cast<size_t>(t) * kOzTileBytes,
+                   static_cast<size_t>(hdr->btiles) * kOzTileBytes, sb, false, row_lim, lim);
     }
   }
 }
@@ -2291,8 +2316,14 @@ cudaError_t launch_ozaki_scale(const double* A, const double* B, const OzakiDims
   if (d.m > 0 && !(oz_fused_a(d) && d.Kt > 0)) {
     const int warps = 8;
     const int64_t blocks = (d.m + warps - 1) / warps;
-    oz_rowmax_kernel<<<static_cast<unsigned>(blocks), warps * 32, 0, s>>>(A, d.m, d.k, rowbits,
-                                                                          status);
+    cudaError_t e = cudaMemsetAsync(rowbits, 0, sizeof(uint64_t) * d.m, s);
+    if (e != cudaSuccess) return e;
+    const int64_t runs = (d.k + kRowMaxRun - 1) / kRowMaxRun;  // k <= 2^31: below 2^20
+    for (int64_t y = 0; y < runs; y += 32768) {
+      const unsigned now = static_cast<unsigned>(runs - y < 32768 ? runs - y : 32768);
+      oz_rowmax_kernel<<<dim3(static_cast<unsigned>(blocks), now), warps * 32, 0, s>>>(
+          A, d.m, d.k, y, reinterpret_cast<unsigned long long*>(rowbits), status);
+    }
   }
   if (d.n > 0) {
     cudaError_t e = cudaMemsetAsync(colbits, 0, sizeof(uint64_t) * d.n, s);
@@ -2307,39 +2338,51 @@ cudaError_t launch_ozaki_scale(const double* A, const double* B, const OzakiDims
   return cudaGetLastError();
 }
 
+template <int kKind, bool kDiff>
+static cudaError_t launch_split_t(const double* A, const double* B, const OzakiDims& d,
+                                  uint64_t* rowbits, const uint64_t* colbits, uint8_t* aslices,
+                                  uint8_t* bslices, int* status, cudaStream_t s) {
+  const Splitter<kKind, kDiff> sa{d.S, d.beta, 0u}, sb{d.S, d.beta, 0x80008000u};
+  if (d.Mt > 0 && kKind != kKindE4m3 && oz_fused_a(d)) {
+    if constexpr (kKind != kKindE4m3) {
+      const int R = d.Kt <= 2 ? 8 : d.Kt <= 4 ? 4 : d.Kt <= 8 ? 2 : 1;
+      const size_t smem = R * static_cast<size_t>(d.Kt) * kOzTileK * sizeof(double);
+      auto kern = oz_scale_split_a_kernel<Splitter<kKind, kDiff>>;
+      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                                           static_cast<int>(smem));
+      if (e != cudaSuccess) return e;
+      kern<<<static_cast<unsigned>(d.Mt * kOzTileRows / R), 256, smem, s>>>(
+          A, d.m, d.k, rowbits, sa, R, d.Mt, d.Kt, aslices, status);
+    }
+  } else if (d.Mt > 0) {
+    oz_split_a_kernel<<<dim3(static_cast<unsigned>(d.Kt), static_cast<unsigned>(d.Mt)), 256, 0,
+                        s>>>(A, d.m, d.k, rowbits, sa, d.Mt, d.Kt, aslices);
+  }
+  if (d.Nt > 0)
+    oz_split_b_kernel<<<dim3(static_cast<unsigned>(d.Kt), static_cast<unsigned>(d.Nt),
+                             kOzTileK / kSplitBRows),
+                        256, 0, s>>>(B, d.k, d.n, colbits, sb, d.Nt, d.Kt, bslices,
+                                     ozaki_b_halves(d));
+  return cudaGetLastError();
+}
+
 cudaError_t launch_ozaki_split(const double* A, const double* B, const OzakiDims& d,
                                uint64_t* rowbits, const uint64_t* colbits,
                                uint8_t* aslices, uint8_t* bslices, int* status,
                                cudaStream_t s) {
   if (d.Kt == 0) return cudaSuccess;
-  if (d.Mt > 0 && oz_fused_a(d)) {
-    const size_t smem = static_cast<size_t>(d.Kt) * kOzTileK * sizeof(double);
-    cudaError_t e = cudaFuncSetAttribute(oz_scale_split_a_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    oz_scale_split_a_kernel<<<static_cast<unsigned>(d.Mt * kOzTileRows), 256, smem, s>>>(
-        A, d.m, d.k, rowbits, d.S, d.beta, d.Mt, d.Kt, aslices, d.rn != 0, d.kara, status);
-  } else if (d.Mt > 0) {
-    dim3 grid(static_cast<unsigned>(d.Kt), static_cast<unsigned>(d.Mt));
-    if (d.fp8)
-      oz_split_a_kernel<16><<<grid, 256, 0, s>>>(A, d.m, d.k, rowbits, d.S, d.beta, d.Mt, d.Kt,
-                                                 aslices, false, 0);
-    else
-      oz_split_a_kernel<8><<<grid, 256, 0, s>>>(A, d.m, d.k, rowbits, d.S, d.beta, d.Mt, d.Kt,
-                                                aslices, d.rn != 0, d.kara);
-  }
-  if (d.Nt > 0) {
-    dim3 grid(static_cast<unsigned>(d.Kt), static_cast<unsigned>(d.Nt), kOzTileK / kSplitBRows);
-    if (d.fp8)
-      oz_split_b_kernel<16><<<grid, 256, 0, s>>>(B, d.k, d.n, colbits, d.S, d.beta, d.Nt, d.Kt,
-                                                 bslices, false, false, 0);
-    else
-      oz_split_b_kernel<8><<<grid, 256, 0, s>>>(B, d.k, d.n, colbits, d.S, d.beta, d.Nt, d.Kt,
-                                                bslices, d.rn != 0, ozaki_b_halves(d),
-                                                d.kara ? -1 : 0);
-  }
-  return cudaGetLastError();
+  auto go = [&](auto kind, auto diff) {
+    return launch_split_t<decltype(kind)::value, decltype(diff)::value>(
+        A, B, d, rowbits, colbits, aslices, bslices, status, s);
+  };
+  auto either = [&](auto kind) {
+    return d.kara ? go(kind, std::true_type{}) : go(kind, std::false_type{});
+  };
+  if (d.fp8) return go(std::integral_constant<int, kKindE4m3>{}, std::false_type{});
+  if (d.rn) return either(std::integral_constant<int, 2>{});
+  if (d.beta == 7 && d.S <= 9) return either(std::integral_constant<int, 0>{});
+  if (d.beta == 8 && d.S <= 8) return either(std::integral_constant<int, 1>{});
+  return go(std::integral_constant<int, kKindOther>{}, std::false_type{});
 }
 
 int g_sm_count = 0;
@@ -2368,29 +2411,51 @@ static cudaError_t launch_oz_gemm_t(const Tiles& tiles, int64_t grid, int S, int
 }
 
 // Split-k recombination (steps 3-4 after a split product): D_g of every C
-// element is the exact int64 sum of the k ranges' partials, added in range
-// order; then the fold and the final scaling of the slice GEMM's epilogue,
-// with the exact phase taken from the full k.  Thread idx walks the
-// elements column by column (consecutive threads: consecutive rows, i.e.
-// contiguous partials in the column-major tiles).
+// element is the exact int64 sum of the k ranges' partials, then the fold and
+// the final scaling of the slice GEMM's epilogue, with the exact phase taken
+// from the full k.  A block takes 256 / kRows elements down the columns
+// (consecutive threads: consecutive rows, i.e. contiguous partials in the
+// column-major tiles); kRows threads share an element's ranges and one of them
+// folds: eight from 32 ranges on (128 ranges of 128 x 128, S = 6: 23 us, one
+// thread for all ranges 110 us), one below (4096 x 128, 9 ranges).
+template <int kRows>
 __global__ void __launch_bounds__(256) oz_splitk_fold_kernel(
     const uint64_t* __restrict__ P, const uint64_t* __restrict__ rowbits,
     const uint64_t* __restrict__ colbits, double* __restrict__ C, int64_t m, int64_t n,
-    int64_t Mt, int64_t Nt, int64_t Kt, int64_t splits, int S, int beta, int eoff) {
-  const int64_t idx = static_cast<int64_t>(blockIdx.x) * blockDim.x + threadIdx.x;
-  if (idx >= m * n) return;
-  const int64_t col = idx / m, row = idx - (idx / m) * m;
+    int64_t Mt, int64_t Nt, int64_t splits, int S, int beta, int gx, int eoff) {
+  constexpr int E = 256 / kRows;
+  __shared__ long long part[kRows > 1 ? kOzMaxSlices : 1][kRows][E];
+  const int tx = threadIdx.x % E, ty = threadIdx.x / E;
+  const int64_t idx = static_cast<int64_t>(blockIdx.x) * E + tx;
+  const bool live = idx < m * n;
+  const int64_t col = live ? idx / m : 0, row = live ? idx - col * m : 0;
   constexpr int64_t kTileWords = kOzTileRows * kOzTileRows;
   const int64_t tile = (row / kOzTileRows) * Nt + col / kOzTileRows;
   const uint64_t* p = P + tile * S * kTileWords + (col % kOzTileRows) * kOzTileRows +
                       row % kOzTileRows;
   const int64_t range_stride = Mt * Nt * S * kTileWords;
-  const int gx = oz_exact_from(S, beta, Kt);
+  auto sum = [&](int g) {
+    long long d = 0;
+#pragma unroll 8
+    for (int64_t sp = ty; sp < splits; sp += kRows)
+      d += static_cast<long long>(__ldcs(p + sp * range_stride + (g - 2) * kTileWords));
+    return d;
+  };
+  if constexpr (kRows > 1) {
+    for (int g = 2; g <= S + 1; ++g) part[g - 2][ty][tx] = live ? sum(g) : 0;
+    __syncthreads();
+    if (ty != 0) return;
+  }
+  if (!live) return;
   uint64_t st = 0;
   for (int g = S + 1; g >= 2; --g) {
     long long dval = 0;
-    const uint64_t* q = p + static_cast<int64_t>(g - 2) * kTileWords;
-    for (int64_t sp = 0; sp < splits; ++sp) dval += static_cast<long long>(__ldcs(q + sp * range_stride));
+    if constexpr (kRows > 1) {
+#pragma unroll
+      for (int q = 0; q < kRows; ++q) dval += part[g - 2][q][tx];
+    } else {
+      dval = sum(g);
+    }
     st = fold_step(st, dval, g, gx, S, beta);
   }
   C[row * n + col] = final_scale(
@@ -2469,9 +2534,13 @@ cudaError_t launch_ozaki_gemm(const uint8_t* aslices, const uint8_t* bslices,
         launch_oz_gemm_t<long long, false>(tiles, grid, d.S, d.beta, window, status, s);
     if (e != cudaSuccess) return e;
     const int64_t total = d.m * d.n;
-    oz_splitk_fold_kernel<<<static_cast<unsigned>((total + 255) / 256), 256, 0, s>>>(
-        sums, rowbits, colbits, C, d.m, d.n, d.Mt, d.Nt, d.Kt, splits, d.S, d.beta,
-        d.rn ? 2 : 0);
+    auto fold = [&](auto kern, int64_t per_block) {
+      kern<<<static_cast<unsigned>((total + per_block - 1) / per_block), 256, 0, s>>>(
+          sums, rowbits, colbits, C, d.m, d.n, d.Mt, d.Nt, splits, d.S, d.beta,
+          ozaki_exact_from(d.S, d.beta, d.Kt), d.rn ? 2 : 0);
+    };
+    if (splits >= 32) fold(oz_splitk_fold_kernel<8>, 32);
+    else fold(oz_splitk_fold_kernel<1>, 256);
     return cudaGetLastError();
   }
   // the paired kernel; when a diagonal's sum over all of k may pass int32,

@@ -740,7 +740,7 @@ bool choose_cut(const OzakiDims& d, int64_t rest, int64_t pairs, KaraArgs& a) {
   for (int parts = 1; parts <= a.prog.nseg; ++parts) {
     const int worst = cut_segments(a.prog, parts, part);
     const int segs = (a.prog.nseg + parts - 1) / parts;
-    for (int ranges = least; ranges < least + 16 && ranges <= d.Kt; ++ranges) {
+    for (int ranges = least; ranges <= kara_max_ranges(d); ++ranges) {
       if (static_cast<size_t>(rest * ranges * nslots) > kara_cut_slots(d)) break;
       const int64_t waves = (rest * parts * ranges + pairs - 1) / pairs;
       const double cost = waves * (static_cast<double>((d.Kt + ranges - 1) / ranges) * worst +

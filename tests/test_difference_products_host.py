@@ -46,6 +46,8 @@ int main() {
   CHECK(kara_chosen(ozaki_dims(129, 64, 129, 7, 7)));
   CHECK(!kara_chosen(ozaki_dims(128, 64, 1024, 7, 7)));
   CHECK(!kara_chosen(ozaki_dims(1024, 64, 128, 7, 7)));
+  CHECK(kara_chosen(ozaki_dims(1024, 300, 100, 7, 7)));
+  CHECK(!kara_chosen(ozaki_dims(32768, 1024, 64, 7, 7)));
   CHECK(!kara_chosen(ozaki_dims(1024, 1024, 1024, 2, 7)));
   CHECK(!kara_chosen(ozaki_dims(1024, 1024, 1024, 10, 7)));
   CHECK(kara_chosen(ozaki_dims(8192, 8192, 8192, 7, 7)));

@@ -28,6 +28,9 @@ def _emulated(A, B, mode, S):
     (mxm.MODE_EMUL_I8, 7, 129, 129, 129),      # a second tile row, column, k-block of one
     (mxm.MODE_EMUL_I8, 8, 385, 1040, 257),     # odd tile counts; 9 k-blocks: two windows
     (mxm.MODE_EMUL_I8, 3, 300, 200, 257),
+    (mxm.MODE_EMUL_I8, 7, 100, 300, 77),       # a single tile-row and tile-column
+    (mxm.MODE_EMUL_RN8, 6, 90, 1000, 600),
+    (mxm.MODE_EMUL_BF16, 6, 700, 260, 128),
     (mxm.MODE_EMUL_I8, 4, 260, 300, 513),
     (mxm.MODE_EMUL_I8, 5, 513, 17, 300),
     (mxm.MODE_EMUL_I8, 6, 257, 2100, 130),     # few tiles: cut along k too
