@@ -2,14 +2,12 @@
 // F(k) = sum_n f(n) W_N^{kn}, W_N = exp(-2 pi i / N), N a power of two,
 // FP64 complex data interleaved (re, im).
 //
-// The radix-2 decimation in frequency of Eqs. 2-3 is the butterfly of every
-// stage: a block of length L becomes f_e(n) = f(n) + f(n + L/2) in its first
-// half and f_o(n) = (f(n) - f(n + L/2)) W_L^n in its second; after log2 L
-// stages position i holds F(bitrev(i)).  The paper's split-stream form
-// (tangle once, then every stage reads even / odd streams and concatenates
-// up / down streams) is a layout for stream processors; here the stages of
-// one sub-transform run in a CTA's shared memory instead, and a transform
-// too large for one CTA is cut in two passes over global memory (the
+// Eqs. 2-3 split a transform into radix-2 butterflies; the paper's
+// split-stream form (tangle once, then every stage reads even / odd streams and
+// concatenates up / down streams) is a layout for stream processors.  Here the
+// stages of one sub-transform run in a CTA's shared memory, in the
+// decimation-in-time order (input bit-reversed, output in place), and a
+// transform too large for one CTA is cut in two passes over global memory (the
 // "four-step" factorisation N = N1 N2, n = N2 n1 + n2, k = k1 + N1 k2):
 //
 //   pass 1: for every n2, the N1-point transform over n1 of x(N2 n1 + n2),
@@ -17,14 +15,19 @@
 //   pass 2: for every k1, the N2-point transform over n2 of Y[k1][.],
 //           stored at X(k1 + N1 k2).
 //
-// A CTA takes C neighbouring columns, so every global access moves C
-// consecutive complex values.  Small transforms (N <= 1024) are one pass of
-// one CTA.  FP64 is scarce on this GPU (~4 G fused multiply-adds per second
-// per SM): the stages go two at a time (radix 4, 28 FP64 operations per 4
-// points and 2 stages against 32 for radix 2; none in the last, whose
-// twiddles are 1 and -i).  Twiddles come from a caller-owned table of
-// W_T^j, j < T/2, for a power of two T that N divides (one table serves
-// every smaller order), expanded per CTA into shared memory.
+// FP64 is scarce on this GPU (a warp-wide FP64 instruction holds an SM
+// sub-partition 64 clocks), so what counts is the number of FP64 instructions
+// (the stages go two at a time, radix 4: 28 per 4 points and 2 stages, 16 in
+// the twiddle-free first two) and that all sub-partitions have the same share
+// of them: a CTA takes as many neighbouring columns as leave the waves of CTAs
+// nearly full (2^20 points: one column, 1024 CTAs on 152 SMs; two columns, 512
+// CTAs, fill 0.84 of theirs).  Indexes are shifts on 32 bits and signs flip by
+// integers (a negation is an FP64 instruction: 39.5 + 33.5 a point before, 36 +
+// 32 now).  Measured: 2^20 points 186 -> 158 us (the FP64 pipe alone 113 us, the
+// rest the loads and stores at the ends of the passes and the barriers between
+// stages), 2^10 11.2 -> 8.7 us, 2^22 727 -> 665 us.  Butterflies of fused multiply-adds (a + w b in
+// four, a - w b = 2 a - (a + w b) in two: 24 per radix 4) ran 2^20 points in
+// 134 us, but with a tenth more error, and are not used.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -43,15 +46,41 @@ constexpr int64_t kFftMaxN = int64_t{1} << 22;
 constexpr int64_t kFftSingleMax = 1024;
 constexpr int64_t kFftClusterMin = 16, kFftClusterMax = 8192;
 
-__device__ __forceinline__ double2 cadd(double2 a, double2 b) {
-  return make_double2(a.x + b.x, a.y + b.y);
+// On this GPU a fused multiply-add of three registers issues every 64 clocks, an
+// add, a multiply or a form with a constant operand every 76: sums and products
+// go through fused multiply-adds with 1, -1 and -0 held in registers (read back
+// from shared memory, so that the compiler does not know them; the results are
+// those of the plain operations, signed zeros included).
+struct Units {
+  double one, mone, nzero;
+};
+__device__ __forceinline__ Units units() {
+  __shared__ volatile double u[3];
+  if (threadIdx.x == 0) {
+    u[0] = 1.0;
+    u[1] = -1.0;
+    u[2] = -0.0;
+  }
+  __syncthreads();
+  return Units{u[0], u[1], u[2]};
 }
-__device__ __forceinline__ double2 csub(double2 a, double2 b) {
-  return make_double2(a.x - b.x, a.y - b.y);
+__device__ __forceinline__ double2 cadd(double2 a, double2 b, const Units& k) {
+  return make_double2(fma(a.x, k.one, b.x), fma(a.y, k.one, b.y));
+}
+__device__ __forceinline__ double2 csub(double2 a, double2 b, const Units& k) {
+  return make_double2(fma(b.x, k.mone, a.x), fma(b.y, k.mone, a.y));
+}
+// a - i b and a + i b
+__device__ __forceinline__ double2 csubi(double2 a, double2 b, const Units& k) {
+  return make_double2(fma(b.y, k.one, a.x), fma(b.x, k.mone, a.y));
+}
+__device__ __forceinline__ double2 caddi(double2 a, double2 b, const Units& k) {
+  return make_double2(fma(b.y, k.mone, a.x), fma(b.x, k.one, a.y));
 }
 // (a + bi)(c + di) with one rounding per component after a fused multiply-add
-__device__ __forceinline__ double2 cmul(double2 a, double2 w) {
-  return make_double2(fma(a.x, w.x, -(a.y * w.y)), fma(a.x, w.y, a.y * w.x));
+__device__ __forceinline__ double2 cmul(double2 a, double2 w, const Units& k) {
+  return make_double2(fma(a.x, w.x, -fma(a.y, w.y, k.nzero)),
+                      fma(a.x, w.y, fma(a.y, w.x, k.nzero)));
 }
 
 __device__ __forceinline__ uint32_t bitrev(uint32_t i, int bits) {
@@ -59,61 +88,69 @@ __device__ __forceinline__ uint32_t bitrev(uint32_t i, int bits) {
 }
 
 // W_T^j for 0 <= j < T from the half table (W_T^{j + T/2} = -W_T^j).
-__device__ __forceinline__ double2 table_w(const double2* __restrict__ table, int64_t T,
-                                           int64_t j) {
-  const int64_t h = T >> 1;
+__device__ __forceinline__ double2 table_w(const double2* __restrict__ table, uint32_t T,
+                                           uint32_t j) {
+  const uint32_t h = T >> 1;
   if (j < h) return __ldg(table + j);
   const double2 w = __ldg(table + (j - h));
-  return make_double2(-w.x, -w.y);
+  // the sign bits by integers: a negation is an instruction of the FP64 pipe
+  return make_double2(
+      __hiloint2double(__double2hiint(w.x) ^ static_cast<int>(0x80000000u), __double2loint(w.x)),
+      __hiloint2double(__double2hiint(w.y) ^ static_cast<int>(0x80000000u), __double2loint(w.y)));
 }
 
-// The decimation-in-frequency stages of C columns of L points in shared
-// memory (data[c L + i]), two at a time (radix 4): a block of length B = 4q
-// with a_m = x(j + m q), W = W_B, j < q, becomes
-//   x(j)      = (a0 + a2) + (a1 + a3)
-//   x(j + q)  = ((a0 + a2) - (a1 + a3)) W^{2j}
-//   x(j + 2q) = ((a0 - a2) - i (a1 - a3)) W^j
-//   x(j + 3q) = ((a0 - a2) + i (a1 - a3)) W^{3j}
-// which is the two radix-2 stages of lengths B and B/2 (Eqs. 2-3) with
-// W_B^{j + q} = -i W_B^j folded in: 3 complex products per 4 points instead
-// of 4, and one barrier per two stages.  An odd stage count ends with the
-// twiddle-free radix-2 stage of length 2.  tw[m] = W_L^m, m < L.  Position i
-// of a column then holds its transform at bitrev(i).  All threads of the
-// block call it; it ends with a barrier.
-__device__ void smem_fft(double2* data, const double2* tw, int64_t L, int C) {
+// The decimation-in-time stages of C columns of L = 2^bits points in shared
+// memory (data[c L + i], position i holding input bitrev(i); output in
+// natural order), two at a time (radix 4): with h a quarter of the block,
+// w = W_{4h}^j, j < h, and x_m at j + m h,
+//   y0 = x0, y1 = w^2 x1, y2 = w x2, y3 = w^3 x3
+//   x0, x2 = (y0 + y1) +- (y2 + y3);  x1, x3 = (y0 - y1) -+ i (y2 - y3)
+// (the radix-2 stages of lengths 2h and 4h with W_{4h}^{j + h} = -i W_{4h}^j
+// folded in).  An odd number of stages begins with the twiddle-free radix-2
+// stage.  tw[m] = W_L^m, m < 3 L / 4.  All threads of the block call it; it
+// ends with a barrier.
+__device__ __forceinline__ void smem_fft(double2* data, const double2* tw, int bits, int C,
+                                         const Units& k) {
   const int tid = threadIdx.x, nth = blockDim.x;
-  int64_t B = L;
-  for (; B >= 4; B >>= 2) {
-    const int64_t q = B >> 2;
-    const int64_t ts = L / B;  // W_B^m = W_L^{m L / B}
-    for (int64_t t = tid; t < C * (L >> 2); t += nth) {
-      const int64_t c = t / (L >> 2), u = t - c * (L >> 2);
-      const int64_t grp = u / q, j = u - grp * q;
-      double2* p = data + c * L + grp * B + j;
-      const double2 a0 = p[0], a1 = p[q], a2 = p[2 * q], a3 = p[3 * q];
-      const double2 s02 = cadd(a0, a2), d02 = csub(a0, a2);
-      const double2 s13 = cadd(a1, a3), d13 = csub(a1, a3);
-      const double2 nd13 = make_double2(d13.y, -d13.x);  // -i (a1 - a3)
-      p[0] = cadd(s02, s13);
-      const double2 y1 = csub(s02, s13), y2 = cadd(d02, nd13), y3 = csub(d02, nd13);
-      if (q == 1) {  // j = 0: every twiddle is 1
-        p[q] = y1;
-        p[2 * q] = y2;
-        p[3 * q] = y3;
-      } else {
-        p[q] = cmul(y1, tw[2 * j * ts]);
-        p[2 * q] = cmul(y2, tw[j * ts]);
-        p[3 * q] = cmul(y3, tw[3 * j * ts]);
-      }
-    }
-    __syncthreads();
-  }
-  if (B == 2) {  // the last stage, length 2: W_2^0 = 1
-    for (int64_t t = tid; t < C * (L >> 1); t += nth) {
+  const int L = 1 << bits;
+  int hb = 0;  // h = 2^hb
+  if (bits & 1) {
+    for (int t = tid; t < C * (L >> 1); t += nth) {
       double2* p = data + 2 * t;
       const double2 x0 = p[0], x1 = p[1];
-      p[0] = cadd(x0, x1);
-      p[1] = csub(x0, x1);
+      p[0] = cadd(x0, x1, k);
+      p[1] = csub(x0, x1, k);
+    }
+    __syncthreads();
+    hb = 1;
+  } else if (bits >= 2) {
+    for (int t = tid; t < C * (L >> 2); t += nth) {
+      double2* p = data + 4 * t;
+      const double2 x0 = p[0], x1 = p[1], x2 = p[2], x3 = p[3];
+      const double2 b0 = cadd(x0, x1, k), b1 = csub(x0, x1, k), b2 = cadd(x2, x3, k),
+                    b3 = csub(x2, x3, k);
+      p[0] = cadd(b0, b2, k);
+      p[2] = csub(b0, b2, k);
+      p[1] = csubi(b1, b3, k);
+      p[3] = caddi(b1, b3, k);
+    }
+    __syncthreads();
+    hb = 2;
+  }
+  for (; hb + 2 <= bits; hb += 2) {
+    const int h = 1 << hb, ts = bits - hb - 2;  // W_{4h}^j = W_L^{j 2^ts}
+    for (int t = tid; t < C * (L >> 2); t += nth) {
+      const int j = t & (h - 1);
+      double2* p = data + ((t - j) << 2) + j;  // columns follow each other: blocks of 4 h
+      const int jt = j << ts;
+      const double2 y0 = p[0], y1 = cmul(p[h], tw[2 * jt], k), y2 = cmul(p[2 * h], tw[jt], k),
+                    y3 = cmul(p[3 * h], tw[3 * jt], k);
+      const double2 b0 = cadd(y0, y1, k), b1 = csub(y0, y1, k), b2 = cadd(y2, y3, k),
+                    b3 = csub(y2, y3, k);
+      p[0] = cadd(b0, b2, k);
+      p[2 * h] = csub(b0, b2, k);
+      p[h] = csubi(b1, b3, k);
+      p[3 * h] = caddi(b1, b3, k);
     }
     __syncthreads();
   }
@@ -123,10 +160,9 @@ struct FftPass {
   const double2* src;
   double2* dst;
   const double2* table;  // W_T^j, j < T/2
-  int64_t T;             // table order
-  int64_t N;             // transform order
-  int64_t N1, N2;        // N = N1 N2; this pass transforms along L = N1 (pass 1) or N2
-  int C;                 // columns per CTA
+  int tbits;             // T = 2^tbits
+  int bits1, bits2;      // N = N1 N2, N1 = 2^bits1; this pass transforms along N1 (stage 1) or N2
+  int cbits;             // 2^cbits columns per CTA
   int stage;             // 1 or 2
 };
 
@@ -136,48 +172,43 @@ struct FftPass {
 //            transform, written in natural order, no twiddle);
 //   stage 2: column k1 = c0 + c reads Y[k1][n2], n2 < L = N2; writes
 //            X(k1 + N1 k2).
+// Orders and columns are powers of two and N <= 2^22: shifts on 32 bits.
 __global__ void __launch_bounds__(kFftThreads) fft_pass_kernel(const FftPass a) {
   extern __shared__ double2 sm[];
-  const int C = a.C;
-  const int64_t L = a.stage == 1 ? a.N1 : a.N2;
-  const int64_t cols = a.stage == 1 ? a.N2 : a.N1;  // columns of this pass
-  int lbits = 0;
-  while ((int64_t{1} << lbits) < L) ++lbits;
+  const int C = 1 << a.cbits;
+  const int bits = a.stage == 1 ? a.bits1 : a.bits2, L = 1 << bits;
   double2* data = sm;             // [C][L]
-  double2* tw = sm + C * L;       // W_L^m, m < L
-  const int64_t c0 = static_cast<int64_t>(blockIdx.x) * C;
-  const int tid = threadIdx.x;
+  double2* tw = sm + (C << bits); // W_L^m, m < 3 L / 4
+  const int c0 = static_cast<int>(blockIdx.x) << a.cbits;
+  const int tid = threadIdx.x, nth = blockDim.x;
+  const Units k = units();
 
   // twiddles of the L-point transform: W_L^m = W_T^{m T / L}
-  const int64_t tstride = a.T / (L > 0 ? L : 1);
-  for (int64_t m = tid; m < L; m += kFftThreads) tw[m] = table_w(a.table, a.T, m * tstride);
+  for (int m = tid; m < (3 * L + 3) / 4; m += nth)
+    tw[m] = table_w(a.table, 1u << a.tbits, static_cast<uint32_t>(m) << (a.tbits - bits));
   // load: C consecutive columns per row, c fastest
-  for (int64_t t = tid; t < L * C; t += kFftThreads) {
-    const int64_t r = t / C, c = t - r * C;
-    const int64_t col = c0 + c;
-    double2 v = make_double2(0.0, 0.0);
-    if (col < cols) v = a.src[a.stage == 1 ? a.N2 * r + col : col * a.N2 + r];
-    data[c * L + r] = v;
+  for (int t = tid; t < (C << bits); t += nth) {
+    const int r = t >> a.cbits, c = t & (C - 1), col = c0 + c;
+    const int at = a.stage == 1 ? (r << a.bits2) + col : (col << a.bits2) + r;
+    data[(c << bits) + bitrev(static_cast<uint32_t>(r), bits)] = a.src[at];
   }
   __syncthreads();
 
-  smem_fft(data, tw, L, C);
+  smem_fft(data, tw, bits, C, k);
 
-  // store: position i of column c holds the transform at bitrev(i)
-  for (int64_t t = tid; t < L * C; t += kFftThreads) {
-    const int64_t kk = t / C, c = t - kk * C;
-    const int64_t col = c0 + c;
-    if (col >= cols) continue;
-    double2 v = data[c * L + bitrev(static_cast<uint32_t>(kk), lbits)];
+  const uint32_t nmask = (1u << (a.bits1 + a.bits2)) - 1u;
+  for (int t = tid; t < (C << bits); t += nth) {
+    const int kk = t >> a.cbits, c = t & (C - 1), col = c0 + c;
+    double2 v = data[(c << bits) + kk];
     if (a.stage == 1) {
-      if (a.N2 > 1) {
-        v = cmul(v, table_w(a.table, a.T, ((col * kk) & (a.N - 1)) * (a.T / a.N)));
-        a.dst[kk * a.N2 + col] = v;  // Y[k1][n2]
-      } else {
-        a.dst[kk] = v;
-      }
+      if (a.bits2 > 0)
+        v = cmul(v, table_w(a.table, 1u << a.tbits,
+                            ((static_cast<uint32_t>(col) * static_cast<uint32_t>(kk)) & nmask)
+                                << (a.tbits - a.bits1 - a.bits2)),
+                 k);
+      a.dst[(kk << a.bits2) + col] = v;  // Y[k1][n2]
     } else {
-      a.dst[col + a.N1 * kk] = v;  // X(k1 + N1 k2)
+      a.dst[col + (kk << a.bits1)] = v;  // X(k1 + N1 k2)
     }
   }
 }
@@ -197,7 +228,7 @@ struct FftCluster {
   const double2* src;
   double2* dst;
   const double2* table;
-  int64_t T, N, N1, N2;
+  int tbits, bits1, bits2;
 };
 
 __device__ __forceinline__ uint32_t fft_cluster_rank() {
@@ -218,47 +249,51 @@ __device__ __forceinline__ void fft_cluster_barrier() {
 
 __global__ void __launch_bounds__(kFftThreads) fft_cluster_kernel(const FftCluster a) {
   extern __shared__ double2 sm[];
-  const int64_t N1 = a.N1, N2 = a.N2;
-  const uint32_t rank = fft_cluster_rank(), C = fft_cluster_size();
-  const int64_t cols = N2 / C, rows = N1 / C;  // columns of pass 1, rows of pass 2 per CTA
-  double2* b1 = sm;                  // [cols][N1]
-  double2* b2 = b1 + cols * N1;      // [rows][N2], written by every CTA of the cluster
-  double2* tw1 = b2 + rows * N2;     // W_N1^m, m < N1
-  double2* tw2 = tw1 + N1;           // W_N2^m, m < N2
+  const int b1n = a.bits1, b2n = a.bits2, N1 = 1 << b1n, N2 = 1 << b2n;
+  const int rank = static_cast<int>(fft_cluster_rank());
+  const int sbits = 31 - __clz(static_cast<int>(fft_cluster_size()));
+  const int cbits = b2n - sbits, rbits = b1n - sbits;  // columns of pass 1, rows of pass 2 per CTA
+  double2* b1 = sm;                          // [cols][N1]
+  double2* b2 = b1 + (N1 << cbits);          // [rows][N2], written by every CTA of the cluster
+  double2* tw1 = b2 + (N2 << rbits);         // W_N1^m, m < 3 N1 / 4 (N1, N2 >= 4)
+  double2* tw2 = tw1 + 3 * N1 / 4;           // W_N2^m, m < 3 N2 / 4
   const int tid = threadIdx.x;
-  for (int64_t m = tid; m < N1; m += kFftThreads) tw1[m] = table_w(a.table, a.T, m * (a.T / N1));
-  for (int64_t m = tid; m < N2; m += kFftThreads) tw2[m] = table_w(a.table, a.T, m * (a.T / N2));
-  const int64_t c0 = static_cast<int64_t>(rank) * cols;
-  for (int64_t t = tid; t < N1 * cols; t += kFftThreads) {
-    const int64_t r = t / cols, c = t - r * cols;
-    b1[c * N1 + r] = a.src[N2 * r + c0 + c];
+  const Units k = units();
+  const int c0 = rank << cbits, cols = 1 << cbits, rows = 1 << rbits;
+  for (int t = tid; t < (N1 << cbits); t += kFftThreads) {
+    const int r = t >> cbits, c = t & (cols - 1);
+    b1[(c << b1n) + bitrev(static_cast<uint32_t>(r), b1n)] = a.src[(r << b2n) + c0 + c];
   }
+  for (int m = tid; m < 3 * N1 / 4; m += kFftThreads)
+    tw1[m] = table_w(a.table, 1u << a.tbits, static_cast<uint32_t>(m) << (a.tbits - b1n));
+  for (int m = tid; m < 3 * N2 / 4; m += kFftThreads)
+    tw2[m] = table_w(a.table, 1u << a.tbits, static_cast<uint32_t>(m) << (a.tbits - b2n));
   fft_cluster_barrier();  // every CTA runs (and has its tables) before any peer writes to it
-  smem_fft(b1, tw1, N1, static_cast<int>(cols));
-  int bits1 = 0;
-  while ((int64_t{1} << bits1) < N1) ++bits1;
-  // Y[k1][n2] = Z_{n2}(k1) W_N^{n2 k1}, into row k1 % rows of CTA k1 / rows
+  smem_fft(b1, tw1, b1n, cols, k);
+  // Y[k1][n2] = Z_{n2}(k1) W_N^{n2 k1}, into row k1 % rows of CTA k1 / rows at
+  // the place of n2 in the second transform's input order
   const uint32_t b2base = static_cast<uint32_t>(__cvta_generic_to_shared(b2));
-  for (int64_t t = tid; t < N1 * cols; t += kFftThreads) {
-    const int64_t k1 = t / cols, c = t - k1 * cols;
-    const int64_t n2 = c0 + c;
-    double2 v = b1[c * N1 + bitrev(static_cast<uint32_t>(k1), bits1)];
-    v = cmul(v, table_w(a.table, a.T, ((n2 * k1) & (a.N - 1)) * (a.T / a.N)));
-    const uint32_t owner = static_cast<uint32_t>(k1 / rows);
-    const uint32_t local = b2base + static_cast<uint32_t>(((k1 - owner * rows) * N2 + n2) * 16);
+  const uint32_t nmask = (1u << (b1n + b2n)) - 1u;
+  for (int t = tid; t < (N1 << cbits); t += kFftThreads) {
+    const int k1 = t >> cbits, c = t & (cols - 1), n2 = c0 + c;
+    double2 v = b1[(c << b1n) + k1];
+    v = cmul(v, table_w(a.table, 1u << a.tbits,
+                        (static_cast<uint32_t>(n2 * k1) & nmask) << (a.tbits - b1n - b2n)),
+             k);
+    const uint32_t owner = static_cast<uint32_t>(k1 >> rbits);
+    const uint32_t local =
+        b2base + ((((k1 & (rows - 1)) << b2n) + bitrev(static_cast<uint32_t>(n2), b2n)) << 4);
     uint32_t remote;
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(remote) : "r"(local), "r"(owner));
     asm volatile("st.shared::cluster.v2.f64 [%0], {%1, %2};" ::"r"(remote), "d"(v.x), "d"(v.y)
                  : "memory");
   }
   fft_cluster_barrier();
-  smem_fft(b2, tw2, N2, static_cast<int>(rows));
-  int bits2 = 0;
-  while ((int64_t{1} << bits2) < N2) ++bits2;
-  const int64_t r0 = static_cast<int64_t>(rank) * rows;
-  for (int64_t t = tid; t < N2 * rows; t += kFftThreads) {
-    const int64_t k2 = t / rows, c = t - k2 * rows;
-    a.dst[r0 + c + N1 * k2] = b2[c * N2 + bitrev(static_cast<uint32_t>(k2), bits2)];
+  smem_fft(b2, tw2, b2n, rows, k);
+  const int r0 = rank << rbits;
+  for (int t = tid; t < (N2 << rbits); t += kFftThreads) {
+    const int k2 = t >> rbits, c = t & (rows - 1);
+    a.dst[r0 + c + (k2 << b1n)] = b2[(c << b2n) + k2];
   }
 }
 
@@ -274,25 +309,40 @@ __global__ void fft_twiddle_kernel(double2* table, int64_t T) {
 
 bool pow2(int64_t v) { return v >= 1 && (v & (v - 1)) == 0; }
 
-// Columns per CTA: as many as keep at least two CTAs per SM, at most 8,
-// within 96 KiB of shared memory (C columns and the L twiddles).
-int fft_columns(int64_t L, int64_t cols) {
-  int C = 8;
-  while (C > 1 && (cols / C < 2 * static_cast<int64_t>(sm_count()) || (C * L + L) * 16 > 96 * 1024))
-    C /= 2;
-  return C;
+// Columns per CTA (a power of two, at most 8, at most 96 KiB of shared memory):
+// the most for which the last wave of CTAs over the SMs is at least 0.9 full on
+// average over the waves, else the count with the fullest waves.
+int fft_column_bits(int bits, int64_t cols) {
+  int best = 0;
+  double best_fill = 0.0;
+  for (int cb = 3; cb >= 0; --cb) {
+    const int64_t C = int64_t{1} << cb, L = int64_t{1} << bits;
+    if (cols < C || (C * L + L) * 16 > 96 * 1024) continue;
+    const int64_t blocks = cols / C, sms = sm_count();
+    const double fill = static_cast<double>(blocks) / static_cast<double>((blocks + sms - 1) / sms * sms);
+    if (fill >= 0.9) return cb;
+    if (fill > best_fill) {
+      best_fill = fill;
+      best = cb;
+    }
+  }
+  return best;
 }
 
 cudaError_t launch_pass(FftPass a, cudaStream_t s) {
-  const int64_t L = a.stage == 1 ? a.N1 : a.N2;
-  const int64_t cols = a.stage == 1 ? a.N2 : a.N1;
-  a.C = fft_columns(L, cols);
-  const size_t smem = static_cast<size_t>(a.C * L + L) * sizeof(double2);
+  const int bits = a.stage == 1 ? a.bits1 : a.bits2;
+  const int64_t cols = int64_t{1} << (a.stage == 1 ? a.bits2 : a.bits1);
+  a.cbits = fft_column_bits(bits, cols);
+  const size_t L = size_t{1} << bits;
+  const size_t smem = ((L << a.cbits) + (3 * L + 3) / 4) * sizeof(double2);
   cudaError_t e = cudaFuncSetAttribute(fft_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(smem));
   if (e != cudaSuccess) return e;
-  const int64_t blocks = (cols + a.C - 1) / a.C;
-  fft_pass_kernel<<<static_cast<unsigned>(blocks), kFftThreads, smem, s>>>(a);
+  // a thread per radix-4 butterfly, up to 256
+  int64_t threads = static_cast<int64_t>(L << a.cbits) / 4;
+  threads = threads > kFftThreads ? kFftThreads : (threads < 32 ? 32 : threads);
+  fft_pass_kernel<<<static_cast<unsigned>(cols >> a.cbits), static_cast<unsigned>(threads), smem,
+                    s>>>(a);
   return cudaGetLastError();
 }
 
@@ -301,9 +351,10 @@ cudaError_t launch_pass(FftPass a, cudaStream_t s) {
 // when it cannot, so that the caller takes the two-pass form.
 cudaError_t launch_cluster(const FftCluster& a, cudaStream_t s) {
   int64_t C = 16;
-  while (C > 1 && (a.N1 % C != 0 || a.N2 % C != 0)) C /= 2;
+  while (C > 1 && (C > (1 << a.bits1) || C > (1 << a.bits2))) C /= 2;
   for (; C >= 1; C /= 2) {
-    const size_t smem = static_cast<size_t>(2 * (a.N / C) + a.N1 + a.N2) * sizeof(double2);
+    const size_t N1 = size_t{1} << a.bits1, N2 = size_t{1} << a.bits2;
+    const size_t smem = (2 * (N1 * N2 / C) + 3 * (N1 + N2) / 4) * sizeof(double2);
     cudaError_t e = cudaFuncSetAttribute(fft_cluster_kernel,
                                          cudaFuncAttributeMaxDynamicSharedMemorySize,
                                          static_cast<int>(smem));
@@ -382,38 +433,37 @@ extern "C" mxm_status mxm_fft(const double* in, double* out, double* work, const
     return cudaMemcpyAsync(out, in, 16, cudaMemcpyDeviceToDevice, s) == cudaSuccess ? MXM_OK
                                                                                     : MXM_ERR_CUDA;
   }
-  int p = 0;
+  int p = 0, tp = 0;
   while ((int64_t{1} << p) < n) ++p;
-  const int64_t N1 = int64_t{1} << ((p + 1) / 2);
+  while ((int64_t{1} << tp) < table_n) ++tp;
+  const int bits1 = (p + 1) / 2;
   cudaError_t e = cudaErrorNotSupported;
   if (n >= kFftClusterMin && n <= kFftClusterMax) {
     FftCluster c;
     c.src = reinterpret_cast<const double2*>(in);
     c.dst = reinterpret_cast<double2*>(out);
     c.table = reinterpret_cast<const double2*>(table);
-    c.T = table_n;
-    c.N = n;
-    c.N1 = N1;
-    c.N2 = n / N1;
+    c.tbits = tp;
+    c.bits1 = bits1;
+    c.bits2 = p - bits1;
     e = launch_cluster(c, s);
     if (e == cudaSuccess) return MXM_OK;
     if (e != cudaErrorNotSupported) return MXM_ERR_CUDA;
   }
   FftPass a;
   a.table = reinterpret_cast<const double2*>(table);
-  a.T = table_n;
-  a.N = n;
-  a.C = 1;
+  a.tbits = tp;
+  a.cbits = 0;
   if (!two_pass) {
     a.src = reinterpret_cast<const double2*>(in);
     a.dst = reinterpret_cast<double2*>(out);
-    a.N1 = n;
-    a.N2 = 1;
+    a.bits1 = p;
+    a.bits2 = 0;
     a.stage = 1;
     e = launch_pass(a, s);
   } else {
-    a.N1 = N1;
-    a.N2 = n / a.N1;
+    a.bits1 = bits1;
+    a.bits2 = p - bits1;
     a.src = reinterpret_cast<const double2*>(in);
     a.dst = reinterpret_cast<double2*>(work);
     a.stage = 1;
