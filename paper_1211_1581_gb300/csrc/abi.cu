@@ -189,7 +189,7 @@ OzakiDims emul_dims(int mode, int64_t m, int64_t k, int64_t n, int slices, const
     OzakiDims w = d;
     w.splits = 1;
     if (kara_chosen(w)) {
-      w.kara = 1;
+      w.kara = kara_short(w) ? 2 : 1;
       w.pair = 1;
       w.raster = p.raster > 0 ? p.raster : kDefaultRaster;
       return w;
@@ -424,7 +424,7 @@ static mxm_status gemm_host_panels(DeviceState* ds, int mode, const double* hA, 
   const int64_t w = host_panel_cols(h, n, ds->sm_count);
   const int64_t P = (m + h - 1) / h, Q = (n + w - 1) / w;
   OzakiDims dp = ozaki_dims(h, k, w, slices, beta, rn);  // the largest block, no split-k
-  dp.kara = kara && kara_chosen(dp) ? 1 : 0;
+  dp.kara = kara && kara_chosen(dp) ? (kara_short(dp) ? 2 : 1) : 0;
   const OzakiLayout L = ozaki_layout(dp);
   // per compute stream: row scales, A planes, running sums of one block
   const size_t rb_bytes = align_up(sizeof(uint64_t) * size_t(h), 1024);

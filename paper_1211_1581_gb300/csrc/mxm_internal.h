@@ -101,8 +101,9 @@ struct OzakiDims {
                        //    persistent walk over C tiles
   int kb_alt;          // 1: alternate the k-block direction from one diagonal
                        //    (pair) to the next
-  int kara;            // 1: difference products on 256 x 256 C tiles (ozaki_kara.cu);
-                       //    the operands have kara_planes(S) digit planes
+  int kara;            // 1: difference products on 256 x 256 C tiles (ozaki_kara.cu),
+                       //    2: on 256 x 128 tiles (little k); the operands have
+                       //    kara_planes(S) digit planes
 };
 
 // Default walk: groups of 8 tile-rows (4 pair-rows on CTA pairs); the
@@ -159,7 +160,7 @@ inline OzakiDims ozaki_dims_splitk(int64_t m, int64_t k, int64_t n, int S, int b
 // tiles): bf16 digits without split-k, chosen where the dims are made (two
 // or more tile-rows of A; products that share B planes share the choice,
 // a single tile-row then leaving the second CTA of its pairs idle).
-inline bool ozaki_b_halves(const OzakiDims& d) { return d.pair != 0 && !d.fp8 && !d.kara; }
+inline bool ozaki_b_halves(const OzakiDims& d) { return d.pair != 0 && !d.fp8 && d.kara != 1; }
 inline bool ozaki_cta2(const OzakiDims& d) {
   return ozaki_b_halves(d) && d.splits <= 1 && d.Mt >= 1;
 }
@@ -287,6 +288,10 @@ inline size_t kara_cut_slots(const OzakiDims& d) {
   return most <= cap ? most : (least > cap ? least : cap);
 }
 inline size_t kara_scratch_bytes(const OzakiDims& d) {
+  if (d.kara == 2) {  // per CTA S slots of a 128 x 128 tile
+    const int64_t t = (d.Mt + 1) / 2 * d.Nt;
+    return kKaraSlotBytes * (size_t)(t < kKaraPairs ? t : kKaraPairs) * d.S;
+  }
   const size_t whole = kara_min_ranges(d) > 1 ? 0 : (size_t)kara_tiles(d) * d.S;
   return 2 * kKaraSlotBytes * (whole + kara_cut_slots(d));
 }
@@ -341,6 +346,7 @@ inline OzakiLayout ozaki_layout(const OzakiDims& d) {
 }
 
 
+constexpr int kKaraShortSlices = 7;
 // The choice: the workspace (digit and difference planes, segment slots) up
 // to kKaraMaxBytes (6.8 GB at 8192^3, 27 GB at 16384^3); not for a part of a
 // wave with little k, where the planes and slots cost more than the products
@@ -349,12 +355,25 @@ inline OzakiLayout ozaki_layout(const OzakiDims& d) {
 // only as long as the product is small enough to be bound by latency (155 x
 // 305 x 98, S = 7: 3x; 64 x 8192 x 8192, S = 6: 956 us against 906).
 constexpr size_t kKaraMaxBytes = (size_t)32 << 30;
+// Little k: 256 x 128 tiles, where the epilogue sets the pace and there are
+// tiles for most CTA pairs.  Measured against 256 x 256 tiles (S = 7): up to
+// three k-blocks (4096 x 128 x 4096 255 us against 384, 16384 x 256 x 16384 4.5
+// ms against 5.6, 2048 x 256 x 2048 121 against 134), four with many tiles (8192 x
+// 512 x 8192 1780 against 1859, but 2048 x 512 x 2048 175 against 169), up to
+// eight where all tiles are one wave (1024 x 512 x 2048 109 against 126).
+inline bool kara_short(const OzakiDims& d) {
+  if (!kara_fits(d) || !ozaki_narrow(d) || d.S > kKaraShortSlices || d.Mt < 2) return false;
+  const int64_t tiles = (d.Mt + 1) / 2 * d.Nt;
+  if (tiles < 40) return false;
+  return d.Kt <= 3 || (d.Kt <= 4 && tiles >= 512) || (d.Kt <= 8 && tiles <= kKaraPairs);
+}
 inline bool kara_chosen(const OzakiDims& d) {
   if (!kara_fits(d)) return false;
-  if (d.Kt <= 4 && kara_tiles(d) > 16 && kara_tiles(d) < 48) return false;
-  if ((d.Mt == 1 || d.Nt == 1) && (d.Kt < 2 || kara_tiles(d) * d.Kt > 256)) return false;
+  const bool is_short = kara_short(d);
+  if (!is_short && d.Kt <= 4 && kara_tiles(d) > 16 && kara_tiles(d) < 48) return false;
+  if (!is_short && (d.Mt == 1 || d.Nt == 1) && (d.Kt < 2 || kara_tiles(d) * d.Kt > 256)) return false;
   OzakiDims w = d;
-  w.kara = 1;
+  w.kara = is_short ? 2 : 1;
   return ozaki_layout(w).total <= kKaraMaxBytes;
 }
 

@@ -35,6 +35,15 @@
 // HBM-bound): inside this one it held up the MMAs, the two windows in flight
 // covering only 8 us of it.
 //
+// Little k (kara_short): the segments are so short that the epilogue, not the
+// MMAs, sets the pace, and the slots of all tiles, written and read back by the
+// fold kernel, would go through memory (16384 x 256 x 16384, S = 6: 4.5 ms, 12 GB
+// of slots).  There C tiles are 256 x 128: with 32 columns a thread the sums T
+// and N_g both fit the registers, the segments interleave (P_1, P_2, N_3, P_3,
+// N_4, ..), D_g = T + N_g goes to the CTA's own slots once (64 KiB each, 58 MB
+// over all CTAs at S = 6: they stay in L2), and the thread folds its own D_g at
+// the end of the tile, while four windows of 128 columns let the MMAs run on.
+//
 // The tiles of the last, partly filled wave are cut by segments, and by ranges
 // of k where that is not enough to fill it: a work unit is then part of a
 // tile's list over part of k and leaves every segment's own sums in a slot,
@@ -53,12 +62,18 @@ namespace {
 constexpr int kThreads = 640;   // warp 0 copies, warp 1 issues (rank 0) or relays (rank 1),
                                 // warps 4-19 run the epilogue
 constexpr int kEpiWarps = 16;
-constexpr int kCPW = 64;        // columns of the C tile per epilogue warp
 constexpr int kSlots = 7;       // ring of operand tiles: A and B alternate
-constexpr int kN = 256;         // columns of a C tile, and of an accumulator window
+// columns of a C tile and of an accumulator window, windows, and columns of the
+// tile per epilogue warp of the two forms
+template <bool kShort>
+struct Form {
+  static constexpr int kN = kShort ? 128 : 256, kBufs = kShort ? 4 : 2, kCPW = kShort ? 32 : 64;
+  static constexpr int kBBytes = kShort ? kOzTileBytes / 2 : kOzTileBytes;
+  static constexpr int kSlotVec = kOzTileRows * kN / 4;  // int4 of a segment's sums of one CTA
+};
 constexpr uint32_t kTmemCols = 512;
 constexpr int kMmas = kOzTileK / 16;
-constexpr int kSlotInts = kOzTileRows * kN;  // one segment's sums of one CTA
+constexpr int kFoldCols = 256, kFoldVec = kOzTileRows * kFoldCols / 4;  // the fold kernel's tiles
 constexpr int kMaxProducts = 40, kMaxSegs = 20, kMaxS = kKaraMaxSlices;
 
 // The products of a tile in order, and the segments they form.
@@ -81,7 +96,7 @@ struct KaraArgs {
   int4* cut_scratch;    // per cut tile, rank and k range: 2 S - 2 slots, N_g in g - 3,
                         // P_s in S - 2 + s
   int64_t m, n;
-  int Mt, Nt, Kt;
+  int Mt, Nt, Kt, Mp, Np;  // Mp, Np: C tiles down and across
   int tiles, full_tiles;  // 256 x 256 C tiles; those done whole
   int raster;
   int S, beta, eoff, gx;
@@ -94,7 +109,7 @@ struct KaraArgs {
 struct __align__(1024) KaraSmem {
   uint8_t slot[kSlots][kOzTileBytes];
   uint64_t full[kSlots], empty[kSlots];
-  uint64_t accfull[2], accempty[2];
+  uint64_t accfull[4], accempty[4];
   uint32_t tmem_base;
   int abort_flag;
 };
@@ -110,10 +125,9 @@ struct KUnit {
 };
 // C tile t of the walk (tile_coords in 32 bits).
 __device__ __forceinline__ void kara_coords(const KaraArgs& a, int t, int& tm, int& tn) {
-  const int Mp = (a.Mt + 1) / 2, Np = (a.Nt + 1) / 2;
-  const int grp = t / (a.raster * Np), first = grp * a.raster;
-  const int gsz = Mp - first < a.raster ? Mp - first : a.raster;
-  const int in = t - first * Np;
+  const int grp = t / (a.raster * a.Np), first = grp * a.raster;
+  const int gsz = a.Mp - first < a.raster ? a.Mp - first : a.raster;
+  const int in = t - first * a.Np;
   tn = in / gsz;
   tm = first + in - tn * gsz;
 }
@@ -207,8 +221,8 @@ __device__ __forceinline__ double i64_pow2(long long y, int p) {
 // Sum: int, or long long where a D_g may pass 2^31.
 __device__ __forceinline__ double sum_pow2(int d, int p) { return i32_times_pow2(d, p); }
 __device__ __forceinline__ double sum_pow2(long long d, int p) { return i64_pow2(d, p); }
-template <typename Sum>
-__device__ __forceinline__ void fold_columns(const Sum (&d)[kMaxS - 1][4], const Sum (&d2)[4],
+template <typename Sum, int kLen>
+__device__ __forceinline__ void fold_columns(const Sum (&d)[kLen][4], const Sum (&d2)[4],
                                              int S, int beta, int gx, double (&out)[4]) {
   long long y[4];
 #pragma unroll
@@ -229,13 +243,13 @@ __device__ __forceinline__ void fold_columns(const Sum (&d)[kMaxS - 1][4], const
     }
   };
 #pragma unroll
-  for (int i = 1; i < kMaxS - 1; ++i)
+  for (int i = 1; i < kLen; ++i)
     if (i <= S - 2 && i <= S + 1 - gx) exact(d[i], beta * i);  // uniform
   if (gx <= 2) exact(d2, beta * (S - 1));
 #pragma unroll
   for (int c = 0; c < 4; ++c) out[c] = i64_pow2(y[c], -beta * (S + 1));
 #pragma unroll
-  for (int i = 1; i < kMaxS - 1; ++i) {
+  for (int i = 1; i < kLen; ++i) {
     const int g = S + 1 - i;
     if (g >= 3 && g < gx) {  // uniform
 #pragma unroll
@@ -270,8 +284,11 @@ __device__ __forceinline__ void store4(double* p, const double (&v)[4]) {
                : "memory");
 }
 
+template <bool kShort>
 __global__ void __launch_bounds__(kThreads, 1)
     oz_kara_kernel(const __grid_constant__ KaraArgs a, int* __restrict__ status) {
+  using F = Form<kShort>;
+  constexpr int kN = F::kN, kBufs = F::kBufs, kCPW = F::kCPW;
   extern __shared__ uint8_t smem_raw[];
   KaraSmem& sm = *reinterpret_cast<KaraSmem*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                               ~static_cast<uintptr_t>(1023));
@@ -285,7 +302,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       mbar_init(&sm.full[i], leader ? 2 : 1);  // rank 0: + the relay's arrival
       mbar_init(&sm.empty[i], 1);
     }
-    for (int i = 0; i < 2; ++i) {
+    for (int i = 0; i < kBufs; ++i) {
       mbar_init(&sm.accfull[i], 1);
       mbar_init(&sm.accempty[i], 2 * kEpiWarps);
     }
@@ -311,11 +328,11 @@ __global__ void __launch_bounds__(kThreads, 1)
       // ------------------------------------------------ producer (bulk copies)
       KRing r;
       bool ok = true;
-      auto load = [&](const uint8_t* src) {  // nullptr: nothing there (past the last tile)
+      auto load = [&](const uint8_t* src, uint32_t bytes) {  // nullptr: nothing there (past the last tile)
         if (!mbar_wait_bounded(&sm.empty[r.slot], r.phase ^ 1u, abort_flag, status)) return false;
         if (src != nullptr) {
-          mbar_arrive_expect_tx(&sm.full[r.slot], kOzTileBytes);
-          bulk_g2s(sm.slot[r.slot], src, kOzTileBytes, &sm.full[r.slot]);
+          mbar_arrive_expect_tx(&sm.full[r.slot], bytes);
+          bulk_g2s(sm.slot[r.slot], src, bytes, &sm.full[r.slot]);
         } else {
           mbar_arrive(&sm.full[r.slot]);
         }
@@ -326,21 +343,24 @@ __global__ void __launch_bounds__(kThreads, 1)
       const size_t b_plane = static_cast<size_t>(a.Nt) * a.Kt * kOzTileBytes;
       for (int u = unit0; u < nunits && ok; u += unit_step) {
         const KUnit k = kunit(a, u);
-        const int ta = 2 * k.tm + static_cast<int>(rank), tb = 2 * k.tn + static_cast<int>(rank);
+        const int ta = 2 * k.tm + static_cast<int>(rank);
+        const int tb = kShort ? k.tn : 2 * k.tn + static_cast<int>(rank);
         const bool alive = ta < a.Mt, blive = tb < a.Nt;
         const uint8_t* a0 = a.aslices + static_cast<size_t>(ta) * a.Kt * kOzTileBytes;
-        const uint8_t* b0 = a.bslices + static_cast<size_t>(tb) * a.Kt * kOzTileBytes;
+        // short: the CTA's half of the tile (oz_chunk_offset_halves)
+        const uint8_t* b0 = a.bslices + static_cast<size_t>(tb) * a.Kt * kOzTileBytes +
+                            (kShort ? rank * F::kBBytes : 0);
         const int p1 = seg_begin(a, k.s1);
         for (int p = seg_begin(a, k.s0); p < p1 && ok; ++p) {
           const uint8_t* ap = a0 + a.prog.pa[p] * a_plane;
           const uint8_t* bp = b0 + a.prog.pb[p] * b_plane;
           MXM_BOUNDS(!alive || in_range(ap, a.Kt * kOzTileBytes, a.aslices,
                                         a.aslices + a_plane * kara_planes(a.S)), status);
-          MXM_BOUNDS(!blive || in_range(bp, a.Kt * kOzTileBytes, a.bslices,
+          MXM_BOUNDS(!blive || in_range(bp, (a.Kt - 1) * kOzTileBytes + F::kBBytes, a.bslices,
                                         a.bslices + b_plane * kara_planes(a.S)), status);
           for (int kb = k.kb0; kb < k.kb1 && ok; ++kb)
-            ok = load(alive ? ap + static_cast<size_t>(kb) * kOzTileBytes : nullptr) &&
-                 load(blive ? bp + static_cast<size_t>(kb) * kOzTileBytes : nullptr);
+            ok = load(alive ? ap + static_cast<size_t>(kb) * kOzTileBytes : nullptr, kOzTileBytes) &&
+                 load(blive ? bp + static_cast<size_t>(kb) * kOzTileBytes : nullptr, F::kBBytes);
         }
       }
       // tail: wait until every slot is released, so that no copy or commit
@@ -371,8 +391,7 @@ __global__ void __launch_bounds__(kThreads, 1)
       const uint32_t idesc = idesc_bf16_f32(256, kN);
       const uint64_t desc0 = sw128_kmajor_desc(smem_u32(sm.slot[0]));
       KRing r;
-      int buf = 0;
-      uint32_t uses[2] = {0u, 0u};
+      uint32_t win = 0;  // windows started
       bool ok = true;
       bool seen_a = false, seen_b = false;  // the next slots were seen full (mbar_test)
       auto wait_full = [&](bool& seen) -> bool {
@@ -402,14 +421,12 @@ __global__ void __launch_bounds__(kThreads, 1)
             }
             const int sb = r.slot;
             r.advance();
-            if (cnt == 0) {  // a window starts: its buffer must have been drained
-              const uint32_t w = buf ? uses[1] : uses[0];
-              if (w > 0 && !mbar_wait_bounded<false, true>(&sm.accempty[buf], (w - 1u) & 1u,
-                                                            abort_flag, status)) {
-                ok = false;
-                break;
-              }
-              if (buf) ++uses[1]; else ++uses[0];
+            const int buf = win % kBufs;
+            if (cnt == 0 && win >= kBufs &&  // a window starts: its buffer must have been drained
+                !mbar_wait_bounded<false, true>(&sm.accempty[buf], (win / kBufs - 1u) & 1u,
+                                                abort_flag, status)) {
+              ok = false;
+              break;
             }
             tc_fence_after();
             const uint64_t da = desc0 + static_cast<uint64_t>(sa) * (kOzTileBytes >> 4);
@@ -422,7 +439,9 @@ __global__ void __launch_bounds__(kThreads, 1)
             for (int kk = 0; kk < kMmas; ++kk) {
               const uint64_t off =
                   static_cast<uint64_t>((kk >> 2) * (kOzAtomBytes >> 4) + (kk & 3) * 2);
-              if (kk < nmma) mma_bf16_ss_pair(d, da + off, db + off, idesc, kk > 0 ? 1u : acc0);
+              const uint64_t boff =  // short: atoms of 64 rows, 8 KiB apart
+                  kShort ? static_cast<uint64_t>((kk >> 2) * (kOzAtomBytes >> 5) + (kk & 3) * 2) : off;
+              if (kk < nmma) mma_bf16_ss_pair(d, da + off, db + boff, idesc, kk > 0 ? 1u : acc0);
               if (kk == kMmas / 2 - 1) {  // half-way: the slots the next waits are on
                 seen_a = mbar_test<true>(&sm.full[nx.slot], nx.phase);
                 nx.advance();
@@ -433,7 +452,7 @@ __global__ void __launch_bounds__(kThreads, 1)
             mma_commit_pair(&sm.empty[sb], static_cast<uint16_t>(0x3));
             if (++cnt == window || st + 1 == steps) {
               mma_commit_pair(&sm.accfull[buf], static_cast<uint16_t>(0x3));
-              buf ^= 1;
+              ++win;
               cnt = 0;
             }
             if (++kb == k.kb1) kb = k.kb0;
@@ -452,16 +471,15 @@ __global__ void __launch_bounds__(kThreads, 1)
     const int S = a.S;
     // this thread's 4-column groups: group c of a slot at + c * 128
     const int own = cg * (kCPW / 4) * kOzTileRows + row_in_tile;
-    constexpr int kSlotVec = kSlotInts / 4;
-    int buf = 0;
-    uint32_t fulls[2] = {0u, 0u};
+    constexpr int kSlotVec = F::kSlotVec;
+    uint32_t win = 0;  // windows drained
     bool ok = true;
-    int D[kCPW];
+    int D[kCPW];                   // a segment's sums; short: T
+    int Ng[kShort ? kCPW : 1];     // short: N_g
 
     auto wait_window = [&]() -> bool {
-      const uint32_t f = buf ? fulls[1] : fulls[0];
-      if (!mbar_wait_bounded(&sm.accfull[buf], f & 1u, abort_flag, status)) return false;
-      if (buf) ++fulls[1]; else ++fulls[0];
+      if (!mbar_wait_bounded(&sm.accfull[win % kBufs], (win / kBufs) & 1u, abort_flag, status))
+        return false;
       tc_fence_after();
       return true;
     };
@@ -469,15 +487,16 @@ __global__ void __launch_bounds__(kThreads, 1)
       tc_fence_before();
       __syncwarp();
       if (lane == 0) {
+        uint64_t* const empty = &sm.accempty[win % kBufs];
         if (!leader)
-          mbar_arrive_remote_release(smem_in_cta(&sm.accempty[buf], 0));  // the issuer is in rank 0
+          mbar_arrive_remote_release(smem_in_cta(empty, 0));  // the issuer is in rank 0
         else
-          mbar_arrive(&sm.accempty[buf]);
+          mbar_arrive(empty);
       }
-      buf ^= 1;
+      ++win;
     };
-    // every window of segment s added into D
-    auto drain = [&](int s, int kblocks) -> bool {
+    // every window of segment s added into X
+    auto drain = [&](int s, int kblocks, int (&X)[kCPW]) -> bool {
       const int window = a.prog.g[s] >= kSquare ? a.win_p : a.win_n;
       const int steps = kblocks * (a.prog.end[s] - seg_begin(a, s));
       for (int st = 0; st < steps; st += window) {
@@ -485,10 +504,10 @@ __global__ void __launch_bounds__(kThreads, 1)
 #pragma unroll
         for (int h = 0; h < kCPW / 16; ++h) {
           uint32_t r[16];
-          tmem_ld16(t_lane + static_cast<uint32_t>(buf * kN + h * 16), r);
+          tmem_ld16(t_lane + static_cast<uint32_t>((win % kBufs) * kN + h * 16), r);
           tmem_wait_ld();
 #pragma unroll
-          for (int i = 0; i < 16; ++i) D[h * 16 + i] += __float2int_rz(__uint_as_float(r[i]));
+          for (int i = 0; i < 16; ++i) X[h * 16 + i] += __float2int_rz(__uint_as_float(r[i]));
         }
         free_window();
       }
@@ -515,30 +534,113 @@ __global__ void __launch_bounds__(kThreads, 1)
       const KUnit k = kunit(a, u);
       const int64_t row0 = (2 * static_cast<int64_t>(k.tm) + rank) * kOzTileRows;
       const int64_t col0 = static_cast<int64_t>(k.tn) * kN + cg * kCPW;
-      int4* const base =
-          k.cut < 0
-              ? a.full_scratch + (static_cast<size_t>(k.tile) * 2 + rank) * S * kSlotVec
-              : a.cut_scratch + (static_cast<size_t>(k.cut) * 2 + rank) * (2 * S - 2) * kSlotVec;
       // a part of the tile outside C (warp-uniform): its windows are drained only
       const bool keep = row0 + quarter * 32 < a.m && col0 < a.n;
-      for (int s = k.s0; s < k.s1 && ok; ++s) {
-        const int g = a.prog.g[s];
-        const bool square = g >= kSquare;
-        const int sq = g - kSquare;
-        int4* const slot =
-            base + static_cast<size_t>(k.cut >= 0 ? (square ? S - 2 + sq : g - 3)
-                                                  : (square ? sq - 1 : g - 2)) * kSlotVec;
-        if (k.cut < 0 && !square) {
-          if (keep) get(slot);  // T_g; in flight until the first window is read
-        } else if (k.cut >= 0 || sq == 1) {
+      if constexpr (kShort) {
+        // ---------------- short: P_1, P_2, N_3, P_3, .., P_{S-1}, N_S, N_{S+1}
+        int4* const base = a.full_scratch + static_cast<size_t>(blockIdx.x) * S * kSlotVec;
 #pragma unroll
-          for (int i = 0; i < kCPW; ++i) D[i] = 0;
+        for (int i = 0; i < kCPW; ++i) D[i] = 0;
+        for (int s = 0; s < k.s1 && ok; ++s) {
+          const int g = a.prog.g[s];
+          if (g >= kSquare) {
+            ok = drain(s, a.Kt, D);
+            if (ok && keep && g == kSquare + 1) {
+#pragma unroll
+              for (int c = 0; c < kCPW / 4; ++c)
+                st_cg4(base + own + c * kOzTileRows,
+                       make_int4(D[4 * c], D[4 * c + 1], D[4 * c + 2], D[4 * c + 3]));
+            }
+          } else {
+#pragma unroll
+            for (int i = 0; i < kCPW; ++i) Ng[i] = 0;
+            ok = drain(s, a.Kt, Ng);
+            if (ok && keep) {
+              int4* const slot = base + static_cast<size_t>(g - 2) * kSlotVec;
+#pragma unroll
+              for (int c = 0; c < kCPW / 4; ++c)
+                st_cg4(slot + own + c * kOzTileRows,
+                       make_int4(D[4 * c] + Ng[4 * c], D[4 * c + 1] + Ng[4 * c + 1],
+                                 D[4 * c + 2] + Ng[4 * c + 2], D[4 * c + 3] + Ng[4 * c + 3]));
+            }
+          }
         }
-        ok = drain(s, k.kb1 - k.kb0);
-        if (!ok || !keep) continue;
-        put(slot);
-        // D_{S+1} starts from T_S as well (the fold takes P_1 = D_2 out of it)
-        if (k.cut < 0 && sq == S - 1) put(slot + kSlotVec);
+        if (!ok) break;
+        if (!keep) continue;
+        const int64_t row = row0 + row_in_tile;
+        const bool row_ok = row < a.m;
+        const int er = row_ok ? exponent_from_absbits(a.rowbits[row]) + a.eoff : 0;
+        // lane l holds the exponent of this warp's column l
+        const int64_t lcol = col0 + lane;
+        const int ec = lcol < a.n ? exponent_from_absbits(__ldg(a.colbits + lcol)) : 0;
+        double* const crow = a.C + (row_ok ? row : 0) * a.n;
+        const bool vec = (a.n & 3) == 0 && (reinterpret_cast<uintptr_t>(a.C) & 31) == 0;
+        const int groups = a.n - col0 >= kCPW ? kCPW / 4 : static_cast<int>((a.n - col0 + 3) / 4);
+        // a group's slots are read one group ahead (T and N_g are dead here)
+        int4 nx[kKaraShortSlices - 1], nx2;
+        auto read = [&](int c) {
+          const int4* p = base + own + c * kOzTileRows;
+#pragma unroll
+          for (int i = 0; i < kKaraShortSlices - 1; ++i)
+            if (i < S - 1) nx[i] = __ldcg(p + static_cast<size_t>(S - 1 - i) * kSlotVec);
+          nx2 = __ldcg(p);  // D_2 = P_1
+        };
+#pragma unroll
+        for (int i = 0; i < kKaraShortSlices - 1; ++i) nx[i] = make_int4(0, 0, 0, 0);
+        read(0);
+#pragma unroll 1
+        for (int c = 0; c < groups; ++c) {
+          int d[kKaraShortSlices - 1][4];
+          const int d2[4] = {nx2.x, nx2.y, nx2.z, nx2.w};
+#pragma unroll
+          for (int i = 0; i < kKaraShortSlices - 1; ++i) {
+            d[i][0] = nx[i].x;
+            d[i][1] = nx[i].y;
+            d[i][2] = nx[i].z;
+            d[i][3] = nx[i].w;
+          }
+          if (c + 1 < groups) read(c + 1);
+#pragma unroll
+          for (int j = 0; j < 4; ++j) d[0][j] -= d2[j];  // the pair (1, S) was taken directly
+          double out[4];
+          fold_columns(d, d2, S, a.beta, a.gx, out);
+          const int64_t col = col0 + 4 * c;
+#pragma unroll
+          for (int j = 0; j < 4; ++j)
+            out[j] = scale_by(out[j], er + __shfl_sync(0xFFFFFFFFu, ec, 4 * c + j));
+          if (!row_ok) continue;
+          if (vec && col + 4 <= a.n) {
+            store4(crow + col, out);
+          } else {
+#pragma unroll
+            for (int j = 0; j < 4; ++j)
+              if (col + j < a.n) crow[col + j] = out[j];
+          }
+        }
+      } else {
+        int4* const base =
+            k.cut < 0
+                ? a.full_scratch + (static_cast<size_t>(k.tile) * 2 + rank) * S * kSlotVec
+                : a.cut_scratch + (static_cast<size_t>(k.cut) * 2 + rank) * (2 * S - 2) * kSlotVec;
+        for (int s = k.s0; s < k.s1 && ok; ++s) {
+          const int g = a.prog.g[s];
+          const bool square = g >= kSquare;
+          const int sq = g - kSquare;
+          int4* const slot =
+              base + static_cast<size_t>(k.cut >= 0 ? (square ? S - 2 + sq : g - 3)
+                                                    : (square ? sq - 1 : g - 2)) * kSlotVec;
+          if (k.cut < 0 && !square) {
+            if (keep) get(slot);  // T_g; in flight until the first window is read
+          } else if (k.cut >= 0 || sq == 1) {
+#pragma unroll
+            for (int i = 0; i < kCPW; ++i) D[i] = 0;
+          }
+          ok = drain(s, k.kb1 - k.kb0, D);
+          if (!ok || !keep) continue;
+          put(slot);
+          // D_{S+1} starts from T_S as well (the fold takes P_1 = D_2 out of it)
+          if (k.cut < 0 && sq == S - 1) put(slot + kSlotVec);
+        }
       }
     }
   }
@@ -568,7 +670,7 @@ constexpr int kFoldThreads = 128;
 template <bool kCut, typename Sum>
 __global__ void __launch_bounds__(kFoldThreads) oz_kara_fold_kernel(
     const __grid_constant__ KaraArgs a, int part0) {
-  constexpr int kSlotVec = kSlotInts / 4;
+  constexpr int kSlotVec = kFoldVec;
   const int S = a.S;
   const int part = part0 + blockIdx.y;  // (tile, rank) among the kind's tiles
   const int t = (kCut ? a.full_tiles : 0) + (part >> 1), rank = part & 1;
@@ -576,7 +678,7 @@ __global__ void __launch_bounds__(kFoldThreads) oz_kara_fold_kernel(
   kara_coords(a, t, tm, tn);
   const int v = blockIdx.x * kFoldThreads + threadIdx.x;  // column group v / 128, row v % 128
   const int64_t row = (2 * static_cast<int64_t>(tm) + rank) * kOzTileRows + (v & 127);
-  const int64_t col = static_cast<int64_t>(tn) * kN + 4 * (v >> 7);
+  const int64_t col = static_cast<int64_t>(tn) * kFoldCols + 4 * (v >> 7);
   if (row >= a.m || col >= a.n) return;
   Sum d[kMaxS - 1][4], d2[4];  // D_{S+1} .. D_3, and D_2
   if constexpr (kCut) {
@@ -678,8 +780,9 @@ __global__ void __launch_bounds__(kFoldThreads) oz_kara_fold_kernel(
   }
 }
 
-// The products and segments of S slices: the squares, then the N_g.
-void build_prog(int S, KaraProg& pr) {
+// The products and segments of S slices: the squares, then the N_g; inter: P_1,
+// then each square with the N_g that follows it.
+void build_prog(int S, bool inter, KaraProg& pr) {
   int np = 0, ns = 0;
   auto square = [&](int s) {
     pr.pa[np] = pr.pb[np] = static_cast<uint8_t>(s - 1);
@@ -703,8 +806,17 @@ void build_prog(int S, KaraProg& pr) {
     pr.end[ns] = static_cast<uint8_t>(np);
     pr.g[ns++] = static_cast<uint8_t>(g);
   };
-  for (int s = 1; s <= S - 1; ++s) square(s);
-  for (int g = 3; g <= S + 1; ++g) ndiag(g);
+  if (inter) {
+    square(1);
+    for (int s = 2; s <= S - 1; ++s) {
+      square(s);
+      ndiag(s + 1);
+    }
+    ndiag(S + 1);
+  } else {
+    for (int s = 1; s <= S - 1; ++s) square(s);
+    for (int g = 3; g <= S + 1; ++g) ndiag(g);
+  }
   pr.nseg = ns;
 }
 
@@ -785,10 +897,14 @@ cudaError_t launch_ozaki_kara(const uint8_t* aslices, const uint8_t* bslices,
   a.win_n = kara_window_stages(d);
   const int64_t klast = d.k - (d.Kt - 1) * kOzTileK;
   a.last_mmas = static_cast<int>((klast + 15) / 16);
+  const bool is_short = d.kara == 2;
   const int64_t Mp = (d.Mt + 1) / 2;
+  a.Mp = static_cast<int>(Mp);
+  a.Np = static_cast<int>(is_short ? d.Nt : (d.Nt + 1) / 2);
   a.raster = static_cast<int>(d.raster < Mp ? (d.raster > 0 ? d.raster : kDefaultRaster) : Mp);
-  build_prog(d.S, a.prog);
-  cudaError_t e = cudaFuncSetAttribute(oz_kara_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
+  build_prog(d.S, is_short, a.prog);
+  const auto kern = is_short ? oz_kara_kernel<true> : oz_kara_kernel<false>;
+  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
                                        static_cast<int>(kSmemBytes));
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
@@ -804,31 +920,31 @@ cudaError_t launch_ozaki_kara(const uint8_t* aslices, const uint8_t* bslices,
   cfg.numAttrs = 1;
   cfg.gridDim = dim3(2, 1, 1);
   int clusters = 0;
-  e = cudaOccupancyMaxActiveClusters(&clusters, oz_kara_kernel, &cfg);
+  e = cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg);
   if (e != cudaSuccess) return e;
   if (clusters < 1) return cudaErrorLaunchOutOfResources;
   const int64_t pairs = clusters < kKaraPairs ? clusters : kKaraPairs;
   // whole waves of tiles, then the rest, cut where that is shorter
-  const int64_t tiles = kara_tiles(d);
+  const int64_t tiles = static_cast<int64_t>(a.Mp) * a.Np;
   a.tiles = static_cast<int>(tiles);
   const bool wide = kara_min_ranges(d) > 1;  // every tile is cut along k
-  const int64_t rest = wide ? tiles : tiles % pairs;
+  const int64_t rest = is_short ? 0 : wide ? tiles : tiles % pairs;
   a.full_tiles = static_cast<int>(tiles - rest);
   a.parts = a.ranges = 1;
   if (rest > 0 && !choose_cut(d, rest, pairs, a)) a.full_tiles = a.tiles;
   a.full_scratch = reinterpret_cast<int4*>(scratch);
-  a.cut_scratch = a.full_scratch + static_cast<size_t>(a.full_tiles) * 2 * d.S * (kSlotInts / 4);
+  a.cut_scratch = a.full_scratch + static_cast<size_t>(a.full_tiles) * 2 * d.S * kFoldVec;
   const int64_t units = a.full_tiles + (tiles - a.full_tiles) * a.parts * a.ranges;
   const int64_t use = units < pairs ? units : pairs;
   cfg.gridDim = dim3(static_cast<unsigned>(2 * use), 1, 1);
-  e = cudaLaunchKernelEx(&cfg, oz_kara_kernel, a, status);
-  if (e != cudaSuccess) return e;
+  e = cudaLaunchKernelEx(&cfg, kern, a, status);
+  if (e != cudaSuccess || is_short) return e;
   // (tile, rank) parts on the y axis of the grid, at most kFoldParts per launch
   constexpr int64_t kFoldParts = 32768;
   auto fold = [&](auto kern, int64_t parts) {
     for (int64_t p0 = 0; p0 < parts; p0 += kFoldParts) {
       const int64_t now = parts - p0 < kFoldParts ? parts - p0 : kFoldParts;
-      kern<<<dim3(kSlotInts / 4 / kFoldThreads, static_cast<unsigned>(now)), kFoldThreads, 0, s>>>(
+      kern<<<dim3(kFoldVec / kFoldThreads, static_cast<unsigned>(now)), kFoldThreads, 0, s>>>(
           a, static_cast<int>(p0));
     }
   };

@@ -72,6 +72,31 @@ def test_many_tiles_match_the_products_one_by_one(m, k, n, raster):
                    "sampled entries")
 
 
+@pytest.mark.parametrize("mode,S,m,k,n", [
+    (mxm.MODE_EMUL_I8, 7, 1300, 100, 1050),    # 256 x 128 tiles: 54, one wave, odd tile-rows
+    (mxm.MODE_EMUL_I8, 3, 1281, 384, 1025),
+    (mxm.MODE_EMUL_I8, 6, 2600, 257, 1100),    # 99: a second wave
+    (mxm.MODE_EMUL_RN8, 6, 1290, 300, 1100),   # several windows a segment
+    (mxm.MODE_EMUL_BF16, 6, 1300, 1000, 1030),
+    (mxm.MODE_EMUL_RN8, 7, 2050, 129, 2050),
+])
+def test_little_k(mode, S, m, k, n):
+    A, B = inputs.gemm_operands("spread", m, k, n, seed=4, cfg=44)
+    dA, dB = torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda()
+    C = torch.full((m, n), float("nan"), dtype=torch.float64, device="cuda")
+    D = torch.full((m, n), float("nan"), dtype=torch.float64, device="cuda")
+    mxm.mxm_gemm(mode, dA, dB, C, slices=S)
+    mxm.mxm_gemm_plan(mode, dA, dB, D, slices=S, plan=mxm.Plan(0, 0, 1, 1))
+    assert mxm.mxm_get_device_status() == mxm.MXM_OK
+    assert torch.equal(C, D)
+    rng = np.random.default_rng(m)
+    ii, jj = rng.integers(0, m, 60), rng.integers(0, n, 60)
+    ii[0], jj[0] = m - 1, n - 1
+    # an entry depends on its row of A and its column of B alone
+    want = np.diagonal(_emulated(A[ii], B[:, jj], mode, S))
+    assert_bitwise(C.cpu().numpy()[ii, jj], want, "sampled entries")
+
+
 def test_smaller_caller_workspace_takes_the_products_one_by_one():
     """A caller workspace of the size the products one by one need (what
     mxm_workspace_size gives under a single-CTA plan) still runs, with the same
