@@ -1144,7 +1144,7 @@ struct OzGrouped {
 // out-of-line form cost the grouped short-k GEMM ~1 % in call overhead and
 // the 8192^3 product nothing).
 __device__ __forceinline__ double final_scale(uint64_t st, int e) {
-  return ldexp_rn(__longlong_as_double(static_cast<long long>(st)), e);
+  return scale_by(__longlong_as_double(static_cast<long long>(st)), e);
 }
 
 __device__ __noinline__ uint64_t fold_step(uint64_t st, long long dval, int g, int gx, int S,
@@ -1165,21 +1165,25 @@ __device__ __noinline__ uint64_t fold_step(uint64_t st, long long dval, int g, i
 // last exact step and the conversion to FP64 at g == gx, an FP64 addition
 // below.  fold_kind is fold_step with the kind fixed by the caller (inline:
 // the paired kernel folds 8 elements at a time with one kind per diagonal
-// pair, straight-line code); on the first diagonal st is 0.
+// pair, straight-line code); on the first diagonal st is 0.  The digit sums
+// stay int32 until they are used, a term is built from its bits and the last
+// scaling moves the exponent field (int64 products, int64 to FP64 conversions
+// and ldexp before: 2000 ragged i8 products of S = 8 in one group 7538 us, now
+// 7449; 32768 x 1024 x 64 rn8 379 -> 363 us).
 constexpr int kFoldInt = 0, kFoldConv = 1, kFoldFp = 2, kFoldNone = 3;
 __device__ __forceinline__ int fold_kind_of(int g, int gx) {
   return g > gx ? kFoldInt : (g == gx ? kFoldConv : kFoldFp);
 }
-template <int K>
-__device__ __forceinline__ uint64_t fold_kind(uint64_t st, long long d, int g, int S, int beta) {
+template <int K, typename Sum>
+__device__ __forceinline__ uint64_t fold_kind(uint64_t st, Sum d, int g, int S, int beta) {
   if constexpr (K == kFoldFp) {
     const double acc = __longlong_as_double(static_cast<long long>(st));
     return static_cast<uint64_t>(
-        __double_as_longlong(__dadd_rn(acc, i64_times_pow2(d, -beta * g))));  // term exact
+        __double_as_longlong(__dadd_rn(acc, sum_pow2(d, -beta * g))));  // term exact
   } else {
-    const long long y = static_cast<long long>(st) + d * (1ll << (beta * (S + 1 - g)));
+    const long long y = add_shifted(static_cast<long long>(st), d, beta * (S + 1 - g));
     if constexpr (K == kFoldConv)
-      return static_cast<uint64_t>(__double_as_longlong(i64_times_pow2(y, -beta * (S + 1))));
+      return static_cast<uint64_t>(__double_as_longlong(i64_pow2(y, -beta * (S + 1))));
     else
       return static_cast<uint64_t>(y);
   }
@@ -1559,7 +1563,7 @@ __global__ void __launch_bounds__(128 + 32 * kEpiW, 1)
                 } else {
                   const uint64_t prev =
                       first ? 0ull : ((static_cast<uint64_t>(r[2 * i + 1]) << 32) | r[2 * i]);
-                  st[i] = fold_kind<K>(prev, static_cast<long long>(D[i]), g, S, beta);
+                  st[i] = fold_kind<K>(prev, D[i], g, S, beta);
                 }
               }
               if (last) {
@@ -2235,7 +2239,8 @@ __global__ void __launch_bounds__(kP2Threads, 1)
             }
 #pragma unroll
             for (int i = 0; i < 8; ++i) {
-              long long d0 = D0[i], d1 = D1[i];
+              using Sum = std::conditional_t<kSpill, long long, int>;
+              Sum d0 = D0[i], d1 = D1[i];
               if constexpr (kSpill) {
                 const size_t sc =
                     static_cast<size_t>(half * 64 + ch * 8 + i) * kOzTileRows + row_in_tile;
@@ -2252,7 +2257,7 @@ __global__ void __launch_bounds__(kP2Threads, 1)
                 const int64_t col = cbase + i;
                 if (row_ok && col < j.n)
                   j.C[row * j.n + col] =
-                      ldexp_rn(__longlong_as_double(static_cast<long long>(cur[i])),
+                      scale_by(__longlong_as_double(static_cast<long long>(cur[i])),
                                er + exponent_from_absbits(__ldg(j.colbits + col)) + j.eoff);
               }
             } else {

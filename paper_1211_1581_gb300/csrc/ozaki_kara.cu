@@ -172,55 +172,12 @@ struct KRing {
   }
 };
 
-// d 2^p as a double (exact), for an int32 d and a normal result.
-__device__ __forceinline__ double i32_times_pow2(int d, int p) {
-  const uint32_t sign = static_cast<uint32_t>(d) & 0x80000000u;
-  const uint32_t mag = static_cast<uint32_t>(d < 0 ? -d : d);  // 2^31 for INT_MIN
-  const int lz = __clz(static_cast<int>(mag));
-  const uint32_t norm = mag << lz;  // top bit set (mag != 0); lz = 32: shifted out
-  const uint32_t hi = sign | (static_cast<uint32_t>(1023 + 31 - lz + p) << 20) |
-                      ((norm >> 11) & 0x000FFFFFu);
-  const uint32_t lo = norm << 21;
-  return __hiloint2double(mag ? static_cast<int>(hi) : 0, mag ? static_cast<int>(lo) : 0);
-}
-
-// x 2^e: the exponent field moved when x and the result are normal (or x is
-// zero), the general form otherwise.
-__device__ __noinline__ double scale_slow(double x, int e) { return ldexp_rn(x, e); }
-__device__ __forceinline__ double scale_by(double x, int e) {
-  const uint32_t hi = static_cast<uint32_t>(__double2hiint(x));
-  const int be = static_cast<int>((hi >> 20) & 0x7FFu);
-  const int nb = be + e;
-  if (be >= 1 && be <= 2046 && nb >= 1 && nb <= 2046)
-    return __hiloint2double(static_cast<int>(hi + (static_cast<uint32_t>(e) << 20)),
-                            __double2loint(x));
-  return scale_slow(x, e);
-}
-
-// y 2^p as a double (exact), for |y| < 2^53 and a normal result.
-__device__ __forceinline__ double i64_pow2(long long y, int p) {
-  const int sg = static_cast<int>(y >> 63);
-  const uint64_t mag = static_cast<uint64_t>((y ^ sg) - sg);
-  const uint32_t h = static_cast<uint32_t>(mag >> 32), l = static_cast<uint32_t>(mag);
-  const bool wide = h != 0;
-  const uint32_t top = wide ? h : l, next = wide ? l : 0u;
-  const int lz = __clz(static_cast<int>(top));
-  const uint32_t n1 = __funnelshift_lc(next, top, lz), n0 = next << (lz & 31);  // normalised
-  const uint32_t be = static_cast<uint32_t>(1023 + (wide ? 63 : 31) - lz + p);
-  const uint32_t hi = (static_cast<uint32_t>(sg) & 0x80000000u) | (be << 20) |
-                      ((n1 >> 11) & 0x000FFFFFu);
-  const uint32_t lo = __funnelshift_r(n0, n1, 11);
-  return __hiloint2double(top ? static_cast<int>(hi) : 0, top ? static_cast<int>(lo) : 0);
-}
-
 // Fold the diagonals d[0] = D_{S+1}, .., d[S-2] = D_3, then d2 = D_2, of four
 // neighbouring elements in the order of step 4 (exact int64 partial for
 // g >= gx, FP64 additions after).  Straight-line over the longest list (D_2
 // apart: indexed by S it would put the list into local memory); the bounds
 // are uniform.
 // Sum: int, or long long where a D_g may pass 2^31.
-__device__ __forceinline__ double sum_pow2(int d, int p) { return i32_times_pow2(d, p); }
-__device__ __forceinline__ double sum_pow2(long long d, int p) { return i64_pow2(d, p); }
 template <typename Sum, int kLen>
 __device__ __forceinline__ void fold_columns(const Sum (&d)[kLen][4], const Sum (&d2)[4],
                                              int S, int beta, int gx, double (&out)[4]) {
@@ -228,19 +185,8 @@ __device__ __forceinline__ void fold_columns(const Sum (&d)[kLen][4], const Sum 
 #pragma unroll
   for (int c = 0; c < 4; ++c) y[c] = d[0][c];  // diagonal S + 1 is always exact
   auto exact = [&](const Sum (&v)[4], int sh) {
-    if constexpr (sizeof(Sum) == 8) {
 #pragma unroll
-      for (int c = 0; c < 4; ++c) y[c] += static_cast<long long>(static_cast<uint64_t>(v[c]) << sh);
-    } else if (sh < 31) {
-      const int w = 1 << sh;
-#pragma unroll
-      for (int c = 0; c < 4; ++c) y[c] += static_cast<long long>(v[c]) * w;  // one IMAD.WIDE
-    } else {
-#pragma unroll
-      for (int c = 0; c < 4; ++c)
-        y[c] += static_cast<long long>(
-            static_cast<uint64_t>(static_cast<uint32_t>(v[c]) << (sh - 32)) << 32);
-    }
+    for (int c = 0; c < 4; ++c) y[c] = add_shifted(y[c], v[c], sh);
   };
 #pragma unroll
   for (int i = 1; i < kLen; ++i)
