@@ -349,30 +349,29 @@ template <int G>
 cudaError_t launch_cg_g(CgArgs a, int C, cudaStream_t s) {
   // the copy of A takes what shared memory is left, up to the whole matrix;
   // a CTA whose rows hold more values reads them from L2 instead
-  int dev = 0, optin = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e != cudaSuccess) return e;
-  e = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
-  if (e != cudaSuccess) return e;
-  cudaFuncAttributes fa;
-  e = cudaFuncGetAttributes(&fa, cg_cluster_kernel<G>);
+  static PerDevice limit;
+  int most = 0;  // dynamic shared memory that the kernel may use
+  cudaError_t e = limit.get(&most, [](int* v) {
+    int dev = 0, optin = 0;
+    cudaFuncAttributes fa;
+    cudaError_t q = cudaGetDevice(&dev);
+    if (q == cudaSuccess)
+      q = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (q == cudaSuccess) q = cudaFuncGetAttributes(&fa, cg_cluster_kernel<G>);
+    if (q != cudaSuccess) return q;
+    *v = optin - static_cast<int>(fa.sharedSizeBytes);
+    q = cudaFuncSetAttribute(cg_cluster_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, *v);
+    if (q != cudaSuccess) return q;
+    return cudaFuncSetAttribute(cg_cluster_kernel<G>,
+                                cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  });
   if (e != cudaSuccess) return e;
   a.rows_cap = (a.n + C - 1) / C;
-  const int64_t room = static_cast<int64_t>(optin) - static_cast<int64_t>(fa.sharedSizeBytes) -
-                       static_cast<int64_t>(cg_smem_bytes(a.n, C, 0)) -
+  const int64_t room = static_cast<int64_t>(most) - static_cast<int64_t>(cg_smem_bytes(a.n, C, 0)) -
                        (a.rows_cap + 1) * static_cast<int64_t>(sizeof(int32_t));
   a.nnz_cap = room > 0 ? room / static_cast<int64_t>(sizeof(double) + sizeof(int32_t)) : 0;
   if (a.nnz_cap > a.nnz) a.nnz_cap = a.nnz;
   const size_t smem = cg_smem_bytes(a.n, C, a.nnz_cap);
-  e = cudaFuncSetAttribute(cg_cluster_kernel<G>,
-                                       cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
-  if (e != cudaSuccess) return e;
-  if (C > 8) {
-    e = cudaFuncSetAttribute(cg_cluster_kernel<G>, cudaFuncAttributeNonPortableClusterSizeAllowed,
-                             1);
-    if (e != cudaSuccess) return e;
-  }
   cudaLaunchConfig_t cfg = {};
   cfg.gridDim = dim3(static_cast<unsigned>(C), 1, 1);
   cfg.blockDim = dim3(kCgThreads, 1, 1);

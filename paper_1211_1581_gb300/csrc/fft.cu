@@ -45,6 +45,10 @@ constexpr int kFftThreads = 256;
 constexpr int64_t kFftMaxN = int64_t{1} << 22;
 constexpr int64_t kFftSingleMax = 1024;
 constexpr int64_t kFftClusterMin = 16, kFftClusterMax = 8192;
+constexpr int kFftClusterBits = 13;  // log2 of kFftClusterMax
+// most dynamic shared memory of a CTA: of a pass (the rule of fft_column_bits),
+// of a cluster (what a CTA may have beside its static part)
+constexpr size_t kFftPassSmem = 96 * 1024, kFftClusterSmem = 200 * 1024;
 
 // On this GPU a fused multiply-add of three registers issues every 64 clocks, an
 // add, a multiply or a form with a constant operand every 76: sums and products
@@ -335,8 +339,8 @@ cudaError_t launch_pass(FftPass a, cudaStream_t s) {
   a.cbits = fft_column_bits(bits, cols);
   const size_t L = size_t{1} << bits;
   const size_t smem = ((L << a.cbits) + (3 * L + 3) / 4) * sizeof(double2);
-  cudaError_t e = cudaFuncSetAttribute(fft_pass_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(smem));
+  static PerDevice limit;
+  const cudaError_t e = allow_smem(limit, fft_pass_kernel, kFftPassSmem);
   if (e != cudaSuccess) return e;
   // a thread per radix-4 butterfly, up to 256
   int64_t threads = static_cast<int64_t>(L << a.cbits) / 4;
@@ -350,37 +354,58 @@ cudaError_t launch_pass(FftPass a, cudaStream_t s) {
 // divides both factors), if the device can place it; cudaErrorNotSupported
 // when it cannot, so that the caller takes the two-pass form.
 cudaError_t launch_cluster(const FftCluster& a, cudaStream_t s) {
-  int64_t C = 16;
-  while (C > 1 && (C > (1 << a.bits1) || C > (1 << a.bits2))) C /= 2;
-  for (; C >= 1; C /= 2) {
+  static PerDevice limit, wide, fits[kFftClusterBits + 1];
+  cudaError_t e = allow_smem(limit, fft_cluster_kernel, kFftClusterSmem);
+  if (e != cudaSuccess) return e;
+  int done = 0;
+  e = wide.get(&done, [](int* v) {
+    *v = 1;
+    return cudaFuncSetAttribute(fft_cluster_kernel,
+                                cudaFuncAttributeNonPortableClusterSizeAllowed, 1);
+  });
+  if (e != cudaSuccess) return e;
+  cudaLaunchAttribute attr[1];
+  cudaLaunchConfig_t cfg = {};
+  auto configure = [&](int64_t C) {
     const size_t N1 = size_t{1} << a.bits1, N2 = size_t{1} << a.bits2;
-    const size_t smem = (2 * (N1 * N2 / C) + 3 * (N1 + N2) / 4) * sizeof(double2);
-    cudaError_t e = cudaFuncSetAttribute(fft_cluster_kernel,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(smem));
-    if (e != cudaSuccess) return e;
-    if (C > 8 && (e = cudaFuncSetAttribute(fft_cluster_kernel,
-                                           cudaFuncAttributeNonPortableClusterSizeAllowed, 1)) !=
-                     cudaSuccess)
-      return e;
-    cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3(static_cast<unsigned>(C), 1, 1);
     cfg.blockDim = dim3(kFftThreads, 1, 1);
-    cfg.dynamicSmemBytes = smem;
+    cfg.dynamicSmemBytes = (2 * (N1 * N2 / C) + 3 * (N1 + N2) / 4) * sizeof(double2);
     cfg.stream = s;
-    cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeClusterDimension;
     attr[0].val.clusterDim.x = static_cast<unsigned>(C);
     attr[0].val.clusterDim.y = 1;
     attr[0].val.clusterDim.z = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    int clusters = 0;
-    if ((e = cudaOccupancyMaxActiveClusters(&clusters, fft_cluster_kernel, &cfg)) != cudaSuccess)
-      return e;
-    if (clusters >= 1) return cudaLaunchKernelEx(&cfg, fft_cluster_kernel, a);
-  }
-  return cudaErrorNotSupported;
+  };
+  // the cluster size that the device places, 0: none
+  auto largest = [&](int* size) {
+    int64_t C = 16;
+    while (C > 1 && (C > (1 << a.bits1) || C > (1 << a.bits2))) C /= 2;
+    for (*size = 0; C >= 1; C /= 2) {
+      configure(C);
+      int clusters = 0;
+      const cudaError_t q = cudaOccupancyMaxActiveClusters(&clusters, fft_cluster_kernel, &cfg);
+      if (q != cudaSuccess) return q;
+      if (clusters >= 1) {
+        *size = static_cast<int>(C);
+        break;
+      }
+    }
+    return cudaSuccess;
+  };
+  int size = 0;
+  // bits1 - bits2 is 0 or 1, so their sum names the shape
+  if ((e = fits[a.bits1 + a.bits2].get(&size, largest)) != cudaSuccess) return e;
+  if (size == 0) return cudaErrorNotSupported;
+  configure(size);
+  e = cudaLaunchKernelEx(&cfg, fft_cluster_kernel, a);
+  if (e == cudaSuccess) return e;
+  // a context with fewer SMs than the one that was asked: ask for this one
+  cudaGetLastError();
+  if ((e = largest(&size)) != cudaSuccess) return e;
+  return size == 0 ? cudaErrorNotSupported : cudaLaunchKernelEx(&cfg, fft_cluster_kernel, a);
 }
 
 }  // namespace

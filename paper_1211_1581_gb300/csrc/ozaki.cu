@@ -2353,8 +2353,8 @@ static cudaError_t launch_split_t(const double* A, const double* B, const OzakiD
       const int R = d.Kt <= 2 ? 8 : d.Kt <= 4 ? 4 : d.Kt <= 8 ? 2 : 1;
       const size_t smem = R * static_cast<size_t>(d.Kt) * kOzTileK * sizeof(double);
       auto kern = oz_scale_split_a_kernel<Splitter<kKind, kDiff>>;
-      cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                           static_cast<int>(smem));
+      static PerDevice limit;
+      cudaError_t e = allow_smem(limit, kern, kFusedRowMaxK * sizeof(double));
       if (e != cudaSuccess) return e;
       kern<<<static_cast<unsigned>(d.Mt * kOzTileRows / R), 256, smem, s>>>(
           A, d.m, d.k, rowbits, sa, R, d.Mt, d.Kt, aslices, status);
@@ -2407,8 +2407,8 @@ static cudaError_t launch_oz_gemm_t(const Tiles& tiles, int64_t grid, int S, int
                                     int window, int* status, cudaStream_t s) {
   if (grid <= 0) return cudaSuccess;
   auto kern = oz_gemm_kernel<Acc, kFloat, Tiles, kEpiW>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(kGemmSmemBytes));
+  static PerDevice limit;
+  cudaError_t e = allow_smem(limit, kern, kGemmSmemBytes);
   if (e != cudaSuccess) return e;
   kern<<<static_cast<unsigned>(grid), 128 + 32 * kEpiW, kGemmSmemBytes, s>>>(tiles, S, beta,
                                                                               window, status);
@@ -2476,8 +2476,9 @@ static cudaError_t launch_gemm2_pairs(const OzSingle& tiles, const OzakiDims& d,
   auto kern = tiles.spill != nullptr ? oz_gemm2_kernel<OzSingle, FmtBf16Pair, true>
                                      : oz_gemm2_kernel<OzSingle, FmtBf16Pair, false>;
   const size_t kSmem = gemm2_smem_bytes<FmtBf16Pair>();
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(kSmem));
+  static PerDevice limit[2], held[2];
+  const int which = tiles.spill != nullptr;
+  cudaError_t e = allow_smem(limit[which], kern, kSmem);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3(kP2Threads, 1, 1);
@@ -2492,7 +2493,9 @@ static cudaError_t launch_gemm2_pairs(const OzSingle& tiles, const OzakiDims& d,
   cfg.numAttrs = 1;
   cfg.gridDim = dim3(2, 1, 1);
   int clusters = 0;
-  e = cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg);
+  e = held[which].get(&clusters, [&](int* v) {
+    return cudaOccupancyMaxActiveClusters(v, kern, &cfg);
+  });
   if (e != cudaSuccess) return e;
   if (clusters < 1) return cudaErrorLaunchOutOfResources;
   const int64_t units = (d.Mt + 1) / 2 * d.Nt;
@@ -2526,8 +2529,8 @@ cudaError_t launch_ozaki_gemm(const uint8_t* aslices, const uint8_t* bslices,
     if (splits > 1 || !ozaki_narrow(d.S, d.beta, d.Kt)) return cudaErrorNotSupported;
     auto kern = oz_gemm2_kernel<OzSingle, FmtE4m3>;
     const size_t kSmem = gemm2_smem_bytes<FmtE4m3>();
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                         static_cast<int>(kSmem));
+    static PerDevice limit;
+    cudaError_t e = allow_smem(limit, kern, kSmem);
     if (e != cudaSuccess) return e;
     kern<<<static_cast<unsigned>(grid), kP2Threads, kSmem, s>>>(tiles, d.S, d.beta, window,
                                                                 status);
@@ -2566,8 +2569,8 @@ cudaError_t launch_ozaki_gemm(const uint8_t* aslices, const uint8_t* bslices,
   auto kern = tiles.spill != nullptr ? oz_gemm2_kernel<OzSingle, FmtBf16, true>
                                      : oz_gemm2_kernel<OzSingle, FmtBf16, false>;
   const size_t kSmem = gemm2_smem_bytes<FmtBf16>();
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(kSmem));
+  static PerDevice limit[2];
+  cudaError_t e = allow_smem(limit[tiles.spill != nullptr], kern, kSmem);
   if (e != cudaSuccess) return e;
   kern<<<static_cast<unsigned>(g2), kP2Threads, kSmem, s>>>(tiles, d.S, d.beta, window, status);
   return cudaGetLastError();
@@ -2594,8 +2597,8 @@ cudaError_t launch_ozaki_grouped(uint8_t* ws, int S, int beta, int64_t short_kt,
   if (lt.spill_every < 1) return cudaErrorNotSupported;
   auto kern = oz_gemm2_kernel<OzGrouped, FmtBf16, true>;
   const size_t kSmem = gemm2_smem_bytes<FmtBf16>();
-  e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(kSmem));
+  static PerDevice limit;
+  e = allow_smem(limit, kern, kSmem);
   if (e != cudaSuccess) return e;
   const int grid = sms < kOzSpillCtas ? sms : static_cast<int>(kOzSpillCtas);
   kern<<<grid, kP2Threads, kSmem, s>>>(lt, S, beta, window, status);

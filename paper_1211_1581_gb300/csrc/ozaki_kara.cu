@@ -850,8 +850,8 @@ cudaError_t launch_ozaki_kara(const uint8_t* aslices, const uint8_t* bslices,
   a.raster = static_cast<int>(d.raster < Mp ? (d.raster > 0 ? d.raster : kDefaultRaster) : Mp);
   build_prog(d.S, is_short, a.prog);
   const auto kern = is_short ? oz_kara_kernel<true> : oz_kara_kernel<false>;
-  cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                                       static_cast<int>(kSmemBytes));
+  static PerDevice limit[2], held[2];
+  cudaError_t e = allow_smem(limit[is_short], kern, kSmemBytes);
   if (e != cudaSuccess) return e;
   cudaLaunchConfig_t cfg = {};
   cfg.blockDim = dim3(kThreads, 1, 1);
@@ -866,7 +866,9 @@ cudaError_t launch_ozaki_kara(const uint8_t* aslices, const uint8_t* bslices,
   cfg.numAttrs = 1;
   cfg.gridDim = dim3(2, 1, 1);
   int clusters = 0;
-  e = cudaOccupancyMaxActiveClusters(&clusters, kern, &cfg);
+  e = held[is_short].get(&clusters, [&](int* v) {
+    return cudaOccupancyMaxActiveClusters(v, kern, &cfg);
+  });
   if (e != cudaSuccess) return e;
   if (clusters < 1) return cudaErrorLaunchOutOfResources;
   const int64_t pairs = clusters < kKaraPairs ? clusters : kKaraPairs;
