@@ -234,11 +234,12 @@ mxm_status run_gemm(int mode, const double* A, const double* B, double* C, int64
     e = launch_f64_gemm(A, B, C, d, ws, ws_bytes, status, s);
     profile_mark(ce, 3, s);
   } else if (emul_mode(mode)) {
-    const OzakiDims d = emul_dims(mode, m, k, n, slices, plan, kara);
+    OzakiDims d = emul_dims(mode, m, k, n, slices, plan, kara);
     const OzakiLayout L = ozaki_layout(d);
     uint64_t* rowbits = reinterpret_cast<uint64_t*>(ws + L.rowbits);
     uint64_t* colbits = reinterpret_cast<uint64_t*>(ws + L.colbits);
     CallEvents* ce = profile_begin(s);
+    d.chain = ce == nullptr;  // phases are timed one after the other
     e = launch_ozaki_scale(A, B, d, rowbits, colbits, status, s);
     profile_mark(ce, 1, s);
     if (e == cudaSuccess)

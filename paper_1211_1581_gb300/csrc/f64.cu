@@ -227,6 +227,7 @@ __device__ __forceinline__ F64Spot f64_spot(const F64Balanced& p, int i) {
 
 __global__ void __launch_bounds__(kBalancedThreads, 1) f64_balanced_kernel(
     const F64Balanced p, int* __restrict__ status) {
+  release_next();
   const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
   const int g = lane >> 2, t4 = lane & 3;
   // neighbouring shares on one sub-partition (warps w and w + 4)
@@ -331,6 +332,8 @@ __global__ void __launch_bounds__(kBalancedThreads, 1) f64_balanced_kernel(
 // the workers' parts in order of k.
 __global__ void __launch_bounds__(kBalancedThreads) f64_balanced_reduce_kernel(
     const F64Balanced p) {
+  follow_grid();
+  const double* const slots = after_follow(p.slots);
   const int w0 = blockIdx.x;
   const F64Spot from = p.starts[w0], to = p.starts[w0 + 1];
   if (to.step == 0 || (from.piece == to.piece && from.step > 0)) return;
@@ -345,16 +348,16 @@ __global__ void __launch_bounds__(kBalancedThreads) f64_balanced_reduce_kernel(
   const int64_t pm = piece / p.Np, pn = piece - pm * p.Np;
   for (int e = blockIdx.y * kBalancedThreads + threadIdx.x; e < kPiece * kPiece;
        e += gridDim.y * kBalancedThreads) {
-    double v = p.slots[(static_cast<int64_t>(w0) * 2 + 1) * (kPiece * kPiece) + e];
+    double v = slots[(static_cast<int64_t>(w0) * 2 + 1) * (kPiece * kPiece) + e];
     if (p.ranges == 0) {
 #pragma unroll 8
       for (int w = w0 + 1; w <= w1; ++w)
-        v += __ldcs(p.slots + static_cast<int64_t>(w) * 2 * (kPiece * kPiece) + e);
+        v += __ldcs(slots + static_cast<int64_t>(w) * 2 * (kPiece * kPiece) + e);
     } else {  // shares may be empty: those have no part
       for (int w = w0 + 1; w <= w1; ++w) {
         const F64Spot b = p.starts[w], n = p.starts[w + 1];
         if (b.piece < n.piece || b.step < n.step)
-          v += __ldcs(p.slots + static_cast<int64_t>(w) * 2 * (kPiece * kPiece) + e);
+          v += __ldcs(slots + static_cast<int64_t>(w) * 2 * (kPiece * kPiece) + e);
       }
     }
     const int i = e >> 5, lane = e & 31, q = i & 3;
@@ -396,7 +399,10 @@ cudaError_t launch_f64_gemm(const double* A, const double* B, double* C, const F
   f64_balanced_kernel<<<(p.workers + kWarps - 1) / kWarps, kBalancedThreads, 0, s>>>(p, status);
   if (p.ranges != 1) {
     const unsigned split = p.Mp * p.Np < 304 ? kPiece * kPiece / kBalancedThreads : 1;
-    f64_balanced_reduce_kernel<<<dim3(p.workers, split), kBalancedThreads, 0, s>>>(p);
+    const cudaError_t e = cudaGetLastError();
+    return e != cudaSuccess ? e
+                            : launch_chained(true, f64_balanced_reduce_kernel,
+                                             dim3(p.workers, split), kBalancedThreads, 0, s, p);
   }
   return cudaGetLastError();
 }

@@ -34,6 +34,7 @@
 
 #include "mxm.h"
 #include "mxm_internal.h"
+#include "ptx.cuh"
 
 namespace mxm {
 
@@ -190,6 +191,9 @@ __global__ void __launch_bounds__(kFftThreads) fft_pass_kernel(const FftPass a) 
   // twiddles of the L-point transform: W_L^m = W_T^{m T / L}
   for (int m = tid; m < (3 * L + 3) / 4; m += nth)
     tw[m] = table_w(a.table, 1u << a.tbits, static_cast<uint32_t>(m) << (a.tbits - bits));
+  // the second pass, launched beside the first, waits for its results here
+  follow_grid();
+  release_next();
   // load: C consecutive columns per row, c fastest
   for (int t = tid; t < (C << bits); t += nth) {
     const int r = t >> a.cbits, c = t & (C - 1), col = c0 + c;
@@ -345,9 +349,9 @@ cudaError_t launch_pass(FftPass a, cudaStream_t s) {
   // a thread per radix-4 butterfly, up to 256
   int64_t threads = static_cast<int64_t>(L << a.cbits) / 4;
   threads = threads > kFftThreads ? kFftThreads : (threads < 32 ? 32 : threads);
-  fft_pass_kernel<<<static_cast<unsigned>(cols >> a.cbits), static_cast<unsigned>(threads), smem,
-                    s>>>(a);
-  return cudaGetLastError();
+  return launch_chained(a.stage == 2, fft_pass_kernel,
+                        dim3(static_cast<unsigned>(cols >> a.cbits)),
+                        dim3(static_cast<unsigned>(threads)), smem, s, a);
 }
 
 // One launch on a cluster of C CTAs (the largest power of two <= 16 that

@@ -117,6 +117,7 @@ __global__ void oz_colmax_kernel(const double* __restrict__ B, int64_t k, int64_
                                  unsigned long long* __restrict__ colbits,
                                  int* __restrict__ status) {
   __shared__ uint32_t red[8][32];
+  release_next();  // A's split does not read the column maxima
   const int tx = threadIdx.x & 31, ty = threadIdx.x >> 5;
   const int64_t col = static_cast<int64_t>(blockIdx.x) * 32 + tx;
   const int64_t l0 = static_cast<int64_t>(blockIdx.y) * kColRowsPerBlock;
@@ -546,6 +547,7 @@ __global__ void __launch_bounds__(256) oz_split_a_kernel(
   split_a_tile(A, m, k, rowbits, split, tm, tk,
                aslices + (static_cast<size_t>(tm) * Kt + tk) * kTile,
                static_cast<size_t>(Mt) * Kt * kTile);
+  follow_grid();  // ran beside B's column maxima
 }
 
 // Steps 1 and 2 for A in one pass: a block takes R rows of A (padding rows of
@@ -628,6 +630,7 @@ __global__ void __launch_bounds__(256) oz_scale_split_a_kernel(
     split(v, e, base + static_cast<size_t>(tk) * kOzTileBytes + oz_chunk_offset(r, c),
           slice_stride);
   }
+  follow_grid();  // ran beside B's column maxima
 }
 
 // Whether A's scale and split run fused (bf16 digits, k short enough for a
@@ -645,8 +648,10 @@ __global__ void __launch_bounds__(256) oz_split_b_kernel(
     const Split split, int64_t Nt, int64_t Kt, uint8_t* __restrict__ bslices, bool halves) {
   constexpr size_t kTile = SplitGeo<Split::V>::kTileBytes;
   __shared__ double sb[kSplitBRows][kOzTileRows + 1];
+  follow_grid();
+  release_next();
   const int64_t tk = blockIdx.x, tn = blockIdx.y;
-  split_b_tile(B, k, n, colbits, split, tn, tk,
+  split_b_tile(B, k, n, after_follow(colbits), split, tn, tk,
                bslices + (static_cast<size_t>(tn) * Kt + tk) * kTile,
                static_cast<size_t>(Nt) * Kt * kTile, sb, halves, kOzTileRows,
                SplitGeo<Split::V>::kChunksPerRow, blockIdx.z, blockIdx.z + 1);
@@ -1264,6 +1269,8 @@ __global__ void __launch_bounds__(128 + 32 * kEpiW, 1)
   tc_fence_after();
   const uint32_t tmem = sm.tmem_base;
   volatile int* abort_flag = &sm.abort_flag;
+  follow_grid();
+  release_next();
   const int64_t ntiles = tiles.count();
 
   if (warp < 4) {  // warps 2, 3 idle
@@ -1782,6 +1789,8 @@ __global__ void __launch_bounds__(kP2Threads, 1)
   tc_fence_after();
   const uint32_t tmem = sm.tmem_base;
   volatile int* abort_flag = &sm.abort_flag;
+  follow_grid();
+  release_next();
   // work units: C tiles, or (pairs) 256-row C tiles shared by the cluster
   int64_t nunits;
   if constexpr (kPair)
@@ -2356,19 +2365,23 @@ static cudaError_t launch_split_t(const double* A, const double* B, const OzakiD
       static PerDevice limit;
       cudaError_t e = allow_smem(limit, kern, kFusedRowMaxK * sizeof(double));
       if (e != cudaSuccess) return e;
-      kern<<<static_cast<unsigned>(d.Mt * kOzTileRows / R), 256, smem, s>>>(
-          A, d.m, d.k, rowbits, sa, R, d.Mt, d.Kt, aslices, status);
+      e = launch_chained(d.chain, kern, dim3(static_cast<unsigned>(d.Mt * kOzTileRows / R)), 256,
+                         smem, s, A, d.m, d.k, rowbits, sa, R, d.Mt, d.Kt, aslices, status);
+      if (e != cudaSuccess) return e;
     }
   } else if (d.Mt > 0) {
-    oz_split_a_kernel<<<dim3(static_cast<unsigned>(d.Kt), static_cast<unsigned>(d.Mt)), 256, 0,
-                        s>>>(A, d.m, d.k, rowbits, sa, d.Mt, d.Kt, aslices);
+    const cudaError_t e = launch_chained(
+        d.chain, oz_split_a_kernel<Splitter<kKind, kDiff>>,
+        dim3(static_cast<unsigned>(d.Kt), static_cast<unsigned>(d.Mt)), 256, 0, s, A, d.m, d.k,
+        rowbits, sa, d.Mt, d.Kt, aslices);
+    if (e != cudaSuccess) return e;
   }
-  if (d.Nt > 0)
-    oz_split_b_kernel<<<dim3(static_cast<unsigned>(d.Kt), static_cast<unsigned>(d.Nt),
+  if (d.Nt == 0) return cudaSuccess;
+  return launch_chained(d.chain, oz_split_b_kernel<Splitter<kKind, kDiff>>,
+                        dim3(static_cast<unsigned>(d.Kt), static_cast<unsigned>(d.Nt),
                              kOzTileK / kSplitBRows),
-                        256, 0, s>>>(B, d.k, d.n, colbits, sb, d.Nt, d.Kt, bslices,
-                                     ozaki_b_halves(d));
-  return cudaGetLastError();
+                        256, 0, s, B, d.k, d.n, colbits, sb, d.Nt, d.Kt, bslices,
+                        ozaki_b_halves(d));
 }
 
 cudaError_t launch_ozaki_split(const double* A, const double* B, const OzakiDims& d,
@@ -2404,15 +2417,14 @@ int sm_count() {
 
 template <typename Acc, bool kFloat, typename Tiles, int kEpiW = 8>
 static cudaError_t launch_oz_gemm_t(const Tiles& tiles, int64_t grid, int S, int beta,
-                                    int window, int* status, cudaStream_t s) {
+                                    int window, int* status, cudaStream_t s, bool chain = false) {
   if (grid <= 0) return cudaSuccess;
   auto kern = oz_gemm_kernel<Acc, kFloat, Tiles, kEpiW>;
   static PerDevice limit;
   cudaError_t e = allow_smem(limit, kern, kGemmSmemBytes);
   if (e != cudaSuccess) return e;
-  kern<<<static_cast<unsigned>(grid), 128 + 32 * kEpiW, kGemmSmemBytes, s>>>(tiles, S, beta,
-                                                                              window, status);
-  return cudaGetLastError();
+  return launch_chained(chain, kern, dim3(static_cast<unsigned>(grid)), 128 + 32 * kEpiW,
+                        kGemmSmemBytes, s, tiles, S, beta, window, status);
 }
 
 // Split-k recombination (steps 3-4 after a split product): D_g of every C
@@ -2425,11 +2437,13 @@ static cudaError_t launch_oz_gemm_t(const Tiles& tiles, int64_t grid, int S, int
 // thread for all ranges 110 us), one below (4096 x 128, 9 ranges).
 template <int kRows>
 __global__ void __launch_bounds__(256) oz_splitk_fold_kernel(
-    const uint64_t* __restrict__ P, const uint64_t* __restrict__ rowbits,
+    const uint64_t* P, const uint64_t* __restrict__ rowbits,
     const uint64_t* __restrict__ colbits, double* __restrict__ C, int64_t m, int64_t n,
     int64_t Mt, int64_t Nt, int64_t splits, int S, int beta, int gx, int eoff) {
   constexpr int E = 256 / kRows;
   __shared__ long long part[kRows > 1 ? kOzMaxSlices : 1][kRows][E];
+  follow_grid();
+  P = after_follow(P);
   const int tx = threadIdx.x % E, ty = threadIdx.x / E;
   const int64_t idx = static_cast<int64_t>(blockIdx.x) * E + tx;
   const bool live = idx < m * n;
@@ -2484,11 +2498,13 @@ static cudaError_t launch_gemm2_pairs(const OzSingle& tiles, const OzakiDims& d,
   cfg.blockDim = dim3(kP2Threads, 1, 1);
   cfg.dynamicSmemBytes = kSmem;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   cfg.gridDim = dim3(2, 1, 1);
@@ -2503,6 +2519,7 @@ static cudaError_t launch_gemm2_pairs(const OzSingle& tiles, const OzakiDims& d,
   if (pairs > max_ctas / 2) pairs = max_ctas / 2;
   if (pairs < 1) pairs = 1;
   cfg.gridDim = dim3(static_cast<unsigned>(2 * pairs), 1, 1);
+  cfg.numAttrs = d.chain ? 2 : 1;
   return cudaLaunchKernelEx(&cfg, kern, tiles, d.S, d.beta, window, status);
 }
 
@@ -2532,24 +2549,22 @@ cudaError_t launch_ozaki_gemm(const uint8_t* aslices, const uint8_t* bslices,
     static PerDevice limit;
     cudaError_t e = allow_smem(limit, kern, kSmem);
     if (e != cudaSuccess) return e;
-    kern<<<static_cast<unsigned>(grid), kP2Threads, kSmem, s>>>(tiles, d.S, d.beta, window,
-                                                                status);
-    return cudaGetLastError();
+    return launch_chained(d.chain, kern, dim3(static_cast<unsigned>(grid)), kP2Threads, kSmem, s,
+                          tiles, d.S, d.beta, window, status);
   }
   if (splits > 1) {
     // one diagonal at a time, each k range's D_g to the partials, then the fold
     cudaError_t e =
-        launch_oz_gemm_t<long long, false>(tiles, grid, d.S, d.beta, window, status, s);
+        launch_oz_gemm_t<long long, false>(tiles, grid, d.S, d.beta, window, status, s, d.chain);
     if (e != cudaSuccess) return e;
     const int64_t total = d.m * d.n;
     auto fold = [&](auto kern, int64_t per_block) {
-      kern<<<static_cast<unsigned>((total + per_block - 1) / per_block), 256, 0, s>>>(
-          sums, rowbits, colbits, C, d.m, d.n, d.Mt, d.Nt, splits, d.S, d.beta,
-          ozaki_exact_from(d.S, d.beta, d.Kt), d.rn ? 2 : 0);
+      return launch_chained(d.chain, kern,
+                            dim3(static_cast<unsigned>((total + per_block - 1) / per_block)), 256,
+                            0, s, sums, rowbits, colbits, C, d.m, d.n, d.Mt, d.Nt, splits, d.S,
+                            d.beta, ozaki_exact_from(d.S, d.beta, d.Kt), d.rn ? 2 : 0);
     };
-    if (splits >= 32) fold(oz_splitk_fold_kernel<8>, 32);
-    else fold(oz_splitk_fold_kernel<1>, 256);
-    return cudaGetLastError();
+    return splits >= 32 ? fold(oz_splitk_fold_kernel<8>, 32) : fold(oz_splitk_fold_kernel<1>, 256);
   }
   // the paired kernel; when a diagonal's sum over all of k may pass int32,
   // with the spill area that follows the running sums (grid capped to it)
@@ -2572,8 +2587,8 @@ cudaError_t launch_ozaki_gemm(const uint8_t* aslices, const uint8_t* bslices,
   static PerDevice limit[2];
   cudaError_t e = allow_smem(limit[tiles.spill != nullptr], kern, kSmem);
   if (e != cudaSuccess) return e;
-  kern<<<static_cast<unsigned>(g2), kP2Threads, kSmem, s>>>(tiles, d.S, d.beta, window, status);
-  return cudaGetLastError();
+  return launch_chained(d.chain, kern, dim3(static_cast<unsigned>(g2)), kP2Threads, kSmem, s,
+                        tiles, d.S, d.beta, window, status);
 }
 
 cudaError_t launch_ozaki_grouped(uint8_t* ws, int S, int beta, int64_t short_kt, int* status,

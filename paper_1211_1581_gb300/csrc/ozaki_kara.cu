@@ -265,6 +265,8 @@ __global__ void __launch_bounds__(kThreads, 1)
   tc_fence_after();
   const uint32_t tmem = sm.tmem_base;
   volatile int* abort_flag = &sm.abort_flag;
+  follow_grid();
+  release_next();
   const int nunits = kunits(a);
   const int unit0 = blockIdx.x >> 1, unit_step = gridDim.x >> 1;
 
@@ -618,6 +620,8 @@ __global__ void __launch_bounds__(kFoldThreads) oz_kara_fold_kernel(
     const __grid_constant__ KaraArgs a, int part0) {
   constexpr int kSlotVec = kFoldVec;
   const int S = a.S;
+  follow_grid();
+  release_next();
   const int part = part0 + blockIdx.y;  // (tile, rank) among the kind's tiles
   const int t = (kCut ? a.full_tiles : 0) + (part >> 1), rank = part & 1;
   int tm, tn;
@@ -633,7 +637,7 @@ __global__ void __launch_bounds__(kFoldThreads) oz_kara_fold_kernel(
     // added first, with 64-bit ones each range's D_g are.
     constexpr bool kWide = sizeof(Sum) == 8;
     const size_t range = 2 * static_cast<size_t>(2 * S - 2) * kSlotVec;
-    const int4* p = a.cut_scratch + static_cast<size_t>(part >> 1) * a.ranges * range +
+    const int4* p = after_follow(a.cut_scratch) + static_cast<size_t>(part >> 1) * a.ranges * range +
                     static_cast<size_t>(rank) * (2 * S - 2) * kSlotVec + v;
     int ng[kMaxS - 1][4], sq[kMaxS - 1][4];  // N_{S+1} .. N_3, P_{S-1} .. P_1
     auto clear = [&]() {
@@ -692,7 +696,8 @@ __global__ void __launch_bounds__(kFoldThreads) oz_kara_fold_kernel(
     }
     if (!kWide) combine();
   } else {
-    const int4* p = a.full_scratch + static_cast<size_t>(part) * S * kSlotVec + v;
+    const int4* p =
+        after_follow(a.full_scratch) + static_cast<size_t>(part) * S * kSlotVec + v;
 #pragma unroll
     for (int i = 0; i < kMaxS - 1; ++i) {
       const int4 x = i < S - 1 ? __ldcs(p + static_cast<size_t>(S - 1 - i) * kSlotVec)
@@ -857,11 +862,13 @@ cudaError_t launch_ozaki_kara(const uint8_t* aslices, const uint8_t* bslices,
   cfg.blockDim = dim3(kThreads, 1, 1);
   cfg.dynamicSmemBytes = kSmemBytes;
   cfg.stream = s;
-  cudaLaunchAttribute attr[1];
+  cudaLaunchAttribute attr[2];
   attr[0].id = cudaLaunchAttributeClusterDimension;
   attr[0].val.clusterDim.x = 2;
   attr[0].val.clusterDim.y = 1;
   attr[0].val.clusterDim.z = 1;
+  attr[1].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  attr[1].val.programmaticStreamSerializationAllowed = 1;
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   cfg.gridDim = dim3(2, 1, 1);
@@ -885,22 +892,24 @@ cudaError_t launch_ozaki_kara(const uint8_t* aslices, const uint8_t* bslices,
   const int64_t units = a.full_tiles + (tiles - a.full_tiles) * a.parts * a.ranges;
   const int64_t use = units < pairs ? units : pairs;
   cfg.gridDim = dim3(static_cast<unsigned>(2 * use), 1, 1);
+  cfg.numAttrs = d.chain ? 2 : 1;
   e = cudaLaunchKernelEx(&cfg, kern, a, status);
   if (e != cudaSuccess || is_short) return e;
   // (tile, rank) parts on the y axis of the grid, at most kFoldParts per launch
   constexpr int64_t kFoldParts = 32768;
   auto fold = [&](auto kern, int64_t parts) {
-    for (int64_t p0 = 0; p0 < parts; p0 += kFoldParts) {
+    for (int64_t p0 = 0; p0 < parts && e == cudaSuccess; p0 += kFoldParts) {
       const int64_t now = parts - p0 < kFoldParts ? parts - p0 : kFoldParts;
-      kern<<<dim3(kFoldVec / kFoldThreads, static_cast<unsigned>(now)), kFoldThreads, 0, s>>>(
-          a, static_cast<int>(p0));
+      e = launch_chained(d.chain, kern,
+                         dim3(kFoldVec / kFoldThreads, static_cast<unsigned>(now)), kFoldThreads,
+                         0, s, a, static_cast<int>(p0));
     }
   };
   fold(oz_kara_fold_kernel<false, int>, 2 * static_cast<int64_t>(a.full_tiles));
   const int64_t cut = 2 * (tiles - a.full_tiles);
   if (wide) fold(oz_kara_fold_kernel<true, long long>, cut);
   else fold(oz_kara_fold_kernel<true, int>, cut);
-  return cudaGetLastError();
+  return e;
 }
 
 }  // namespace mxm

@@ -12,6 +12,24 @@
 
 namespace mxm {
 
+// Launches that overlap their predecessor (launch_chained).  follow_grid: wait
+// until the grids before this one have ended and their writes are visible (at
+// once in an ordinary launch); release_next: the next grid may be launched.
+__device__ __forceinline__ void follow_grid() {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+__device__ __forceinline__ void release_next() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+// A pointer to an earlier grid's results, known only from here on: loads that
+// the compiler may move (__ldg, __ldcs, restrict) stay behind follow_grid.
+template <typename T>
+__device__ __forceinline__ T* after_follow(T* p) {
+  asm volatile("" : "+l"(p)::"memory");
+  return p;
+}
+
+
 // ------------------------------------------------------------ bounds checks
 // The MXM_DEBUG_BOUNDS build (libmxm_debug.so) checks tile coordinates, the
 // sources of bulk copies and tensor-memory column ranges in the kernels; a
