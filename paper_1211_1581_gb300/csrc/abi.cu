@@ -188,7 +188,7 @@ OzakiDims emul_dims(int mode, int64_t m, int64_t k, int64_t n, int slices, const
   if (kara && p.cta == 0 && p.splitk <= 1) {
     OzakiDims w = d;
     w.splits = 1;
-    if (kara_chosen(w)) {
+    if (kara_chosen(w) || kara_one_block(w)) {
       w.kara = kara_short(w) ? 2 : 1;
       w.pair = 1;
       w.raster = p.raster > 0 ? p.raster : kDefaultRaster;
@@ -217,6 +217,16 @@ size_t workspace_bytes(int mode, int64_t m, int64_t k, int64_t n, int slices,
   if (mode == MXM_MODE_EMUL_FP8) return ozaki_layout(fp8_dims(m, k, n, slices, p)).total;
   if (mode == MXM_MODE_BF16_F32ACC) return ozaki_layout(ozaki_dims(m, k, n, 1, 8)).total;
   return 0;
+}
+
+// The size that a caller is told: the most, but for one k-block of one tile-row
+// or tile-column, where the segment slots are many times the planes (256 x 128
+// x 128, S = 7: 6.7 MB instead of 0.9), the least; a workspace with more room,
+// the library's own among them, is still used.
+size_t workspace_told(int mode, int64_t m, int64_t k, int64_t n, int slices, const mxm_plan& p) {
+  const bool thin = emul_mode(mode) &&
+                    kara_one_block(ozaki_dims(m, k, n, slices, mode_beta(mode), mode_rn(mode)));
+  return workspace_bytes(mode, m, k, n, slices, p, !thin);
 }
 
 // Launch sequence of one product whose workspace is already in place.
@@ -333,7 +343,7 @@ const char* mxm_status_string(mxm_status s) {
 
 size_t mxm_workspace_size(int mode, int64_t m, int64_t k, int64_t n, int slices) {
   if (check_mode(mode, slices) != MXM_OK) return 0;
-  return workspace_bytes(mode, m, k, n, slices);
+  return workspace_told(mode, m, k, n, slices, kNoPlan);
 }
 
 mxm_status mxm_gemm_plan(int mode, const double* A, const double* B, double* C, int64_t m,
@@ -371,7 +381,7 @@ size_t mxm_workspace_size_plan(int mode, int64_t m, int64_t k, int64_t n, int sl
                                const mxm_plan* plan) {
   const mxm_plan p = plan ? *plan : kNoPlan;
   if (check_mode(mode, slices) != MXM_OK || !plan_ok(mode, p)) return 0;
-  return workspace_bytes(mode, m, k, n, slices, p);
+  return workspace_told(mode, m, k, n, slices, p);
 }
 
 mxm_status mxm_f64(const double* A, const double* B, double* C, int64_t m, int64_t k, int64_t n,

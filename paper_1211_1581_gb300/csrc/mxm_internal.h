@@ -373,6 +373,14 @@ inline bool kara_short(const OzakiDims& d) {
   if (tiles < 40) return false;
   return d.Kt <= 3 || (d.Kt <= 4 && tiles >= 512) || (d.Kt <= 8 && tiles <= kKaraPairs);
 }
+// One k-block of one tile-row or tile-column: one by one, a lone CTA takes the
+// diagonals of a tile in turn; here the segments are shared out over the SMs
+// (64^3, S = 7: 35 us against 74; 4096 x 64 x 64, 16 tiles, 52 against 81; with
+// 64 tiles there is a CTA for each: 16384 x 64 x 64 74 against 75).  Apart from
+// kara_chosen because a caller is not asked for its workspace (workspace_told).
+inline bool kara_one_block(const OzakiDims& d) {
+  return kara_fits(d) && d.Kt == 1 && (d.Mt == 1 || d.Nt == 1) && kara_tiles(d) <= 16;
+}
 inline bool kara_chosen(const OzakiDims& d) {
   if (!kara_fits(d)) return false;
   const bool is_short = kara_short(d);

@@ -111,7 +111,8 @@ __global__ void oz_rowmax_kernel(const double* __restrict__ A, int64_t m, int64_
 }
 
 // max_l |b_lj| for 32 columns per block, rows split over blockIdx.y; the
-// per-block maxima meet in colbits by atomicMax (colbits zeroed first).
+// per-block maxima meet in colbits by atomicMax (colbits zeroed first; one
+// block of rows, k up to 256, stores them: a small call is launches and gaps).
 constexpr int kColRowsPerBlock = 256;
 __global__ void oz_colmax_kernel(const double* __restrict__ B, int64_t k, int64_t n,
                                  unsigned long long* __restrict__ colbits,
@@ -135,7 +136,10 @@ __global__ void oz_colmax_kernel(const double* __restrict__ B, int64_t k, int64_
       for (int64_t l = l0; l < l1; ++l) lo = max(lo, lo_word(__ldg(B + l * n + col)));
     // the block maxima of a column meet in the same form: hi 2^32 beats any lo
     const uint64_t mx = max_bits(mh, lo);
-    atomicMax(colbits + col, static_cast<unsigned long long>(mx));
+    if (gridDim.y == 1)
+      colbits[col] = mx;
+    else
+      atomicMax(colbits + col, static_cast<unsigned long long>(mx));
     if (mx >= kInfBits) atomicOr(status, kStatusNonFinite);
   }
 }
@@ -2340,8 +2344,10 @@ cudaError_t launch_ozaki_scale(const double* A, const double* B, const OzakiDims
     }
   }
   if (d.n > 0) {
-    cudaError_t e = cudaMemsetAsync(colbits, 0, sizeof(uint64_t) * d.n, s);
-    if (e != cudaSuccess) return e;
+    if (d.k <= 0 || d.k > kColRowsPerBlock) {
+      const cudaError_t e = cudaMemsetAsync(colbits, 0, sizeof(uint64_t) * d.n, s);
+      if (e != cudaSuccess) return e;
+    }
     if (d.k > 0) {
       dim3 grid(static_cast<unsigned>((d.n + 31) / 32),
                 static_cast<unsigned>((d.k + kColRowsPerBlock - 1) / kColRowsPerBlock));

@@ -128,3 +128,29 @@ def test_smaller_caller_workspace_takes_the_products_one_by_one():
     finally:
         torch.cuda.synchronize()
         mxm.mxm_set_workspace(None)
+
+
+@pytest.mark.parametrize("m,k,n", [(1, 1, 1), (64, 64, 64), (128, 128, 128), (129, 128, 128),
+                                   (128, 127, 129), (4096, 64, 64), (100, 30, 4096),
+                                   (4097, 64, 64)])
+@pytest.mark.parametrize("mode,S", [(mxm.MODE_EMUL_I8, 3), (mxm.MODE_EMUL_I8, 7),
+                                    (mxm.MODE_EMUL_BF16, 8), (mxm.MODE_EMUL_RN8, 6)])
+def test_one_block_of_one_tile_row_or_column(mode, S, m, k, n):
+    """Up to 16 tiles the library's own workspace takes the difference products,
+    a caller's of the size it was told takes the digit products one by one, as
+    does a single-CTA plan: the same bits."""
+    A, B = inputs.gemm_operands("spread", m, k, n, seed=5, cfg=71)
+    a, b = torch.from_numpy(A).cuda(), torch.from_numpy(B).cuda()
+    outs = [torch.full((m, n), float("nan"), dtype=torch.float64, device="cuda")
+            for _ in range(3)]
+    mxm.mxm_gemm(mode, a, b, outs[0], slices=S)
+    mxm.mxm_gemm_plan(mode, a, b, outs[1], slices=S, plan=mxm.Plan(cta=1))
+    ws = torch.empty(mxm.mxm_workspace_size(mode, m, k, n, S), dtype=torch.uint8, device="cuda")
+    mxm.mxm_set_workspace(ws)
+    try:
+        mxm.mxm_gemm(mode, a, b, outs[2], slices=S)
+        torch.cuda.synchronize()
+    finally:
+        mxm.mxm_set_workspace(None)
+    assert mxm.mxm_get_device_status() == mxm.MXM_OK
+    assert torch.equal(outs[0], outs[1]) and torch.equal(outs[0], outs[2])
