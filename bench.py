@@ -75,7 +75,7 @@ def profiled_traffic():
     summary, if the kernel sources still hash as they did at capture."""
     import hashlib
     import re
-    summary = os.path.join(ROOT, "profiles", "oz_gemm2_n8192_dram.md")
+    summary = os.path.join(ROOT, "profiles", "oz_kara_n8192_dram.md")
     if not os.path.exists(summary):
         return None
     text = open(summary).read()
@@ -84,7 +84,7 @@ def profiled_traffic():
     if not mt or not mh:
         return None
     h = hashlib.sha256()
-    for rel in ("csrc/ozaki.cu", "csrc/ptx.cuh", "csrc/mxm_internal.h"):
+    for rel in ("csrc/ozaki_kara.cu", "csrc/ptx.cuh", "csrc/mxm_internal.h"):
         with open(os.path.join(ROOT, "paper_1211_1581_gb300", rel), "rb") as fh:
             h.update(fh.read())
     return int(mt.group(1)) if h.hexdigest() == mh.group(1) else None

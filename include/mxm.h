@@ -392,8 +392,9 @@ int64_t mxm_cg_max_n(void);
 /*
  * mxm_fft -- the forward 1-D complex DFT of mod2f (Sec. 3.3, Eq. 1):
  * out(k) = sum_{j<n} in(j) exp(-2 pi i k j / n), 0 <= k < n, computed by
- * radix-2 decimation in frequency (Eqs. 2-3) in shared memory, in one pass
- * (n <= 1024) or two passes through `work` (the four-step factorisation).
+ * the stages of Eqs. 2-3 two at a time (radix 4), decimated in time, in shared
+ * memory, in one launch (n <= 8192) or two passes through `work` (the
+ * four-step factorisation).
  * Arguments (device memory; complex FP64 interleaved re, im; 16-byte
  * aligned):
  *   in      n complex values (read);
