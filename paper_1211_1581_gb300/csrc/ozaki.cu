@@ -1525,16 +1525,15 @@ __global__ void __launch_bounds__(128 + 32 * kEpiW, 1)
         }
         if (!ok) break;
         if (!kFloat && j.partial != nullptr) {
-          // split-k: this range's exact D_g, column-major in the tile (a
-          // warp's 32 lanes store 256 contiguous bytes per column)
+          // split-k: this range's exact D_g, as int32 or int64, column-major in
+          // the tile (a warp's 32 lanes store whole lines)
           if (!rows_live) continue;
-          uint64_t* p = j.partial + static_cast<size_t>(g - 2) * (kOzTileRows * kOzTileRows) +
-                        static_cast<size_t>(cg * kCPW) * kOzTileRows + row_in_tile;
+          Acc* p = reinterpret_cast<Acc*>(j.partial) +
+                   static_cast<size_t>(g - 2) * (kOzTileRows * kOzTileRows) +
+                   static_cast<size_t>(cg * kCPW) * kOzTileRows + row_in_tile;
 #pragma unroll
           for (int i = 0; i < kCPW; ++i)
-            if (cg * kCPW + i < ncols)
-              __stcg(reinterpret_cast<unsigned long long*>(p + i * kOzTileRows),
-                     static_cast<unsigned long long>(static_cast<long long>(D[i])));
+            if (cg * kCPW + i < ncols) __stcg(p + i * kOzTileRows, D[i]);
           continue;
         }
         if (!rows_live) continue;
@@ -2440,8 +2439,9 @@ static cudaError_t launch_oz_gemm_t(const Tiles& tiles, int64_t grid, int S, int
 // (consecutive threads: consecutive rows, i.e. contiguous partials in the
 // column-major tiles); kRows threads share an element's ranges and one of them
 // folds: eight from 32 ranges on (128 ranges of 128 x 128, S = 6: 23 us, one
-// thread for all ranges 110 us), one below (4096 x 128, 9 ranges).
-template <int kRows>
+// thread for all ranges 110 us), one below (4096 x 128, 9 ranges).  Part: the
+// type of the partials.
+template <int kRows, typename Part>
 __global__ void __launch_bounds__(256) oz_splitk_fold_kernel(
     const uint64_t* P, const uint64_t* __restrict__ rowbits,
     const uint64_t* __restrict__ colbits, double* __restrict__ C, int64_t m, int64_t n,
@@ -2456,14 +2456,16 @@ __global__ void __launch_bounds__(256) oz_splitk_fold_kernel(
   const int64_t col = live ? idx / m : 0, row = live ? idx - col * m : 0;
   constexpr int64_t kTileWords = kOzTileRows * kOzTileRows;
   const int64_t tile = (row / kOzTileRows) * Nt + col / kOzTileRows;
-  const uint64_t* p = P + tile * S * kTileWords + (col % kOzTileRows) * kOzTileRows +
-                      row % kOzTileRows;
-  const int64_t range_stride = Mt * Nt * S * kTileWords;
+  // a tile's room is that of int64 partials
+  constexpr int64_t kPer = sizeof(uint64_t) / sizeof(Part);
+  const Part* p = reinterpret_cast<const Part*>(P + tile * S * kTileWords) +
+                  (col % kOzTileRows) * kOzTileRows + row % kOzTileRows;
+  const int64_t range_stride = Mt * Nt * S * kTileWords * kPer;
   auto sum = [&](int g) {
     long long d = 0;
 #pragma unroll 8
     for (int64_t sp = ty; sp < splits; sp += kRows)
-      d += static_cast<long long>(__ldcs(p + sp * range_stride + (g - 2) * kTileWords));
+      d += __ldcs(p + sp * range_stride + (g - 2) * kTileWords);
     return d;
   };
   if constexpr (kRows > 1) {
@@ -2560,8 +2562,17 @@ cudaError_t launch_ozaki_gemm(const uint8_t* aslices, const uint8_t* bslices,
   }
   if (splits > 1) {
     // one diagonal at a time, each k range's D_g to the partials, then the fold
-    cudaError_t e =
-        launch_oz_gemm_t<long long, false>(tiles, grid, d.S, d.beta, window, status, s, d.chain);
+    // (int32 sums, stores half as wide and 16 epilogue warps where every
+    // range's D_g fits: 128 x 65536 x 128, S = 6, 227 -> 210 us, 128 x 9000 x 2000
+    // 343 -> 310)
+    OzakiDims range = d;
+    range.Kt = (d.Kt + splits - 1) / splits;
+    const bool narrow = ozaki_narrow(range);
+    const cudaError_t e =
+        narrow ? launch_oz_gemm_t<int, false, OzSingle, 16>(tiles, grid, d.S, d.beta, window,
+                                                            status, s, d.chain)
+               : launch_oz_gemm_t<long long, false>(tiles, grid, d.S, d.beta, window, status, s,
+                                                    d.chain);
     if (e != cudaSuccess) return e;
     const int64_t total = d.m * d.n;
     auto fold = [&](auto kern, int64_t per_block) {
@@ -2570,7 +2581,11 @@ cudaError_t launch_ozaki_gemm(const uint8_t* aslices, const uint8_t* bslices,
                             0, s, sums, rowbits, colbits, C, d.m, d.n, d.Mt, d.Nt, splits, d.S,
                             d.beta, ozaki_exact_from(d.S, d.beta, d.Kt), d.rn ? 2 : 0);
     };
-    return splits >= 32 ? fold(oz_splitk_fold_kernel<8>, 32) : fold(oz_splitk_fold_kernel<1>, 256);
+    if (narrow)
+      return splits >= 32 ? fold(oz_splitk_fold_kernel<8, int>, 32)
+                          : fold(oz_splitk_fold_kernel<1, int>, 256);
+    return splits >= 32 ? fold(oz_splitk_fold_kernel<8, long long>, 32)
+                        : fold(oz_splitk_fold_kernel<1, long long>, 256);
   }
   // the paired kernel; when a diagonal's sum over all of k may pass int32,
   // with the spill area that follows the running sums (grid capped to it)
