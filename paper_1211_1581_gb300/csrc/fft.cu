@@ -25,7 +25,8 @@
 // integers (a negation is an FP64 instruction: 39.5 + 33.5 a point before, 36 +
 // 32 now).  Measured: 2^20 points 186 -> 158 us (the FP64 pipe alone 113 us, the
 // rest the loads and stores at the ends of the passes and the barriers between
-// stages), 2^10 11.2 -> 8.7 us, 2^22 727 -> 665 us.  Butterflies of fused multiply-adds (a + w b in
+// stages; 6 us less since the second pass is launched beside the first), 2^10 11.2
+// -> 8.7 us, 2^22 727 -> 665 us.  Butterflies of fused multiply-adds (a + w b in
 // four, a - w b = 2 a - (a + w b) in two: 24 per radix 4) ran 2^20 points in
 // 134 us, but with a tenth more error, and are not used.
 #include <cuda_runtime.h>
