@@ -35,6 +35,7 @@
 
 #include <cstdint>
 
+#include "cg_rows.h"
 #include "mxm.h"
 #include "mxm_internal.h"
 
@@ -209,10 +210,10 @@ __device__ __forceinline__ double cg_product(const CgGridArgs& a, int64_t lo, in
       }
       if (sub == 0) prow = __ldcg(p + row);
     }
-    int j = b + sub;
+    RowWalk w = row_walk(b, e, sub);
     double t = 0.0;
     // the most values any lane of the warp has left (the warp runs together)
-    int m = __reduce_max_sync(0xFFFFFFFFu, j < e ? (e - j + G - 1) / G : 0);
+    int m = __reduce_max_sync(0xFFFFFFFFu, w.count(G));
     for (; m > 0; m -= kBatch) {
       double v[kBatch], pv[kBatch];
       int c[kBatch];
@@ -220,9 +221,9 @@ __device__ __forceinline__ double cg_product(const CgGridArgs& a, int64_t lo, in
       for (int u = 0; u < kBatch; ++u) {
         c[u] = -1;
         v[u] = 0.0;
-        if (j + u * G < e) {
-          c[u] = __ldg(a.indx + j + u * G);
-          v[u] = __ldg(a.vals + j + u * G);
+        if (w.has(u * G)) {
+          c[u] = __ldg(a.indx + w.at + u * G);
+          v[u] = __ldg(a.vals + w.at + u * G);
           bad |= c[u] < 0 || c[u] >= n;
         }
       }
@@ -235,7 +236,7 @@ __device__ __forceinline__ double cg_product(const CgGridArgs& a, int64_t lo, in
 #pragma unroll
       for (int u = 0; u < kBatch; ++u)
         if (u < m) t = fma(v[u], pv[u], t);  // uniform
-      j = j + kBatch * G;
+      w.advance(kBatch * G);
     }
 #pragma unroll
     for (int o = G / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
