@@ -350,26 +350,40 @@ int cg_grid_group(int64_t n, int64_t nnz) {
   return g;
 }
 
+// The most dynamic shared memory of a block and the most blocks at once are asked
+// of the device once, and the limit raised once: solves of different orders from
+// two threads would lower it under each other between a call and its launch.
 template <int G>
 mxm_status launch_grid(CgGridArgs a, cudaStream_t s) {
-  int dev = 0, optin = 0, sms = 0, per_sm = 0;
-  cudaFuncAttributes fa;
-  if (cudaGetDevice(&dev) != cudaSuccess ||
-      cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev) !=
-          cudaSuccess ||
-      cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev) != cudaSuccess ||
-      cudaFuncGetAttributes(&fa, cg_grid_kernel<G>) != cudaSuccess)
+  static PerDevice limit, held;
+  int most = 0, blocks = 0;
+  const cudaError_t e = limit.get(&most, [](int* v) {
+    int dev = 0, optin = 0;
+    cudaFuncAttributes fa;
+    cudaError_t q = cudaGetDevice(&dev);
+    if (q == cudaSuccess)
+      q = cudaDeviceGetAttribute(&optin, cudaDevAttrMaxSharedMemoryPerBlockOptin, dev);
+    if (q == cudaSuccess) q = cudaFuncGetAttributes(&fa, cg_grid_kernel<G>);
+    if (q != cudaSuccess) return q;
+    *v = optin - static_cast<int>(fa.sharedSizeBytes);
+    return cudaFuncSetAttribute(cg_grid_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize, *v);
+  });
+  if (e != cudaSuccess) return MXM_ERR_CUDA;
+  if (held.get(&blocks, [&](int* v) {  // a block fills an SM's registers, whatever its memory
+        int dev = 0, sms = 0, per_sm = 0;
+        cudaError_t q = cudaGetDevice(&dev);
+        if (q == cudaSuccess) q = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+        if (q == cudaSuccess)
+          q = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cg_grid_kernel<G>, kCgGThreads,
+                                                            static_cast<size_t>(most));
+        *v = sms * per_sm;
+        return q;
+      }) != cudaSuccess)
     return MXM_ERR_CUDA;
   a.rows_cap = (a.n + kCgBlocks - 1) / kCgBlocks;
   size_t smem = 3 * static_cast<size_t>(a.rows_cap) * sizeof(double);
-  a.in_smem = smem + fa.sharedSizeBytes <= static_cast<size_t>(optin) ? 1 : 0;
+  a.in_smem = smem <= static_cast<size_t>(most) ? 1 : 0;
   if (!a.in_smem) smem = 0;
-  if (cudaFuncSetAttribute(cg_grid_kernel<G>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           static_cast<int>(smem)) != cudaSuccess ||
-      cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, cg_grid_kernel<G>, kCgGThreads,
-                                                    smem) != cudaSuccess)
-    return MXM_ERR_CUDA;
-  int blocks = sms * per_sm;
   if (blocks > kCgBlocks) blocks = kCgBlocks;
   if (blocks < 1) return MXM_ERR_CUDA;
   if (cudaMemsetAsync(a.w.st, 0, sizeof(CgState), s) != cudaSuccess) return MXM_ERR_CUDA;
