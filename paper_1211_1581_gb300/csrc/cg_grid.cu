@@ -17,17 +17,21 @@
 // the latency of one gather).
 //
 // Rows are shared out by number: block b of kCgBlocks owns rows
-// [b n / kCgBlocks, (b + 1) n / kCgBlocks), its q, r and x live in shared
-// memory when they fit (n up to ~1.4 million), p, gathered by everybody, in
-// global memory.  The product is bound by the FP64 pipe on this GPU (a
-// warp-wide fused multiply-add holds an SM sub-partition 64 clocks, however
-// many lanes are live) and by latency, so a row is given as few lanes as keep
-// every thread on rows (one lane a row from 156,000 rows on: no shuffle tree,
-// all 32 lanes live; the lanes' strided loads of values and columns meet in
-// L1), and a lane has eight values, columns and gathers in flight.
+// [b n / kCgBlocks, (b + 1) n / kCgBlocks).  Where that gives a block more than
+// twice the mean of the values, the rows are cut by work instead (cg_rows.h),
+// once per solve: of 200,000 rows the first 1316 of 658 values, the rest of 3,
+// 466 -> 101 us a step.  A block's q, r and x live in shared memory when they
+// fit (n up to ~1.4 million; a block that the cut by work gives more rows than
+// the mean keeps them in global memory), p, gathered by everybody, in global
+// memory.  The product is bound by the FP64 pipe on this GPU (a warp-wide fused
+// multiply-add holds an SM sub-partition 64 clocks, however many lanes are live)
+// and by latency, so a row is given as few lanes as keep every thread on rows
+// (one lane a row from 156,000 rows on: no shuffle tree, all 32 lanes live; the
+// lanes' strided loads of values and columns meet in L1), and a lane has eight
+// values, columns and gathers in flight.
 //
-// The number of blocks and the lanes per row depend on n and nnz only, and
-// every sum has a fixed order: the rounding of a solve does not depend on the
+// The shares depend on the row pointers, the lanes per row on n and nnz only,
+// and every sum has a fixed order: the rounding of a solve does not depend on the
 // device (a device with room for fewer blocks gives each several).  Every
 // wait at a barrier is bounded: after kWaitLimitNs it raises the abort word,
 // records MXM_ERR_TIMEOUT and every block leaves.
@@ -45,8 +49,8 @@ namespace {
 
 constexpr int kCgGThreads = 1024;
 constexpr int kCgGWarps = kCgGThreads / 32;
-constexpr int kCgBlocks = 152;        // row shares (one per SM of a GB300), as a constant
 constexpr int64_t kCgGMaxShares = 1216;  // doubles per share table in the workspace
+static_assert(3 * kCgBlocks <= kCgGMaxShares, "a share table, then the shares' rows");
 constexpr int kBatch = 8;             // values, columns and gathers of a lane in flight
 
 struct CgState {
@@ -86,8 +90,8 @@ struct CgGridArgs {
   double* x;
   CgWork w;
   int64_t n, nnz;
-  int64_t rows_cap;   // most rows of a share
-  int in_smem;        // q, r and x of the shares in shared memory
+  int64_t rows_cap;   // most rows of a share by number
+  int in_smem;        // q, r and x of a share of that many rows in shared memory
   double stop;
   int32_t max_iters;
   int32_t* iters;
@@ -248,25 +252,28 @@ __device__ __forceinline__ double cg_product(const CgGridArgs& a, int64_t lo, in
   return pq;
 }
 
-template <int G>
-__global__ void __launch_bounds__(kCgGThreads, 1) cg_grid_kernel(const CgGridArgs a) {
-  extern __shared__ double dsm[];
-  __shared__ double red[kCgGThreads + 6];
-  __shared__ int flag;
+// A solve.  kByWork: the shares' rows as this block has left them in `span`;
+// compiled apart, since the way to them costs 1.5 us a step (and the rows by
+// number are a product and a division).
+template <int G, bool kByWork>
+__device__ __forceinline__ void cg_solve(const CgGridArgs& a, double* dsm, double* red, int& flag,
+                                         const int64_t* span) {
   const int tid = threadIdx.x;
   const bool many = gridDim.x < kCgBlocks;  // several shares a block: their vectors in memory
-  const bool smem = a.in_smem && !many;
   CgState* const st = a.w.st;
   unsigned long long target = 0;
   bool bad = false;
-  auto lo_of = [&](int s) { return a.n * s / kCgBlocks; };
+  auto lo_of = [&](int s) { return kByWork ? __ldcg(span + 2 * s) : share_by_rows(a.n, s); };
+  auto hi_of = [&](int s) { return kByWork ? __ldcg(span + 2 * s + 1) : share_by_rows(a.n, s + 1); };
+  const bool smem = a.in_smem && !many &&
+                    (!kByWork || hi_of(blockIdx.x) - lo_of(blockIdx.x) <= a.rows_cap);
   auto q_of = [&](int64_t lo) { return smem ? dsm : a.w.q + lo; };
   auto r_of = [&](int64_t lo) { return smem ? dsm + a.rows_cap : a.w.r + lo; };
   auto x_of = [&](int64_t lo) { return smem ? dsm + 2 * a.rows_cap : a.x + lo; };
 
   // x0 = 0, r0 = p0 = b, shares of (b, b)
   for (int s = blockIdx.x; s < kCgBlocks; s += gridDim.x) {
-    const int64_t lo = lo_of(s), hi = lo_of(s + 1);
+    const int64_t lo = lo_of(s), hi = hi_of(s);
     double* const r = r_of(lo);
     double* const x = x_of(lo);
     double bb = 0.0;
@@ -287,7 +294,7 @@ __global__ void __launch_bounds__(kCgGThreads, 1) cg_grid_kernel(const CgGridArg
   bool brk = false;
   while (ok && r2 > a.stop && k < a.max_iters) {
     for (int s = blockIdx.x; s < kCgBlocks; s += gridDim.x) {
-      const int64_t lo = lo_of(s), hi = lo_of(s + 1);
+      const int64_t lo = lo_of(s), hi = hi_of(s);
       const double pq = block_total(cg_product<G>(a, lo, hi, q_of(lo), bad), red);
       if (tid == 0) a.w.part_pq[s] = pq;
     }
@@ -299,7 +306,7 @@ __global__ void __launch_bounds__(kCgGThreads, 1) cg_grid_kernel(const CgGridArg
       break;
     }
     for (int s = blockIdx.x; s < kCgBlocks; s += gridDim.x) {
-      const int64_t lo = lo_of(s), own = lo_of(s + 1) - lo;
+      const int64_t lo = lo_of(s), own = hi_of(s) - lo;
       const double* const q = q_of(lo);
       double* const r = r_of(lo);
       double rr = 0.0;
@@ -315,7 +322,7 @@ __global__ void __launch_bounds__(kCgGThreads, 1) cg_grid_kernel(const CgGridArg
     shares_total(a.w.part_rr, red, r2, false, r2n, beta);
     r2 = r2n;
     for (int s = blockIdx.x; s < kCgBlocks; s += gridDim.x) {
-      const int64_t lo = lo_of(s), own = lo_of(s + 1) - lo;
+      const int64_t lo = lo_of(s), own = hi_of(s) - lo;
       const double* const r = r_of(lo);
       double* const x = x_of(lo);
 #pragma unroll 4
@@ -330,7 +337,7 @@ __global__ void __launch_bounds__(kCgGThreads, 1) cg_grid_kernel(const CgGridArg
     if (!(ok = grid_barrier(st, target, &flag, a.status))) break;
   }
   if (smem) {  // each thread's own elements
-    const int64_t lo = lo_of(blockIdx.x), own = lo_of(blockIdx.x + 1) - lo;
+    const int64_t lo = lo_of(blockIdx.x), own = hi_of(blockIdx.x) - lo;
     for (int64_t i = tid; i < own; i += kCgGThreads) a.x[lo + i] = x_of(lo)[i];
   }
   if (blockIdx.x == 0 && tid == 0) {
@@ -339,6 +346,30 @@ __global__ void __launch_bounds__(kCgGThreads, 1) cg_grid_kernel(const CgGridArg
     if (brk) atomicOr(a.status, kStatusBreakdown);
   }
   if (bad) atomicOr(a.status, kStatusBounds);
+}
+
+template <int G>
+__global__ void __launch_bounds__(kCgGThreads, 1) cg_grid_kernel(const CgGridArgs a) {
+  extern __shared__ double dsm[];
+  __shared__ double red[kCgGThreads + 6];
+  __shared__ int flag;
+  const int tid = threadIdx.x;
+  // the shares' rows: by number, or (the same choice in every block) by work,
+  // each block then looking up its own and keeping them behind the share table
+  bool too_long = false;
+  if (tid < kCgBlocks) {
+    const int64_t first = __ldg(a.rowp + share_by_rows(a.n, tid));
+    too_long = share_too_long(__ldg(a.rowp + share_by_rows(a.n, tid + 1)) - first, a.nnz);
+  }
+  if (__syncthreads_or(too_long)) {
+    int64_t* const span = reinterpret_cast<int64_t*>(a.w.part_pq + kCgBlocks);
+    for (int s = blockIdx.x; s < kCgBlocks; s += gridDim.x)
+      if (tid < 2) span[2 * s + tid] = share_by_work(a.rowp, a.n, a.nnz, s + tid);
+    __syncthreads();
+    cg_solve<G, true>(a, dsm, red, flag, span);
+  } else {
+    cg_solve<G, false>(a, dsm, red, flag, nullptr);
+  }
 }
 
 // Lanes per row: the fewest that give every thread of a share a row.

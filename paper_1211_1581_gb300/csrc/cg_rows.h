@@ -27,4 +27,40 @@ __host__ __device__ inline RowWalk row_walk(int32_t begin, int32_t end, int32_t 
   return RowWalk{static_cast<int64_t>(begin) + sub, end};
 }
 
+// Rows are shared out over kCgBlocks blocks (one per SM of a 152-SM GPU, a
+// constant: the rounding of a solve does not depend on the device): share s
+// takes rows [begin of s, begin of s + 1).
+//
+// By number where the values come out even.
+constexpr int kCgBlocks = 152;
+__host__ __device__ inline int64_t share_by_rows(int64_t n, int s) { return n * s / kCgBlocks; }
+
+// Whether a share by number holds so many values that the shares are taken by
+// work instead: more than twice the mean, and kShareSlack (four values a thread)
+// beyond that, so that the chance differences of short shares do not count.
+constexpr int64_t kShareSlack = 4096;
+__host__ __device__ inline bool share_too_long(int64_t values, int64_t nnz) {
+  return values > 2 * (nnz / kCgBlocks) + kShareSlack;
+}
+
+// By work: the row pointer plus kRowWork a row (its own part of the three dot
+// products and vector updates of a step, five multiply-adds) grows from 0 to the
+// whole work; the share begins at the first row at or past s parts of it.  Row
+// pointers that are not in order give some other cut; the cuts still never
+// decrease with s (each step of the search goes right for every larger s).
+constexpr int64_t kRowWork = 5;
+__host__ __device__ inline int64_t share_by_work(const int32_t* rowp, int64_t n, int64_t nnz,
+                                                 int s) {
+  if (s <= 0) return 0;
+  if (s >= kCgBlocks) return n;
+  const int64_t want = (nnz + kRowWork * n) * s / kCgBlocks;  // < 2^42 before the division
+  int64_t lo = 0, hi = n;
+  while (lo < hi) {
+    const int64_t mid = (lo + hi) >> 1;
+    if (rowp[mid] + kRowWork * mid < want) lo = mid + 1;
+    else hi = mid;
+  }
+  return lo;
+}
+
 }  // namespace mxm

@@ -75,3 +75,70 @@ void check() {
   CHECK(w.count(32) == (INT_MAX - 32) / 32 + 1 && w.count(1) == INT_MAX - 31);
 }
 """)
+
+
+def test_shares_of_uneven_rows(tmp_path):
+    """The cut by work covers every row once and gives no share more than its
+    part of the work and one row; it is taken where neighbouring rows hold most
+    of the values and not for rows of one length, or of chance lengths.  Row
+    pointers out of order still give cuts that never decrease."""
+    run(tmp_path, r"""
+static std::vector<int> pointers(const std::vector<int>& len) {
+  std::vector<int> p(1, 0);
+  for (int l : len) p.push_back(p.back() + l);
+  return p;
+}
+static bool by_work(const std::vector<int>& p) {
+  const long long n = static_cast<long long>(p.size()) - 1;
+  for (int s = 0; s < kCgBlocks; ++s)
+    if (share_too_long(p[share_by_rows(n, s + 1)] - p[share_by_rows(n, s)], p[n])) return true;
+  return false;
+}
+void check() {
+  unsigned long long seed = 1;
+  auto rnd = [&](int m) { return static_cast<int>((seed = seed * 6364136223846793005ull + 1442695040888963407ull) >> 33) % m; };
+  std::vector<std::vector<int>> uneven, even;
+  std::vector<int> l(200000, 3);
+  for (int i = 0; i < 1316; ++i) l[i] = 658;
+  uneven.push_back(l);
+  l.assign(160001, 2); l[80000] = 160001;
+  uneven.push_back(l);
+  l.assign(5000, 2); l[4999] = 5000;
+  uneven.push_back(l);
+  l.assign(100, 0); l[7] = 3000000;
+  uneven.push_back(l);
+  l.assign(1, 1000000);
+  uneven.push_back(l);
+  for (int n : {1, 100, 151, 152, 153, 12288, 200000}) {
+    l.assign(n, 7);
+    even.push_back(l);
+    for (int& v : l) v = rnd(33);
+    even.push_back(l);
+    l.assign(n, 0);
+    even.push_back(l);
+  }
+  for (const auto& len : uneven) CHECK(by_work(pointers(len)));
+  for (const auto& len : even) CHECK(!by_work(pointers(len)));
+  uneven.insert(uneven.end(), even.begin(), even.end());
+  for (const auto& len : uneven) {
+    const std::vector<int> p = pointers(len);
+    const long long n = static_cast<long long>(len.size()), nnz = p[n];
+    const long long part = (nnz + kRowWork * n) / kCgBlocks + 1;
+    CHECK(share_by_work(p.data(), n, nnz, 0) == 0 && share_by_work(p.data(), n, nnz, kCgBlocks) == n);
+    for (int s = 0; s < kCgBlocks; ++s) {
+      const long long lo = share_by_work(p.data(), n, nnz, s), hi = share_by_work(p.data(), n, nnz, s + 1);
+      CHECK(lo <= hi && hi <= n);
+      CHECK(lo == hi || (p[hi - 1] + kRowWork * (hi - 1)) - (p[lo] + kRowWork * lo) <= part);
+    }
+  }
+  for (int r = 0; r < 200; ++r) {  // anything at all in the row pointers
+    const int n = 1 + rnd(3000);
+    std::vector<int> p(n + 1);
+    for (int& v : p) v = (rnd(2) ? 1 : -1) * rnd(INT_MAX);
+    for (int s = 0; s < kCgBlocks; ++s) {
+      const long long lo = share_by_work(p.data(), n, 100000, s), hi = share_by_work(p.data(), n, 100000, s + 1);
+      CHECK(0 <= lo && lo <= hi && hi <= n);
+    }
+  }
+}
+""")
