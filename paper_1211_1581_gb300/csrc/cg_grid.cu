@@ -28,7 +28,11 @@
 // and by latency, so a row is given as few lanes as keep every thread on rows
 // (one lane a row from 156,000 rows on: no shuffle tree, all 32 lanes live; the
 // lanes' strided loads of values and columns meet in L1), and a lane has eight
-// values, columns and gathers in flight.
+// values, columns and gathers in flight.  Rows that are long beside the mean
+// are taken by a whole warp, very long ones by the block (row_limit,
+// block_limit): with those 1316 rows of 658 values 101 -> 29 us a step, a
+// diagonal matrix of 160,001 rows bordered by one full row and column 16.5 ms ->
+// 73 us, of 10^6 rows 103 ms -> 0.30 ms.
 //
 // The shares depend on the row pointers, the lanes per row on n and nnz only,
 // and every sum has a fixed order: the rounding of a solve does not depend on the
@@ -90,6 +94,7 @@ struct CgGridArgs {
   double* x;
   CgWork w;
   int64_t n, nnz;
+  int32_t row_limit, block_limit;  // longest row of the lanes, of a warp (cg_rows.h)
   int64_t rows_cap;   // most rows of a share by number
   int in_smem;        // q, r and x of a share of that many rows in shared memory
   double stop;
@@ -189,9 +194,105 @@ __device__ bool grid_barrier(CgState* st, unsigned long long& target, int* flag,
   return *flag != 0;
 }
 
+// The pointers of a row (none: past the end, or the pointers are not in order);
+// returns its length.
+__device__ __forceinline__ int row_pointers(const CgGridArgs& a, int64_t row, int64_t hi, int& b,
+                                            int& e) {
+  b = e = 0;
+  if (row < hi) {
+    b = __ldg(a.rowp + row);
+    e = __ldg(a.rowp + row + 1);
+    if (b < 0 || e < b || e > a.nnz) b = e = 0;
+  }
+  return e - b;
+}
+
+// Thread `sub` of T's part of a row's sum.
+template <int T>
+__device__ __forceinline__ double cg_long_row(const CgGridArgs& a, int b, int e, int sub, bool& bad) {
+  const double* const p = a.w.p;
+  const int n = static_cast<int>(a.n);
+  double t = 0.0;
+  for (RowWalk w = row_walk(b, e, sub); w.has(0); w.advance(kBatch * T)) {
+    double v[kBatch], pv[kBatch];
+    int c[kBatch];
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) {
+      c[u] = -1;
+      v[u] = 0.0;
+      if (w.has(u * T)) {
+        c[u] = __ldg(a.indx + w.at + u * T);
+        v[u] = __ldg(a.vals + w.at + u * T);
+        bad |= c[u] < 0 || c[u] >= n;
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) {
+      pv[u] = 0.0;
+      if (c[u] >= 0 && c[u] < n) pv[u] = __ldcg(p + c[u]);
+      else v[u] = 0.0;
+    }
+#pragma unroll
+    for (int u = 0; u < kBatch; ++u) t = fma(v[u], pv[u], t);
+  }
+  return t;
+}
+
+// The rows of [lo, hi) that cg_product has left out: neighbours to different
+// warps, then (huge) those for the whole block one after another.  Returns
+// this thread's part of (p, q).  Out of line: its registers are its own.
+struct LongRows {
+  double pq;
+  bool bad;
+};
+__device__ __noinline__ LongRows cg_long_rows(const CgGridArgs& a, int64_t lo, int64_t hi,
+                                              double* qs, bool huge, double* red) {
+  const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+  const double* const p = a.w.p;
+  double pq = 0.0;
+  bool bad = false;
+  int b, e;
+  for (int64_t base = lo; base < hi; base += kCgGThreads) {
+    const int len = row_pointers(a, base + lane * kCgGWarps + warp, hi, b, e);
+    for (uint32_t todo = __ballot_sync(0xFFFFFFFFu, len > a.row_limit && len <= a.block_limit);
+         todo != 0; todo &= todo - 1) {
+      const int src = __ffs(todo) - 1;
+      double t = cg_long_row<32>(a, __shfl_sync(0xFFFFFFFFu, b, src),
+                                 __shfl_sync(0xFFFFFFFFu, e, src), lane, bad);
+#pragma unroll
+      for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
+      if (lane == 0) {
+        const int64_t row = base + src * kCgGWarps + warp;
+        qs[row - lo] = t;
+        pq = fma(__ldcg(p + row), t, pq);
+      }
+    }
+  }
+  if (!huge) return LongRows{pq, bad};  // block-uniform
+  for (int64_t base = lo; base < hi; base += kCgGThreads) {
+    if (!__syncthreads_or(row_pointers(a, base + tid, hi, b, e) > a.block_limit)) continue;
+    for (int64_t base32 = base; base32 < base + kCgGThreads; base32 += 32) {  // all warps alike
+      const int len = row_pointers(a, base32 + lane, hi, b, e);
+      for (uint32_t todo = __ballot_sync(0xFFFFFFFFu, len > a.block_limit); todo != 0;
+           todo &= todo - 1) {
+        const int src = __ffs(todo) - 1;
+        const double t =
+            block_total(cg_long_row<kCgGThreads>(a, __shfl_sync(0xFFFFFFFFu, b, src),
+                                                 __shfl_sync(0xFFFFFFFFu, e, src), tid, bad), red);
+        if (tid == 0) {
+          qs[base32 + src - lo] = t;
+          pq = fma(__ldcg(p + base32 + src), t, pq);
+        }
+      }
+    }
+  }
+  return LongRows{pq, bad};
+}
+
 // q = A p on rows [lo, hi) (qs[row - lo]); returns this thread's part of
-// (p, q).  G lanes a row; a warp takes 32 / G rows at a time.
-template <int G>
+// (p, q).  G lanes a row; a warp takes 32 / G rows at a time.  kUneven: rows
+// longer than row_limit are left out.
+template <int G, bool kUneven>
 __device__ __forceinline__ double cg_product(const CgGridArgs& a, int64_t lo, int64_t hi,
                                              double* qs, bool& bad) {
   constexpr int R = 32 / G;
@@ -205,11 +306,16 @@ __device__ __forceinline__ double cg_product(const CgGridArgs& a, int64_t lo, in
     const int64_t row = base + grp;
     int b = 0, e = 0;
     double prow = 0.0;
-    if (row < hi) {
+    bool own = row < hi;
+    if (own) {
       b = __ldg(a.rowp + row);
       e = __ldg(a.rowp + row + 1);
       if (b < 0 || e < b || e > a.nnz) {
         bad = true;
+        b = e = 0;
+      }
+      if (kUneven && e - b > a.row_limit) {
+        own = false;
         b = e = 0;
       }
       if (sub == 0) prow = __ldcg(p + row);
@@ -244,7 +350,7 @@ __device__ __forceinline__ double cg_product(const CgGridArgs& a, int64_t lo, in
     }
 #pragma unroll
     for (int o = G / 2; o > 0; o >>= 1) t += __shfl_xor_sync(0xFFFFFFFFu, t, o);
-    if (row < hi && sub == 0) {
+    if (own && sub == 0) {
       qs[row - lo] = t;
       pq = fma(prow, t, pq);
     }
@@ -252,21 +358,21 @@ __device__ __forceinline__ double cg_product(const CgGridArgs& a, int64_t lo, in
   return pq;
 }
 
-// A solve.  kByWork: the shares' rows as this block has left them in `span`;
-// compiled apart, since the way to them costs 1.5 us a step (and the rows by
-// number are a product and a division).
-template <int G, bool kByWork>
+// A solve.  kUneven: the shares' rows as this block has left them in `span`, rows
+// beyond row_limit (longest: the block's longest row) done apart; compiled apart,
+// since this costs 1.5 us a step.  Both meet at the same barriers.
+template <int G, bool kUneven>
 __device__ __forceinline__ void cg_solve(const CgGridArgs& a, double* dsm, double* red, int& flag,
-                                         const int64_t* span) {
+                                         const int64_t* span, bool any_long, bool any_huge) {
   const int tid = threadIdx.x;
   const bool many = gridDim.x < kCgBlocks;  // several shares a block: their vectors in memory
   CgState* const st = a.w.st;
   unsigned long long target = 0;
   bool bad = false;
-  auto lo_of = [&](int s) { return kByWork ? __ldcg(span + 2 * s) : share_by_rows(a.n, s); };
-  auto hi_of = [&](int s) { return kByWork ? __ldcg(span + 2 * s + 1) : share_by_rows(a.n, s + 1); };
+  auto lo_of = [&](int s) { return kUneven ? __ldcg(span + 2 * s) : share_by_rows(a.n, s); };
+  auto hi_of = [&](int s) { return kUneven ? __ldcg(span + 2 * s + 1) : share_by_rows(a.n, s + 1); };
   const bool smem = a.in_smem && !many &&
-                    (!kByWork || hi_of(blockIdx.x) - lo_of(blockIdx.x) <= a.rows_cap);
+                    (!kUneven || hi_of(blockIdx.x) - lo_of(blockIdx.x) <= a.rows_cap);
   auto q_of = [&](int64_t lo) { return smem ? dsm : a.w.q + lo; };
   auto r_of = [&](int64_t lo) { return smem ? dsm + a.rows_cap : a.w.r + lo; };
   auto x_of = [&](int64_t lo) { return smem ? dsm + 2 * a.rows_cap : a.x + lo; };
@@ -295,7 +401,13 @@ __device__ __forceinline__ void cg_solve(const CgGridArgs& a, double* dsm, doubl
   while (ok && r2 > a.stop && k < a.max_iters) {
     for (int s = blockIdx.x; s < kCgBlocks; s += gridDim.x) {
       const int64_t lo = lo_of(s), hi = hi_of(s);
-      const double pq = block_total(cg_product<G>(a, lo, hi, q_of(lo), bad), red);
+      double pq = cg_product<G, kUneven>(a, lo, hi, q_of(lo), bad);
+      if (kUneven && any_long) {
+        const LongRows rest = cg_long_rows(a, lo, hi, q_of(lo), any_huge, red);
+        pq += rest.pq;
+        bad |= rest.bad;
+      }
+      pq = block_total(pq, red);
       if (tid == 0) a.w.part_pq[s] = pq;
     }
     if (!(ok = grid_barrier(st, target, &flag, a.status))) break;
@@ -354,22 +466,40 @@ __global__ void __launch_bounds__(kCgGThreads, 1) cg_grid_kernel(const CgGridArg
   __shared__ double red[kCgGThreads + 6];
   __shared__ int flag;
   const int tid = threadIdx.x;
-  // the shares' rows: by number, or (the same choice in every block) by work,
-  // each block then looking up its own and keeping them behind the share table
+  // The shares' rows: by number, or (the same choice in every block) by work,
+  // each block then looking its own up and keeping them behind the share table.
+  int64_t* const span = reinterpret_cast<int64_t*>(a.w.part_pq + kCgBlocks);
   bool too_long = false;
   if (tid < kCgBlocks) {
     const int64_t first = __ldg(a.rowp + share_by_rows(a.n, tid));
     too_long = share_too_long(__ldg(a.rowp + share_by_rows(a.n, tid + 1)) - first, a.nnz);
   }
-  if (__syncthreads_or(too_long)) {
-    int64_t* const span = reinterpret_cast<int64_t*>(a.w.part_pq + kCgBlocks);
-    for (int s = blockIdx.x; s < kCgBlocks; s += gridDim.x)
+  const bool by_work = __syncthreads_or(too_long) != 0;
+  int longest = 0;  // of the block's rows, by this thread
+  for (int s = blockIdx.x; s < kCgBlocks; s += gridDim.x) {
+    int64_t lo = share_by_rows(a.n, s), hi = share_by_rows(a.n, s + 1);
+    if (by_work) {
       if (tid < 2) span[2 * s + tid] = share_by_work(a.rowp, a.n, a.nnz, s + tid);
-    __syncthreads();
-    cg_solve<G, true>(a, dsm, red, flag, span);
-  } else {
-    cg_solve<G, false>(a, dsm, red, flag, nullptr);
+      __syncthreads();
+      lo = __ldcg(span + 2 * s);
+      hi = __ldcg(span + 2 * s + 1);
+    }
+    for (int64_t i = lo + tid; i < hi; i += kCgGThreads) {
+      int b, e;
+      longest = max(longest, row_pointers(a, i, hi, b, e));
+    }
   }
+  const bool any_long = __syncthreads_or(longest > a.row_limit) != 0;
+  if (!by_work && !any_long) {
+    cg_solve<G, false>(a, dsm, red, flag, nullptr, false, false);
+    return;
+  }
+  if (!by_work)
+    for (int s = blockIdx.x; s < kCgBlocks; s += gridDim.x)
+      if (tid < 2) span[2 * s + tid] = share_by_rows(a.n, s + tid);
+  // (a barrier of the block: the span is read after it)
+  const bool any_huge = __syncthreads_or(longest > a.block_limit) != 0;
+  cg_solve<G, true>(a, dsm, red, flag, span, any_long, any_huge);
 }
 
 // Lanes per row: the fewest that give every thread of a share a row.
@@ -411,6 +541,8 @@ mxm_status launch_grid(CgGridArgs a, cudaStream_t s) {
         return q;
       }) != cudaSuccess)
     return MXM_ERR_CUDA;
+  a.row_limit = row_limit(a.n, a.nnz, G);
+  a.block_limit = block_limit(a.row_limit);
   a.rows_cap = (a.n + kCgBlocks - 1) / kCgBlocks;
   size_t smem = 3 * static_cast<size_t>(a.rows_cap) * sizeof(double);
   a.in_smem = smem <= static_cast<size_t>(most) ? 1 : 0;
@@ -446,6 +578,7 @@ mxm_status cg_grid_solve(const double* vals, const int32_t* indx, const int32_t*
   a.w = cg_work(work, n);
   a.n = n;
   a.nnz = nnz;
+  a.row_limit = a.block_limit = 0;
   a.rows_cap = 0;
   a.in_smem = 0;
   a.stop = stop;

@@ -63,4 +63,18 @@ __host__ __device__ inline int64_t share_by_work(const int32_t* rowp, int64_t n,
   return lo;
 }
 
+// Rows longer than row_limit are not left to the G lanes that a row has by the
+// mean length: a warp takes each, and above block_limit a whole block.  Four
+// times the mean is no longer even; 256 values a lane take 32 rounds of eight
+// loads, some 40 us, about a whole step.  A warp goes through block_limit values
+// in 64 rounds.
+__host__ __device__ inline int32_t row_limit(int64_t n, int64_t nnz, int G) {
+  const int64_t four = 4 * ((nnz + n - 1) / n), most = four > 256 * G ? four : 256 * G;
+  return static_cast<int32_t>(most < INT32_MAX ? most : INT32_MAX);
+}
+__host__ __device__ inline int32_t block_limit(int32_t row_limit) {
+  const int64_t most = row_limit > 2048 ? 8 * static_cast<int64_t>(row_limit) : 16384;
+  return static_cast<int32_t>(most < INT32_MAX ? most : INT32_MAX);
+}
+
 }  // namespace mxm

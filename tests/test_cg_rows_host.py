@@ -142,3 +142,22 @@ void check() {
   }
 }
 """)
+
+
+def test_limits_of_long_rows(tmp_path):
+    """Rows up to four times the mean, and up to 256 values a lane, stay with
+    their lanes; the limits do not overflow at the largest counts."""
+    run(tmp_path, r"""
+void check() {
+  for (long long n : {1ll, 152ll, 5000ll, 160001ll, 1000000ll, 2147483647ll})
+    for (long long nnz : {0ll, 1ll, 3 * n, 40 * n, 2147483647ll})
+      for (int G = 1; G <= 32; G *= 2) {
+        if (nnz > 2147483647ll) continue;
+        const long long r = row_limit(n, nnz, G), b = block_limit(static_cast<int>(r));
+        CHECK(r >= 256 * G && (r == INT_MAX || r >= 4 * (nnz / n)));
+        CHECK(b >= 16384 && (b == INT_MAX || b >= 8 * r) && b >= r);
+      }
+  CHECK(row_limit(160001, 480001, 1) == 256 && block_limit(256) == 16384);
+  CHECK(row_limit(1000, 2147483647, 32) == 4 * 2147484);
+}
+""")
