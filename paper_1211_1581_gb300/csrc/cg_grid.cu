@@ -42,6 +42,7 @@
 #include <cuda_runtime.h>
 
 #include <cstdint>
+#include <type_traits>
 
 #include "cg_rows.h"
 #include "mxm.h"
@@ -213,7 +214,7 @@ __device__ __forceinline__ double cg_long_row(const CgGridArgs& a, int b, int e,
   const double* const p = a.w.p;
   const int n = static_cast<int>(a.n);
   double t = 0.0;
-  for (RowWalk w = row_walk(b, e, sub); w.has(0); w.advance(kBatch * T)) {
+  for (auto w = row_walk<int64_t>(b, e, sub); w.has(0); w.advance(kBatch * T)) {
     double v[kBatch], pv[kBatch];
     int c[kBatch];
 #pragma unroll
@@ -291,7 +292,7 @@ __device__ __noinline__ LongRows cg_long_rows(const CgGridArgs& a, int64_t lo, i
 
 // q = A p on rows [lo, hi) (qs[row - lo]); returns this thread's part of
 // (p, q).  G lanes a row; a warp takes 32 / G rows at a time.  kUneven: rows
-// longer than row_limit are left out.
+// longer than row_limit are left out; any number of values, else kNarrowValues.
 template <int G, bool kUneven>
 __device__ __forceinline__ double cg_product(const CgGridArgs& a, int64_t lo, int64_t hi,
                                              double* qs, bool& bad) {
@@ -320,7 +321,7 @@ __device__ __forceinline__ double cg_product(const CgGridArgs& a, int64_t lo, in
       }
       if (sub == 0) prow = __ldcg(p + row);
     }
-    RowWalk w = row_walk(b, e, sub);
+    auto w = row_walk<std::conditional_t<kUneven, int64_t, int32_t>>(b, e, sub);
     double t = 0.0;
     // the most values any lane of the warp has left (the warp runs together)
     int m = __reduce_max_sync(0xFFFFFFFFu, w.count(G));
@@ -359,8 +360,8 @@ __device__ __forceinline__ double cg_product(const CgGridArgs& a, int64_t lo, in
 }
 
 // A solve.  kUneven: the shares' rows as this block has left them in `span`, rows
-// beyond row_limit (longest: the block's longest row) done apart; compiled apart,
-// since this costs 1.5 us a step.  Both meet at the same barriers.
+// beyond row_limit done apart, positions in 64 bits; compiled apart, since the
+// way to the rows alone costs 1.5 us a step.  Both meet at the same barriers.
 template <int G, bool kUneven>
 __device__ __forceinline__ void cg_solve(const CgGridArgs& a, double* dsm, double* red, int& flag,
                                          const int64_t* span, bool any_long, bool any_huge) {
@@ -461,7 +462,7 @@ __device__ __forceinline__ void cg_solve(const CgGridArgs& a, double* dsm, doubl
 }
 
 template <int G>
-__global__ void __launch_bounds__(kCgGThreads, 1) cg_grid_kernel(const CgGridArgs a) {
+__global__ void __launch_bounds__(kCgGThreads, 1) cg_grid_kernel(const __grid_constant__ CgGridArgs a) {
   extern __shared__ double dsm[];
   __shared__ double red[kCgGThreads + 6];
   __shared__ int flag;
@@ -490,7 +491,7 @@ __global__ void __launch_bounds__(kCgGThreads, 1) cg_grid_kernel(const CgGridArg
     }
   }
   const bool any_long = __syncthreads_or(longest > a.row_limit) != 0;
-  if (!by_work && !any_long) {
+  if (!by_work && !any_long && a.nnz <= kNarrowValues) {
     cg_solve<G, false>(a, dsm, red, flag, nullptr, false, false);
     return;
   }

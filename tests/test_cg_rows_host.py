@@ -46,15 +46,16 @@ def test_rows_at_the_largest_count_of_values(tmp_path):
     rows that end at or near INT32_MAX and however long the lane goes on
     beside a longer row of its warp."""
     run(tmp_path, r"""
-void check() {
-  const int kBatch = 8, ends[] = {INT_MAX, INT_MAX - 1, INT_MAX - 100, INT_MAX - 224, 70000, 100};
+const int kBatch = 8;
+template <typename Pos>
+static void walks(const std::vector<int>& ends) {
   for (int end : ends)
     for (int G = 1; G <= 32; G *= 2)
       for (int len : {0, 1, 7, 31, 32, 33, 100}) {
         const int begin = end - len;
         std::vector<int> seen(len, 0);
         for (int sub = 0; sub < G; ++sub) {
-          RowWalk w = row_walk(begin, end, sub);
+          auto w = row_walk<Pos>(begin, end, sub);
           int own = 0;
           for (int m = w.count(G) + 40 * kBatch; m > 0; m -= kBatch) {  // a longer row beside it
             for (int u = 0; u < kBatch; ++u)
@@ -70,9 +71,22 @@ void check() {
         }
         for (int v : seen) CHECK(v == 1);
       }
-  // one row of all the values
-  RowWalk w = row_walk(0, INT_MAX, 31);
+}
+void check() {
+  walks<int64_t>({INT_MAX, INT_MAX - 1, INT_MAX - 100, INT_MAX - 224, 70000, 100});
+  walks<int32_t>({kNarrowValues, kNarrowValues - 1, 70000, 100});
+  // one row of all the values, and a lane of the last row beside it to its end
+  auto w = row_walk<int64_t>(0, INT_MAX, 31);
   CHECK(w.count(32) == (INT_MAX - 32) / 32 + 1 && w.count(1) == INT_MAX - 31);
+  for (int G = 1; G <= 32; G *= 2) {
+    auto one = row_walk<int32_t>(0, kNarrowValues, 0);
+    auto last = row_walk<int32_t>(kNarrowValues - 1, kNarrowValues, G - 1);
+    for (int m = one.count(G); m > 0; m -= kBatch) {
+      const bool mine = last.has(0) && last.at == kNarrowValues - 1;
+      for (int u = 0; u < kBatch; ++u) CHECK(last.has(u * G) == (mine && u == 0));
+      last.advance(kBatch * G);
+    }
+  }
 }
 """)
 
