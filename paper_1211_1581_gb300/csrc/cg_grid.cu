@@ -37,7 +37,7 @@
 // The shares depend on the row pointers, the lanes per row on n and nnz only,
 // and every sum has a fixed order: the rounding of a solve does not depend on the
 // device (a device with room for fewer blocks gives each several).  Every
-// wait at a barrier is bounded: after kWaitLimitNs it raises the abort word,
+// wait at a barrier is bounded: after cg_wait_limit_ns it raises the abort word,
 // records MXM_ERR_TIMEOUT and every block leaves.
 #include <cuda_runtime.h>
 
@@ -99,6 +99,7 @@ struct CgGridArgs {
   int64_t rows_cap;   // most rows of a share by number
   int in_smem;        // q, r and x of a share of that many rows in shared memory
   double stop;
+  uint64_t wait_ns;
   int32_t max_iters;
   int32_t* iters;
   double* r2;
@@ -162,7 +163,8 @@ __device__ __forceinline__ uint64_t timer_ns() {
 
 // All blocks; what each wrote before is visible to all after.  false: a wait
 // gave up (here or in another block).
-__device__ bool grid_barrier(CgState* st, unsigned long long& target, int* flag, int* status) {
+__device__ bool grid_barrier(CgState* st, unsigned long long& target, int* flag, uint64_t limit_ns,
+                             int* status) {
   target += gridDim.x;
   __syncthreads();
   if (threadIdx.x == 0) {
@@ -181,7 +183,7 @@ __device__ bool grid_barrier(CgState* st, unsigned long long& target, int* flag,
           ok = 0;
           break;
         }
-        if (timer_ns() - t0 > kWaitLimitNs) {
+        if (timer_ns() - t0 > limit_ns) {
           atomicExch(&st->abort, 1);
           atomicOr(status, kStatusTimeout);
           ok = 0;
@@ -394,7 +396,7 @@ __device__ __forceinline__ void cg_solve(const CgGridArgs& a, double* dsm, doubl
     bb = block_total(bb, red);
     if (tid == 0) a.w.part_rr[s] = bb;
   }
-  bool ok = grid_barrier(st, target, &flag, a.status);
+  bool ok = grid_barrier(st, target, &flag, a.wait_ns, a.status);
   double r2 = 0.0, unused;
   if (ok) shares_total(a.w.part_rr, red, 1.0, false, r2, unused);
   int32_t k = 0;
@@ -411,7 +413,7 @@ __device__ __forceinline__ void cg_solve(const CgGridArgs& a, double* dsm, doubl
       pq = block_total(pq, red);
       if (tid == 0) a.w.part_pq[s] = pq;
     }
-    if (!(ok = grid_barrier(st, target, &flag, a.status))) break;
+    if (!(ok = grid_barrier(st, target, &flag, a.wait_ns, a.status))) break;
     double pAp, alpha, r2n, beta;
     shares_total(a.w.part_pq, red, r2, true, pAp, alpha);
     if (!(pAp > 0.0)) {  // the same in every block: the same shares, the same order
@@ -431,7 +433,7 @@ __device__ __forceinline__ void cg_solve(const CgGridArgs& a, double* dsm, doubl
       rr = block_total(rr, red);
       if (tid == 0) a.w.part_rr[s] = rr;
     }
-    if (!(ok = grid_barrier(st, target, &flag, a.status))) break;
+    if (!(ok = grid_barrier(st, target, &flag, a.wait_ns, a.status))) break;
     shares_total(a.w.part_rr, red, r2, false, r2n, beta);
     r2 = r2n;
     for (int s = blockIdx.x; s < kCgBlocks; s += gridDim.x) {
@@ -447,7 +449,7 @@ __device__ __forceinline__ void cg_solve(const CgGridArgs& a, double* dsm, doubl
     }
     if (blockIdx.x == 0 && tid == 0 && a.r2_hist != nullptr) a.r2_hist[k] = r2;
     ++k;
-    if (!(ok = grid_barrier(st, target, &flag, a.status))) break;
+    if (!(ok = grid_barrier(st, target, &flag, a.wait_ns, a.status))) break;
   }
   if (smem) {  // each thread's own elements
     const int64_t lo = lo_of(blockIdx.x), own = hi_of(blockIdx.x) - lo;
@@ -583,6 +585,7 @@ mxm_status cg_grid_solve(const double* vals, const int32_t* indx, const int32_t*
   a.rows_cap = 0;
   a.in_smem = 0;
   a.stop = stop;
+  a.wait_ns = cg_wait_limit_ns(nnz);
   a.max_iters = max_iters;
   a.iters = iters;
   a.r2 = r2;

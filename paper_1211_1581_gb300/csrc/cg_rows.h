@@ -6,6 +6,8 @@
 
 #include <cuda_runtime.h>
 
+#include "mxm_internal.h"
+
 namespace mxm {
 
 // A lane's way through the values [begin, end) of a row, 0 <= begin <= end <=
@@ -80,6 +82,15 @@ __host__ __device__ inline int32_t row_limit(int64_t n, int64_t nnz, int G) {
 __host__ __device__ inline int32_t block_limit(int32_t row_limit) {
   const int64_t most = row_limit > 2048 ? 8 * static_cast<int64_t>(row_limit) : 16384;
   return static_cast<int32_t>(most < INT32_MAX ? most : INT32_MAX);
+}
+
+// How long a block waits for the others at a barrier.  The wait is for their
+// work, most of all for a block that holds one row of nearly all the values: 0.3
+// ns a value by a whole block, 0.8 by lanes that each have few rows.  So the limit
+// grows with the number of values, five times what they may take (2^31 values:
+// 10.6 s).
+__host__ __device__ inline uint64_t cg_wait_limit_ns(int64_t nnz) {
+  return kWaitLimitNs + 4 * static_cast<uint64_t>(nnz);
 }
 
 }  // namespace mxm

@@ -175,3 +175,15 @@ void check() {
   CHECK(row_limit(1000, 2147483647, 32) == 4 * 2147484);
 }
 """)
+
+
+def test_wait_limit_grows_with_the_values(tmp_path):
+    """A block may hold a row of all the values: the wait for it allows ns for
+    each beyond the usual limit, and stays bounded."""
+    run(tmp_path, r"""
+void check() {
+  CHECK(cg_wait_limit_ns(0) == kWaitLimitNs);
+  for (long long nnz : {1000ll, 60000000ll, 2147483647ll})
+    CHECK(cg_wait_limit_ns(nnz) >= kWaitLimitNs + 4 * nnz && cg_wait_limit_ns(nnz) < 20000000000ull);
+}
+""")

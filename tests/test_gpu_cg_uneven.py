@@ -140,3 +140,28 @@ def test_wrong_pointers_and_columns():
     bad = indx.copy()
     bad[rowp[100] + 200] = n
     run_cg(rowp, bad, vals, b, 0.0, 3, expect=mxm.MXM_ERR_INVALID_ARG, engine=mxm.CG_GRAPH)
+
+
+def test_one_row_of_twenty_million_values():
+    """One block's product of such a row is not taken for a block that is lost:
+    the step ends without MXM_ERR_TIMEOUT and its iterate is alpha b."""
+    n = 20_000_000
+    w = 0.1 / n
+    rowp = torch.cat((torch.zeros(1, dtype=torch.int64),
+                      n + 2 * torch.arange(n, dtype=torch.int64))).to(torch.int32).cuda()
+    indx = torch.empty(3 * n - 2, dtype=torch.int32, device="cuda")
+    vals = torch.empty(3 * n - 2, dtype=torch.float64, device="cuda")
+    indx[:n] = torch.arange(n, dtype=torch.int32, device="cuda")
+    vals[:n] = w
+    vals[0] = 4.0
+    indx[n::2] = 0
+    indx[n + 1::2] = torch.arange(1, n, dtype=torch.int32, device="cuda")
+    vals[n::2] = w
+    vals[n + 1::2] = 2.0
+    b = torch.ones(n, dtype=torch.float64, device="cuda")
+    x = torch.empty_like(b)
+    it, _ = mxm.mxm_cg(vals, indx, rowp, b, x, 0.0, 1, engine=mxm.CG_GRAPH)
+    assert mxm.mxm_get_device_status() == mxm.MXM_OK and int(it) == 1
+    # b = 1: (b, b) = n, (b, A b) = 4 + 2 (n - 1) + 2 w (n - 1)
+    alpha = n / (4 + 2 * (n - 1) + 2 * w * (n - 1))
+    assert float((x - alpha).abs().max()) <= 4 * n * U * alpha
