@@ -214,8 +214,10 @@ size_t mxm_workspace_size(int mode, int64_t m, int64_t k, int64_t n, int slices)
  * library then never allocates for mxm_f64 / mxm_f64_emul / mxm_gemm, which
  * makes them safe to capture in a CUDA graph.  d_ws == NULL returns to the
  * library-owned workspace (grown with cudaMalloc on demand, outside
- * capture).  The paper has no counterpart (its calls take arrays the caller
- * owns and nothing else); this is the library's memory contract.
+ * capture; a size beyond what a call cannot do without that the device had no
+ * memory for is not asked for again until this function is called).  The paper
+ * has no counterpart (its calls take arrays the caller owns and nothing else);
+ * this is the library's memory contract.
  *   stream  the stream the caller's next calls run on: the switch waits for
  *           the work already queued there (which may still use the previous
  *           workspace), and frees a library-owned previous workspace after

@@ -11,6 +11,7 @@
 #include "mxm.h"
 #include "mxm_internal.h"
 #include "ptx.cuh"
+#include "workspace.h"
 
 namespace mxm {
 
@@ -24,9 +25,7 @@ constexpr int kMaxDevices = 64;
 struct DeviceState {
   bool init = false;
   int* status = nullptr;       // device address of g_device_status
-  void* ws = nullptr;          // workspace base
-  size_t ws_bytes = 0;
-  bool ws_owned = true;        // allocated by the library
+  Workspace ws;
   int sm_count = 0;
   cudaStream_t h2d = nullptr;  // streams of the pipelined host path: copies in,
   cudaStream_t d2h = nullptr;  // copies out, and a second compute stream
@@ -90,30 +89,32 @@ bool stream_capturing(cudaStream_t s) {
   return cs != cudaStreamCaptureStatusNone;
 }
 
-// Make sure the current device's workspace holds `need` bytes.
-mxm_status ensure_workspace(DeviceState* st, size_t need, cudaStream_t s) {
-  if (need <= st->ws_bytes) return MXM_OK;
-  if (!st->ws_owned) return MXM_ERR_WORKSPACE_TOO_SMALL;
-  if (stream_capturing(s)) return MXM_ERR_NO_WORKSPACE;
-  if (st->ws) {
-    if (cudaDeviceSynchronize() != cudaSuccess) return cuda_fail();
-    cudaFree(st->ws);
-    st->ws = nullptr;
-    st->ws_bytes = 0;
-  }
-  size_t grow = need + need / 8;
-  grow = align_up(grow, size_t(2) << 20);
-  if (cudaMalloc(&st->ws, grow) != cudaSuccess) {
+struct CudaAllocator {
+  cudaStream_t s;
+  bool capturing() const { return stream_capturing(s); }
+  bool synchronize() const { return cudaDeviceSynchronize() == cudaSuccess; }
+  bool allocate(void** p, size_t bytes) const {
+    if (cudaMalloc(p, bytes) == cudaSuccess) return true;
     cudaGetLastError();
-    if (cudaMalloc(&st->ws, need) != cudaSuccess) {
-      cudaGetLastError();
-      st->ws = nullptr;
-      return cuda_fail();
-    }
-    grow = need;
+    *p = nullptr;
+    return false;
   }
-  st->ws_bytes = grow;
-  return MXM_OK;
+  void release(void* p) const { cudaFree(p); }
+  bool available(size_t* bytes) const {
+    size_t total = 0;
+    return cudaMemGetInfo(bytes, &total) == cudaSuccess;
+  }
+};
+
+// The workspace of a call: `most` bytes where they can be had (*all), else the
+// `least` that it runs with.
+mxm_status call_workspace(DeviceState* ds, size_t most, size_t least, cudaStream_t s, bool* all) {
+  CudaAllocator a{s};
+  *all = true;
+  if (most <= least) return workspace_need(ds->ws, most, a);
+  if (workspace_want(ds->ws, most, least, a)) return MXM_OK;
+  *all = false;
+  return workspace_need(ds->ws, least, a);
 }
 
 bool overlaps(const void* a, size_t abytes, const void* b, size_t bbytes) {
@@ -363,12 +364,10 @@ mxm_status mxm_gemm_plan(int mode, const double* A, const double* B, double* C, 
   // had, else (a caller workspace sized for less, a capture, no memory) the
   // products one by one, with the same bits (native: fewer workers)
   bool most = true;
-  if (ensure_workspace(ds, workspace_bytes(mode, m, k, n, slices, p), s) != MXM_OK) {
-    most = false;
-    st = ensure_workspace(ds, workspace_bytes(mode, m, k, n, slices, p, false), s);
-    if (st != MXM_OK) return st;
-  }
-  return run_gemm(mode, A, B, C, m, k, n, slices, static_cast<uint8_t*>(ds->ws), ds->ws_bytes,
+  st = call_workspace(ds, workspace_bytes(mode, m, k, n, slices, p),
+                      workspace_bytes(mode, m, k, n, slices, p, false), s, &most);
+  if (st != MXM_OK) return st;
+  return run_gemm(mode, A, B, C, m, k, n, slices, static_cast<uint8_t*>(ds->ws.base), ds->ws.bytes,
                   ds->status, s, p, most);
 }
 
@@ -429,26 +428,36 @@ static int64_t host_panel_cols(int64_t h, int64_t n, int sms) {
 
 static mxm_status gemm_host_panels(DeviceState* ds, int mode, const double* hA, const double* hB,
                                    double* hC, int64_t m, int64_t k, int64_t n, int slices,
-                                   int64_t h, cudaStream_t s, bool kara) {
+                                   int64_t h, cudaStream_t s) {
   const int beta = mode_beta(mode);
   const bool rn = mode_rn(mode);
   const int64_t w = host_panel_cols(h, n, ds->sm_count);
   const int64_t P = (m + h - 1) / h, Q = (n + w - 1) / w;
-  OzakiDims dp = ozaki_dims(h, k, w, slices, beta, rn);  // the largest block, no split-k
-  dp.kara = kara && kara_chosen(dp) ? (kara_short(dp) ? 2 : 1) : 0;
-  const OzakiLayout L = ozaki_layout(dp);
-  // per compute stream: row scales, A planes, running sums of one block
-  const size_t rb_bytes = align_up(sizeof(uint64_t) * size_t(h), 1024);
-  const size_t ap_bytes = L.bslices - L.aslices;
-  const size_t sm_bytes = L.total - L.sums;
-  const size_t per_buf = rb_bytes + ap_bytes + sm_bytes;
-  // per column panel: column scales and B planes
-  const size_t per_col = (L.aslices - L.colbits) + (L.sums - L.bslices);
   const size_t ab = align_up(sizeof(double) * size_t(m) * size_t(k), 1024);
   const size_t bb = align_up(sizeof(double) * size_t(k) * size_t(n), 1024);
   const size_t cb = align_up(sizeof(double) * size_t(m) * size_t(n), 1024);
-  mxm_status st = ensure_workspace(ds, ab + bb + cb + size_t(Q) * per_col + 2 * per_buf, s);
+  OzakiDims dp = ozaki_dims(h, k, w, slices, beta, rn);  // the largest block, no split-k
+  OzakiLayout L;
+  size_t rb_bytes = 0, ap_bytes = 0, per_buf = 0, per_col = 0;
+  const auto lay_out = [&](bool kara) -> size_t {
+    dp.kara = kara && kara_chosen(dp) ? (kara_short(dp) ? 2 : 1) : 0;
+    L = ozaki_layout(dp);
+    // per compute stream: row scales, A planes, running sums of one block
+    rb_bytes = align_up(sizeof(uint64_t) * size_t(h), 1024);
+    ap_bytes = L.bslices - L.aslices;
+    per_buf = rb_bytes + ap_bytes + (L.total - L.sums);
+    // per column panel: column scales and B planes
+    per_col = (L.aslices - L.colbits) + (L.sums - L.bslices);
+    return ab + bb + cb + size_t(Q) * per_col + 2 * per_buf;
+  };
+  // as mxm_gemm: without the difference products where their workspace cannot
+  // be had
+  bool kara = true;
+  const size_t least = lay_out(false);
+  mxm_status st = call_workspace(ds, lay_out(true), least, s, &kara);
   if (st != MXM_OK) return st;
+  if (!kara && stream_capturing(s)) return MXM_ERR_NO_WORKSPACE;  // the path synchronises
+  lay_out(kara);
   if (ds->h2d == nullptr && cudaStreamCreateWithFlags(&ds->h2d, cudaStreamNonBlocking) != cudaSuccess)
     return cuda_fail();
   if (ds->d2h == nullptr && cudaStreamCreateWithFlags(&ds->d2h, cudaStreamNonBlocking) != cudaSuccess)
@@ -457,7 +466,7 @@ static mxm_status gemm_host_panels(DeviceState* ds, int mode, const double* hA, 
     return cuda_fail();
   if (ds->c2 == nullptr && cudaStreamCreateWithFlags(&ds->c2, cudaStreamNonBlocking) != cudaSuccess)
     return cuda_fail();
-  uint8_t* base = static_cast<uint8_t*>(ds->ws);
+  uint8_t* base = static_cast<uint8_t*>(ds->ws.base);
   double* dA = reinterpret_cast<double*>(base);
   double* dB = reinterpret_cast<double*>(base + ab);  // column panel j at dB + j w k (k x wj)
   double* dC = reinterpret_cast<double*>(base + ab + bb);  // block (i, j) at dC + (i n + j w h)
@@ -593,26 +602,17 @@ mxm_status mxm_gemm_host(int mode, const double* hA, const double* hB, double* h
   if ((st = current_state(&ds)) != MXM_OK) return st;
   if (emul_mode(mode) && k > 0) {
     const int64_t h = host_panel_rows(m, n, ds->sm_count);
-    if (h > 0) {
-      // as mxm_gemm: without the difference products where their workspace
-      // cannot be had
-      st = gemm_host_panels(ds, mode, hA, hB, hC, m, k, n, slices, h, s, true);
-      if (st == MXM_ERR_WORKSPACE_TOO_SMALL || (st == MXM_ERR_CUDA && ds->ws == nullptr))
-        st = gemm_host_panels(ds, mode, hA, hB, hC, m, k, n, slices, h, s, false);
-      return st;
-    }
+    if (h > 0) return gemm_host_panels(ds, mode, hA, hB, hC, m, k, n, slices, h, s);
   }
   const size_t ab = align_up(sizeof(double) * size_t(m) * size_t(k), 1024);
   const size_t bb = align_up(sizeof(double) * size_t(k) * size_t(n), 1024);
   const size_t cb = align_up(sizeof(double) * size_t(m) * size_t(n), 1024);
   bool most = true;
-  if (ensure_workspace(ds, ab + bb + cb + workspace_bytes(mode, m, k, n, slices), s) != MXM_OK) {
-    most = false;
-    st = ensure_workspace(ds, ab + bb + cb + workspace_bytes(mode, m, k, n, slices, kNoPlan, false),
-                          s);
-    if (st != MXM_OK) return st;
-  }
-  uint8_t* base = static_cast<uint8_t*>(ds->ws);
+  st = call_workspace(ds, ab + bb + cb + workspace_bytes(mode, m, k, n, slices),
+                      ab + bb + cb + workspace_bytes(mode, m, k, n, slices, kNoPlan, false), s,
+                      &most);
+  if (st != MXM_OK) return st;
+  uint8_t* base = static_cast<uint8_t*>(ds->ws.base);
   double* dA = reinterpret_cast<double*>(base);
   double* dB = reinterpret_cast<double*>(base + ab);
   double* dC = reinterpret_cast<double*>(base + ab + bb);
@@ -624,7 +624,7 @@ mxm_status mxm_gemm_host(int mode, const double* hA, const double* hB, double* h
       return cuda_fail();
   }
   st = run_gemm(mode, dA, dB, dC, m, k, n, slices, base + ab + bb + cb,
-                ds->ws_bytes - (ab + bb + cb), ds->status, s, kNoPlan, most);
+                ds->ws.bytes - (ab + bb + cb), ds->status, s, kNoPlan, most);
   if (st != MXM_OK) return st;
   if (cudaMemcpyAsync(hC, dC, sizeof(double) * size_t(m) * size_t(n), cudaMemcpyDeviceToHost, s) !=
       cudaSuccess)
@@ -644,18 +644,15 @@ mxm_status mxm_set_workspace(void* d_ws, size_t bytes, void* stream) {
   if (stream_capturing(s)) return MXM_ERR_UNSUPPORTED;
   // work already queued on `stream` may still use the previous workspace
   if (cudaStreamSynchronize(s) != cudaSuccess) return cuda_fail();
-  if (ds->ws_owned && ds->ws) {
+  if (ds->ws.owned && ds->ws.base != nullptr) {
     if (cudaDeviceSynchronize() != cudaSuccess) return cuda_fail();
-    cudaFree(ds->ws);
+    cudaFree(ds->ws.base);
   }
-  if (d_ws == nullptr) {
-    ds->ws = nullptr;
-    ds->ws_bytes = 0;
-    ds->ws_owned = true;
-  } else {
-    ds->ws = d_ws;
-    ds->ws_bytes = bytes;
-    ds->ws_owned = false;
+  ds->ws = Workspace();
+  if (d_ws != nullptr) {
+    ds->ws.base = d_ws;
+    ds->ws.bytes = bytes;
+    ds->ws.owned = false;
   }
   return MXM_OK;
 }
