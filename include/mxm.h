@@ -86,8 +86,8 @@ const char* mxm_status_string(mxm_status s);
  * with any correct FP64 evaluation within |C - AB|_ij <= 2 k u (|A||B|)_ij,
  * u = 2^-53, and are bit-exact whenever every partial sum is exact (e.g.
  * small-integer matrices).  Uses library workspace (partial sums of the
- * pieces of C that two of the GPU's equal shares of the work meet in,
- * mxm_workspace_size(MXM_MODE_F64, ...) bytes).
+ * pieces of C that two of the GPU's equal shares of the work meet in, 20 MB at
+ * most).
  */
 mxm_status mxm_f64(const double* A, const double* B, double* C, int64_t m, int64_t k,
                    int64_t n, void* stream);
@@ -195,13 +195,15 @@ mxm_status mxm_gemm_host(int mode, const double* hA, const double* hB, double* h
 /*
  * mxm_workspace_size -- bytes of device workspace one mxm_gemm call of mode
  * `mode` on an m x k by k x n product (Sec. 3.1 shapes) with `slices` slices
- * needs (the FP64 path: partial sums of 32 x 32 pieces of C, and never less
- * than the tile copies of A and B an earlier form held; the emulated modes: row and column scales, the digit planes of
+ * needs (the FP64 path: partial sums of 32 x 32 pieces of C, 20 MB at most, and
+ * where it is larger the size of the tile copies of A and B that an earlier form
+ * held; the emulated modes: row and column scales, the digit planes of
  * the Ozaki split and of the difference products, the segment sums, running
  * sums or split-k partials).  An emulated call on a smaller caller workspace
  * runs without the difference products (same bits) as long as it holds
- * mxm_workspace_size_plan of a plan with cta = 1; a native call on a smaller
- * one cuts the work into fewer shares.  Host arithmetic
+ * mxm_workspace_size_plan of a plan with cta = 1; a native call needs no more
+ * than those 20 MB (nothing for k < 32), and on a smaller workspace that holds
+ * the tile copies cuts the work into fewer shares.  Host arithmetic
  * only, no device call.  Returns 0 for an empty product (m, n or k <= 0),
  * an unknown mode or a slice count the mode does not take.  The paper has no
  * counterpart; size a buffer for mxm_set_workspace with it.

@@ -223,8 +223,11 @@ size_t workspace_bytes(int mode, int64_t m, int64_t k, int64_t n, int slices,
 // The size that a caller is told: the most, but for one k-block of one tile-row
 // or tile-column, where the segment slots are many times the planes (256 x 128
 // x 128, S = 7: 6.7 MB instead of 0.9), the least; a workspace with more room,
-// the library's own among them, is still used.
+// the library's own among them, is still used.  Native products:
+// f64_workspace_told.
 size_t workspace_told(int mode, int64_t m, int64_t k, int64_t n, int slices, const mxm_plan& p) {
+  if (mode == MXM_MODE_F64)
+    return m > 0 && k > 0 && n > 0 ? f64_workspace_told(native_dims(m, k, n, p)) : 0;
   const bool thin = emul_mode(mode) &&
                     kara_one_block(ozaki_dims(m, k, n, slices, mode_beta(mode), mode_rn(mode)));
   return workspace_bytes(mode, m, k, n, slices, p, !thin);

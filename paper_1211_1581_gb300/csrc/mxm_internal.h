@@ -453,19 +453,28 @@ inline int64_t f64_workers(const F64Dims& d) {
   return steps < 1 ? 1 : (steps < 1216 ? steps : 1216);
 }
 
-// Workspace of a native product: the workers' slots, and never less than
-// before, when it held zero-padded 128 x 16 tile copies of A and B and the
-// partial tiles of the k ranges (a size callers may have kept).
-inline size_t f64_workspace_least(const F64Dims& d) {
+// Workspace of a native product: the workers' slots, 20 MB at most, and what the
+// library allocates for it.
+inline size_t f64_workspace(const F64Dims& d) {
+  return d.ranges == 1 ? 0 : (size_t)(f64_workers(d) + 1) * kF64WorkerBytes;
+}
+// The size that an earlier form of the product needed, zero-padded 128 x 16 tile
+// copies of A and B and the partial tiles of the k ranges: buffers of it are
+// kept by callers.  A product runs in the smaller of the two, and callers are
+// told the larger.
+inline size_t f64_workspace_kept(const F64Dims& d) {
   const size_t packs = align_up((size_t)(d.Mt + d.Nt) * d.Kt * kF64TileBytes, 1024);
   const size_t partials =
       d.splits > 1 ? (size_t)d.splits * d.Mt * d.Nt * kF64BM * kF64BN * sizeof(double) : 0;
   return align_up(packs + partials, 1024);
 }
-inline size_t f64_workspace(const F64Dims& d) {
-  const size_t least = f64_workspace_least(d);
-  const size_t slots = d.ranges == 1 ? 0 : (size_t)(f64_workers(d) + 1) * kF64WorkerBytes;
-  return slots > least ? slots : least;
+inline size_t f64_workspace_least(const F64Dims& d) {
+  const size_t slots = f64_workspace(d), kept = f64_workspace_kept(d);
+  return slots < kept ? slots : kept;
+}
+inline size_t f64_workspace_told(const F64Dims& d) {
+  const size_t slots = f64_workspace(d), kept = f64_workspace_kept(d);
+  return slots > kept ? slots : kept;
 }
 
 // C = A.B with ws_bytes of workspace (fewer slots: fewer workers).
