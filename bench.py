@@ -70,6 +70,11 @@ def load_peaks():
     return {"hbm_gbs": 6800.0, "bf16_tflops": 1900.0, "bf16_tflops_sustained": 1700.0}, "fallback"
 
 
+# what the profiled product kernel is compiled from
+PRODUCT_SOURCES = ("csrc/ozaki_kara.cu", "csrc/ozaki_fold.cuh", "csrc/ptx.cuh",
+                   "csrc/mxm_internal.h")
+
+
 def profiled_traffic():
     """DRAM bytes per launch of the product kernel from the committed ncu
     summary, if the kernel sources still hash as they did at capture."""
@@ -84,7 +89,7 @@ def profiled_traffic():
     if not mt or not mh:
         return None
     h = hashlib.sha256()
-    for rel in ("csrc/ozaki_kara.cu", "csrc/ptx.cuh", "csrc/mxm_internal.h"):
+    for rel in PRODUCT_SOURCES:
         with open(os.path.join(ROOT, "paper_1211_1581_gb300", rel), "rb") as fh:
             h.update(fh.read())
     return int(mt.group(1)) if h.hexdigest() == mh.group(1) else None
@@ -122,11 +127,13 @@ def sample_entries(n_rows, n_cols, count, seed):
     return np.array(ii, dtype=np.int64), np.array(jj, dtype=np.int64)
 
 
-def digit_products(S: int) -> int:
-    """Digit products the slice GEMM runs for S slices: S - 1 squares, one
-    difference product per pair s < t, s + t <= S + 1, and the pair (1, S) by
-    two products (fewer than three slices: all pairs one by one)."""
-    if S < 3 or S > 9:
+def digit_products(S: int, beta: int = 7) -> int:
+    """Digit products the slice GEMM runs for S slices of beta bits at the
+    benchmark's size: S - 1 squares, one difference product per pair s < t,
+    s + t <= S + 1, and the pair (1, S) by two products (fewer than three slices,
+    or more than 64 bits: all pairs one by one).  Truncated 8-bit digits of long
+    k run the same products over ranges of k."""
+    if S < 3 or S > 9 or beta * S > 64:
         return S * (S + 1) // 2
     return S - 1 + sum((g - 1) // 2 for g in range(3, S + 2)) + 1
 
@@ -347,7 +354,7 @@ def run_ours(args):
     ii, jj = sample_entries(n, n, 1024, seed=8192)
     C_sampled = C[torch.from_numpy(ii).cuda(), torch.from_numpy(jj).cuda()].cpu().numpy()
 
-    pairs = digit_products(S)
+    pairs = digit_products(S, beta)
     gemm_ms = phase_ms[2] / max(calls, 1)
     achieved = pairs * flops / (gemm_ms * 1e-3) / 1e12
     peak, peak_key, peak_why = choose_bf16_peak(peaks, clk)
@@ -399,9 +406,7 @@ def run_ours(args):
             ph, c_ = mxm.mxm_profile_read()
             mxm.mxm_profile_enable(False)
             t = a0.elapsed_time(a1) / steps
-            # truncated 8-bit digits of long k go one product at a time
-            p_ = (digit_products(s_) if mode == mxm.MODE_EMUL_RN8 or s_ * 255 ** 2 * n < 2 ** 31
-                  else s_ * (s_ + 1) // 2)
+            p_ = digit_products(s_, 8)
             gms = ph[2] / max(c_, 1)
             modes[name] = {"slices": s_, "digit_bits": 8,
                            "digits": "balanced, rounded to nearest" if mode == mxm.MODE_EMUL_RN8
@@ -506,7 +511,8 @@ def run_ours(args):
                            "parallelism": f"replicas x{world}"},
                 "roofline": roofline, "cpu_baseline": cpu, "e2e": e2e, "clocks": clk,
                 # per step: column maxima of B, the fused scale + split of A, the
-                # split of B, the product (and one memset of the column maxima)
+                # split of B, the product and its folds (and one memset of the
+                # column maxima)
                 "gpu_launches": launches_per_product(n) * args.steps, "modes": modes, "check": check,
                 "check_all_entries": check_all}
         print(json.dumps(line))
