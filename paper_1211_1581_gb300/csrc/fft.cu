@@ -43,7 +43,6 @@ int sm_count();
 
 namespace {
 
-constexpr int kFftThreads = 256;
 constexpr int64_t kFftMaxN = int64_t{1} << 22;
 constexpr int64_t kFftSingleMax = 1024;
 constexpr int64_t kFftClusterMin = 16, kFftClusterMax = 8192;
@@ -318,30 +317,10 @@ __global__ void fft_twiddle_kernel(double2* table, int64_t T) {
 
 bool pow2(int64_t v) { return v >= 1 && (v & (v - 1)) == 0; }
 
-// Columns per CTA (a power of two, at most 8, at most 96 KiB of shared memory):
-// the most for which the last wave of CTAs over the SMs is at least 0.9 full on
-// average over the waves, else the count with the fullest waves.
-int fft_column_bits(int bits, int64_t cols) {
-  int best = 0;
-  double best_fill = 0.0;
-  for (int cb = 3; cb >= 0; --cb) {
-    const int64_t C = int64_t{1} << cb, L = int64_t{1} << bits;
-    if (cols < C || (C * L + L) * 16 > 96 * 1024) continue;
-    const int64_t blocks = cols / C, sms = sm_count();
-    const double fill = static_cast<double>(blocks) / static_cast<double>((blocks + sms - 1) / sms * sms);
-    if (fill >= 0.9) return cb;
-    if (fill > best_fill) {
-      best_fill = fill;
-      best = cb;
-    }
-  }
-  return best;
-}
-
 cudaError_t launch_pass(FftPass a, cudaStream_t s) {
   const int bits = a.stage == 1 ? a.bits1 : a.bits2;
   const int64_t cols = int64_t{1} << (a.stage == 1 ? a.bits2 : a.bits1);
-  a.cbits = fft_column_bits(bits, cols);
+  a.cbits = fft_column_bits(bits, cols, sm_count());
   const size_t L = size_t{1} << bits;
   const size_t smem = ((L << a.cbits) + (3 * L + 3) / 4) * sizeof(double2);
   static PerDevice limit;

@@ -652,6 +652,35 @@ cudaError_t allow_smem(PerDevice& site, Kernel kern, size_t bytes) {
   });
 }
 
+// ---------------------------------------------------------------- FFT
+constexpr int kFftThreads = 256;
+
+// log2 of the columns per CTA of a pass over `cols` transforms of 2^bits points (a
+// power of two, at most 8, at most 96 KiB of shared memory): the most for which
+// the last wave of CTAs over the SMs is at least 0.9 full on average over the
+// waves, else the count with the fullest waves; of equally full ones the fewest
+// columns that leave every thread of a CTA a butterfly of four points.  Fewer
+// CTAs than SMs have too few warps to hide latency: 2^19 points with 128 CTAs of
+// four columns in the first pass 121 us, 512 of one 101; 2^18 with 128 of four in
+// both 59.1, 256 of two 57.0; but 2^17 with less than 1024 points a CTA 38.6
+// instead of 36.6.
+inline int fft_column_bits(int bits, int64_t cols, int64_t sms) {
+  int best = 0;
+  double best_fill = 0.0;
+  for (int cb = 3; cb >= 0; --cb) {
+    const int64_t C = int64_t{1} << cb, L = int64_t{1} << bits;
+    if (cols < C || (C * L + L) * 16 > 96 * 1024) continue;
+    const int64_t blocks = cols / C;
+    const double fill = static_cast<double>(blocks) / static_cast<double>((blocks + sms - 1) / sms * sms);
+    if (fill >= 0.9) return cb;
+    if (fill > best_fill || (fill == best_fill && C * L >= 4 * kFftThreads)) {
+      best_fill = fill;
+      best = cb;
+    }
+  }
+  return best;
+}
+
 // Comparison modes (not FP64-accurate).
 cudaError_t launch_bf16_gemm(const double* A, const double* B, double* C, const OzakiDims& d,
                              uint8_t* aplane, uint8_t* bplane, int* status, cudaStream_t s);
