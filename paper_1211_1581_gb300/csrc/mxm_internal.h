@@ -652,6 +652,15 @@ cudaError_t allow_smem(PerDevice& site, Kernel kern, size_t bytes) {
   });
 }
 
+// Whether the fold of a split-k product of m rows, `blocks` blocks of it, is
+// launched beside the slice GEMM.  The GEMM's CTAs leave no registers for a fold
+// block, so blocks launched early all settle on the first SMs that are free; with
+// few rows every lane of their loads is a sector of its own, and those SMs are
+// long at it.  S = 7, beside against after: 1 x 4096 x 4096 402 us against 281, 4
+// rows 299 against 275, 8 rows 282 against 274, 16 rows 277 against 276; 1 x 65536
+// x 1 (one block) 157 against 160.
+inline bool splitk_fold_chained(int64_t m, int64_t blocks) { return m >= 16 || blocks <= 8; }
+
 // ---------------------------------------------------------------- FFT
 constexpr int kFftThreads = 256;
 

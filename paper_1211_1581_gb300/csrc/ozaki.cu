@@ -2576,10 +2576,11 @@ cudaError_t launch_ozaki_gemm(const uint8_t* aslices, const uint8_t* bslices,
     if (e != cudaSuccess) return e;
     const int64_t total = d.m * d.n;
     auto fold = [&](auto kern, int64_t per_block) {
-      return launch_chained(d.chain, kern,
-                            dim3(static_cast<unsigned>((total + per_block - 1) / per_block)), 256,
-                            0, s, sums, rowbits, colbits, C, d.m, d.n, d.Mt, d.Nt, splits, d.S,
-                            d.beta, ozaki_exact_from(d.S, d.beta, d.Kt), d.rn ? 2 : 0);
+      const int64_t blocks = (total + per_block - 1) / per_block;
+      return launch_chained(d.chain && splitk_fold_chained(d.m, blocks), kern,
+                            dim3(static_cast<unsigned>(blocks)), 256, 0, s, sums, rowbits, colbits,
+                            C, d.m, d.n, d.Mt, d.Nt, splits, d.S, d.beta,
+                            ozaki_exact_from(d.S, d.beta, d.Kt), d.rn ? 2 : 0);
     };
     if (narrow)
       return splits >= 32 ? fold(oz_splitk_fold_kernel<8, int>, 32)
