@@ -50,12 +50,14 @@ __host__ __device__ inline bool share_too_long(int64_t values, int64_t nnz) {
   return values > 2 * (nnz / kCgBlocks) + kShareSlack;
 }
 
-// By work: the row pointer plus kRowWork a row (its own part of the three dot
-// products and vector updates of a step, five multiply-adds) grows from 0 to the
-// whole work; the share begins at the first row at or past s parts of it.  Row
-// pointers that are not in order give some other cut; the cuts still never
+// By work: the row pointer plus kRowWork a row grows from 0 to the whole work; the
+// share begins at the first row at or past s parts of it.  A row counts as one
+// value: a lane's strided loads and gathers cost far more than the row's part of
+// the dot products and vector updates (10^6 rows, the first tenth of 41 values,
+// the rest of 5: 112 us a step; counted as two 117, as five 133; by number 233).
+// Row pointers that are not in order give some other cut; the cuts still never
 // decrease with s (each step of the search goes right for every larger s).
-constexpr int64_t kRowWork = 5;
+constexpr int64_t kRowWork = 1;
 __host__ __device__ inline int64_t share_by_work(const int32_t* rowp, int64_t n, int64_t nnz,
                                                  int s) {
   if (s <= 0) return 0;
