@@ -29,7 +29,8 @@ constexpr int kStatusWorkspace = 4;
 constexpr int kStatusBounds = 8;
 constexpr int kStatusBreakdown = 16;
 
-// Every bounded wait inside a kernel gives up after this long.
+// Every bounded wait inside a kernel gives up after this long (the barriers of
+// cg_grid.cu, where the others may be at work on long rows, later: cg_rows.h).
 constexpr unsigned long long kWaitLimitNs = 2000000000ull;  // 2 s
 
 // Split-k for products with fewer C tiles than SMs: the k-blocks of every
@@ -359,7 +360,11 @@ constexpr int kKaraShortSlices = 7;
 // save (measured at 512 x 512 x 4096, S = 7: 154 us against 148); and with a
 // single tile-row or tile-column, where half of a 256 x 256 tile is empty,
 // only as long as the product is small enough to be bound by latency (155 x
-// 305 x 98, S = 7: 3x; 64 x 8192 x 8192, S = 6: 956 us against 906).
+// 305 x 98, S = 7: 3x; 64 x 8192 x 8192, S = 6: 956 us against 906).  Against the
+// one-by-one products as they are now, over 294 products that take the difference
+// products: 1.59 times as fast in the geometric mean, 21 of them slower, most
+// one tile-row beside many tile-columns with two k-blocks (128 x 200 x 16384, S =
+// 8: 154 us against 127).
 constexpr size_t kKaraMaxBytes = (size_t)32 << 30;
 // Little k: 256 x 128 tiles, where the epilogue sets the pace and there are
 // tiles for most CTA pairs.  Measured against 256 x 256 tiles (S = 7): up to

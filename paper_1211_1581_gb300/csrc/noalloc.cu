@@ -14,8 +14,8 @@
 // The array lives in every GPU that loads the library, until the process
 // exits.  Every call shares it, so calls that overlap on the GPU (different
 // streams, or several host threads) race; the array keeps the previous
-// call's contents, and the launch sequence clears what must start at zero
-// (the column maxima, reduced with atomicMax) before using it.
+// call's contents, and the launch sequence clears what must start at zero (the
+// column maxima where they are reduced with atomicMax) before using it.
 #include <cuda_runtime.h>
 
 #include <cstdint>
@@ -108,9 +108,10 @@ extern "C" mxm_status mxm_f64_emul_noalloc(const double* A, const double* B, dou
 
   uint64_t* rowbits = reinterpret_cast<uint64_t*>(ws + L.rowbits);
   uint64_t* colbits = reinterpret_cast<uint64_t*>(ws + L.colbits);
-  // launch_ozaki_scale zeroes the column maxima before reducing into them;
-  // the row maxima, every digit-plane byte (padding included), the running
-  // sums and the split-k partials are written before they are read.
+  // launch_ozaki_scale writes the column maxima (k <= 256) or zeroes them before
+  // reducing into them; the row maxima, every digit-plane byte (padding
+  // included), the running sums and the split-k partials are written before
+  // they are read.
   cudaError_t e = launch_ozaki_scale(A, B, d, rowbits, colbits, status, s);
   if (e == cudaSuccess)
     e = launch_ozaki_split(A, B, d, rowbits, colbits, ws + L.aslices, ws + L.bslices,
